@@ -82,13 +82,6 @@ struct BoxCount {
   uint32_t why = 0;    // fallback reason: 0 none, 1 square too wide (or too many runs), 2 too few hits, 3 tie
 };
 
-// unwrapped coarse-cell index of an unwrapped coordinate x, -L <= x < 2L
-__device__ __forceinline__ int box_ucell(int64_t x, int n, const uint32_t* __restrict__ bnd, float inv_w, int64_t L) {
-  if (x < 0) return cell_of_tab((uint32_t)(x + L), n, bnd, inv_w) - n;
-  if (x >= L) return cell_of_tab((uint32_t)(x - L), n, bnd, inv_w) + n;
-  return cell_of_tab((uint32_t)x, n, bnd, inv_w);
-}
-
 // exact minimum-image offset and squared distance of pj from the particle
 __device__ __forceinline__ uint64_t box_offset(const Ctx& C, int2 pj, int32_t& dx, int32_t& dy) {
   dx = (int32_t)((uint32_t)pj.x - C.px);
@@ -120,18 +113,20 @@ __device__ __forceinline__ uint64_t box_dist2(const Ctx& C, int2 pj) {
 constexpr int kGroup = 4;
 
 template <class HB, class V>
-__device__ __forceinline__ bool box_walk(HB& H, const Rep& R, const uint32_t* __restrict__ bounds,
-                                         const GridView& G, const int2* __restrict__ pos, const Ctx& C, int64_t a,
-                                         BoxCount& bc, V& v) {
+__device__ __forceinline__ bool box_walk(HB& H, const Rep& R, const GridView& G, const int2* __restrict__ pos,
+                                         const Ctx& C, int64_t a, BoxCount& bc, V& v) {
   const int64_t Lx = C.Lx, Ly = C.Ly;
   if (2 * (2 * a + 1) >= Lx || 2 * (2 * a + 1) >= Ly) return false;
   const int nx = R.nc[0], ny = R.nc[1];
-  const uint32_t* bx = bounds + R.bnd[0];
-  const uint32_t* by = bounds + R.bnd[1];
   const int64_t qx0 = (int64_t)C.px - a, qx1 = (int64_t)C.px + a;
   const int64_t qy0 = (int64_t)C.py - a, qy1 = (int64_t)C.py + a;
-  const int ucx0 = box_ucell(qx0, nx, bx, R.inv_w[0], Lx), ucx1 = box_ucell(qx1, nx, bx, R.inv_w[0], Lx);
-  const int ucy0 = box_ucell(qy0, ny, by, R.inv_w[1], Ly), ucy1 = box_ucell(qy1, ny, by, R.inv_w[1], Ly);
+  const int ucx0 = ucell2(qx0, nx, R.sh[0], Lx), ucx1 = ucell2(qx1, nx, R.sh[0], Lx);
+  const int ucy0 = ucell2(qy0, ny, R.sh[1], Ly), ucy1 = ucell2(qy1, ny, R.sh[1], Ly);
+  // in-cell offsets of the square's corners in their own cells
+  const uint32_t fx0 = cell_frac((uint32_t)(qx0 < 0 ? qx0 + Lx : qx0), R.sh[0]);
+  const uint32_t fx1 = cell_frac((uint32_t)(qx1 >= Lx ? qx1 - Lx : qx1), R.sh[0]);
+  const uint32_t fy0 = cell_frac((uint32_t)(qy0 < 0 ? qy0 + Ly : qy0), R.sh[1]);
+  const uint32_t fy1 = cell_frac((uint32_t)(qy1 >= Ly ? qy1 - Ly : qy1), R.sh[1]);
   if (ucx1 - ucx0 + 1 > nx || ucy1 - ucy0 + 1 > ny) return false;
   bc.tries += 1;
   // enumeration cursor over (coarse cell, row of sub-cells): runs are listed
@@ -165,15 +160,11 @@ __device__ __forceinline__ bool box_walk(HB& H, const Rep& R, const uint32_t* __
         row = 0;
         row_end = 0;
         if (split) {
-          const int64_t y0c = cell_lo_tab(ucy, ny, by, Ly);
-          const int64_t wy = cell_lo_tab(ucy + 1, ny, by, Ly) - y0c;
-          const int64_t x0c = cell_lo_tab(ucx, nx, bx, Lx);
-          const int64_t wx = cell_lo_tab(ucx + 1, nx, bx, Lx) - x0c;
           s = __ldg(G.sub_s + gc);
-          sx0 = sub_idx(max(qx0 - x0c, (int64_t)0), wx, s);
-          sx1 = sub_idx(min(qx1 - x0c, wx - 1), wx, s);
-          row = sub_idx(max(qy0 - y0c, (int64_t)0), wy, s);
-          row_end = sub_idx(min(qy1 - y0c, wy - 1), wy, s);
+          sx0 = ucx == ucx0 ? sub_of(fx0, s) : 0;
+          sx1 = ucx == ucx1 ? sub_of(fx1, s) : s - 1;
+          row = ucy == ucy0 ? sub_of(fy0, s) : 0;
+          row_end = ucy == ucy1 ? sub_of(fy1, s) : s - 1;
         }
         ++ucx;
       }

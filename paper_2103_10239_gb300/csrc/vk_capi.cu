@@ -160,8 +160,9 @@ float default_occupancy(const vk_params& p, int dim, int64_t n_total, int n_rep)
   return dim == 2 ? 256.0f : 1.5f;
 }
 
-// per-replica search grid for a target occupancy; fills nc, c0 and the cell
-// boundary tables (bnd[b] = ceil(b * L / nc), the first coordinate of cell b)
+// per-replica search grid for a target occupancy; fills nc and c0, and sh
+// (2D) or the cell boundary tables (3D: bnd[b] = ceil(b * L / nc), the first
+// coordinate of cell b)
 void plan_cells(vk_sim* s, float occ) {
   int64_t c0 = 0;
   s->bounds_h.clear();
@@ -170,23 +171,20 @@ void plan_cells(vk_sim* s, float occ) {
     double vol = 1.0;
     for (int a = 0; a < s->dim; ++a) vol *= (double)R.L[a];
     const double side = std::pow((double)occ * vol / (double)std::max<int64_t>(1, R.n), 1.0 / s->dim);
-    int64_t cells = 1;
-    for (int a = 0; a < 3; ++a) {
-      if (a >= s->dim) {
-        R.nc[a] = 1;
-        continue;
+    if (s->dim == 2) {
+      plan_grid2(R, side);
+    } else {
+      for (int a = 0; a < 3; ++a) {
+        double ncd = std::floor((double)R.L[a] / side);
+        ncd = std::max(1.0, std::min(ncd, std::min((double)R.L[a], 65536.0)));
+        R.nc[a] = (int32_t)ncd;
+        R.bnd[a] = (int32_t)s->bounds_h.size();
+        R.inv_w[a] = (float)R.nc[a] / (float)R.L[a];
+        for (int64_t b = 0; b <= R.nc[a]; ++b)
+          s->bounds_h.push_back((uint32_t)((b * (int64_t)R.L[a] + R.nc[a] - 1) / R.nc[a]));
       }
-      double ncd = std::floor((double)R.L[a] / side);
-      ncd = std::max(1.0, std::min(ncd, std::min((double)R.L[a], 65536.0)));
-      R.nc[a] = (int32_t)ncd;
-      cells *= R.nc[a];
     }
-    for (int a = 0; a < 3; ++a) {
-      R.bnd[a] = (int32_t)s->bounds_h.size();
-      R.inv_w[a] = (float)R.nc[a] / (float)R.L[a];
-      for (int64_t b = 0; b <= R.nc[a]; ++b)
-        s->bounds_h.push_back((uint32_t)((b * (int64_t)R.L[a] + R.nc[a] - 1) / R.nc[a]));
-    }
+    const int64_t cells = (int64_t)R.nc[0] * R.nc[1] * R.nc[2];
     R.c0 = c0;
     c0 += cells;
   }
@@ -300,11 +298,11 @@ vk_status clear_phi(vk_sim* s) {
 }
 
 // kernels of the search+update phase: for 2D kNN the radius-first kernel,
-// the deferred-particle kernel and the walk-list kernel (one kernel with the
-// walk only); one for 3D kNN and for the metric rule; the Voronoi kernel and
+// the kernel of the particles it hands on and that of the few that need the
+// whole box; one for 3D kNN and for the metric rule; the Voronoi kernel and
 // its overflow kernel
 int search_launches(const vk_sim* s) {
-  if (s->prm.rule == VK_RULE_KNN) return (s->dim == 2 && s->prm.knn_search == 0) ? 3 : 1;
+  if (s->prm.rule == VK_RULE_KNN) return s->dim == 2 ? 3 : 1;
   if (s->prm.rule == VK_RULE_METRIC) return 1;
   return 2;
 }
@@ -319,7 +317,7 @@ vk_status enqueue_step(vk_sim* s) {
   else if (s->prm.rule == VK_RULE_METRIC) VK_CUDA(s, launch_metric_step(s->g, s->b, P, s->stream));
   else if (s->dim == 2) VK_CUDA(s, launch_voronoi_step(s->g, s->b, P, s->stream));
   else VK_CUDA(s, launch_voronoi3_step(s->g, s->b, P, s->prm.voronoi3_kernel, s->stream));
-  const int deferred_launches = (s->prm.rule == VK_RULE_KNN && s->dim == 2 && s->prm.knn_search == 0) ? 2 : 0;
+  const int deferred_launches = (s->prm.rule == VK_RULE_KNN && s->dim == 2) ? 2 : 0;
   if ((st = record_end(s, 0, e0, search_launches(s) - deferred_launches))) return st;
   if (deferred_launches) {
     if ((st = record_begin(s, 5, &e0))) return st;
@@ -475,7 +473,7 @@ vk_status build_sim(int32_t n_rep, const int64_t* n_r, const int32_t* pos_q, con
   const size_t fv = dim == 2 ? sizeof(float2) : sizeof(float4);
   cudaError_t e = cudaSuccess;
   const size_t N = (size_t)total;
-  if ((e = cudaMalloc(&s->b.S_pos, pv * N)) || (e = cudaMalloc(&s->b.S_dir, fv * N)) ||
+  if ((e = cudaMalloc(&s->b.S_pos, pv * (N + kPosPad))) || (e = cudaMalloc(&s->b.S_dir, fv * N)) ||
       (e = dalloc(&s->b.S_id, N)) || (e = cudaMalloc(&s->b.U_pos, pv * N)) || (e = cudaMalloc(&s->b.U_dir, fv * N)) ||
       (e = dalloc(&s->b.U_id, N)) || (e = dalloc(&s->b.U_rank, N)) ||
       (e = dalloc(&s->b.phi_acc, 3 * (size_t)s->phi_cap * n_rep)) || (e = dalloc(&s->b.d_step, 1)) ||
@@ -608,8 +606,7 @@ vk_status vk_get_neighbors(vk_sim* s, int32_t replica, int64_t* offsets, int32_t
     const int k = s->prm.k;
     int32_t* out_d = nullptr;
     VK_CUDA(s, dalloc(&out_d, (size_t)n * k));
-    cudaError_t e = s->dim == 2 ? launch_knn2_export(s->g, s->b, k, replica, (int)n, out_d, s->stream,
-                                                     step_params(s))
+    cudaError_t e = s->dim == 2 ? launch_knn2_export(s->g, s->b, replica, (int)n, out_d, s->stream, step_params(s))
                                 : launch_knn_export(s->g, s->b, k, replica, (int)n, out_d, s->stream);
     if (e == cudaSuccess) {
       ids_h.resize((size_t)n * k);

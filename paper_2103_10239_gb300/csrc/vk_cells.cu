@@ -65,12 +65,14 @@ __global__ void __launch_bounds__(kBlock) count_kernel(const Rep* __restrict__ r
   const int64_t s = R.p0 + li;
   int32_t p[3];
   unpack(U_pos[s], p);
-  int c[3] = {0, 0, 0};
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) c[a] = cell_of_tab((uint32_t)p[a], R.nc[a], bounds + R.bnd[a], R.inv_w[a]);
   int64_t lin = 0;
+  if (DIM == 2) {
+    lin = linear_cell<2>(R, p) - R.c0;
+  } else {
 #pragma unroll
-  for (int a = DIM - 1; a >= 0; --a) lin = lin * R.nc[a] + c[a];
+    for (int a = DIM - 1; a >= 0; --a)
+      lin = lin * R.nc[a] + cell_of_tab((uint32_t)p[a], R.nc[a], bounds + R.bnd[a], R.inv_w[a]);
+  }
   atomicAdd(counts + R.c0 + lin, 1u);
 }
 
@@ -90,7 +92,7 @@ __global__ void __launch_bounds__(kBlock) sub_count_kernel(const Rep* __restrict
   int32_t p[3];
   unpack(U_pos[s], p);
   int64_t gc, g;
-  locate_tab<DIM>(R, G, bounds, p, &gc, &g);
+  locate<DIM>(R, G, bounds, p, &gc, &g);
   U_rank[s] = atomicAdd(sub_count + g, 1u);
 }
 
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(kBlock) scatter_kernel(const Rep* __restrict__
   int32_t p[3];
   unpack(pv, p);
   int64_t gc, g;
-  locate_tab<DIM>(R, G, bounds, p, &gc, &g);
+  locate<DIM>(R, G, bounds, p, &gc, &g);
   const uint32_t dst = G.sub_off[g] + U_rank[s];
   S_pos[dst] = pv;
   S_dir[dst] = U_dir[s];

@@ -11,8 +11,10 @@
 //   * a per-replica table (Rep) and a per-block task table (BlockTask), so a
 //     256-thread block never straddles two replicas.
 #pragma once
-#include <cstdint>
+#include <algorithm>
 #include <climits>
+#include <cmath>
+#include <cstdint>
 #include <cuda_runtime.h>
 
 namespace vk {
@@ -40,6 +42,7 @@ struct Rep {
   uint32_t replica;
   int32_t bnd[3];  // offset of the axis' cell-boundary table in the bounds array
   float inv_w[3];  // nc / L (estimate of the cell index; corrected exactly)
+  int32_t sh[2];   // 2D: coarse cells are 2^sh grid units wide (1..31; the last one ends at L)
   uint32_t r0q;    // metric rule: interaction radius in grid units, rint(r0 * 2^F)
 };
 
@@ -59,8 +62,8 @@ struct StepParams {
   uint32_t seed_lo, seed_hi;
   int32_t n_rep;
   int32_t phi_cap;
-  // 2D kNN search: 0 = radius first (per-particle walk as the last resort),
-  // 1 = per-particle walk only
+  // kNN search: 0 = radius first, one thread per particle; 1 = the general
+  // search only (2D: groups of lanes and larger squares; 3D: the ring walk)
   int32_t knn_search;
   // radius-first search square: halo_alpha * (the particle's k-th distance at
   // the previous step) + halo_beta * (grid step per unit heading)
@@ -196,9 +199,31 @@ __device__ __forceinline__ int64_t cell_lo_tab(int b, int n, const uint32_t* __r
   return (int64_t)__ldg(bnd + b);
 }
 
+// 2D grid: coarse cells are 2^sh grid units wide, so that the coarse cell of a
+// coordinate is a shift and its sub-cell the high word of one product; the
+// table and division forms cost 10 to 100 instructions per lookup, and the
+// search does several per particle.  The last cell of an axis ends at L; its
+// sub-cells are laid out as if it were whole.
+__device__ __forceinline__ uint32_t cell_frac(uint32_t p, int sh) { return p << (32 - sh); }
+// floor(u * s / 2^sh) of the in-cell offset u, frac = cell_frac(p, sh)
+__device__ __forceinline__ int sub_of(uint32_t frac, int s) { return (int)__umulhi(frac, (uint32_t)s); }
+// first (unwrapped) coordinate of unwrapped cell b, -n <= b < 2n
+__device__ __forceinline__ int64_t cell_lo2(int b, int n, int sh, int64_t L) {
+  if (b < 0) return ((int64_t)(b + n) << sh) - L;
+  if (b >= n) return ((int64_t)(b - n) << sh) + L;
+  return (int64_t)b << sh;
+}
+// unwrapped cell of an unwrapped coordinate, -L <= x < 2L
+__device__ __forceinline__ int ucell2(int64_t x, int n, int sh, int64_t L) {
+  if (x < 0) return (int)((uint32_t)(x + L) >> sh) - n;
+  if (x >= L) return (int)((uint32_t)(x - L) >> sh) + n;
+  return (int)((uint32_t)x >> sh);
+}
+
 // global cell index of a position in replica R (x fastest)
 template <int DIM>
 __device__ __forceinline__ int64_t linear_cell(const Rep& R, const int32_t* p) {
+  if (DIM == 2) return R.c0 + (int64_t)((uint32_t)p[1] >> R.sh[1]) * R.nc[0] + ((uint32_t)p[0] >> R.sh[0]);
   int64_t c = 0;
 #pragma unroll
   for (int a = DIM - 1; a >= 0; --a) c = c * R.nc[a] + cell_of(p[a], R.nc[a], R.L[a]);
@@ -211,8 +236,11 @@ __device__ __forceinline__ int wrap_index(int x, int n) {
 }
 
 __device__ __forceinline__ int32_t wrap_add(int32_t p, int32_t d, uint32_t L) {
-  int64_t q = ((int64_t)p + (int64_t)d) % (int64_t)L;
-  if (q < 0) q += (int64_t)L;
+  int64_t q = (int64_t)p + (int64_t)d;
+  if (q < 0 || q >= (int64_t)L) {  // rare: the 64-bit remainder is a long call
+    q %= (int64_t)L;
+    if (q < 0) q += (int64_t)L;
+  }
   return (int32_t)q;
 }
 
@@ -245,67 +273,24 @@ struct GridView {
   const uint32_t* __restrict__ sub_off;   // sub-cell -> first slot
 };
 
-// sub-cell (sx, sy) of a point at in-cell offset u in a cell of width w
-__device__ __forceinline__ int sub_index(int64_t u, int64_t w, int s) {
-  return (int)((u * s) / w);
-}
-
-// global sub-cell index of a position (2D), given its coarse cell
+// Coarse cell and sub-cell (global indices) of a position: shifts in 2D,
+// the per-replica boundary tables in 3D (whose cells are never split).
 template <int DIM>
-__device__ __forceinline__ int64_t sub_cell_of(const Rep& R, const GridView& G, const int32_t* p, int64_t gcell) {
-  const int s = G.sub_s[gcell];
-  int64_t j = 0;
-  if (DIM == 2 && s > 1) {
-    const int cx = cell_of(p[0], R.nc[0], R.L[0]), cy = cell_of(p[1], R.nc[1], R.L[1]);
-    const int64_t x0 = cell_lo(cx, R.nc[0], R.L[0]), y0 = cell_lo(cy, R.nc[1], R.L[1]);
-    const int64_t wx = cell_lo(cx + 1, R.nc[0], R.L[0]) - x0, wy = cell_lo(cy + 1, R.nc[1], R.L[1]) - y0;
-    j = (int64_t)sub_index(p[1] - y0, wy, s) * s + sub_index(p[0] - x0, wx, s);
-  }
-  return (int64_t)G.sub_base[gcell] + j;
-}
-
-// sub-cell index of offset u (0 <= u < w) in a cell of width w split s ways:
-// floor(u*s/w), from a float estimate corrected with exact products
-__device__ __forceinline__ int sub_idx(int64_t u, int64_t w, int s) {
-  int j = min(max((int)((float)u * ((float)s / (float)w)), 0), s - 1);
-  const int64_t us = u * s;
-  while (j > 0 && us < (int64_t)j * w) --j;
-  while (j < s - 1 && us >= (int64_t)(j + 1) * w) ++j;
-  return j;
-}
-
-// Coarse cell and sub-cell (global indices) of a position, from the
-// per-replica boundary tables (no 64-bit division); the same cells as
-// linear_cell / sub_cell_of.
-template <int DIM>
-__device__ __forceinline__ void locate_tab(const Rep& R, const GridView& G, const uint32_t* __restrict__ bounds,
-                                           const int32_t* p, int64_t* gcell, int64_t* gsub) {
-  int c[3] = {0, 0, 0};
+__device__ __forceinline__ void locate(const Rep& R, const GridView& G, const uint32_t* __restrict__ bounds,
+                                       const int32_t* p, int64_t* gcell, int64_t* gsub) {
+  if (DIM == 2) {
+    *gcell = linear_cell<2>(R, p);
+    const int s = G.sub_s[*gcell];
+    *gsub = (int64_t)G.sub_base[*gcell] + sub_of(cell_frac((uint32_t)p[1], R.sh[1]), s) * s +
+            sub_of(cell_frac((uint32_t)p[0], R.sh[0]), s);
+  } else {
+    int64_t lin = 0;
 #pragma unroll
-  for (int a = 0; a < DIM; ++a) c[a] = cell_of_tab((uint32_t)p[a], R.nc[a], bounds + R.bnd[a], R.inv_w[a]);
-  int64_t lin = 0;
-#pragma unroll
-  for (int a = DIM - 1; a >= 0; --a) lin = lin * R.nc[a] + c[a];
-  *gcell = R.c0 + lin;
-  const int s = G.sub_s[*gcell];
-  int64_t j = 0;
-  if (DIM == 2 && s > 1) {
-    const uint32_t* bx = bounds + R.bnd[0];
-    const uint32_t* by = bounds + R.bnd[1];
-    const int64_t x0 = __ldg(bx + c[0]), wx = (int64_t)__ldg(bx + c[0] + 1) - x0;
-    const int64_t y0 = __ldg(by + c[1]), wy = (int64_t)__ldg(by + c[1] + 1) - y0;
-    j = (int64_t)sub_idx(p[1] - y0, wy, s) * s + sub_idx(p[0] - x0, wx, s);
+    for (int a = DIM - 1; a >= 0; --a)
+      lin = lin * R.nc[a] + cell_of_tab((uint32_t)p[a], R.nc[a], bounds + R.bnd[a], R.inv_w[a]);
+    *gcell = R.c0 + lin;
+    *gsub = (int64_t)G.sub_base[*gcell];
   }
-  *gsub = (int64_t)G.sub_base[*gcell] + j;
-}
-
-// upper bound (integer) of the square root of r2; r2 may be ~0ull (infinite)
-__device__ __forceinline__ int64_t radius_upper(uint64_t r2) {
-  if (r2 >= (1ull << 62)) return INT64_MAX / 4;
-  const float f = sqrtf((float)r2) * 1.0000005f;
-  int64_t r = (int64_t)f + 1;
-  while ((uint64_t)r * (uint64_t)r < r2) ++r;
-  return r;
 }
 
 // Walk the 3D grid around the particle at pi (3D coarse cells are never
@@ -608,6 +593,31 @@ __device__ __forceinline__ void set_status(int32_t* status, int32_t code) {
 // host-side launchers (defined in the .cu files)
 namespace vk {
 
+// 2D grid of a replica: cells of about `side` grid units, rounded to a power
+// of two (the cell count varies by a factor of two either way around the
+// target; the search time is flat over that range) and at most 65536 per
+// axis.  Boxes of only a few cells get at least four per axis, so that a
+// search square seldom meets a cell through two periodic images; not where
+// that would multiply the cells of a box much longer than wide.
+inline void plan_grid2(Rep& R, double side) {
+  auto cells = [](uint32_t L, int sh) { return (int64_t)(((uint64_t)L + (1ull << sh) - 1) >> sh); };
+  int wide[2], fine[2];
+  for (int a = 0; a < 2; ++a) {
+    int sh = std::max(1, std::min(31, (int)std::lround(std::log2(std::max(side, 1.0)))));
+    while (sh < 31 && cells(R.L[a], sh) > 65536) ++sh;
+    while (sh > 1 && (1ull << (sh - 1)) >= R.L[a]) --sh;
+    wide[a] = fine[a] = sh;
+    while (fine[a] > 1 && (4ull << fine[a]) > R.L[a]) --fine[a];
+  }
+  const bool few = cells(R.L[0], fine[0]) * cells(R.L[1], fine[1]) <= std::max<int64_t>(64, R.n / 8);
+  for (int a = 0; a < 2; ++a) {
+    R.sh[a] = few ? fine[a] : wide[a];
+    R.nc[a] = (int32_t)cells(R.L[a], R.sh[a]);
+    R.inv_w[a] = 0.f;
+  }
+  R.nc[2] = 1;
+}
+
 // streaming multiprocessors of the current device (for fixed-size grids)
 inline int device_sm_count() {
   int dev = 0, sms = 0;
@@ -616,6 +626,10 @@ inline int device_sm_count() {
     return 1;
   return sms;
 }
+
+// the 2D search reads sorted positions in aligned groups of four: the array
+// ends in this many unused slots
+constexpr int64_t kPosPad = 4;
 
 struct Buffers {
   // sorted current state
@@ -640,7 +654,7 @@ struct Buffers {
   int64_t* d_step;
   int32_t* d_status;
   int2* ovf_list;      // 2 N entries of (slot, replica): Voronoi cells too large for the main kernel;
-                       // 2D kNN: deferred particles (first half) and particles for the walk (second)
+                       // 2D kNN: deferred particles (first half) and those that need the whole box (second)
   int32_t* ovf_count;  // 2 counters for those lists, cleared by the scatter of every step
   // 2D kNN: each particle's k-th neighbor distance (grid units) found at the
   // previous step, in S order, and the one found now in U order (0 = unknown);
@@ -695,13 +709,13 @@ cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int k, int re
                               cudaStream_t st);
 
 // vk_knn2d.cu (the 2D kNN hot path)
-// search + update of every particle (radius first: those it can serve; the
+// search + update of every particle (those one square each can serve; the
 // rest is listed) ...
 cudaError_t launch_knn2_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
-// ... and of the listed particles (deferred squares, then the walk); no-op for the walk-only search
+// ... and of the listed particles (larger squares, then the whole box)
 cudaError_t launch_knn2_finish(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
-cudaError_t launch_knn2_export(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out,
-                               cudaStream_t st, const StepParams& P);
+cudaError_t launch_knn2_export(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out, cudaStream_t st,
+                               const StepParams& P);
 // one-time kernel attributes (shared memory of the radius-first search)
 cudaError_t prepare_knn2();
 

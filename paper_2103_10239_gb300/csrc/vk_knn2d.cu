@@ -1,501 +1,418 @@
 // vk_knn2d.cu -- the 2D k-nearest-neighbor rule fused with the Vicsek update
 // (Sec. "Metric and topological flocking models": each particle aligns with
-// its k nearest neighbors at any distance; Eq. 1 and Eq. 2).  This is the
-// benchmark's hot kernel, written for issue efficiency:
-//   * cell indices and cell boundaries come from per-replica tables (no
-//     64-bit division on the search path);
-//   * a row segment of coarse cells without sub-grids is one run of the
-//     sorted arrays (detected from the sub-cell bases, no per-cell branch);
-//   * minimum-image differences in int32, exact int64 squared distances, a
-//     register top-k ordered by (D, id);
-//   * the block's order-parameter partials are combined by the last warp to
-//     finish (no barrier that would hold finished warps).
-// The search is the two-level walk documented in vk_internal.cuh.
+// its k nearest neighbors at any distance; Eq. 1 and Eq. 2).
+//
+// Radius first: each particle knows roughly how far its k-th neighbor is (its
+// k-th distance at the last step, kept as a hint in the state), so it scans,
+// once, the square [p - a, p + a] with a a little above that distance: the
+// sub-cell rows of the one to four coarse cells that the square meets, each a
+// contiguous run of the sorted arrays.  Nothing outside the square is closer
+// than a + 1, so k hits within it are the k nearest.
+//
+//   * knn2_box_step_kernel: one thread per particle, one square each.  The
+//     kernel is bound by instruction issue (a few cache lines of data per
+//     particle, DRAM below 2 % of its rate), so the whole selection runs on
+//     32-bit keys: the FP32 squared distance with its low bits replaced by
+//     the hit's number, inserted into a register list by min / max (two
+//     instructions an entry).  A key orders two candidates with certainty
+//     when the keys differ by two steps or more (2^-18 relative); a list with
+//     a closer pair (about one particle in 5000) or with fewer than k hits is
+//     handed on.
+//   * knn2_second_kernel: long lists of handed-on particles get larger squares
+//     by the same one-thread search.
+//   * knn2_group_kernel: short lists, and what is left: 16 lanes per particle
+//     scan the rows of larger squares together and rank the hits exactly, by
+//     (int64 squared distance, id).
+//
+// Measured (GB300, us per step, 64-bit list / 32-bit keys and power-of-two
+// cells): 4M clustered, k = 7: first square 2372 / 1175, listed particles
+// 1232 / 594; 50,021 uniform, k = 16, vectorial noise: 178 / 35, 183 / 36;
+// 2048 uniform: 45 / 26, 48 / 26.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "vk_box2d.cuh"
-
-// resident 256-thread blocks per SM the step kernels are compiled for
-// (register budget): the per-particle walk, and the radius-first search
-#ifndef VK_KNN2_MIN_BLOCKS
-#define VK_KNN2_MIN_BLOCKS 4
-#endif
-#ifndef VK_KNN2_BOX_BLOCKS
-#define VK_KNN2_BOX_BLOCKS 3
-#endif
-// ... and the deferred-particle kernel (a few larger squares per particle)
-#ifndef VK_KNN2_DEFER_BLOCKS
-#define VK_KNN2_DEFER_BLOCKS 2
-#endif
 
 namespace vk {
 
 namespace {
 
-// Top-k in registers: exact squared distances and sorted slots, ordered by
-// (D, id).  For k < KC the first KC-k entries are sentinels (D = 0, slot -1)
-// that order before every real candidate, so the threshold is always entry
-// KC-1 and no register array is indexed dynamically.  Ids are only read to
-// break an exact distance tie.
+constexpr int kBlk = 128;  // threads per block of the step kernel (a block task is split)
+constexpr int kSplit = kBlock / kBlk;
+
+// KC keys per thread: room for k <= KC - 1 neighbors and the one after them.
+// CAP hits buffered per thread (about 1.3 k + 1 are expected), numbered in
+// BITS bits.
+template <int KC> struct BoxCfg;
+template <> struct BoxCfg<8> { static constexpr int CAP = 24, BITS = 5, BLOCKS = 6; };
+template <> struct BoxCfg<12> { static constexpr int CAP = 32, BITS = 5, BLOCKS = 5; };
+template <> struct BoxCfg<17> { static constexpr int CAP = 48, BITS = 6, BLOCKS = 3; };
+template <> struct BoxCfg<33> { static constexpr int CAP = 64, BITS = 6, BLOCKS = 2; };
+constexpr int kRuns = 8;  // slot runs listed before they are scanned
+
 template <int KC>
-struct Top {
-  uint64_t d[KC];
-  int32_t slot[KC];
+struct BoxShared {
+  uint2 hit[BoxCfg<KC>::CAP][kBlk];  // (slot, bits of the FP32 squared distance), one column per thread
+  uint2 run[kRuns][kBlk];            // (first slot, length << 4 | image shift codes)
 };
 
+// the slot behind a key of the list
 template <int KC>
-__device__ __forceinline__ void top_init(Top<KC>& T, int k) {
+__device__ __forceinline__ int32_t key_slot(const BoxShared<KC>& H, uint32_t key) {
+  return (int32_t)H.hit[key & ((1u << BoxCfg<KC>::BITS) - 1u)][threadIdx.x].x;
+}
+
+// The k nearest of the particle at slot `self` from the square of half-width
+// a = ceil(r), as keys t[KC-1-k .. KC-2] in order (the first entries are
+// sentinels, so that no register array is indexed dynamically); false when
+// the square cannot decide, with the radius to try next.
+//
+// Every slot of the square with FP32 squared distance <= tau goes to the
+// thread's hit column, and the column is merged into t after the scan, where
+// the warp's threads have met again (and whenever the column is full: the KC
+// best then stay, and tau shrinks to the k-th).  With a field of view of at
+// most a half-plane, candidates behind the particle are dropped in the scan
+// (exactly); the rest of the view test is the merge's.
+template <int KC, bool FOV>
+__device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const GridView& G,
+                                           const int2* __restrict__ pos, int32_t self, int2 p, const View& vw,
+                                           float radius, int k, uint32_t* t, float* r_next, BoxCount& bc) {
+  constexpr int B = BoxCfg<KC>::BITS, CAP = BoxCfg<KC>::CAP;
+  const int32_t a = (int32_t)ceilf(fminf(radius, 1.0e9f));
+  *r_next = (float)a;
+  const uint32_t Lx = R.L[0], Ly = R.L[1];
+  bc.why = 1u;  // too wide for the minimum image, or a coarse cell met through two periodic images
+  if (4ll * a + 2 >= (int64_t)Lx || 4ll * a + 2 >= (int64_t)Ly) return false;
+  const int nx = R.nc[0], ny = R.nc[1], shx = R.sh[0], shy = R.sh[1];
+  const int tid = (int)threadIdx.x;
+  // corners wrapped into the box, their unwrapped coarse cells and in-cell fractions
+  const bool wx0 = p.x < a, wy0 = p.y < a;
+  const bool wx1 = (uint32_t)p.x + (uint32_t)a >= Lx, wy1 = (uint32_t)p.y + (uint32_t)a >= Ly;
+  const uint32_t x0 = (uint32_t)p.x - (uint32_t)a + (wx0 ? Lx : 0u), x1 = (uint32_t)p.x + (uint32_t)a - (wx1 ? Lx : 0u);
+  const uint32_t y0 = (uint32_t)p.y - (uint32_t)a + (wy0 ? Ly : 0u), y1 = (uint32_t)p.y + (uint32_t)a - (wy1 ? Ly : 0u);
+  const int ucx0 = (int)(x0 >> shx) - (wx0 ? nx : 0), ucx1 = (int)(x1 >> shx) + (wx1 ? nx : 0);
+  const int ucy0 = (int)(y0 >> shy) - (wy0 ? ny : 0), ucy1 = (int)(y1 >> shy) + (wy1 ? ny : 0);
+  if (ucx1 - ucx0 >= nx || ucy1 - ucy0 >= ny) return false;
+  const uint32_t fx0 = cell_frac(x0, shx), fx1 = cell_frac(x1, shx);
+  const uint32_t fy0 = cell_frac(y0, shy), fy1 = cell_frac(y1, shy);
+  bc.tries += 1;
+  // below (a + 1)^2 by more than the rounding of the distances
+  const float a1 = (float)a + 1.0f;
+  float tau = a1 * a1 * (1.0f - 9.5367431640625e-07f);
+  const uint32_t edge = __float_as_uint(tau) >> B;
 #pragma unroll
-  for (int s = 0; s < KC; ++s) {
-    T.d[s] = s < KC - k ? 0ull : ~0ull;
-    T.slot[s] = -1;
-  }
-}
-
-// insert candidate slot q at squared distance D, known to order before the
-// current last entry; an exact distance tie is decided by the ids (a real
-// candidate never orders before a sentinel)
-template <int KC>
-__device__ __forceinline__ void top_insert(Top<KC>& T, uint64_t D, int32_t q, const int32_t* __restrict__ ids) {
-  bool placed = false;
-#pragma unroll
-  for (int s = KC - 1; s > 0; --s) {
-    if (!placed) {
-      bool before = D < T.d[s - 1];
-      if (D == T.d[s - 1]) before = T.slot[s - 1] >= 0 && __ldg(ids + q) < __ldg(ids + T.slot[s - 1]);
-      if (before) {
-        T.d[s] = T.d[s - 1];
-        T.slot[s] = T.slot[s - 1];
-      } else {
-        T.d[s] = D;
-        T.slot[s] = q;
-        placed = true;
-      }
-    }
-  }
-  if (!placed) {
-    T.d[0] = D;
-    T.slot[0] = q;
-  }
-}
-
-template <int KC>
-__device__ __forceinline__ void scan_run(Ctx& C, const int2* __restrict__ pos, const int32_t* __restrict__ ids,
-                                         uint32_t qb, uint32_t qe, Top<KC>& T) {
-  C.n_cand += qe - qb;
-  C.n_runs += 1;
-  for (uint32_t q = qb; q < qe; ++q) {
-    const int2 pj = __ldg(pos + q);
-    int32_t dx = (int32_t)((uint32_t)pj.x - C.px);
-    int32_t dy = (int32_t)((uint32_t)pj.y - C.py);
-    if (dx > C.hix) dx = (int32_t)((uint32_t)dx - C.Lx);
-    else if (dx <= C.lox) dx = (int32_t)((uint32_t)dx + C.Lx);
-    if (dy > C.hiy) dy = (int32_t)((uint32_t)dy - C.Ly);
-    else if (dy <= C.loy) dy = (int32_t)((uint32_t)dy + C.Ly);
-    const uint64_t D = (uint64_t)((int64_t)dx * dx) + (uint64_t)((int64_t)dy * dy);
-    if (D <= T.d[KC - 1] && (int64_t)q != C.self && in_view(C.view, dx, dy, D)) {
-      // an exact tie with the current k-th best is decided by the ids
-      if (D < T.d[KC - 1] || (T.slot[KC - 1] >= 0 && __ldg(ids + q) < __ldg(ids + T.slot[KC - 1])))
-        top_insert<KC>(T, D, (int32_t)q, ids);
-    }
-  }
-}
-
-// first offset of sub-cell b: ceil(b*w/s)
-__device__ __forceinline__ int64_t sub_lo(int b, int64_t w, int s) {
-  const int64_t bw = (int64_t)b * w;
-  int64_t q = (int64_t)((float)bw / (float)s);
-  while (q * s < bw) ++q;
-  while (q > 0 && (q - 1) * s >= bw) --q;
-  return q;
-}
-
-// Resumable generator of the slot runs of the two-level walk, so that the
-// candidate loop exists once in the kernel (instruction-cache footprint).
-// Phase 1: rings of sub-cells in the own coarse cell (when it is split).
-// Phase 2: rings of coarse cells; a row segment without sub-grids is one run,
-// a split cell contributes the rows of its sub-cells that meet the box
-// [p - rad, p + rad], rad^2 >= the current k-th best distance.
-struct RunGen {
-  // fixed
-  const Rep* R;
-  const uint32_t* __restrict__ bx;
-  const uint32_t* __restrict__ by;
-  GridView G;
-  int64_t px, py;
-  int nx, ny, cx, cy;
-  int64_t own;
-  // phase 1 geometry
-  int s1, sx, sy;
-  uint32_t ob0;
-  int64_t cx0, wx1, cy0, wy1;
-  // cursor
-  int phase, r;
-  int bx0, bx1, by0, by1, px0, px1, py0, py1;  // phase 1 block (current and previous ring)
-  int yy, seg;                                  // phase 1 row / segment
-  int lox, hix, loy, hiy, plox, phix, ploy, phiy;
-  int oy;                                       // phase 2 row offset
-  int part, nparts;                             // phase 2 parts of the row
-  int pa[4], pb[4], pu[4];                      // part x0, x1, unwrapped x of x0
-  int64_t rowbase;
-  int ucy;
-  int x;                                        // current cell in a per-cell part (-1: part not started)
-  bool fast;
-  int sr, sr1, sx0r, sx1r;                      // rows of the current split-cell rectangle
-  uint32_t sbase;
-  int sstride;
-  bool in_rect;
-  bool own_done;
-  // the box [p - rad, p + rad] stays within every ring's representative cell
-  // offsets (so a cell meets it at its visited offset only) while rad < safe
-  int64_t safe;
-  int64_t prad;  // radius used to skip rows and cells of the current part (-1: none)
-  // split cells met while the search radius was still unknown, revisited at
-  // the end of the ring (when it usually is known)
-  int ndef;
-  int64_t def_g[4];
-  int def_ucx[4], def_ucy[4];
-};
-
-enum { kRun = 0, kRingEnd = 1, kDone = 2 };
-
-__device__ __forceinline__ void gen_row_parts(RunGen& g) {
-  // parts of row offset g.oy of ring g.r: up to 2 segments, each split by the wrap
-  g.nparts = 0;
-  const int ay = g.ucy < 0 ? g.ucy + g.ny : (g.ucy >= g.ny ? g.ucy - g.ny : g.ucy);
-  g.rowbase = g.R->c0 + (int64_t)ay * g.nx;
-  int sa[2], sb[2], ns = 0;
-  if (g.oy < g.ploy || g.oy > g.phiy) {
-    sa[0] = g.lox; sb[0] = g.hix; ns = 1;
-  } else {
-    if (g.lox <= g.plox - 1) { sa[ns] = g.lox; sb[ns] = g.plox - 1; ++ns; }
-    if (g.phix + 1 <= g.hix) { sa[ns] = g.phix + 1; sb[ns] = g.hix; ++ns; }
-  }
-  for (int q = 0; q < ns; ++q) {
-    const int ua = g.cx + sa[q];
-    const int start = ua < 0 ? ua + g.nx : (ua >= g.nx ? ua - g.nx : ua);
-    const int len = sb[q] - sa[q] + 1;
-    if (start + len <= g.nx) {
-      g.pa[g.nparts] = start; g.pb[g.nparts] = start + len - 1; g.pu[g.nparts] = ua; ++g.nparts;
-    } else {
-      g.pa[g.nparts] = start; g.pb[g.nparts] = g.nx - 1; g.pu[g.nparts] = ua; ++g.nparts;
-      g.pa[g.nparts] = 0; g.pb[g.nparts] = start + len - g.nx - 1; g.pu[g.nparts] = ua + (g.nx - start);
-      ++g.nparts;
-    }
-  }
-  g.part = 0;
-  g.x = -1;
-}
-
-// sub-cell rectangle of split cell gc (unwrapped indices ucx, ucy) meeting
-// the box [p - rad, p + rad]; false if it misses the cell
-__device__ __forceinline__ bool gen_rect(RunGen& g, int64_t gc, int ucx, int ucy, uint64_t r2) {
-  const GridView& G = g.G;
-  const Rep& R = *g.R;
-  const int s = __ldg(G.sub_s + gc);
-  g.sbase = __ldg(G.sub_base + gc);
-  g.sstride = s;
-  if (r2 == ~0ull) {
-    g.sx0r = 0; g.sx1r = s - 1; g.sr = 0; g.sr1 = s - 1;
-    g.in_rect = true;
-    return true;
-  }
-  const int64_t rad = radius_upper(r2);
-  // Rings visit every cell once, at its offset in [-(n-1)/2, n/2].  If the
-  // box [p - rad, p + rad] reaches past that range (few cells per axis, or a
-  // large radius), the cell can meet the box through another periodic image:
-  // then all of it is scanned (every candidate is measured by its minimum
-  // image, so scanning more is always correct).
-  if (rad >= g.safe) {
-    g.sx0r = 0; g.sx1r = s - 1; g.sr = 0; g.sr1 = s - 1;
-    g.in_rect = true;
-    return true;
-  }
-  const int64_t cx0 = cell_lo_tab(ucx, g.nx, g.bx, R.L[0]);
-  const int64_t wx = cell_lo_tab(ucx + 1, g.nx, g.bx, R.L[0]) - cx0;
-  const int64_t cy0 = cell_lo_tab(ucy, g.ny, g.by, R.L[1]);
-  const int64_t wy = cell_lo_tab(ucy + 1, g.ny, g.by, R.L[1]) - cy0;
-  const int64_t lx = g.px - rad - cx0, hx = g.px + rad - cx0;
-  const int64_t ly = g.py - rad - cy0, hy = g.py + rad - cy0;
-  if (hx < 0 || lx >= wx || hy < 0 || ly >= wy) return false;
-  g.sx0r = lx <= 0 ? 0 : sub_idx(lx, wx, s);
-  g.sx1r = hx >= wx ? s - 1 : sub_idx(hx, wx, s);
-  g.sr = ly <= 0 ? 0 : sub_idx(ly, wy, s);
-  g.sr1 = hy >= wy ? s - 1 : sub_idx(hy, wy, s);
-  g.in_rect = true;
-  return true;
-}
-
-__device__ __forceinline__ void gen_ring2(RunGen& g) {
-  const int r = g.r;
-  g.lox = -min(r, (g.nx - 1) / 2); g.hix = min(r, g.nx / 2);
-  g.loy = -min(r, (g.ny - 1) / 2); g.hiy = min(r, g.ny / 2);
-  g.plox = r ? -min(r - 1, (g.nx - 1) / 2) : 1; g.phix = r ? min(r - 1, g.nx / 2) : 0;
-  g.ploy = r ? -min(r - 1, (g.ny - 1) / 2) : 1; g.phiy = r ? min(r - 1, g.ny / 2) : 0;
-  g.oy = g.loy;
-  g.ucy = g.cy + g.oy;
-  gen_row_parts(g);
-}
-
-__device__ __forceinline__ void gen_ring1(RunGen& g) {
-  const int r = g.r, s = g.s1;
-  g.bx0 = max(g.sx - r, 0); g.bx1 = min(g.sx + r, s - 1);
-  g.by0 = max(g.sy - r, 0); g.by1 = min(g.sy + r, s - 1);
-  g.px0 = r ? max(g.sx - r + 1, 0) : 1; g.px1 = r ? min(g.sx + r - 1, s - 1) : 0;
-  g.py0 = r ? max(g.sy - r + 1, 0) : 1; g.py1 = r ? min(g.sy + r - 1, s - 1) : 0;
-  g.yy = g.by0;
-  g.seg = 0;
-}
-
-__device__ __forceinline__ void gen_init(RunGen& g, const Rep& R, const uint32_t* __restrict__ bounds,
-                                         const GridView& G, uint32_t px, uint32_t py, int k) {
-  g.R = &R;
-  g.bx = bounds + R.bnd[0];
-  g.by = bounds + R.bnd[1];
-  g.G = G;
-  g.px = px;
-  g.py = py;
-  g.nx = R.nc[0];
-  g.ny = R.nc[1];
-  g.cx = cell_of_tab(px, g.nx, g.bx, R.inv_w[0]);
-  g.cy = cell_of_tab(py, g.ny, g.by, R.inv_w[1]);
-  g.own = R.c0 + (int64_t)g.cy * g.nx + g.cx;
-  g.safe = min(min((int64_t)px - cell_lo_tab(g.cx - (g.nx - 1) / 2, g.nx, g.bx, R.L[0]),
-                   cell_lo_tab(g.cx + g.nx / 2 + 1, g.nx, g.bx, R.L[0]) - (int64_t)px),
-               min((int64_t)py - cell_lo_tab(g.cy - (g.ny - 1) / 2, g.ny, g.by, R.L[1]),
-                   cell_lo_tab(g.cy + g.ny / 2 + 1, g.ny, g.by, R.L[1]) - (int64_t)py));
-  g.prad = -1;
-  g.own_done = false;
-  g.in_rect = false;
-  g.ndef = 0;
-  g.ob0 = __ldg(G.sub_base + g.own);
-  const uint32_t ob1 = __ldg(G.sub_base + g.own + 1);
-  g.r = 0;
-  // phase 1 (sub-cell rings inside the own cell) bounds the rest of the own
-  // cell by its distance to the scanned sub-block, which needs the own cell
-  // to be narrower than half a period: at least 3 cells per axis
-  if (ob1 - g.ob0 > 1 && g.nx >= 3 && g.ny >= 3) {
-    g.phase = 1;
-    g.s1 = __ldg(G.sub_s + g.own);
-    g.cx0 = __ldg(g.bx + g.cx);
-    g.wx1 = (int64_t)__ldg(g.bx + g.cx + 1) - g.cx0;
-    g.cy0 = __ldg(g.by + g.cy);
-    g.wy1 = (int64_t)__ldg(g.by + g.cy + 1) - g.cy0;
-    g.sx = sub_idx(px - g.cx0, g.wx1, g.s1);
-    g.sy = sub_idx(py - g.cy0, g.wy1, g.s1);
-    // Start with the 3 x 3 block of sub-cells, scanned as whole rows, rather
-    // than the own sub-cell and a ring around it: the own sub-cell (about 2
-    // particles) rarely holds and certifies the k nearest.  Only a very dense
-    // own sub-cell (more than 16 k particles, where the 64 x 64 cap of the
-    // sub-grid leaves dense cluster cores) starts alone.
-    const uint32_t os = g.ob0 + (uint32_t)(g.sy * g.s1 + g.sx);
-    if (__ldg(G.sub_off + os + 1) - __ldg(G.sub_off + os) <= (uint32_t)(16 * k)) {
-      g.r = 1;
-      gen_ring1(g);
-      g.px0 = 1;
-      g.px1 = 0;
-    } else {
-      gen_ring1(g);
-    }
-  } else {
-    g.phase = 2;
-    gen_ring2(g);
-  }
-}
-
-// squared distance bound of the current ring's block (call at kRingEnd);
-// returns ~0ull when the phase has covered everything it can
-__device__ __forceinline__ uint64_t gen_ring_bound(const RunGen& g) {
-  int64_t B = INT64_MAX;
-  if (g.phase == 1) {
-    const int s = g.s1;
-    if (g.bx0 == 0 && g.by0 == 0 && g.bx1 == s - 1 && g.by1 == s - 1) return ~0ull;
-    if (g.bx0 > 0) B = min(B, g.px - (g.cx0 + sub_lo(g.bx0, g.wx1, s)) + 1);
-    if (g.bx1 < s - 1) B = min(B, g.cx0 + sub_lo(g.bx1 + 1, g.wx1, s) - g.px);
-    if (g.by0 > 0) B = min(B, g.py - (g.cy0 + sub_lo(g.by0, g.wy1, s)) + 1);
-    if (g.by1 < s - 1) B = min(B, g.cy0 + sub_lo(g.by1 + 1, g.wy1, s) - g.py);
-  } else {
-    const bool fullx = g.hix - g.lox + 1 == g.nx, fully = g.hiy - g.loy + 1 == g.ny;
-    if (fullx && fully) return ~0ull;
-    const int r = g.r;
-    if (!fullx) {
-      B = min(B, g.px - cell_lo_tab(g.cx - r, g.nx, g.bx, g.R->L[0]) + 1);
-      B = min(B, cell_lo_tab(g.cx + r + 1, g.nx, g.bx, g.R->L[0]) - g.px);
-    }
-    if (!fully) {
-      B = min(B, g.py - cell_lo_tab(g.cy - r, g.ny, g.by, g.R->L[1]) + 1);
-      B = min(B, cell_lo_tab(g.cy + r + 1, g.ny, g.by, g.R->L[1]) - g.py);
-    }
-  }
-  return (uint64_t)B * (uint64_t)B;
-}
-
-// after kRingEnd: move to the next ring (stop=false) or end the phase (stop=true)
-__device__ __forceinline__ bool gen_advance(RunGen& g, bool stop) {
-  if (g.phase == 1) {
-    g.own_done = true;
-    if (!stop) {
-      ++g.r;
-      gen_ring1(g);
-      return true;
-    }
-    g.phase = 2;
-    g.r = 0;
-    gen_ring2(g);
-    return true;
-  }
-  if (stop) return false;
-  ++g.r;
-  const int lox = -min(g.r, (g.nx - 1) / 2), hix = min(g.r, g.nx / 2);
-  const int loy = -min(g.r, (g.ny - 1) / 2), hiy = min(g.r, g.ny / 2);
-  if (lox == g.lox && hix == g.hix && loy == g.loy && hiy == g.hiy) return false;  // nothing new
-  gen_ring2(g);
-  return true;
-}
-
-// next run [qb, qe) of the current ring, or kRingEnd
-__device__ __forceinline__ int gen_next(RunGen& g, uint64_t r2, uint32_t& qb, uint32_t& qe) {
-  const GridView& G = g.G;
-  if (g.phase == 1) {
-    for (;;) {
-      if (g.yy > g.by1) return kRingEnd;
-      const uint32_t rb = g.ob0 + (uint32_t)g.yy * g.s1;
-      const bool oldrow = !(g.yy < g.py0 || g.yy > g.py1 || g.px0 > g.px1);
-      int a, b;
-      if (!oldrow) {
-        a = g.bx0; b = g.bx1;
-        ++g.yy;
-      } else if (g.seg == 0) {
-        a = g.bx0; b = g.px0 - 1;
-        g.seg = 1;
-      } else {
-        a = g.px1 + 1; b = g.bx1;
-        g.seg = 0;
-        ++g.yy;
-      }
-      if (a > b) continue;
-      qb = __ldg(G.sub_off + rb + a);
-      qe = __ldg(G.sub_off + rb + b + 1);
-      return kRun;
-    }
-  }
+  for (int s = 0; s < KC; ++s) t[s] = s < KC - 1 - k ? 0u : 0xFFFFFFFFu;
+  int cnt = 0, merged = 0, got = 0;
+  // cursors over (coarse cell, row of sub-cells) and over the listed runs
+  int ucx = ucx0, ucy = ucy0, row = 0, row_end = -1, s = 1, nrun = 0, r = 0;
+  uint32_t lo = 0, hi = 0, code = 0;  // first and one-past-last sub-cell of the row
+  uint32_t q = 0, qb = 0, len = 0, ox = 0, oy = 0;
+  bool more = true, done = false;
   for (;;) {
-    if (g.in_rect) {  // rows of a split cell's rectangle
-      if (g.sr > g.sr1) {
-        g.in_rect = false;
-        continue;
-      }
-      const uint32_t rb = g.sbase + (uint32_t)g.sr * g.sstride;
-      ++g.sr;
-      qb = __ldg(G.sub_off + rb + g.sx0r);
-      qe = __ldg(G.sub_off + rb + g.sx1r + 1);
-      return kRun;
-    }
-    if (g.part >= g.nparts) {  // next row
-      if (g.oy + 1 > g.hiy) {
-        if (g.ndef > 0) {  // deferred split cells, now with the current radius
-          --g.ndef;
-          gen_rect(g, g.def_g[g.ndef], g.def_ucx[g.ndef], g.def_ucy[g.ndef], r2);
-          continue;
-        }
-        return kRingEnd;
-      }
-      ++g.oy;
-      g.ucy = g.cy + g.oy;
-      gen_row_parts(g);
-      continue;
-    }
-    const int x0 = g.pa[g.part], x1 = g.pb[g.part];
-    if (g.x < 0) {  // start of a part: one run when no cell in it is split
-      // once the radius is known, a row that misses the box is skipped, and
-      // so are (below) its cells that miss it
-      g.prad = -1;
-      if (r2 != ~0ull) {
-        const int64_t rad = radius_upper(r2);
-        if (rad < g.safe) {
-          if (cell_lo_tab(g.ucy, g.ny, g.by, g.R->L[1]) > g.py + rad ||
-              cell_lo_tab(g.ucy + 1, g.ny, g.by, g.R->L[1]) <= g.py - rad) {
-            ++g.part;
-            continue;
+    while (cnt <= CAP - 4) {
+      if (q - qb >= len) {  // next run
+        if (r == nrun) {
+          // list up to kRuns runs, so that one flat loop scans them and the
+          // threads of a warp scan candidates together however their squares split
+          nrun = r = 0;
+          while (more && nrun <= kRuns - 2) {
+            if (row > row_end) {  // next coarse cell
+              if (ucx > ucx1) {
+                ucx = ucx0;
+                ++ucy;
+              }
+              if (ucy > ucy1) {
+                more = false;
+                break;
+              }
+              const int cy = ucy < 0 ? ucy + ny : (ucy >= ny ? ucy - ny : ucy);
+              const int cx = ucx < 0 ? ucx + nx : (ucx >= nx ? ucx - nx : ucx);
+              // shift code per axis: 0 same image, 1 the image at -L, 2 at +L
+              code = (ucx < 0 ? 4u : (ucx >= nx ? 8u : 0u)) | (ucy < 0 ? 1u : (ucy >= ny ? 2u : 0u));
+              const int64_t gc = R.c0 + (int64_t)cy * nx + cx;
+              const uint32_t base = __ldg(G.sub_base + gc);
+              s = __ldg(G.sub_s + gc);
+              const int sx0 = ucx == ucx0 ? sub_of(fx0, s) : 0, sx1 = ucx == ucx1 ? sub_of(fx1, s) : s - 1;
+              row = ucy == ucy0 ? sub_of(fy0, s) : 0;
+              row_end = ucy == ucy1 ? sub_of(fy1, s) : s - 1;
+              lo = base + (uint32_t)(row * s + sx0);
+              hi = lo + (uint32_t)(sx1 - sx0 + 1);
+              bc.cells += 1;
+              ++ucx;
+            }
+            // two rows at a time: their four loads are in flight together
+            const uint32_t step = row < row_end ? (uint32_t)s : 0u;
+            const uint32_t b0 = __ldg(G.sub_off + lo), e0 = __ldg(G.sub_off + hi);
+            const uint32_t b1 = __ldg(G.sub_off + lo + step), e1 = __ldg(G.sub_off + hi + step);
+            if (e0 > b0) H.run[nrun++][tid] = make_uint2(b0, (e0 - b0) << 4 | code);
+            if (step && e1 > b1) H.run[nrun++][tid] = make_uint2(b1, (e1 - b1) << 4 | code);
+            row += 2;
+            lo += 2u * (uint32_t)s;
+            hi += 2u * (uint32_t)s;
           }
-          g.prad = rad;
+          bc.runs += (uint32_t)nrun;
+          if (nrun == 0) {
+            done = true;
+            break;
+          }
         }
+        const uint2 e = H.run[r++][tid];
+        qb = e.x;
+        len = e.y >> 4;
+        q = qb & ~1u;  // 16-byte aligned pairs; the slot before the run is masked
+        // reference shifted into the run's periodic image: dx = x_j - ox exactly
+        ox = (uint32_t)p.x + (e.y & 4u ? Lx : 0u) - (e.y & 8u ? Lx : 0u);
+        oy = (uint32_t)p.y + (e.y & 1u ? Ly : 0u) - (e.y & 2u ? Ly : 0u);
+        bc.cand += len;
       }
-      const uint32_t sb0 = __ldg(G.sub_base + g.rowbase + x0), sb1 = __ldg(G.sub_base + g.rowbase + x1 + 1);
-      if (sb1 - sb0 == (uint32_t)(x1 - x0 + 1)) {
-        ++g.part;
-        qb = __ldg(G.off + g.rowbase + x0);
-        qe = __ldg(G.off + g.rowbase + x1 + 1);
-        return kRun;
+      // four candidates from two 16-byte loads (the arrays are padded by four slots)
+      const int4 A = __ldg(reinterpret_cast<const int4*>(pos + q));
+      const int4 C = __ldg(reinterpret_cast<const int4*>(pos + q + 2));
+      const int32_t xs[4] = {A.x, A.z, C.x, C.z}, ys[4] = {A.y, A.w, C.y, C.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        // branch-free append: written at the next free place, kept only for a hit
+        const int32_t dx = (int32_t)((uint32_t)xs[u] - ox), dy = (int32_t)((uint32_t)ys[u] - oy);
+        const float fx = (float)dx, fy = (float)dy;
+        const float D = __fmaf_rn(fx, fx, __fmul_rn(fy, fy));
+        bool hit = D <= tau && q + (uint32_t)u - qb < len;
+        if (FOV) hit = hit && (vw.cq < 0 || (long long)dx * vw.nxq + (long long)dy * vw.nyq >= 0);
+        H.hit[cnt][tid] = make_uint2(q + (uint32_t)u, __float_as_uint(D));
+        cnt += hit ? 1 : 0;
       }
-      g.x = x0;
-    }
-    if (g.x > x1) {
-      ++g.part;
-      g.x = -1;
-      continue;
-    }
-    if (g.prad >= 0) {
-      const int ucx = g.pu[g.part] + (g.x - x0);
-      if (cell_lo_tab(ucx, g.nx, g.bx, g.R->L[0]) > g.px + g.prad ||
-          cell_lo_tab(ucx + 1, g.nx, g.bx, g.R->L[0]) <= g.px - g.prad) {
-        ++g.x;
-        continue;
+      q += 4;
+      if (q - qb >= len && r == nrun && !more) {
+        done = true;
+        break;
       }
     }
-    // per cell: a maximal run of unsplit cells, or one split cell
-    const int64_t gc = g.rowbase + g.x;
-    uint32_t b0 = __ldg(G.sub_base + gc), b1 = __ldg(G.sub_base + gc + 1);
-    if (b1 - b0 == 1) {
-      const int xs = g.x;
-      while (g.x + 1 <= x1) {
-        const uint32_t c1 = __ldg(G.sub_base + gc + (g.x - xs) + 2);
-        if (c1 - b1 != 1) break;
-        b1 = c1;
-        ++g.x;
+#pragma unroll 2
+    for (int b = merged; b < cnt; ++b) {
+      const uint2 h = H.hit[b][tid];
+      bool keep = (int32_t)h.x != self;
+      if (FOV && vw.cq != 0) {  // (cq = 0: the scan's test was the whole test)
+        const int2 pj = __ldg(pos + h.x);
+        const int64_t dx = min_image((int64_t)pj.x - p.x, Lx), dy = min_image((int64_t)pj.y - p.y, Ly);
+        keep = keep && in_view(vw, (int32_t)dx, (int32_t)dy, (uint64_t)(dx * dx) + (uint64_t)(dy * dy));
       }
-      qb = __ldg(G.off + g.rowbase + xs);
-      qe = __ldg(G.off + g.rowbase + g.x + 1);
-      ++g.x;
-      return kRun;
+      got += keep ? 1 : 0;
+      uint32_t x = keep ? (h.y & ~((1u << B) - 1u)) | (uint32_t)b : 0xFFFFFFFFu;
+#pragma unroll
+      for (int e = 0; e < KC; ++e) {
+        const uint32_t m = min(t[e], x);
+        x = max(t[e], x);
+        t[e] = m;
+      }
     }
-    const int xc = g.x;
-    ++g.x;
-    if (gc == g.own && g.own_done) continue;
-    const int ucx = g.pu[g.part] + (xc - x0);
-    if (r2 == ~0ull && g.ndef < 4) {
-      g.def_g[g.ndef] = gc;
-      g.def_ucx[g.ndef] = ucx;
-      g.def_ucy[g.ndef] = g.ucy;
-      ++g.ndef;
-      continue;
-    }
-    gen_rect(g, gc, ucx, g.ucy, r2);
+    if (done) break;
+    // full column: its KC best move to the front and keep their order
+    merged = 0;
+    uint2 best[KC];
+#pragma unroll
+    for (int e = 0; e < KC; ++e)
+      if (e >= KC - 1 - k && t[e] != 0xFFFFFFFFu) best[e] = H.hit[t[e] & ((1u << B) - 1u)][tid];
+#pragma unroll
+    for (int e = 0; e < KC; ++e)
+      if (e >= KC - 1 - k && t[e] != 0xFFFFFFFFu) {
+        H.hit[merged][tid] = best[e];
+        t[e] = (t[e] & ~((1u << B) - 1u)) | (uint32_t)merged;
+        ++merged;
+      }
+    cnt = merged;
+    if (t[KC - 2] < 0xFF000000u) tau = fminf(tau, __uint_as_float(((t[KC - 2] >> B) + 3u) << B));
   }
+  bc.hits += (uint32_t)got;
+  if ((t[KC - 2] >> B) + 1u < edge) {
+    bool close = false;  // a pair whose order the keys leave open
+#pragma unroll
+    for (int e = 0; e < KC - 1; ++e) close |= e >= KC - 1 - k && (t[e + 1] >> B) - (t[e] >> B) <= 1u;
+    bc.why = close ? 3u : 0u;
+    return !close;
+  }
+  // too few: scale the radius towards about 1.5 k expected hits
+  const float want = 1.5f * (float)k + 1.f;
+  *r_next = (float)a * (got > 0 ? fminf(sqrtf(want / (float)got), 2.f) : 2.f);
+  bc.why = 2u;
+  return false;
 }
 
-template <int KC>
-__device__ __forceinline__ void knn2_search(Ctx& C, const Rep& R, const uint32_t* __restrict__ bounds,
-                                            const GridView& G, const int2* __restrict__ pos,
-                                            const int32_t* __restrict__ ids, Top<KC>& T, int k) {
-  RunGen g;
-  gen_init(g, R, bounds, G, C.px, C.py, k);
-  C.split = g.phase == 1;
-  for (;;) {
-    uint32_t qb = 0, qe = 0;
-    const int ev = gen_next(g, T.d[KC - 1], qb, qe);
-    if (ev == kRun) {
-      scan_run<KC>(C, pos, ids, qb, qe, T);  // the only copy of the candidate loop
-      continue;
+// ---------------------------------------------------------------------------
+// A group of GS lanes searches for one particle, exactly.  Hits (D <= tau)
+// are appended to the group's list by ballot; a nearly full list keeps its k
+// best, and tau follows.  All lanes of the group call every function here.
+// ---------------------------------------------------------------------------
+template <int CAP>
+struct GroupList {
+  unsigned long long d[CAP];
+  int32_t slot[CAP];
+};
+
+template <int KC> struct GroupCfg { static constexpr int CAP = KC <= 12 ? 64 : KC <= 17 ? 96 : 160; };
+
+template <int GS, int CAP, bool FOV>
+struct Group {
+  GroupList<CAP>& L;
+  const int2* __restrict__ pos;
+  const int32_t* __restrict__ ids;
+  unsigned mask;      // the group's lanes
+  int shift, gl;      // its first lane, the lane's number in it
+  int32_t self;
+  Ctx C;
+  int k, cnt;
+  unsigned long long tau;
+  uint32_t n_cand;
+
+  // the k best of the list by (D, id), in order, through put(rank, D, slot)
+  template <class F>
+  __device__ __forceinline__ void rank(F put) {
+    constexpr int E = (CAP + GS - 1) / GS;
+    __syncwarp(mask);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int i = gl + e * GS;
+      if (e * GS >= cnt) break;
+      int r = INT_MAX;
+      unsigned long long D = 0;
+      int32_t q = 0;
+      if (i < cnt) {
+        D = L.d[i];
+        q = L.slot[i];
+        r = 0;
+        for (int j = 0; j < cnt; ++j) {
+          const unsigned long long Dj = L.d[j];
+          bool before = Dj < D;
+          if (Dj == D && j != i) before = __ldg(ids + L.slot[j]) < __ldg(ids + q);
+          r += before ? 1 : 0;
+        }
+      }
+      put(e, r, D, q);
     }
-    // ring end: every unscanned particle (of the phase's region) is at
-    // squared distance >= B2; an equal distance could still win on id
-    const uint64_t B2 = gen_ring_bound(g);
-    const bool stop = (B2 == ~0ull) || (T.d[KC - 1] < B2);
-    if (!gen_advance(g, stop)) break;
   }
-}
+
+  __device__ __forceinline__ void compact() {
+    constexpr int E = (CAP + GS - 1) / GS;
+    int rk[E];
+    unsigned long long dk[E];
+    int32_t qk[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) rk[e] = INT_MAX;
+    rank([&](int e, int r, unsigned long long D, int32_t q) {
+      rk[e] = r;
+      dk[e] = D;
+      qk[e] = q;
+    });
+    __syncwarp(mask);
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (rk[e] < k) {
+        L.d[rk[e]] = dk[e];
+        L.slot[rk[e]] = qk[e];
+      }
+    __syncwarp(mask);
+    cnt = min(cnt, k);
+    if (cnt == k) tau = L.d[k - 1];
+  }
+
+  // the candidates of slots [qb, qe)
+  __device__ __forceinline__ void run(int64_t qb, int64_t qe) {
+    n_cand += (uint32_t)(qe - qb);
+    for (int64_t b = qb; b < qe; b += GS) {
+      const int64_t q = b + gl;
+      bool hit = false;
+      unsigned long long D = 0;
+      if (q < qe && (int32_t)q != self) {
+        int32_t dx, dy;
+        D = box_offset(C, __ldg(pos + q), dx, dy);
+        hit = D <= tau;
+        if (FOV) hit = hit && in_view(C.view, dx, dy, D);
+      }
+      const unsigned m = (__ballot_sync(mask, hit) & mask) >> shift;
+      if (hit) {
+        const int at = cnt + __popc(m & ((1u << gl) - 1u));
+        L.d[at] = D;
+        L.slot[at] = (int32_t)q;
+      }
+      cnt += __popc(m);
+      if (cnt > CAP - GS) compact();
+    }
+  }
+
+  // does the square of half-width a meet some coarse cell of an axis twice
+  // (then the axis is covered whole)?
+  static __device__ __forceinline__ bool spans(uint32_t p, int64_t a, int n, int sh, int64_t L) {
+    return 2 * a + 1 >= L || ucell2((int64_t)p + a, n, sh, L) - ucell2((int64_t)p - a, n, sh, L) >= n;
+  }
+  // sub-cells [*i0, *i1] of unwrapped cell u that meet [p - w, p + w]; false if none does
+  static __device__ __forceinline__ bool clip(uint32_t p, int64_t w, int u, int n, int sh, int64_t L, int s, int* i0,
+                                              int* i1) {
+    const int64_t lo = (int64_t)p - w - cell_lo2(u, n, sh, L), hi = lo + 2 * w;
+    if (hi < 0 || lo >> sh > 0) return false;
+    *i0 = lo <= 0 ? 0 : sub_of(cell_frac((uint32_t)lo, sh), s);
+    *i1 = hi >> sh > 0 ? s - 1 : sub_of(cell_frac((uint32_t)hi, sh), s);
+    return true;
+  }
+
+  // The candidates of the square of half-width a (an axis that it spans is
+  // covered whole).  The lanes look at GS coarse cells at a time, so that
+  // empty ones cost little; a non-empty one is scanned by rows of the
+  // sub-cells that meet the square of half-width min(a, sqrt(tau)): a list
+  // that has filled up on the way leaves little to scan.  True when the
+  // square is the whole box.
+  __device__ __forceinline__ bool square(const Rep& R, const GridView& G, int64_t a) {
+    const int64_t Lx = C.Lx, Ly = C.Ly;
+    const int nx = R.nc[0], ny = R.nc[1], shx = R.sh[0], shy = R.sh[1];
+    const bool fullx = spans(C.px, a, nx, shx, Lx), fully = spans(C.py, a, ny, shy, Ly);
+    const int ux0 = fullx ? 0 : ucell2((int64_t)C.px - a, nx, shx, Lx);
+    const int ux1 = fullx ? nx - 1 : ucell2((int64_t)C.px + a, nx, shx, Lx);
+    const int uy0 = fully ? 0 : ucell2((int64_t)C.py - a, ny, shy, Ly);
+    const int uy1 = fully ? ny - 1 : ucell2((int64_t)C.py + a, ny, shy, Ly);
+    tau = fullx && fully ? ~0ull : (unsigned long long)(a + 1) * (unsigned long long)(a + 1) - 1;
+    unsigned long long at = ~0ull;  // the tau that w was taken for
+    int64_t w = a;
+    for (int uy = uy0; uy <= uy1; ++uy) {
+      const int cy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy);
+      const int64_t rb = R.c0 + (int64_t)cy * nx;
+      for (int uc = ux0; uc <= ux1; uc += GS) {
+        const int lx = uc + gl;
+        const int64_t lc = rb + (lx < 0 ? lx + nx : (lx >= nx ? lx - nx : lx));
+        const bool some = lx <= ux1 && __ldg(G.off + lc) != __ldg(G.off + lc + 1);
+        unsigned cells = (__ballot_sync(mask, some) & mask) >> shift;
+        while (cells) {
+          const int ux = uc + __ffs(cells) - 1;
+          cells &= cells - 1u;
+          const int64_t gc = rb + (ux < 0 ? ux + nx : (ux >= nx ? ux - nx : ux));
+          const uint32_t base = __ldg(G.sub_base + gc);
+          const int s = __ldg(G.sub_s + gc);
+          if (tau != at) {
+            at = tau;
+            if (tau < (unsigned long long)a * (unsigned long long)a)
+              w = min(a, (int64_t)(sqrtf((float)tau) * 1.000001f) + 1);
+          }
+          int sx0 = 0, sx1 = s - 1, r0 = 0, r1 = s - 1;
+          if (!fullx && !clip(C.px, w, ux, nx, shx, Lx, s, &sx0, &sx1)) continue;
+          if (!fully && !clip(C.py, w, uy, ny, shy, Ly, s, &r0, &r1)) continue;
+          for (int rr = r0; rr <= r1; rr += GS) {
+            // each lane looks up one row of sub-cells
+            uint32_t qb = 0, qe = 0;
+            if (rr + gl <= r1) {
+              const uint32_t lo = base + (uint32_t)((rr + gl) * s);
+              qb = __ldg(G.sub_off + lo + sx0);
+              qe = __ldg(G.sub_off + lo + sx1 + 1);
+            }
+            unsigned rows = (__ballot_sync(mask, qe > qb) & mask) >> shift;
+            while (rows) {
+              const int j = shift + __ffs(rows) - 1;
+              rows &= rows - 1u;
+              run(__shfl_sync(mask, qb, j), __shfl_sync(mask, qe, j));
+            }
+          }
+        }
+      }
+    }
+    return fullx && fully;
+  }
+};
 
 // the general update (vectorial noise, FP64 sums), kept out of line
 __device__ __noinline__ void align_advect_general(const Rep& R, const StepParams& P, uint32_t step, int32_t id,
@@ -504,28 +421,42 @@ __device__ __noinline__ void align_advect_general(const Rep& R, const StepParams
   align_advect<2>(R, P, step, id, ni, H, m, pi, pout, nout);
 }
 
-// Eq. (2) alignment + noise and Eq. (1) advection of one particle from its
-// finished top-k; writes the next state and counts the new coarse cell.
-template <int KC, bool FOV = true>
+// Eq. (2) alignment + noise and Eq. (1) advection of one particle; at(j) is
+// the slot of list entry j in [KC-1-k, KC-1) in (D, id) order, -1 where a
+// field of view holds fewer than k.  Writes the next state and counts the new
+// coarse cell.
+template <int KC, class At>
 __device__ __forceinline__ void knn2_update(const Rep& R, const StepParams& P, int64_t step, int64_t s, int2 p,
-                                            float2 nv, int32_t id, const Top<KC>& T,
-                                            const uint32_t* __restrict__ bounds, const float2* __restrict__ S_dir,
+                                            float2 nv, int32_t id, At at, const float2* __restrict__ S_dir,
                                             int2* __restrict__ U_pos, float2* __restrict__ U_dir,
                                             int32_t* __restrict__ U_id, uint32_t* __restrict__ counts, float* nnew) {
-  // Eq. (2): neighbor headings in (D, id) order; with a field of view the
-  // list may be shorter than k (unfilled entries have slot -1)
   HeadSum<2> H;
   H.init();
   const float ni[3] = {nv.x, nv.y, 0.f};
   int m = P.include_self ? 1 : 0;
   if (P.include_self) H.add(ni, P.sum_mode);
 #pragma unroll
-  for (int j = 0; j < KC; ++j) {
-    if (j >= KC - P.k && (!FOV || T.slot[j] >= 0)) {
-      const float2 d = __ldg(S_dir + T.slot[j]);
-      const float v[2] = {d.x, d.y};
+  for (int c = 0; c < KC - 1; c += 8) {
+    // eight headings in flight, then summed in order; a missing entry adds
+    // zero, which changes neither sum nor compensation
+    float2 d[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = c + u;
+      d[u] = make_float2(0.f, 0.f);
+      if (j < KC - 1 && j >= KC - 1 - P.k) {
+        const int32_t q = at(j);
+        if (q >= 0) {
+          d[u] = __ldg(S_dir + q);
+          ++m;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (c + u >= KC - 1) break;
+      const float v[2] = {d[u].x, d[u].y};
       H.add(v, P.sum_mode);
-      ++m;
     }
   }
   const int32_t pi[3] = {p.x, p.y, 0};
@@ -549,287 +480,27 @@ __device__ __forceinline__ void knn2_update(const Rep& R, const StepParams& P, i
     sincosf(R.eta * (u - 0.5f), &sn, &cs);
     nnew[0] = cs * ex - sn * ey;
     nnew[1] = sn * ex + cs * ey;
-    const float hx = P.advect_new ? nnew[0] : nv.x, hy = P.advect_new ? nnew[1] : nv.y;
-    int64_t qx = (int64_t)p.x + grid_step(R.s, hx), qy = (int64_t)p.y + grid_step(R.s, hy);
-    if (qx < 0 || qx >= (int64_t)R.L[0]) {
-      qx %= (int64_t)R.L[0];
-      if (qx < 0) qx += R.L[0];
-    }
-    if (qy < 0 || qy >= (int64_t)R.L[1]) {
-      qy %= (int64_t)R.L[1];
-      if (qy < 0) qy += R.L[1];
-    }
-    pout[0] = (int32_t)qx;
-    pout[1] = (int32_t)qy;
+    pout[0] = wrap_add(p.x, grid_step(R.s, P.advect_new ? nnew[0] : nv.x), R.L[0]);
+    pout[1] = wrap_add(p.y, grid_step(R.s, P.advect_new ? nnew[1] : nv.y), R.L[1]);
   } else {
     align_advect_general(R, P, (uint32_t)step, id, ni, H, m, pi, pout, nnew);
   }
   U_pos[s] = make_int2(pout[0], pout[1]);
   U_dir[s] = make_float2(nnew[0], nnew[1]);
   U_id[s] = id;
-  const uint32_t* bx = bounds + R.bnd[0];
-  const uint32_t* by = bounds + R.bnd[1];
-  const int ncx = cell_of_tab((uint32_t)pout[0], R.nc[0], bx, R.inv_w[0]);
-  const int ncy = cell_of_tab((uint32_t)pout[1], R.nc[1], by, R.inv_w[1]);
-  atomicAdd(counts + R.c0 + (int64_t)ncy * R.nc[0] + ncx, 1u);
-}
-
-// thread-per-particle search + update (the walk of RunGen for every particle)
-template <int KC>
-__global__ void __launch_bounds__(kBlock, VK_KNN2_MIN_BLOCKS) knn2_step_kernel(
-    const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const uint32_t* __restrict__ bounds,
-    const int2* __restrict__ S_pos, const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G,
-    int2* __restrict__ U_pos, float2* __restrict__ U_dir, int32_t* __restrict__ U_id, uint32_t* __restrict__ counts,
-    PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P) {
-  __shared__ PhiShared phs;
-  phi_block_begin(phs);
-  const BlockTask t = tasks[blockIdx.x];
-  const Rep R = reps[t.rep];
-  const int li = t.first + (int)threadIdx.x;
-  const int64_t step = *d_step;
-  float nnew[3] = {0.f, 0.f, 0.f};
-  Ctx C;
-  C.n_cand = 0;
-  C.n_runs = 0;
-  C.split = false;
-  if (li < R.n) {
-    const int64_t s = R.p0 + li;
-    const int2 p = S_pos[s];
-    const float2 nv = S_dir[s];
-    const int32_t id = S_id[s];
-    init_ctx(C, R, s, p);
-    if (P.fov_cq != kViewAll) C.view = make_view(nv, P.fov_cq);
-    Top<KC> T;
-    top_init<KC>(T, P.k);
-    knn2_search<KC>(C, R, bounds, G, S_pos, S_id, T, P.k);
-    knn2_update<KC>(R, P, step, s, p, nv, id, T, bounds, S_dir, U_pos, U_dir, U_id, counts, nnew);
-  }
-  record_search_stats(P.stats, li < R.n, C.n_cand, C.n_runs, C.split);
-  phi_block_end<2>(phs, nnew, phi_acc + ((size_t)(step % P.phi_cap) * (size_t)P.n_rep + (size_t)t.rep) * 3);
-}
-
-// row id of the export table: the ids of T in (D, id) order, -1 past the
-// count found (a field of view may hold fewer than k)
-template <int KC>
-__device__ __forceinline__ void write_row(const Top<KC>& T, const int32_t* __restrict__ S_id, int32_t id, int k,
-                                          int32_t* __restrict__ out) {
-#pragma unroll
-  for (int j = 0; j < KC; ++j)
-    if (j >= KC - k) out[(int64_t)id * k + (j - (KC - k))] = T.slot[j] >= 0 ? __ldg(S_id + T.slot[j]) : -1;
-}
-
-template <int KC>
-__global__ void __launch_bounds__(kBlock, 2) knn2_export_kernel(const Rep* __restrict__ reps, int rep,
-                                                                const uint32_t* __restrict__ bounds,
-                                                                const int2* __restrict__ S_pos,
-                                                                const float2* __restrict__ S_dir,
-                                                                const int32_t* __restrict__ S_id, GridView G, int k,
-                                                                int32_t cq, int32_t* __restrict__ out) {
-  const Rep R = reps[rep];
-  const int li = blockIdx.x * kBlock + (int)threadIdx.x;
-  if (li >= R.n) return;
-  const int64_t s = R.p0 + li;
-  Ctx C;
-  init_ctx(C, R, s, S_pos[s]);
-  if (cq != kViewAll) C.view = make_view(S_dir[s], cq);
-  Top<KC> T;
-  top_init<KC>(T, k);
-  knn2_search<KC>(C, R, bounds, G, S_pos, S_id, T, k);
-  write_row<KC>(T, S_id, S_id[s], k, out);
-}
-
-// ---------------------------------------------------------------------------
-// Radius-first search (the default).  Each particle knows roughly how far
-// its k-th neighbor is: its k-th distance at the previous step, kept as a
-// per-particle hint in the state (particles move by at most v0 dt per step,
-// and neighbors mostly move together).  So it scans, once, every particle of
-// the square [p - a, p + a], a a little above that distance: the sub-cell
-// rows of the one to four coarse cells that overlap the square, each a
-// contiguous run of the sorted arrays.  A candidate whose exact int64
-// squared distance D is <= tau = (a+1)^2 - 1 goes to the particle's short
-// hit list in shared memory; nothing outside the square is that close, so
-// with at least k hits the k best hits by (D, id) are exactly the k nearest.
-// The hits are merged into the register top-k by a branch-free insertion on
-// D.  With fewer than k hits the square doubles and the scan repeats.  Equal
-// distances (the ids must decide), a full hit list, or a square wider than
-// half the period hand the particle to the per-particle walk, which runs in
-// a separate kernel over a device list so that its code and registers stay
-// out of this one; so do particles that need a second square, so that a
-// warp never waits for one particle's rescan.
-// ---------------------------------------------------------------------------
-constexpr int kBoxTries = 4;  // square sizes tried before the walk takes over
-
-
-template <int KC>
-struct BoxHits {
-  static constexpr int kCap = KC + 16;  // buffered hits per particle (merged when full)
-  static constexpr int kRuns = VK_KNN2_BOX_RUNS;  // slot runs of one square
-  int32_t slot[kCap][kBlock];           // one column per thread
-  uint2 run[kRuns][kBlock];             // (first slot, length << 4 | image shift codes)
-};
-
-// Merge the thread's hits into T by a branch-free insertion on D and return
-// how many of them count: the particle itself is skipped, and so is a hit
-// outside the field of view (the view test runs here, per hit, not per
-// candidate in the scan).  Sets *tie if two counted candidates at the same
-// distance met (their order, or which of them is kept, needs the ids: the
-// caller falls back to the walk).
-template <int KC>
-__device__ __forceinline__ int box_merge(const BoxHits<KC>& H, int cnt, const Ctx& C, const int2* __restrict__ pos,
-                                         Top<KC>& T, bool* tie) {
-  bool t = false;
-  int got = 0;
-  for (int b = 0; b < cnt; ++b) {
-    const int32_t q = H.slot[b][threadIdx.x];
-    if ((int64_t)q == C.self) continue;  // the particle is a hit of its own square
-    int32_t dx, dy;
-    const uint64_t D = box_offset(C, __ldg(pos + q), dx, dy);
-    if (!in_view(C.view, dx, dy, D)) continue;
-    ++got;
-    t |= D == T.d[KC - 1];
-    if (D < T.d[KC - 1]) {
-      bool lt_hi = true;
-#pragma unroll
-      for (int s = KC - 1; s > 0; --s) {
-        const bool lt_lo = D < T.d[s - 1];
-        t |= D == T.d[s - 1];
-        const uint64_t nd = lt_lo ? T.d[s - 1] : (lt_hi ? D : T.d[s]);
-        const int32_t ns = lt_lo ? T.slot[s - 1] : (lt_hi ? q : T.slot[s]);
-        T.d[s] = nd;
-        T.slot[s] = ns;
-        lt_hi = lt_lo;
-      }
-      if (lt_hi) {
-        T.d[0] = D;
-        T.slot[0] = q;
-      }
-    }
-  }
-  *tie = *tie || t;
-  return got;
-}
-
-// kNN visitor of the square walk: candidates with D <= tau go to the hit
-// list, which is merged into T when nearly full (tau then shrinks to T's
-// k-th distance) and by the caller at the end.  AHEAD (a view of at most a
-// half-plane, cq >= 0): a candidate behind the particle (d.nq < 0, exact in
-// int64) is out of view and is not buffered; the merge decides the rest.
-template <int KC, bool AHEAD>
-struct KnnVisit {
-  BoxHits<KC>& H;
-  const Ctx& C;
-  const int2* __restrict__ pos;
-  Top<KC>& T;
-  bool* tie;
-  uint64_t tau;
-  int cnt, got;
-  __device__ __forceinline__ void group(uint32_t q, uint32_t n, const int2* pj, uint32_t ox, uint32_t oy) {
-    // branch-free append: every candidate is written at the next free slot,
-    // and the slot advances only for a hit
-#pragma unroll
-    for (int u = 0; u < kGroup; ++u) {
-      const int32_t dx = (int32_t)((uint32_t)pj[u].x - ox), dy = (int32_t)((uint32_t)pj[u].y - oy);
-      const uint64_t D = (uint64_t)((int64_t)dx * dx) + (uint64_t)((int64_t)dy * dy);
-      bool hit = (uint32_t)u < n && D <= tau;
-      if (AHEAD) hit = hit && (long long)dx * C.view.nxq + (long long)dy * C.view.nyq >= 0;
-      H.slot[cnt][threadIdx.x] = (int32_t)(q + (uint32_t)u);
-      cnt += hit ? 1 : 0;
-    }
-    if (cnt > BoxHits<KC>::kCap - kGroup) {  // rare: a nearly full buffer is merged on the spot
-      got += box_merge<KC>(H, cnt, C, pos, T, tie);
-      cnt = 0;
-      if (T.d[KC - 1] < tau) tau = T.d[KC - 1];
-    }
-  }
-};
-
-// Scan the square [p - a, p + a] into T (initialised by the caller): every
-// slot with D <= tau = (a+1)^2 - 1 is a hit.  Nothing outside the square is
-// that close.  Hits are buffered and merged into T at the end (and, rarely,
-// when the buffer fills, after which tau shrinks to T's k-th distance).
-// Returns the number of hits that count (other particles, in view), >= k
-// exactly when T is full, or -1 when the square is too wide for the minimum
-// image or meets a coarse cell through two periodic images.
-template <int KC, bool AHEAD>
-__device__ __forceinline__ int box_scan_v(BoxHits<KC>& H, const Rep& R, const uint32_t* __restrict__ bounds,
-                                          const GridView& G, const int2* __restrict__ pos, const Ctx& C, int64_t a,
-                                          Top<KC>& T, bool* tie, BoxCount& bc) {
-  KnnVisit<KC, AHEAD> v{H, C, pos, T, tie, (uint64_t)(a + 1) * (uint64_t)(a + 1) - 1, 0, 0};
-  if (!box_walk(H, R, bounds, G, pos, C, a, bc, v)) return -1;
-  // after the loop, where the threads have reconverged
-  return v.got + box_merge<KC>(H, v.cnt, C, pos, T, tie);
-}
-
-// the view is the same for every particle: the branch is warp-uniform, and
-// only one copy of the scan loop runs in a given simulation
-template <int KC>
-__device__ __forceinline__ int box_scan(BoxHits<KC>& H, const Rep& R, const uint32_t* __restrict__ bounds,
-                                        const GridView& G, const int2* __restrict__ pos, const Ctx& C, int64_t a,
-                                        Top<KC>& T, bool* tie, BoxCount& bc) {
-  if (C.view.cq >= 0) return box_scan_v<KC, true>(H, R, bounds, G, pos, C, a, T, tie, bc);
-  return box_scan_v<KC, false>(H, R, bounds, G, pos, C, a, T, tie, bc);
+  atomicAdd(counts + linear_cell<2>(R, pout), 1u);
 }
 
 // search radius without a hint: a multiple of the k-th distance expected
 // from the density of the particle's own sub-cell
-__device__ __forceinline__ float box_radius_estimate(const Rep& R, const uint32_t* __restrict__ bounds,
-                                                     const GridView& G, int2 p, int k) {
-  const uint32_t* bx = bounds + R.bnd[0];
-  const uint32_t* by = bounds + R.bnd[1];
-  const int cx = cell_of_tab((uint32_t)p.x, R.nc[0], bx, R.inv_w[0]);
-  const int cy = cell_of_tab((uint32_t)p.y, R.nc[1], by, R.inv_w[1]);
-  const int64_t gc = R.c0 + (int64_t)cy * R.nc[0] + cx;
-  const uint32_t sb0 = __ldg(G.sub_base + gc), sb1 = __ldg(G.sub_base + gc + 1);
-  const int64_t x0 = __ldg(bx + cx), wx = (int64_t)__ldg(bx + cx + 1) - x0;
-  const int64_t y0 = __ldg(by + cy), wy = (int64_t)__ldg(by + cy + 1) - y0;
-  int s = 1;
-  uint32_t cnt;
-  if (sb1 - sb0 > 1) {
-    s = __ldg(G.sub_s + gc);
-    const uint32_t sub = sb0 + (uint32_t)(sub_idx((int64_t)p.y - y0, wy, s) * s + sub_idx((int64_t)p.x - x0, wx, s));
-    cnt = __ldg(G.sub_off + sub + 1) - __ldg(G.sub_off + sub);
-  } else {
-    cnt = __ldg(G.off + gc + 1) - __ldg(G.off + gc);
-  }
-  const float area = (float)wx * (float)wy / ((float)s * (float)s);
+__device__ __forceinline__ float box_radius_estimate(const Rep& R, const GridView& G, int2 p, int k) {
+  const int32_t pi[2] = {p.x, p.y};
+  int64_t gc, gs;
+  locate<2>(R, G, nullptr, pi, &gc, &gs);
+  const float s = (float)__ldg(G.sub_s + gc);
+  const uint32_t cnt = __ldg(G.sub_off + gs + 1) - __ldg(G.sub_off + gs);
+  const float area = (float)(1ull << R.sh[0]) * (float)(1ull << R.sh[1]) / (s * s);
   return 1.6f * sqrtf((float)k * area / (3.14159265f * (float)max(cnt, 1u)));
-}
-
-// The radius-first search of one particle with a first radius r: up to
-// `tries` squares.  A square with fewer than k hits is followed by one with
-// the radius scaled up towards about 1.5 k expected hits (hits grow with the
-// area, the square of the radius).
-// Returns true when T holds the exact top-k; otherwise *r_next is the radius
-// to try next, or -1 when only the walk can serve the particle (a square
-// too wide for the box, or two candidates at the same distance).
-template <int KC>
-__device__ __forceinline__ bool box_search(BoxHits<KC>& H, const Rep& R, const uint32_t* __restrict__ bounds,
-                                           const GridView& G, const int2* __restrict__ pos, const Ctx& C, float r,
-                                           int k, int tries, Top<KC>& T, BoxCount& bc, float* r_next) {
-  for (int tr = 0; tr < tries; ++tr) {
-    const int64_t a = (int64_t)ceilf(fminf(r, 2.0e9f));
-    bool tie = false;
-    top_init<KC>(T, k);
-    const int hits = box_scan<KC>(H, R, bounds, G, pos, C, a, T, &tie, bc);
-    if (hits < 0) {
-      bc.why = 1u;
-      *r_next = -1.f;
-      return false;
-    }
-    if (hits >= k) {
-      bc.hits += (uint32_t)hits;
-      if (!tie) return true;
-      bc.why = 3u;
-      *r_next = -1.f;
-      return false;
-    }
-    const float want = 1.5f * (float)k + 1.f;
-    const float f = hits > 0 ? sqrtf(want / (float)hits) : 2.f;
-    r = (float)a * fminf(f, 2.f);
-  }
-  bc.why = 2u;
-  *r_next = r;
-  return false;
 }
 
 // Tracing: totals of the radius-first counters (stats[5..13]).
@@ -860,198 +531,241 @@ __device__ __forceinline__ void warp_append(bool put, int2 e, int2* __restrict__
   if (put) list[base + __popc(m & ((1u << lane) - 1u))] = e;
 }
 
-// Search + update, radius first, one square per particle.  Particles it
-// cannot serve go on the deferred list (slot, replica) with the radius to
-// try next in U_hint (-1: walk), and knn2_deferred_kernel finishes them: a
-// warp here never waits for one particle's second square.
+// what a search hands its result to: the Vicsek update of a step ...
+template <int KC>
+struct StepOut {
+  const float2* __restrict__ S_dir;
+  int2* __restrict__ U_pos;
+  float2* __restrict__ U_dir;
+  int32_t* __restrict__ U_id;
+  float* __restrict__ U_hint;
+  uint32_t* __restrict__ counts;
+  PhiAcc* __restrict__ phi_acc;
+  const int64_t* __restrict__ d_step;
+  StepParams P;
+  static constexpr bool kStep = true;
+  // by slot: the radius a handed-on particle tries next (its hint replaces it in the end)
+  __device__ __forceinline__ float* radius() const { return U_hint; }
+  template <class At>
+  __device__ __forceinline__ void put(const Rep& R, int64_t step, int64_t s, int2 p, int32_t id, At at, float dk,
+                                      float* nnew) const {
+    knn2_update<KC>(R, P, step, s, p, S_dir[s], id, at, S_dir, U_pos, U_dir, U_id, counts, nnew);
+    U_hint[s] = sqrtf(dk) * 1.0001f + 1.f;
+  }
+};
+// ... or the particle's row of an export table, by id (-1 past the count found)
+template <int KC>
+struct RowOut {
+  const float2* __restrict__ S_dir;
+  const int32_t* __restrict__ S_id;
+  int32_t* __restrict__ out;
+  float* __restrict__ r_next;
+  StepParams P;
+  static constexpr bool kStep = false;
+  __device__ __forceinline__ float* radius() const { return r_next; }
+  template <class At>
+  __device__ __forceinline__ void put(const Rep&, int64_t, int64_t, int2, int32_t id, At at, float, float*) const {
+#pragma unroll
+    for (int j = 0; j < KC - 1; ++j)
+      if (j >= KC - 1 - P.k) {
+        const int32_t q = at(j);
+        out[(int64_t)id * P.k + (j - (KC - 1 - P.k))] = q >= 0 ? __ldg(S_id + q) : -1;
+      }
+  }
+};
+
+// the first radius of a particle
+__device__ __forceinline__ float box_radius(const Rep& R, const GridView& G, int2 p, float hint, const StepParams& P) {
+  return hint > 0.f ? P.halo_alpha * hint + P.halo_beta * fabsf(R.s) : box_radius_estimate(R, G, p, P.k);
+}
+
+// the search of one thread's particle with the square of half-width ceil(r)
+template <int KC, bool FOV, class Out>
+__device__ __forceinline__ bool box_particle(BoxShared<KC>& H, const Rep& R, const GridView& G,
+                                             const int2* __restrict__ S_pos, const int32_t* __restrict__ S_id,
+                                             float r, int64_t s, int64_t step, const Out& out, float* r_next,
+                                             BoxCount& bc, float* nnew) {
+  const int2 p = S_pos[s];
+  View vw;
+  if (FOV) vw = make_view(out.S_dir[s], out.P.fov_cq);
+  uint32_t t[KC];
+  if (!box_search<KC, FOV>(H, R, G, S_pos, (int32_t)s, p, vw, r, out.P.k, t, r_next, bc)) return false;
+  out.put(R, step, s, p, S_id[s], [&](int j) { return key_slot<KC>(H, t[j]); }, __uint_as_float(t[KC - 2]), nnew);
+  return true;
+}
+
+// Search + update, one square per particle.  Particles it cannot serve go on
+// the deferred list (slot, replica) with the radius to try next in U_hint.
 template <int KC, bool FOV>
-__global__ void __launch_bounds__(kBlock, VK_KNN2_BOX_BLOCKS) knn2_box_step_kernel(
-    const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const uint32_t* __restrict__ bounds,
-    const int2* __restrict__ S_pos, const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id,
-    const float* __restrict__ S_hint, GridView G, int2* __restrict__ U_pos, float2* __restrict__ U_dir,
-    int32_t* __restrict__ U_id, float* __restrict__ U_hint, uint32_t* __restrict__ counts,
-    PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P, int2* __restrict__ defer_list,
-    int32_t* __restrict__ defer_count) {
+__global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_box_step_kernel(
+    const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const int2* __restrict__ S_pos,
+    const int32_t* __restrict__ S_id, const float* __restrict__ S_hint, GridView G, StepOut<KC> out,
+    int2* __restrict__ defer_list, int32_t* __restrict__ defer_count) {
   extern __shared__ __align__(16) unsigned char box_smem[];
-  BoxHits<KC>& H = *reinterpret_cast<BoxHits<KC>*>(box_smem);
+  BoxShared<KC>& H = *reinterpret_cast<BoxShared<KC>*>(box_smem);
   __shared__ PhiShared phs;
   phi_block_begin(phs);
-  const BlockTask t = tasks[blockIdx.x];
+  const BlockTask t = tasks[blockIdx.x / kSplit];
   const Rep R = reps[t.rep];
-  const int li = t.first + (int)threadIdx.x;
+  const int li = t.first + (int)(blockIdx.x % kSplit) * kBlk + (int)threadIdx.x;
   const bool valid = li < R.n;
-  const int64_t step = *d_step;
+  const int64_t step = *out.d_step;
   float nnew[3] = {0.f, 0.f, 0.f};
   BoxCount bc;
   bool served = false;
   if (valid) {
     const int64_t s = R.p0 + li;
-    const int2 p = S_pos[s];
-    const float hint = S_hint[s];
-    Ctx C;
-    init_ctx(C, R, s, p);
-    if (FOV) C.view = make_view(S_dir[s], P.fov_cq);
-    Top<KC> T;
-    const float r =
-        hint > 0.f ? P.halo_alpha * hint + P.halo_beta * fabsf(R.s) : box_radius_estimate(R, bounds, G, p, P.k);
-    float r_next = -1.f;
-    served = box_search<KC>(H, R, bounds, G, S_pos, C, r, P.k, 1, T, bc, &r_next);
-    if (served) {
-      knn2_update<KC, FOV>(R, P, step, s, p, S_dir[s], S_id[s], T, bounds, S_dir, U_pos, U_dir, U_id, counts, nnew);
-      U_hint[s] = sqrtf((float)T.d[KC - 1]) * 1.0001f + 1.f;
-    } else {
-      U_hint[s] = r_next;
-    }
+    float r = box_radius(R, G, S_pos[s], S_hint[s], out.P);
+    if (out.P.knn_search == 0) served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, step, out, &r, bc, nnew);
+    if (!served) out.radius()[s] = r;
   }
   warp_append(valid && !served, make_int2((int)(R.p0 + li), t.rep), defer_list, defer_count);
-  record_search_stats(P.stats, served, bc.cand, bc.tries, false);
-  record_box_stats(P.stats, bc);
-  phi_block_end<2>(phs, nnew, phi_acc + ((size_t)(step % P.phi_cap) * (size_t)P.n_rep + (size_t)t.rep) * 3);
+  record_search_stats(out.P.stats, served, bc.cand, bc.tries, false);
+  record_box_stats(out.P.stats, bc);
+  phi_block_end<2>(phs, nnew,
+                   out.phi_acc + ((size_t)(step % out.P.phi_cap) * (size_t)out.P.n_rep + (size_t)t.rep) * 3);
 }
 
-// Search + update of the deferred particles: more squares from the radius
-// the step kernel left in U_hint.  A grid of one thread per particle covers
-// a list of any length (the length is read on the device, so the launch can
-// sit in a CUDA graph); particles that still cannot be served go on the walk
-// list.
 template <int KC, bool FOV>
-__global__ void __launch_bounds__(kBlock, VK_KNN2_DEFER_BLOCKS) knn2_deferred_kernel(
-    const Rep* __restrict__ reps, const uint32_t* __restrict__ bounds, const int2* __restrict__ S_pos,
-    const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G, int2* __restrict__ U_pos,
-    float2* __restrict__ U_dir, int32_t* __restrict__ U_id, float* __restrict__ U_hint,
-    uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P,
-    const int2* __restrict__ defer_list, const int32_t* __restrict__ defer_count, int2* __restrict__ walk_list,
-    int32_t* __restrict__ walk_count) {
+__global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_box_export_kernel(
+    const Rep* __restrict__ reps, int rep, const int2* __restrict__ S_pos, const int32_t* __restrict__ S_id,
+    const float* __restrict__ S_hint, GridView G, RowOut<KC> out, int2* __restrict__ defer_list,
+    int32_t* __restrict__ defer_count) {
   extern __shared__ __align__(16) unsigned char box_smem[];
-  BoxHits<KC>& H = *reinterpret_cast<BoxHits<KC>*>(box_smem);
-  const int total = *defer_count;
-  if ((int)(blockIdx.x * kBlock) >= total) return;  // whole block past the list
-  const int i = blockIdx.x * kBlock + (int)threadIdx.x;
-  const int64_t step = *d_step;
-  float nnew[3] = {0.f, 0.f, 0.f};
-  bool served = false;
-  int rep = 0;
-  BoxCount bc;
-  int2 e = make_int2(0, 0);
-  if (i < total) {
-    e = defer_list[i];
-    const int64_t s = e.x;
-    rep = e.y;
-    const Rep R = reps[e.y];
-    const int2 p = S_pos[s];
-    Ctx C;
-    init_ctx(C, R, s, p);
-    if (FOV) C.view = make_view(S_dir[s], P.fov_cq);
-    Top<KC> T;
-    const float r = U_hint[s];
-    float r_next = -1.f;
-    served = r > 0.f && box_search<KC>(H, R, bounds, G, S_pos, C, r, P.k, kBoxTries, T, bc, &r_next);
-    if (served) {
-      knn2_update<KC, FOV>(R, P, step, s, p, S_dir[s], S_id[s], T, bounds, S_dir, U_pos, U_dir, U_id, counts, nnew);
-      U_hint[s] = sqrtf((float)T.d[KC - 1]) * 1.0001f + 1.f;
-    }
-  }
-  warp_append(i < total && !served, e, walk_list, walk_count);
-  phi_add_warp<2>(phi_acc + (size_t)(step % P.phi_cap) * (size_t)P.n_rep * 3, rep, nnew, served);
-  if (P.stats && served) {
-    atomicAdd(P.stats + 0, (unsigned long long)bc.cand);
-    atomicAdd(P.stats + 1, (unsigned long long)bc.tries);
-    atomicMax(P.stats + 2, (unsigned long long)bc.cand);
-    atomicAdd(P.stats + 3, 1ull);
-  }
-}
-
-// Per-particle walk + update for the particles the radius-first kernels
-// could not serve (squares wider than the box allows, equal distances, no
-// fitting square).  A small fixed grid strides over the (short) list; the
-// stride loop is warp-uniform so that the order-parameter add is too.
-template <int KC>
-__global__ void __launch_bounds__(kBlock, 2) knn2_walk_list_kernel(
-    const Rep* __restrict__ reps, const uint32_t* __restrict__ bounds, const int2* __restrict__ S_pos,
-    const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G, int2* __restrict__ U_pos,
-    float2* __restrict__ U_dir, int32_t* __restrict__ U_id, float* __restrict__ U_hint,
-    uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P,
-    const int2* __restrict__ walk_list, const int32_t* __restrict__ walk_count) {
-  const int total = *walk_count;
-  const int64_t step = *d_step;
-  PhiAcc* step_acc = phi_acc + (size_t)(step % P.phi_cap) * (size_t)P.n_rep * 3;
-  for (int base = blockIdx.x * kBlock; base < total; base += gridDim.x * kBlock) {
-    const int i = base + (int)threadIdx.x;
-    float nnew[3] = {0.f, 0.f, 0.f};
-    int rep = 0;
-    const bool active = i < total;
-    if (active) {
-      const int2 e = walk_list[i];
-      const int64_t s = e.x;
-      rep = e.y;
-      const Rep R = reps[e.y];
-      const int2 p = S_pos[s];
-      Ctx C;
-      init_ctx(C, R, s, p);
-      if (P.fov_cq != kViewAll) C.view = make_view(S_dir[s], P.fov_cq);
-      Top<KC> T;
-      top_init<KC>(T, P.k);
-      knn2_search<KC>(C, R, bounds, G, S_pos, S_id, T, P.k);
-      knn2_update<KC>(R, P, step, s, p, S_dir[s], S_id[s], T, bounds, S_dir, U_pos, U_dir, U_id, counts, nnew);
-      U_hint[s] = sqrtf((float)T.d[KC - 1]) * 1.0001f + 1.f;
-      if (P.stats) {
-        atomicAdd(P.stats + 0, (unsigned long long)C.n_cand);
-        atomicAdd(P.stats + 1, (unsigned long long)C.n_runs);
-        atomicMax(P.stats + 2, (unsigned long long)C.n_cand);
-        atomicAdd(P.stats + 3, 1ull);
-        atomicAdd(P.stats + 4, 1ull);
-      }
-    }
-    phi_add_warp<2>(step_acc, rep, nnew, active);
-  }
-}
-
-template <int KC>
-__global__ void __launch_bounds__(kBlock, 3) knn2_box_export_kernel(
-    const Rep* __restrict__ reps, int rep, const uint32_t* __restrict__ bounds, const int2* __restrict__ S_pos,
-    const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id, const float* __restrict__ S_hint, GridView G,
-    int k, int32_t cq, float alpha, float beta, int32_t* __restrict__ out, int2* __restrict__ walk_list,
-    int32_t* __restrict__ walk_count) {
-  extern __shared__ __align__(16) unsigned char box_smem[];
-  BoxHits<KC>& H = *reinterpret_cast<BoxHits<KC>*>(box_smem);
+  BoxShared<KC>& H = *reinterpret_cast<BoxShared<KC>*>(box_smem);
   const Rep R = reps[rep];
-  const int li = blockIdx.x * kBlock + (int)threadIdx.x;
-  if (li >= R.n) return;
+  const int li = blockIdx.x * kBlk + (int)threadIdx.x;
+  const bool valid = li < R.n;
   const int64_t s = R.p0 + li;
-  const int2 p = S_pos[s];
-  Ctx C;
-  init_ctx(C, R, s, p);
-  if (cq != kViewAll) C.view = make_view(S_dir[s], cq);
-  Top<KC> T;
-  BoxCount bc;
-  const float hint = S_hint ? S_hint[s] : 0.f;
-  const float r = hint > 0.f ? alpha * hint + beta * fabsf(R.s) : box_radius_estimate(R, bounds, G, p, k);
-  float r_next = -1.f;
-  if (!box_search<KC>(H, R, bounds, G, S_pos, C, r, k, kBoxTries, T, bc, &r_next)) {
-    walk_list[atomicAdd(walk_count, 1)] = make_int2((int)s, rep);
-    return;
+  bool served = false;
+  if (valid) {
+    BoxCount bc;
+    float r = box_radius(R, G, S_pos[s], S_hint ? S_hint[s] : 0.f, out.P);
+    if (out.P.knn_search == 0) served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, 0, out, &r, bc, nullptr);
+    if (!served) out.radius()[s] = r;
   }
-  write_row<KC>(T, S_id, S_id[s], k, out);
+  warp_append(valid && !served, make_int2((int)s, rep), defer_list, defer_count);
 }
 
-// the per-particle walk for the listed particles of an export
-template <int KC>
-__global__ void __launch_bounds__(kBlock, 2) knn2_walk_export_list_kernel(
-    const Rep* __restrict__ reps, const uint32_t* __restrict__ bounds, const int2* __restrict__ S_pos,
-    const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G, int k, int32_t cq,
-    int32_t* __restrict__ out, const int2* __restrict__ walk_list, const int32_t* __restrict__ walk_count) {
-  const int total = *walk_count;
-  for (int i = blockIdx.x * kBlock + (int)threadIdx.x; i < total; i += gridDim.x * kBlock) {
-    const int2 e = walk_list[i];
-    const int64_t s = e.x;
-    const Rep R = reps[e.y];
-    Ctx C;
-    init_ctx(C, R, s, S_pos[s]);
-    if (cq != kViewAll) C.view = make_view(S_dir[s], cq);
-    Top<KC> T;
-    top_init<KC>(T, k);
-    knn2_search<KC>(C, R, bounds, G, S_pos, S_id, T, k);
-    write_row<KC>(T, S_id, S_id[s], k, out);
+// Handed-on particles, long lists: one thread each, up to two larger squares;
+// what is left goes on the second list.  A list that would leave most of the
+// chip idle at one thread per particle is left whole to the groups of the
+// next kernel (which serve a particle at 1.4 ns when they fill the chip, a
+// thread at 0.45 ns, but a thread takes about 30 us from start to end).
+constexpr int kLongList = 24576;
+constexpr int kSecondTries = 2;
+
+template <int KC, bool FOV, class Out>
+__global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_second_kernel(
+    const Rep* __restrict__ reps, const int2* __restrict__ S_pos, const int32_t* __restrict__ S_id, GridView G,
+    Out out, const int2* __restrict__ list, const int32_t* __restrict__ count, int2* __restrict__ left_list,
+    int32_t* __restrict__ left_count) {
+  extern __shared__ __align__(16) unsigned char box_smem[];
+  BoxShared<KC>& H = *reinterpret_cast<BoxShared<KC>*>(box_smem);
+  const int total = *count;
+  if (total < kLongList || out.P.knn_search == 1) return;
+  int64_t step = 0;
+  if constexpr (Out::kStep) step = *out.d_step;
+  for (int base = blockIdx.x * kBlk; base < total; base += gridDim.x * kBlk) {
+    const int i = base + (int)threadIdx.x;
+    const bool valid = i < total;
+    int2 e = make_int2(0, 0);
+    float nnew[3] = {0.f, 0.f, 0.f};
+    BoxCount bc;
+    bool served = false;
+    if (valid) {
+      e = list[i];
+      const Rep R = reps[e.y];
+      float r = out.radius()[e.x];
+      for (int tr = 0; tr < kSecondTries && !served; ++tr)
+        served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, e.x, step, out, &r, bc, nnew);
+      if (!served) out.radius()[e.x] = r;
+    }
+    warp_append(valid && !served, e, left_list, left_count);
+    if constexpr (Out::kStep) {
+      phi_add_warp<2>(out.phi_acc + (size_t)(step % out.P.phi_cap) * (size_t)out.P.n_rep * 3, e.y, nnew, served);
+      record_search_stats(out.P.stats, served, bc.cand, bc.tries, false);
+    }
+  }
+}
+
+// The rest: GS lanes each, larger squares until k hits are in one.  A warp
+// takes up to 32 particles, its groups search them one after another, and
+// then every lane updates one, so that the update runs on full warps.  Takes
+// the first list where the kernel above left it (its length is read on the
+// device, so that the launch can sit in a CUDA graph).
+constexpr int kGS = 16;
+constexpr int kGroupBlk = 128;
+
+template <int KC, bool FOV, class Out>
+__global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel(
+    const Rep* __restrict__ reps, const int2* __restrict__ S_pos, const int32_t* __restrict__ S_id, GridView G,
+    Out out, const int2* __restrict__ first_list, const int2* __restrict__ left_list,
+    const int32_t* __restrict__ counts) {
+  constexpr int CAP = GroupCfg<KC>::CAP, NG = 32 / kGS, NW = kGroupBlk / 32;
+  __shared__ GroupList<CAP> lists[kGroupBlk / kGS];
+  __shared__ int32_t res[NW][32][KC - 1];  // slots of the k nearest of the warp's particles
+  __shared__ float res_d[NW][32];          // their k-th squared distance
+  const bool first = counts[0] < kLongList || out.P.knn_search == 1;
+  const int2* __restrict__ list = first ? first_list : left_list;
+  const int total = first ? counts[0] : counts[1];
+  const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
+  const int nw = (int)gridDim.x * NW, w = (int)blockIdx.x * NW + wid;
+  // short lists are spread over all warps, long ones taken 32 at a time
+  const int chunk = min(32, (int)(((int64_t)total + (int64_t)nw * NG - 1) / ((int64_t)nw * NG)) * NG);
+  int64_t step = 0;
+  if constexpr (Out::kStep) step = *out.d_step;
+  const int k = out.P.k;
+  for (int64_t base = (int64_t)w * chunk; base < total; base += (int64_t)nw * chunk) {
+    const int todo = (int)min((int64_t)chunk, (int64_t)total - base);
+    for (int i = lane / kGS; i < todo; i += NG) {
+      const int2 e = list[base + i];
+      const Rep& R = reps[e.y];
+      Group<kGS, CAP, FOV> g{lists[threadIdx.x / kGS], S_pos, S_id, ((1u << kGS) - 1u) << (lane / kGS * kGS),
+                             lane / kGS * kGS, lane % kGS, e.x};
+      init_ctx(g.C, R, e.x, S_pos[e.x]);
+      if (FOV) g.C.view = make_view(out.S_dir[e.x], out.P.fov_cq);
+      g.k = k;
+      float r = out.radius()[e.x];
+      uint32_t tries = 1;
+      g.n_cand = 0;
+      for (;; ++tries) {
+        const int64_t a = (int64_t)ceilf(fminf(r, 4.0e9f));
+        g.cnt = 0;
+        if (g.square(R, G, a) || g.cnt >= k) break;
+        const float want = 1.5f * (float)k + 1.f;
+        r = (float)a * (g.cnt > 0 ? fminf(sqrtf(want / (float)g.cnt), 2.f) : 2.f) + 1.f;
+      }
+      for (int j = g.cnt + g.gl; j < k; j += kGS) res[wid][i][j] = -1;
+      if (g.gl == 0) res_d[wid][i] = 0.f;
+      __syncwarp(g.mask);
+      g.rank([&](int, int rk, unsigned long long D, int32_t q) {
+        if (rk < k) res[wid][i][rk] = q;
+        if (rk == k - 1) res_d[wid][i] = (float)D;
+      });
+      __syncwarp(g.mask);
+      if constexpr (Out::kStep)
+        if (out.P.stats && g.gl == 0) {
+          atomicAdd(out.P.stats + 0, (unsigned long long)g.n_cand);
+          atomicAdd(out.P.stats + 1, (unsigned long long)tries);
+          atomicMax(out.P.stats + 2, (unsigned long long)g.n_cand);
+          atomicAdd(out.P.stats + 3, 1ull);
+          atomicAdd(out.P.stats + 4, 1ull);
+        }
+    }
+    __syncwarp();
+    // every lane one particle
+    int2 e = make_int2(0, 0);
+    float nnew[3] = {0.f, 0.f, 0.f};
+    const bool mine = lane < todo;
+    if (mine) {
+      e = list[base + lane];
+      out.put(reps[e.y], step, e.x, S_pos[e.x], S_id[e.x],
+              [&](int j) { return res[wid][lane][j - (KC - 1 - k)]; }, res_d[wid][lane], nnew);
+    }
+    if constexpr (Out::kStep)
+      phi_add_warp<2>(out.phi_acc + (size_t)(step % out.P.phi_cap) * (size_t)out.P.n_rep * 3, e.y, nnew, mine);
+    __syncwarp();
   }
 }
 
@@ -1064,128 +778,109 @@ GridView view_of(const Buffers& b) {
   return G;
 }
 
-template <int KC>
-constexpr size_t box_smem_bytes() {
-  return sizeof(BoxHits<KC>);
+// blocks of the group kernel: as many as fit at once, fewer for small systems
+int group_blocks(int64_t n) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, (int64_t)device_sm_count() * 6));
 }
-
-// blocks of the deferred-particle kernel: enough threads for a list of every
-// particle (the length is known only on the device; threads past it exit at
-// once), so a long list never queues on a few threads
-int walk_blocks(const Geometry& g) { return (int)std::max<int64_t>(1, (g.n_total + kBlock - 1) / kBlock); }
-
-// blocks of the walk-list kernels: a small fixed grid striding over the
-// (short) list
-int walk_list_blocks(const Geometry& g) {
-  return (int)std::max<int64_t>(1, std::min<int64_t>((g.n_total + kBlock - 1) / kBlock, device_sm_count()));
+// blocks of the second-square kernel (strides over lists of any length)
+template <int KC>
+int second_blocks(int64_t n) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>((n + kBlk - 1) / kBlk, (int64_t)device_sm_count() * BoxCfg<KC>::BLOCKS));
 }
 
 template <int KC>
+StepOut<KC> step_out(const Buffers& b, const StepParams& P) {
+  return {(const float2*)b.S_dir, (int2*)b.U_pos, (float2*)b.U_dir, b.U_id, b.U_hint, b.counts, b.phi_acc, b.d_step, P};
+}
+
+template <int KC, bool FOV>
 cudaError_t step2(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
-  if (P.knn_search == 1 || !b.S_hint) {
-    knn2_step_kernel<KC><<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, b.bounds, (const int2*)b.S_pos,
-                                                       (const float2*)b.S_dir, b.S_id, view_of(b), (int2*)b.U_pos,
-                                                       (float2*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P);
-    if (b.U_hint) cudaMemsetAsync(b.U_hint, 0, sizeof(float) * (size_t)g.n_total, st);
-  } else {
-    // the lists are empty here: the previous scatter (or init) cleared them
-    // a field of view gets its own instantiation, so that the plain rule
-    // carries no view code (registers)
-    auto k = P.fov_cq != kViewAll ? knn2_box_step_kernel<KC, true> : knn2_box_step_kernel<KC, false>;
-    k<<<g.n_tasks, kBlock, box_smem_bytes<KC>(), st>>>(
-        g.reps, g.tasks, b.bounds, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id, b.S_hint, view_of(b),
-        (int2*)b.U_pos, (float2*)b.U_dir, b.U_id, b.U_hint, b.counts, b.phi_acc, b.d_step, P, b.ovf_list,
-        b.ovf_count);
-  }
+  // the lists are empty here: the previous scatter (or init) cleared them
+  knn2_box_step_kernel<KC, FOV><<<g.n_tasks * kSplit, kBlk, sizeof(BoxShared<KC>), st>>>(
+      g.reps, g.tasks, (const int2*)b.S_pos, b.S_id, b.S_hint, view_of(b), step_out<KC>(b, P), b.ovf_list,
+      b.ovf_count);
   return cudaGetLastError();
 }
 
-template <int KC>
+// the listed particles: the first list in the first half of ovf_list, what the
+// second squares leave in the second half
+template <int KC, bool FOV, class Out>
+void finish_lists(const Geometry& g, const Buffers& b, const Out& out, int64_t n, cudaStream_t st) {
+  int2* left = b.ovf_list + g.n_total;
+  knn2_second_kernel<KC, FOV><<<second_blocks<KC>(n), kBlk, sizeof(BoxShared<KC>), st>>>(
+        g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, b.ovf_list, b.ovf_count, left, b.ovf_count + 1);
+  knn2_group_kernel<KC, FOV><<<group_blocks(n), kGroupBlk, 0, st>>>(
+      g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, b.ovf_list, left, b.ovf_count);
+}
+
+template <int KC, bool FOV>
 cudaError_t finish2(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
-  if (P.knn_search == 0 && b.S_hint) {
-    // the deferred list lives in the first half of ovf_list, the walk list in the second
-    auto k = P.fov_cq != kViewAll ? knn2_deferred_kernel<KC, true> : knn2_deferred_kernel<KC, false>;
-    k<<<walk_blocks(g), kBlock, box_smem_bytes<KC>(), st>>>(
-        g.reps, b.bounds, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id, view_of(b), (int2*)b.U_pos,
-        (float2*)b.U_dir, b.U_id, b.U_hint, b.counts, b.phi_acc, b.d_step, P, b.ovf_list, b.ovf_count,
-        b.ovf_list + g.n_total, b.ovf_count + 1);
-    knn2_walk_list_kernel<KC><<<walk_list_blocks(g), kBlock, 0, st>>>(
-        g.reps, b.bounds, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id, view_of(b), (int2*)b.U_pos,
-        (float2*)b.U_dir, b.U_id, b.U_hint, b.counts, b.phi_acc, b.d_step, P, b.ovf_list + g.n_total,
-        b.ovf_count + 1);
-  }
+  finish_lists<KC, FOV>(g, b, step_out<KC>(b, P), g.n_total, st);
   return cudaGetLastError();
 }
 
-template <int KC>
-cudaError_t export2(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out, cudaStream_t st,
+template <int KC, bool FOV>
+cudaError_t export2(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out_ids, cudaStream_t st,
                     const StepParams& P) {
-  const int nb = (n + kBlock - 1) / kBlock;
-  if (nb == 0) return cudaSuccess;
-  if (P.knn_search == 1 || !b.S_hint) {
-    knn2_export_kernel<KC><<<nb, kBlock, 0, st>>>(g.reps, rep, b.bounds, (const int2*)b.S_pos,
-                                                  (const float2*)b.S_dir, b.S_id, view_of(b), k, P.fov_cq, out);
-  } else {
-    cudaError_t e = cudaMemsetAsync(b.ovf_count, 0, sizeof(int32_t), st);
-    if (e != cudaSuccess) return e;
-    knn2_box_export_kernel<KC><<<nb, kBlock, box_smem_bytes<KC>(), st>>>(
-        g.reps, rep, b.bounds, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id, b.S_hint, view_of(b), k,
-        P.fov_cq, P.halo_alpha, P.halo_beta, out, b.ovf_list, b.ovf_count);
-    knn2_walk_export_list_kernel<KC><<<walk_list_blocks(g), kBlock, 0, st>>>(
-        g.reps, b.bounds, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id, view_of(b), k, P.fov_cq, out,
-        b.ovf_list, b.ovf_count);
-    // leave the list empty for the next step
-    e = cudaMemsetAsync(b.ovf_count, 0, sizeof(int32_t), st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaGetLastError();
+  if (n == 0) return cudaSuccess;
+  // the lists are empty between steps; the export clears what it used
+  const RowOut<KC> out{(const float2*)b.S_dir, b.S_id, out_ids, b.U_hint, P};
+  knn2_box_export_kernel<KC, FOV><<<(n + kBlk - 1) / kBlk, kBlk, sizeof(BoxShared<KC>), st>>>(
+      g.reps, rep, (const int2*)b.S_pos, b.S_id, b.S_hint, view_of(b), out, b.ovf_list, b.ovf_count);
+  finish_lists<KC, FOV>(g, b, out, n, st);
+  cudaError_t e = cudaMemsetAsync(b.ovf_count, 0, 2 * sizeof(int32_t), st);
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 template <int KC>
 cudaError_t prepare2() {
-  cudaError_t e = cudaFuncSetAttribute(knn2_box_step_kernel<KC, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)box_smem_bytes<KC>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(knn2_box_step_kernel<KC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)box_smem_bytes<KC>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(knn2_box_export_kernel<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)box_smem_bytes<KC>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(knn2_deferred_kernel<KC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)box_smem_bytes<KC>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(knn2_deferred_kernel<KC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)box_smem_bytes<KC>());
-  return e;
+  const int bytes = (int)sizeof(BoxShared<KC>);
+  const void* f[] = {(const void*)knn2_box_step_kernel<KC, false>, (const void*)knn2_box_step_kernel<KC, true>,
+                      (const void*)knn2_box_export_kernel<KC, false>, (const void*)knn2_box_export_kernel<KC, true>,
+                     (const void*)knn2_second_kernel<KC, false, StepOut<KC>>,
+                     (const void*)knn2_second_kernel<KC, true, StepOut<KC>>,
+                     (const void*)knn2_second_kernel<KC, false, RowOut<KC>>,
+                     (const void*)knn2_second_kernel<KC, true, RowOut<KC>>};
+  for (const void* k : f) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// f(the list size the kernels for k are compiled for, field of view or not)
+template <int KC> using KeyCount = std::integral_constant<int, KC>;
+
+template <class F>
+cudaError_t for_k(const StepParams& P, F f) {
+  auto view = [&](auto kc) { return P.fov_cq != kViewAll ? f(kc, std::true_type{}) : f(kc, std::false_type{}); };
+  if (P.k <= 7) return view(KeyCount<8>{});
+  if (P.k <= 11) return view(KeyCount<12>{});
+  if (P.k <= 16) return view(KeyCount<17>{});
+  return view(KeyCount<33>{});
 }
 
 }  // namespace
 
 cudaError_t prepare_knn2() {
   cudaError_t e = prepare2<8>();
-  if (e == cudaSuccess) e = prepare2<16>();
-  if (e == cudaSuccess) e = prepare2<32>();
+  if (e == cudaSuccess) e = prepare2<12>();
+  if (e == cudaSuccess) e = prepare2<17>();
+  if (e == cudaSuccess) e = prepare2<33>();
   return e;
 }
 
 cudaError_t launch_knn2_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
-  if (P.k <= 8) return step2<8>(g, b, P, st);
-  if (P.k <= 16) return step2<16>(g, b, P, st);
-  return step2<32>(g, b, P, st);
+  return for_k(P, [&](auto kc, auto view) { return step2<kc(), view()>(g, b, P, st); });
 }
 
 cudaError_t launch_knn2_finish(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
-  if (P.k <= 8) return finish2<8>(g, b, P, st);
-  if (P.k <= 16) return finish2<16>(g, b, P, st);
-  return finish2<32>(g, b, P, st);
+  return for_k(P, [&](auto kc, auto view) { return finish2<kc(), view()>(g, b, P, st); });
 }
 
-cudaError_t launch_knn2_export(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out,
-                               cudaStream_t st, const StepParams& P) {
-  if (k <= 8) return export2<8>(g, b, k, rep, n, out, st, P);
-  if (k <= 16) return export2<16>(g, b, k, rep, n, out, st, P);
-  return export2<32>(g, b, k, rep, n, out, st, P);
+cudaError_t launch_knn2_export(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out, cudaStream_t st,
+                               const StepParams& P) {
+  return for_k(P, [&](auto kc, auto view) { return export2<kc(), view()>(g, b, rep, n, out, st, P); });
 }
 
 }  // namespace vk

@@ -112,7 +112,7 @@ __device__ __forceinline__ void metric_update(const Rep& R, const StepParams& P,
 }
 
 __global__ void __launch_bounds__(kBlock) metric2_step_kernel(
-    const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const uint32_t* __restrict__ bounds,
+    const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks,
     const int2* __restrict__ S_pos, const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G,
     int2* __restrict__ U_pos, float2* __restrict__ U_dir, int32_t* __restrict__ U_id, uint32_t* __restrict__ counts,
     PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P) {
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kBlock) metric2_step_kernel(
     MetricSum<2> S;
     S.init();
     MetricVisit2 v{C, S_dir, (uint64_t)R.r0q * (uint64_t)R.r0q, S};
-    if (!box_walk(H, R, bounds, G, S_pos, C, (int64_t)R.r0q, bc, v)) {
+    if (!box_walk(H, R, G, S_pos, C, (int64_t)R.r0q, bc, v)) {
       metric_scan_all2(R, S_pos, C, v);
       bc.cand += (uint32_t)R.n;
       bc.why = 1u;
@@ -147,9 +147,7 @@ __global__ void __launch_bounds__(kBlock) metric2_step_kernel(
     U_pos[s] = make_int2(pout[0], pout[1]);
     U_dir[s] = make_float2(nnew[0], nnew[1]);
     U_id[s] = id;
-    const int ncx = cell_of_tab((uint32_t)pout[0], R.nc[0], bounds + R.bnd[0], R.inv_w[0]);
-    const int ncy = cell_of_tab((uint32_t)pout[1], R.nc[1], bounds + R.bnd[1], R.inv_w[1]);
-    atomicAdd(counts + R.c0 + (int64_t)ncy * R.nc[0] + ncx, 1u);
+    atomicAdd(counts + linear_cell<2>(R, pout), 1u);
   }
   record_search_stats(P.stats, li < R.n, bc.cand, bc.runs, bc.why != 0u);
   phi_block_end<2>(phs, nnew, phi_acc + ((size_t)(step % P.phi_cap) * (size_t)P.n_rep + (size_t)t.rep) * 3);
@@ -235,7 +233,6 @@ __device__ __forceinline__ void sort_row(int32_t* __restrict__ ids, int64_t b, i
 // the neighbor ids of row id at out_off[id] (the slots are collected in
 // out_ids first, then mapped to ids and sorted).
 __global__ void __launch_bounds__(kBlock) metric2_export_kernel(const Rep* __restrict__ reps, int rep,
-                                                                const uint32_t* __restrict__ bounds,
                                                                 const int2* __restrict__ S_pos,
                                                                 const int32_t* __restrict__ S_id, GridView G,
                                                                 int pass, int32_t* __restrict__ deg,
@@ -253,7 +250,7 @@ __global__ void __launch_bounds__(kBlock) metric2_export_kernel(const Rep* __res
     int32_t* row = pass == 1 ? out_ids + out_off[id] : nullptr;
     MetricList2 v{C, (uint64_t)R.r0q * (uint64_t)R.r0q, row, 0};
     BoxCount bc;
-    if (!box_walk(H, R, bounds, G, S_pos, C, (int64_t)R.r0q, bc, v)) {
+    if (!box_walk(H, R, G, S_pos, C, (int64_t)R.r0q, bc, v)) {
       v.w = 0;
       metric_scan_all2(R, S_pos, C, v);
     }
@@ -304,7 +301,7 @@ GridView metric_view(const Buffers& b) {
 
 cudaError_t launch_metric_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
   if (g.dim == 2) {
-    metric2_step_kernel<<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, b.bounds, (const int2*)b.S_pos,
+    metric2_step_kernel<<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, (const int2*)b.S_pos,
                                                       (const float2*)b.S_dir, b.S_id, metric_view(b),
                                                       (int2*)b.U_pos, (float2*)b.U_dir, b.U_id, b.counts,
                                                       b.phi_acc, b.d_step, P);
@@ -322,7 +319,7 @@ cudaError_t launch_metric_export(const Geometry& g, const Buffers& b, int rep, i
   const int nb = (n + kBlock - 1) / kBlock;
   if (nb == 0) return cudaSuccess;
   if (g.dim == 2) {
-    metric2_export_kernel<<<nb, kBlock, 0, st>>>(g.reps, rep, b.bounds, (const int2*)b.S_pos, b.S_id,
+    metric2_export_kernel<<<nb, kBlock, 0, st>>>(g.reps, rep, (const int2*)b.S_pos, b.S_id,
                                                  metric_view(b), pass, deg, out_off, out_ids);
   } else {
     metric3_export_kernel<<<nb, kBlock, 0, st>>>(g.reps, rep, (const int4*)b.S_pos, b.S_id, metric_view(b), pass,

@@ -26,7 +26,7 @@ namespace vk {
 namespace {
 
 constexpr int64_t kNoAllocMaxN = VK_NOALLOC_MAX_N;
-constexpr float kNoAllocOccupancy = 2.0f;
+constexpr float kNoAllocOccupancy = 64.0f;  // particles per coarse cell; dense cells have sub-cells of about 2
 // generous bound of the scratch the layout below needs for kNoAllocMaxN
 constexpr size_t kScratchBytes = (size_t)6 << 20;
 
@@ -39,8 +39,9 @@ std::mutex g_mu;
 void* g_ptr[256] = {nullptr};
 
 // Device address of the scratch on the current device, looked up once per
-// device (the first call on a device does it; that call must not be made
-// while the stream is being captured).
+// device together with the search kernels' shared-memory attributes (the
+// first call on a device does it; that call must not be made while the stream
+// is being captured).
 cudaError_t scratch_ptr(void** out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -50,6 +51,7 @@ cudaError_t scratch_ptr(void** out) {
   if (!g_ptr[dev]) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+    if (e == cudaSuccess) e = prepare_knn2();
     if (e != cudaSuccess) return e;
     g_ptr[dev] = p;
   }
@@ -70,19 +72,17 @@ struct Carver {
 };
 
 // tables, grid bounds and cleared counters for one call
-__global__ void noalloc_setup_kernel(Rep R, BlockTask* tasks, int n_tasks, Rep* rep_out, uint32_t* bounds,
-                                     uint32_t* counts, int64_t n_cells, uint32_t* sub_count, int64_t n_sub,
+__global__ void noalloc_setup_kernel(Rep R, BlockTask* tasks, int n_tasks, Rep* rep_out, uint32_t* counts,
+                                     int64_t n_cells, uint32_t* sub_count, int64_t n_sub, int32_t* list_count,
                                      int32_t* status) {
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   if (tid == 0) {
     *rep_out = R;
     *status = 0;
+    list_count[0] = list_count[1] = 0;
   }
   for (int64_t i = tid; i < n_tasks; i += stride) tasks[i] = BlockTask{0, (int32_t)(i * kBlock)};
-  for (int a = 0; a < 3; ++a)
-    for (int64_t b = tid; b <= R.nc[a]; b += stride)
-      bounds[R.bnd[a] + b] = (uint32_t)((b * (int64_t)R.L[a] + R.nc[a] - 1) / R.nc[a]);
   for (int64_t i = tid; i < n_cells; i += stride) counts[i] = 0u;
   for (int64_t i = tid; i < n_sub; i += stride) sub_count[i] = 0u;
 }
@@ -133,18 +133,8 @@ extern "C" vk_status vk_knn_lists_noalloc(const int32_t* pos_q, int64_t n, const
   R.L[1] = box->box_q[1];
   R.L[2] = 1;
   const double side = std::sqrt((double)kNoAllocOccupancy * (double)R.L[0] * (double)R.L[1] / (double)n);
-  int64_t n_cells = 1;
-  for (int a = 0; a < 3; ++a) {
-    double ncd = a < 2 ? std::floor((double)R.L[a] / side) : 1.0;
-    ncd = std::max(1.0, std::min(ncd, std::min((double)R.L[a], 65536.0)));
-    R.nc[a] = (int32_t)ncd;
-    n_cells *= R.nc[a];
-    R.inv_w[a] = (float)R.nc[a] / (float)R.L[a];
-  }
-  R.bnd[0] = 0;
-  R.bnd[1] = R.nc[0] + 1;
-  R.bnd[2] = R.bnd[1] + R.nc[1] + 1;
-  const int64_t n_bounds = (int64_t)R.nc[0] + R.nc[1] + R.nc[2] + 3;
+  plan_grid2(R, side);
+  const int64_t n_cells = (int64_t)R.nc[0] * R.nc[1];
   const int64_t n_sub = n_cells + n / kSubTarget + 1;
   const int n_tasks = (int)((n + kBlock - 1) / kBlock);
 
@@ -153,13 +143,13 @@ extern "C" vk_status vk_knn_lists_noalloc(const int32_t* pos_q, int64_t n, const
   Carver cv{0};
   const size_t o_upos = cv.take<int2>(n), o_udir = cv.take<float2>(n), o_uid = cv.take<int32_t>(n);
   const size_t o_urank = cv.take<uint32_t>(n);
-  const size_t o_spos = cv.take<int2>(n), o_sdir = cv.take<float2>(n), o_sid = cv.take<int32_t>(n);
+  const size_t o_spos = cv.take<int2>(n + kPosPad), o_sdir = cv.take<float2>(n), o_sid = cv.take<int32_t>(n);
   const size_t o_counts = cv.take<uint32_t>(n_cells), o_offsets = cv.take<uint32_t>(n_cells + 1);
   const size_t o_bsum = cv.take<uint32_t>(2 * ((n_cells + 2047) / 2048 + 1));
   const size_t o_subs = cv.take<uint8_t>(n_cells), o_subbase = cv.take<uint32_t>(n_cells + 1);
   const size_t o_subcount = cv.take<uint32_t>(n_sub), o_suboff = cv.take<uint32_t>(n_sub + 1);
   const size_t o_bsum2 = cv.take<uint32_t>((n_sub + 2047) / 2048 + 1);
-  const size_t o_bounds = cv.take<uint32_t>(n_bounds);
+  const size_t o_list = cv.take<int2>(2 * n), o_lcount = cv.take<int32_t>(2), o_radius = cv.take<float>(n);
   const size_t o_rep = cv.take<Rep>(1), o_tasks = cv.take<BlockTask>(n_tasks), o_status = cv.take<int32_t>(1);
   if (cv.used > kScratchBytes) return VK_ERR_CAPACITY;  // cannot happen for n <= kNoAllocMaxN
   // an error left pending by the caller's earlier work is reported, not
@@ -188,7 +178,9 @@ extern "C" vk_status vk_knn_lists_noalloc(const int32_t* pos_q, int64_t n, const
   b.sub_count = reinterpret_cast<uint32_t*>(base + o_subcount);
   b.sub_off = reinterpret_cast<uint32_t*>(base + o_suboff);
   b.bsum2 = reinterpret_cast<uint32_t*>(base + o_bsum2);
-  b.bounds = reinterpret_cast<uint32_t*>(base + o_bounds);
+  b.ovf_list = reinterpret_cast<int2*>(base + o_list);
+  b.ovf_count = reinterpret_cast<int32_t*>(base + o_lcount);
+  float* radius = reinterpret_cast<float*>(base + o_radius);
   Rep* rep_d = reinterpret_cast<Rep*>(base + o_rep);
   BlockTask* tasks_d = reinterpret_cast<BlockTask*>(base + o_tasks);
   int32_t* status_d = reinterpret_cast<int32_t*>(base + o_status);
@@ -208,18 +200,18 @@ extern "C" vk_status vk_knn_lists_noalloc(const int32_t* pos_q, int64_t n, const
   P.k = k;
   P.n_rep = 1;
   P.phi_cap = 2;
-  P.knn_search = 1;  // the per-particle walk: no hint buffers, no shared-memory attribute to set
   P.fov_cq = kViewAll;
 
-  noalloc_setup_kernel<<<64, 256, 0, st>>>(R, tasks_d, n_tasks, rep_d, b.bounds, b.counts, n_cells, b.sub_count,
-                                           n_sub, status_d);
+  noalloc_setup_kernel<<<64, 256, 0, st>>>(R, tasks_d, n_tasks, rep_d, b.counts, n_cells, b.sub_count,
+                                           n_sub, b.ovf_count, status_d);
   noalloc_load_kernel<<<(int)((n + 255) / 256), 256, 0, st>>>(pos_q, (int32_t)n, R.L[0], R.L[1], (int2*)b.U_pos,
                                                               (float2*)b.U_dir, b.U_id, status_d);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = launch_count(g, b, st);
   if (e == cudaSuccess) e = launch_build(g, b, st);
   if (e == cudaSuccess) e = launch_scatter(g, b, P, 0, st);
-  if (e == cudaSuccess) e = launch_knn2_export(g, b, k, 0, (int)n, out_ids, st, P);
+  b.U_hint = radius;  // no hints to carry over: only the radius of handed-on particles
+  if (e == cudaSuccess) e = launch_knn2_export(g, b, 0, (int)n, out_ids, st, P);
   if (e == cudaSuccess && dev_status)
     e = cudaMemcpyAsync(dev_status, status_d, sizeof(int32_t), cudaMemcpyDefault, st);
   if (e != cudaSuccess) {

@@ -340,13 +340,6 @@ __device__ __forceinline__ bool poly_clip(Poly<CAP>& P, int32_t mx, int32_t my, 
 // sub-cells that meet it, and the walk stops once the scanned block holds
 // it.  run(qb, qe) receives runs of sorted slots.  Returns true if the whole
 // grid was visited.
-__device__ __forceinline__ int unwrapped_cell(int64_t X, int n, int64_t L) {
-  // X within one period of [0, L)
-  if (X < 0) return cell_of((int32_t)(X + L), n, (uint32_t)L) - n;
-  if (X >= L) return cell_of((int32_t)(X - L), n, (uint32_t)L) + n;
-  return cell_of((int32_t)X, n, (uint32_t)L);
-}
-
 // the box holds only minimum images (offsets strictly inside half a period),
 // so that visiting every site once, at its minimum image, is enough
 __device__ __forceinline__ bool within_half(const int64_t* b, int64_t Lx, int64_t Ly) {
@@ -358,7 +351,8 @@ __device__ bool voronoi_walk(const Rep& R, const int32_t* pi, const GridView& G,
   const int nx = R.nc[0], ny = R.nc[1];
   const int64_t Lx = R.L[0], Ly = R.L[1];
   const int64_t px = pi[0], py = pi[1];
-  const int cx = cell_of(pi[0], nx, R.L[0]), cy = cell_of(pi[1], ny, R.L[1]);
+  const int shx = R.sh[0], shy = R.sh[1];
+  const int cx = (int)((uint32_t)pi[0] >> shx), cy = (int)((uint32_t)pi[1] >> shy);
   const int64_t own = R.c0 + (int64_t)cy * nx + cx;
   const int s_own = G.sub_s[own];
   int64_t b[4];
@@ -366,9 +360,13 @@ __device__ bool voronoi_walk(const Rep& R, const int32_t* pi, const GridView& G,
   if (s_own > 1) {
     // ---- rings of sub-cells inside the own coarse cell
     const int s = s_own;
-    const int64_t x0 = cell_lo(cx, nx, Lx), y0 = cell_lo(cy, ny, Ly);
-    const int64_t wx = cell_lo(cx + 1, nx, Lx) - x0, wy = cell_lo(cy + 1, ny, Ly) - y0;
-    const int sx = sub_index(px - x0, wx, s), sy = sub_index(py - y0, wy, s);
+    const int64_t x0 = (int64_t)cx << shx, y0 = (int64_t)cy << shy;
+    const int sx = sub_of(cell_frac((uint32_t)pi[0], shx), s), sy = sub_of(cell_frac((uint32_t)pi[1], shy), s);
+    // sub-cell b begins at offset ceil(b 2^sh / s); b (2^32 / s) rounded up
+    // (down) and shifted bounds it from above (below) by at most a unit or two
+    const uint32_t inv = 0xFFFFFFFFu / (uint32_t)s;
+    auto sub_up = [&](int bq, int sh) { return (int64_t)((((uint64_t)bq * ((uint64_t)inv + 2)) >> (32 - sh)) + 1); };
+    auto sub_dn = [&](int bq, int sh) { return (int64_t)(((uint64_t)bq * (uint64_t)inv) >> (32 - sh)); };
     const uint32_t base = G.sub_base[own];
     for (int r = 0;; ++r) {
       const int bx0 = max(sx - r, 0), bx1 = min(sx + r, s - 1), by0 = max(sy - r, 0), by1 = min(sy + r, s - 1);
@@ -384,8 +382,9 @@ __device__ bool voronoi_walk(const Rep& R, const int32_t* pi, const GridView& G,
         }
       }
       // the scanned sub-block, as offsets from the particle
-      const int64_t xlo = x0 + (bx0 * wx + s - 1) / s - px, xhi = x0 + ((bx1 + 1) * wx + s - 1) / s - 1 - px;
-      const int64_t ylo = y0 + (by0 * wy + s - 1) / s - py, yhi = y0 + ((by1 + 1) * wy + s - 1) / s - 1 - py;
+      const int64_t xlo = x0 + (bx0 ? sub_up(bx0, shx) : 0) - px, ylo = y0 + (by0 ? sub_up(by0, shy) : 0) - py;
+      const int64_t xhi = min(bx1 == s - 1 ? x0 + ((int64_t)1 << shx) : x0 + sub_dn(bx1 + 1, shx), Lx) - 1 - px;
+      const int64_t yhi = min(by1 == s - 1 ? y0 + ((int64_t)1 << shy) : y0 + sub_dn(by1 + 1, shy), Ly) - 1 - py;
       box(b);
       if (b[0] >= xlo && b[1] <= xhi && b[2] >= ylo && b[3] <= yhi && within_half(b, Lx, Ly)) return false;
       if (bx0 == 0 && by0 == 0 && bx1 == s - 1 && by1 == s - 1) break;
@@ -408,7 +407,7 @@ __device__ bool voronoi_walk(const Rep& R, const int32_t* pi, const GridView& G,
     int ox0 = -(nx - 1) / 2, ox1 = nx / 2, oy0 = -(ny - 1) / 2, oy1 = ny / 2;
     bool clx = false, cly = false;
     if (b[0] > -Lx && b[1] < Lx) {
-      const int a0 = unwrapped_cell(px + b[0], nx, Lx) - cx, a1 = unwrapped_cell(px + b[1], nx, Lx) - cx;
+      const int a0 = ucell2(px + b[0], nx, shx, Lx) - cx, a1 = ucell2(px + b[1], nx, shx, Lx) - cx;
       if (a0 >= ox0 && a1 <= ox1) {
         clx = true;
         ox0 = a0;
@@ -416,7 +415,7 @@ __device__ bool voronoi_walk(const Rep& R, const int32_t* pi, const GridView& G,
       }
     }
     if (b[2] > -Ly && b[3] < Ly) {
-      const int a0 = unwrapped_cell(py + b[2], ny, Ly) - cy, a1 = unwrapped_cell(py + b[3], ny, Ly) - cy;
+      const int a0 = ucell2(py + b[2], ny, shy, Ly) - cy, a1 = ucell2(py + b[3], ny, shy, Ly) - cy;
       if (a0 >= oy0 && a1 <= oy1) {
         cly = true;
         oy0 = a0;
@@ -427,7 +426,6 @@ __device__ bool voronoi_walk(const Rep& R, const int32_t* pi, const GridView& G,
       a = max(a, ox0);
       e = min(e, ox1);
       if (a > e) return;
-      const int64_t ucy = (int64_t)cy + oy;
       const int64_t rowbase = R.c0 + (int64_t)wrap_index(cy + oy, ny) * nx;
       uint32_t pend_b = 0, pend_e = 0;
       bool pend = false;
@@ -443,14 +441,15 @@ __device__ bool voronoi_walk(const Rep& R, const int32_t* pi, const GridView& G,
             continue;
           }
           // split cell: the sub-cells meeting the box
-          const int64_t ucx = (int64_t)cx + ox;
-          const int64_t x0 = cell_lo(ucx, nx, Lx), y0 = cell_lo(ucy, ny, Ly);
-          const int64_t wx = cell_lo(ucx + 1, nx, Lx) - x0, wy = cell_lo(ucy + 1, ny, Ly) - y0;
+          const int64_t wx = (int64_t)1 << shx, wy = (int64_t)1 << shy;
+          const int64_t x0 = cell_lo2(cx + ox, nx, shx, Lx), y0 = cell_lo2(cy + oy, ny, shy, Ly);
           const int64_t lx = px + b[0] - x0, hx = px + b[1] - x0;
           const int64_t ly = py + b[2] - y0, hy = py + b[3] - y0;
           if (hx < 0 || lx >= wx || hy < 0 || ly >= wy) continue;
-          const int sx0 = lx <= 0 ? 0 : sub_index(lx, wx, s), sx1 = hx >= wx ? s - 1 : sub_index(hx, wx, s);
-          const int sy0 = ly <= 0 ? 0 : sub_index(ly, wy, s), sy1 = hy >= wy ? s - 1 : sub_index(hy, wy, s);
+          const int sx0 = lx <= 0 ? 0 : sub_of(cell_frac((uint32_t)lx, shx), s);
+          const int sx1 = hx >= wx ? s - 1 : sub_of(cell_frac((uint32_t)hx, shx), s);
+          const int sy0 = ly <= 0 ? 0 : sub_of(cell_frac((uint32_t)ly, shy), s);
+          const int sy1 = hy >= wy ? s - 1 : sub_of(cell_frac((uint32_t)hy, shy), s);
           const uint32_t base = G.sub_base[g];
           for (int yy = sy0; yy <= sy1; ++yy) {
             const uint32_t rb = base + (uint32_t)yy * s;
@@ -481,10 +480,10 @@ __device__ bool voronoi_walk(const Rep& R, const int32_t* pi, const GridView& G,
     if (fullx && fully) return true;
     // stop once the scanned block holds the (current) box
     box(b);
-    const bool inx = fullx || (b[0] >= cell_lo((int64_t)cx - r, nx, Lx) - px &&
-                               b[1] <= cell_lo((int64_t)cx + r + 1, nx, Lx) - 1 - px);
-    const bool iny = fully || (b[2] >= cell_lo((int64_t)cy - r, ny, Ly) - py &&
-                               b[3] <= cell_lo((int64_t)cy + r + 1, ny, Ly) - 1 - py);
+    const bool inx = fullx || (b[0] >= cell_lo2(cx - r, nx, shx, Lx) - px &&
+                               b[1] <= cell_lo2(cx + r + 1, nx, shx, Lx) - 1 - px);
+    const bool iny = fully || (b[2] >= cell_lo2(cy - r, ny, shy, Ly) - py &&
+                               b[3] <= cell_lo2(cy + r + 1, ny, shy, Ly) - 1 - py);
     if (inx && iny && within_half(b, Lx, Ly)) return false;
   }
 }
