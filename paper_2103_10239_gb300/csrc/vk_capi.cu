@@ -316,7 +316,7 @@ vk_status enqueue_step(vk_sim* s) {
   else if (s->prm.rule == VK_RULE_KNN) VK_CUDA(s, launch_knn_step(s->g, s->b, P, s->stream));
   else if (s->prm.rule == VK_RULE_METRIC) VK_CUDA(s, launch_metric_step(s->g, s->b, P, s->stream));
   else if (s->dim == 2) VK_CUDA(s, launch_voronoi_step(s->g, s->b, P, s->stream));
-  else VK_CUDA(s, launch_voronoi3_step(s->g, s->b, P, s->prm.voronoi3_kernel, s->stream));
+  else VK_CUDA(s, launch_voronoi3_step(s->g, s->b, P, s->stream));
   const int deferred_launches = (s->prm.rule == VK_RULE_KNN && s->dim == 2) ? 2 : 0;
   if ((st = record_end(s, 0, e0, search_launches(s) - deferred_launches))) return st;
   if (deferred_launches) {
@@ -491,6 +491,8 @@ vk_status build_sim(int32_t n_rep, const int64_t* n_r, const int32_t* pos_q, con
         (e = dalloc(&s->b.slot_of, N)))
       return bail(cuda_fail(s, e, "Voronoi seed buffers"));
   }
+  if (params->rule == VK_RULE_VORONOI && dim == 3 && (e = prepare_voronoi3()))
+    return bail(cuda_fail(s, e, "3D Voronoi kernels"));
   if (ensure_cells_capacity(s)) return bail(VK_ERR_OOM);
   if ((e = cudaMemsetAsync(s->b.d_step, 0, sizeof(int64_t), s->stream)) ||
       (e = cudaMemsetAsync(s->b.ovf_count, 0, 2 * sizeof(int32_t), s->stream)) ||

@@ -32,7 +32,9 @@
 // with candidates limited to |d| < 2 R (R <= sqrt(3)/2 L) that is box edges up
 // to 2^23 grid units.
 //
-// The builder is plain C++ usable on the host and the device.
+// The predicates are plain C++ for the host and the device.  The kernels
+// (vk_voronoi3.cu) clip with a whole warp; cell_init, cell_clip and
+// face_positive below are the same steps written serially, for the host.
 #pragma once
 #include <cmath>
 #include <cstdint>

@@ -4,11 +4,11 @@
 
 namespace vk {
 
-// search + update of every particle: warp = 0 one thread per cell, 1 one warp
-// per cell (same results); the overflow kernel finishes the cells that
-// outgrow the main kernel's
-cudaError_t launch_voronoi3_step(const Geometry& g, const Buffers& b, const StepParams& P, int warp,
-                                 cudaStream_t st);
+// one-time kernel attributes (shared memory of the larger cells)
+cudaError_t prepare_voronoi3();
+// search + update of every particle (one warp per cell), then of the
+// particles whose cell outgrew the first kernel's
+cudaError_t launch_voronoi3_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
 // pass 0: deg[id] = neighbor count; pass 1: the ids of row id at out_off[id], sorted by id
 cudaError_t launch_voronoi3_export(const Geometry& g, const Buffers& b, int rep, int n, int pass, int32_t* deg,
                                    const int64_t* out_off, int32_t* out_ids, cudaStream_t st);
