@@ -6,28 +6,27 @@
 // Instead of a global (serial) triangulation, every particle builds its own
 // Voronoi cell by half-plane clipping, which is embarrassingly parallel:
 //   * the cell starts as the square bounded by the particle's own periodic
-//     images (+-L_x, 0), (0, +-L_y);
-//   * candidates arrive ring by ring from the cell grid; each one clips the
-//     convex polygon by its bisector.  The polygon is a cyclic list of the
-//     sites that define its edges; a vertex is the circumcenter of the particle
-//     (at the origin) and two consecutive sites.  "Vertex beyond the bisector
-//     of m" is exactly incircle(0, a, b, m) > 0, i.e. 2 m.V > |m|^2: decided
-//     from an FP32 estimate of V with a rigorous error bound, else by an FP32
-//     filter of the incircle determinant, else exactly in int128;
+//     images (+-L_x, 0), (0, +-L_y), and every candidate of the cell grid clips
+//     it by its bisector.  The polygon is a cyclic list of the sites that define
+//     its edges; a vertex is the circumcenter of the particle (at the origin)
+//     and two consecutive sites.  "Vertex beyond the bisector of m" is exactly
+//     incircle(0, a, b, m) > 0, i.e. 2 m.V > |m|^2: decided from an FP32
+//     estimate of V with a rigorous error bound, else by an FP32 filter of the
+//     incircle determinant, else exactly in int128;
 //   * a site can still cut the cell only inside the union of the disks
 //     through the particle centred at the vertices (the disk of V holds the
 //     points closer to V than the particle is); its bounding box, the
-//     relevance box, only shrinks.  The walk skips rows and cells that miss
-//     it and stops once the scanned block holds it;
-//   * a cell that outgrows 32 edges or needs more than kHeavy candidates
-//     (a particle bordering a void) is finished by the overflow kernel, one
-//     warp per cell: the lanes test 32 candidates at a time against the
+//     relevance box, only shrinks;
+//   * ordinary cells: vk_voronoi_fast.cuh.  A cell that outgrows 16 edges, meets
+//     more than kHeavy candidates (a particle bordering a void), reaches half a
+//     period or has coincident particles is finished by the overflow kernel,
+//     one warp per cell: the lanes test 32 candidates at a time against the
 //     current cell and one lane applies the few that cut it;
 //   * neighbors are the sites of edges with positive length (an edge between
 //     two coincident vertices, i.e. four cocircular points, is dropped);
 //   * coincident particles form one site (see Poly).
 // Exact predicates need |relative coordinates| < 1.5 * 2^30, hence L_q <= 2^30.
-#include "vk_voronoi.cuh"
+#include "vk_voronoi_fast.cuh"
 
 namespace vk {
 
@@ -76,62 +75,150 @@ __device__ __forceinline__ void voronoi_update(const Rep& R, const StepParams& P
 constexpr uint32_t kHeavyHint = VK_VOR_HEAVY_HINT > 0 ? VK_VOR_HEAVY_HINT : 0xFFFFFFFFu;
 constexpr uint32_t kHeavyKeep = VK_VOR_HEAVY_HINT > 0 ? VK_VOR_HEAVY_HINT / 2 : 0xFFFFFFFFu;
 
-// Main kernel: cells of up to kFastCap edges.  Particles whose cell outgrows
-// it are appended to the overflow list and finished by the overflow kernel.
-// resident 256-thread blocks per SM the main kernel is compiled for
+// Main kernel: the ordinary cells, eight lanes each (vk_voronoi_fast.cuh).
+// The others go on the overflow list.  A warp builds the cells of 4 x ROUNDS
+// consecutive particles, four at a time, and then updates them, one per lane.
+// A cell that met more than kSeedMin candidates keeps its neighbors as the
+// next step's seeds: a particle beside a void has a wide box until its own
+// neighbors bound the cell, while the nearest particles bound an ordinary one
+// as well.
+constexpr uint32_t kSeedMin = 160;
+constexpr int kCellBlk = 128;
+// resident blocks per SM the main kernel is compiled for
 #ifndef VK_VOR_MIN_BLOCKS
-#define VK_VOR_MIN_BLOCKS 2
+#define VK_VOR_MIN_BLOCKS 4
 #endif
-// threads per block of the main kernel: each 256-particle block task is
-// split into kBlock / VK_VOR_BLOCK blocks, so that the few slow cells (void
-// rims) hold back smaller blocks and the SMs stay evenly loaded
-#ifndef VK_VOR_BLOCK
-#define VK_VOR_BLOCK 256
-#endif
-constexpr int kVorBlock = VK_VOR_BLOCK;
-constexpr int kVorSplit = kBlock / kVorBlock;
 
-__global__ void __launch_bounds__(kVorBlock, VK_VOR_MIN_BLOCKS * kVorSplit) voronoi_step_kernel(
+template <int ROUNDS>
+__global__ void __launch_bounds__(kCellBlk, VK_VOR_MIN_BLOCKS) voronoi_step_kernel(
     const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const int2* __restrict__ S_pos,
     const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G,
     int2* __restrict__ U_pos, float2* __restrict__ U_dir, int32_t* __restrict__ U_id,
     uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams Pm,
-    int2* __restrict__ ovf_list, int32_t* __restrict__ ovf_count, int32_t* status, int32_t* __restrict__ vor_seed,
+    int2* __restrict__ ovf_list, int32_t* __restrict__ ovf_count, int32_t* __restrict__ vor_seed,
     int32_t* __restrict__ vor_seed_n, const int32_t* __restrict__ slot_of) {
   __shared__ PhiShared phs;
   phi_block_begin(phs);
-  const BlockTask t = tasks[blockIdx.x / kVorSplit];
-  const Rep R = reps[t.rep];
-  const int li = t.first + (int)(blockIdx.x % kVorSplit) * kVorBlock + (int)threadIdx.x;
+  constexpr int kPerBlock = kCellBlk / kCG * ROUNDS, kPerWarp = 4 * ROUNDS, kBlocks = kBlock / kPerBlock;
+  const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
+  const BlockTask t = tasks[blockIdx.x / kBlocks];
+  const Rep& R = reps[t.rep];
+  const int li0 = t.first + (int)(blockIdx.x % kBlocks) * kPerBlock + wid * kPerWarp;
   const int64_t step = *d_step;
-  float nnew[3] = {0.f, 0.f, 0.f};
-  uint32_t n_cand = 0, n_runs = 0;
-  if (li < R.n) {
-    const int64_t s = R.p0 + li;
+  Cell8 c;
+  c.gl = lane & (kCG - 1);
+  c.base = lane & ~(kCG - 1);
+  // of the warp's particle number `lane`
+  HeadSum<2> sum;
+  sum.init();
+  int my_m = -1;
+  uint32_t my_seen = 0;
+#pragma unroll 1
+  for (int r = 0; r < ROUNDS; ++r) {
+    const int li = li0 + 4 * r + lane / kCG;
+    const bool on = li < R.n;
+    if (!__any_sync(kAll, on)) break;
+    const int64_t s = R.p0 + (on ? li : 0);
     const int2 p = S_pos[s];
-    const float2 nv = S_dir[s];
-    const int32_t pi[3] = {p.x, p.y, 0};
-    const float ni[3] = {nv.x, nv.y, 0.f};
     const int32_t id = S_id[s];
     const int64_t gi = R.p0 + id;
-    const int32_t sw = vor_seed ? vor_seed_n[gi] : 0;
-    const Seeds sd{vor_seed ? vor_seed + gi * kVorSeed : nullptr, sw & kSeedCount, slot_of};
-    Poly<kFastCap> P;
-    uint32_t seen = 0;
+    const int32_t sw = vor_seed && on ? vor_seed_n[gi] : 0;
+    const Seeds sd{vor_seed ? vor_seed + gi * kVorSeed : nullptr, min(sw & kSeedCount, kVorSeed), slot_of};
     // a cell that was heavy at the last step goes straight to the warp kernel
-    const bool ok = !(sw & kSeedHeavy) &&
-                    (Pm.stats ? voronoi_cell(R, s, pi, id, S_pos, S_id, G, P, status, kHeavy, sd, &seen, &n_cand,
-                                             &n_runs)
-                              : voronoi_cell(R, s, pi, id, S_pos, S_id, G, P, status, kHeavy, sd, &seen));
-    if (ok) {
-      voronoi_update(R, Pm, step, s, P, pi, ni, id, S_dir, U_pos, U_dir, U_id, counts, nnew,
-                     vor_seed ? vor_seed + gi * kVorSeed : nullptr, vor_seed_n + gi, seen > kHeavyHint);
-    } else {
-      const int q = atomicAdd(ovf_count, 1);
-      ovf_list[q] = make_int2((int)s, t.rep);
+    const bool mine = on && !(sw & kSeedHeavy);
+    c.build(mine, R, s, p, S_pos, G, sd, kHeavy);
+    const bool ok = mine && !c.other;
+    if (on && !ok && c.gl == 0) ovf_list[atomicAdd(ovf_count, 1)] = make_int2((int)s, t.rep);
+    // neighbors: the sites of edges of positive length, ordered by id
+    const unsigned kept = c.neighbor_edges();
+    const int cnt = __popc(kept);
+    const bool big = __any_sync(kAll, c.m > 8);
+    int32_t nid[2];
+    float2 d[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    int rank[2] = {0, 0};
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      nid[i] = INT_MAX;
+      if (ok && (kept >> (c.gl + 8 * i) & 1u)) {
+        nid[i] = __ldg(S_id + c.slot[i]);
+        d[i] = __ldg(S_dir + c.slot[i]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kCG; ++j) {
+      const int32_t o = __shfl_sync(kAll, nid[0], c.base + j);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) rank[i] += o < nid[i] ? 1 : 0;
+    }
+    if (big)
+#pragma unroll
+      for (int j = 0; j < kCG; ++j) {
+        const int32_t o = __shfl_sync(kAll, nid[1], c.base + j);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) rank[i] += o < nid[i] ? 1 : 0;
+      }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (nid[i] == INT_MAX) rank[i] = -1;
+    HeadSum<2> H;
+    H.init();
+    if (Pm.include_self) {
+      const float2 nv = S_dir[s];
+      const float ni[2] = {nv.x, nv.y};
+      H.add(ni, Pm.sum_mode);
+    }
+    for (int k = 0; __any_sync(kAll, ok && k < cnt); ++k) {
+      const bool second = rank[1] == k;
+      const unsigned who = c.group_bits(rank[0] == k || second);
+      const int from = c.base + (who ? __ffs(who) - 1 : 0);
+      const float v[2] = {__shfl_sync(kAll, second ? d[1].x : d[0].x, from),
+                          __shfl_sync(kAll, second ? d[1].y : d[0].y, from)};
+      if (who) H.add(v, Pm.sum_mode);
+    }
+    if (vor_seed && ok) {
+      const bool keep = c.n_seen > kSeedMin;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (keep && rank[i] >= 0 && rank[i] < kVorSeed) vor_seed[gi * kVorSeed + rank[i]] = nid[i];
+      if (c.gl == 0) vor_seed_n[gi] = keep ? min(cnt, kVorSeed) | (c.n_seen > kHeavyHint ? kSeedHeavy : 0) : 0;
+    }
+    // hand the sums to the lanes of these four particles
+    const int from = (lane & 3) * kCG;
+    const bool take = lane >> 2 == r;
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const float ts = __shfl_sync(kAll, H.s[a], from), tc = __shfl_sync(kAll, H.c[a], from);
+      const double td = Pm.sum_mode == 2 ? __shfl_sync(kAll, H.d[a], from) : 0.0;
+      if (take) {
+        sum.s[a] = ts;
+        sum.c[a] = tc;
+        sum.d[a] = td;
+      }
+    }
+    const int tm = __shfl_sync(kAll, ok ? cnt : -1, from);
+    const uint32_t tn = __shfl_sync(kAll, c.n_seen, from);
+    if (take) {
+      my_m = tm;
+      my_seen = tn;
     }
   }
-  record_search_stats(Pm.stats, li < R.n, n_cand, n_runs);
+  float nnew[3] = {0.f, 0.f, 0.f};
+  const bool valid = lane < kPerWarp && li0 + lane < R.n;
+  if (my_m >= 0) {
+    const int64_t s = R.p0 + li0 + lane;
+    const int2 p = S_pos[s];
+    const float2 nv = S_dir[s];
+    const int32_t id = S_id[s];
+    const int32_t pi[3] = {p.x, p.y, 0};
+    const float ni[3] = {nv.x, nv.y, 0.f};
+    int32_t pout[3] = {0, 0, 0};
+    align_advect<2>(R, Pm, (uint32_t)step, id, ni, sum, my_m + (Pm.include_self ? 1 : 0), pi, pout, nnew);
+    U_pos[s] = make_int2(pout[0], pout[1]);
+    U_dir[s] = make_float2(nnew[0], nnew[1]);
+    U_id[s] = id;
+    atomicAdd(counts + linear_cell<2>(R, pout), 1u);
+  }
+  record_search_stats(Pm.stats, valid, my_seen, 0, my_m < 0);
   phi_block_end<2>(phs, nnew, phi_acc + ((size_t)(step % Pm.phi_cap) * (size_t)Pm.n_rep + (size_t)t.rep) * 3);
 }
 
@@ -233,12 +320,17 @@ static GridView grid_view(const Buffers& b) {
 
 cudaError_t launch_voronoi_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
   const GridView G = grid_view(b);
-  voronoi_step_kernel<<<g.n_tasks * kVorSplit, kVorBlock, 0, st>>>(g.reps, g.tasks, (const int2*)b.S_pos, (const float2*)b.S_dir,
-                                                    b.S_id, G, (int2*)b.U_pos, (float2*)b.U_dir, b.U_id,
-                                                    b.counts, b.phi_acc, b.d_step, P, b.ovf_list,
-                                                    b.ovf_count, b.d_status, b.vor_seed, b.vor_seed_n,
-                                                    b.slot_of);
-  voronoi_overflow_kernel<<<device_sm_count(), 32 * kOvfWarps, 0, st>>>(g.reps, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id,
+  // 32 cells per warp (one full update) where that still fills the chip, 4 in small systems
+  auto step = [&](auto kernel, int rounds) {
+    kernel<<<g.n_tasks * (kBlock / (kCellBlk / kCG * rounds)), kCellBlk, 0, st>>>(
+        g.reps, g.tasks, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id, G, (int2*)b.U_pos, (float2*)b.U_dir,
+        b.U_id, b.counts, b.phi_acc, b.d_step, P, b.ovf_list, b.ovf_count, b.vor_seed, b.vor_seed_n, b.slot_of);
+  };
+  const int64_t fill = (int64_t)device_sm_count() * VK_VOR_MIN_BLOCKS * (kCellBlk / kCG) * 3;
+  if (g.n_total >= 8 * fill) step(voronoi_step_kernel<8>, 8);
+  else if (g.n_total >= 2 * fill) step(voronoi_step_kernel<2>, 2);
+  else step(voronoi_step_kernel<1>, 1);
+  voronoi_overflow_kernel<<<device_sm_count() * 4, 32 * kOvfWarps, 0, st>>>(g.reps, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id,
                                               G, (int2*)b.U_pos, (float2*)b.U_dir, b.U_id,
                                               b.counts, b.phi_acc, b.d_step, P, b.ovf_list, b.ovf_count,
                                               b.d_status, b.vor_seed, b.vor_seed_n, b.slot_of);
