@@ -299,10 +299,10 @@ vk_status clear_phi(vk_sim* s) {
 
 // kernels of the search+update phase: for 2D kNN the radius-first kernel,
 // the kernel of the particles it hands on and that of the few that need the
-// whole box; one for 3D kNN and for the metric rule; the Voronoi kernel and
+// whole box; two for 3D kNN; one for the metric rule; the Voronoi kernel and
 // its overflow kernel
 int search_launches(const vk_sim* s) {
-  if (s->prm.rule == VK_RULE_KNN) return s->dim == 2 ? 3 : 1;
+  if (s->prm.rule == VK_RULE_KNN) return s->dim == 2 ? 3 : 2;
   if (s->prm.rule == VK_RULE_METRIC) return 1;
   return 2;
 }
@@ -483,7 +483,7 @@ vk_status build_sim(int32_t n_rep, const int64_t* n_r, const int32_t* pos_q, con
       (e = dalloc(&s->tasks_d, s->tasks_h.size())))
     return bail(cuda_fail(s, e, "cudaMalloc"));
   if (params->rule == VK_RULE_KNN) {
-    if ((e = dalloc(&s->b.S_hint, N)) || (e = dalloc(&s->b.U_hint, N)) || (dim == 2 && (e = prepare_knn2())))
+    if ((e = dalloc(&s->b.S_hint, N)) || (e = dalloc(&s->b.U_hint, N)) || (e = dim == 2 ? prepare_knn2() : prepare_knn3()))
       return bail(cuda_fail(s, e, "kNN search buffers"));
   }
   if (params->rule == VK_RULE_VORONOI && dim == 2 && !params->voronoi_rebuild) {

@@ -703,7 +703,8 @@ cudaError_t launch_hints_by_id(const Buffers& b, int64_t p0, int32_t n, cudaStre
 cudaError_t launch_import_state(const Geometry& g, const Buffers& b, int rep, int64_t p0, int32_t n,
                                 const int32_t* pos_in, const float* dir_in, cudaStream_t st);
 
-// vk_knn.cu (3D)
+// vk_knn.cu (3D); one-time kernel attributes first
+cudaError_t prepare_knn3();
 cudaError_t launch_knn_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
 cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out,
                               cudaStream_t st);

@@ -3,14 +3,18 @@
 // so the relation is not reciprocal) fused with the Vicsek update of Eq. (1)
 // and Eq. (2), in 3D (the 2D rule, the benchmark's, is in vk_knn2d.cu).
 //
-// One thread per particle, in cell-sorted order.  The search walks rings of
-// cells around the particle's cell; each row segment of a ring is one
-// contiguous run of the sorted arrays.  The k best (exact int64 squared
-// distance, id) pairs live in registers, sorted.  After ring r the search
-// stops once the k-th best distance is below the exact integer distance from
-// the particle to the boundary of the scanned (2r+1)^d block.
+// One thread per particle, in cell-sorted order, radius first: the cube around
+// the particle a little wider than its k-th distance at the last step; 16 lanes
+// each for the particles that this cube cannot serve.  The lists are exported by
+// a ring walk: it walks rings of cells around the particle's cell (each row
+// segment of a ring is one contiguous run of the sorted arrays), keeps the k
+// best (exact int64 squared distance, id) pairs in registers, and stops once
+// the k-th best distance is below the exact integer distance from the particle
+// to the boundary of the scanned (2r+1)^d block.
+#include <algorithm>
 #include <climits>
 
+#include "vk_group.cuh"
 #include "vk_internal.cuh"
 
 namespace vk {
@@ -101,12 +105,32 @@ __device__ __forceinline__ void knn_search(const Rep& R, int64_t self, const int
 // Radius first (3D): each particle scans the cube [p - a, p + a]^3, a a
 // little above its k-th neighbor distance at the previous step, as the
 // x-row segments of the cells it meets (each a contiguous run of the sorted
-// arrays, with the periodic image it lies in).  Every candidate with exact
-// squared distance D <= tau = (a+1)^2 - 1 goes into the register top-k by
-// (D, id); nothing outside the cube is that close, so once the k-th best is
-// <= tau the list is exact, ties included.  Otherwise one larger cube, then
-// the ring walk.
+// arrays, with the periodic image it lies in).  Nothing outside the cube is
+// closer than a + 1.  As in 2D (vk_knn2d.cu) the selection runs on 32-bit
+// keys, the FP32 squared distance with the hit's number in its low bits: a
+// 64-bit list with ids cost eight compares and moves per hit, run by the few
+// lanes that had one: 1943 us per step at 1M particles; this takes 1058, and 86
+// for the particles handed on.
+// Candidates within the cube's inscribed ball are buffered and merged after
+// the scan by min / max; a list whose order the keys leave open, or with too
+// few hits, is handed on.
 // ---------------------------------------------------------------------------
+constexpr int kBlk3 = 128;
+constexpr int kSplit3 = kBlock / kBlk3;
+constexpr int kRuns3 = 8;
+
+// KC keys (k <= KC - 1 and the one after them), CAP buffered hits (about 2.2 k
+// + 1 are expected) numbered in BITS bits
+template <int KC> struct CubeCfg;
+template <> struct CubeCfg<8> { static constexpr int CAP = 32, BITS = 5, BLOCKS = 5; };
+template <> struct CubeCfg<17> { static constexpr int CAP = 64, BITS = 6, BLOCKS = 3; };
+template <> struct CubeCfg<33> { static constexpr int CAP = 96, BITS = 7, BLOCKS = 2; };
+
+template <int KC>
+struct CubeShared {
+  uint2 hit[CubeCfg<KC>::CAP][kBlk3];  // (slot, bits of the FP32 squared distance), one column per thread
+  uint2 run[kRuns3][kBlk3];            // (first slot, length << 6 | image codes)
+};
 
 // unwrapped cell index of an unwrapped coordinate, -L <= x < 2L
 __device__ __forceinline__ int ucell3(int64_t x, int n, const uint32_t* __restrict__ bnd, float inv_w, int64_t L) {
@@ -115,64 +139,137 @@ __device__ __forceinline__ int ucell3(int64_t x, int n, const uint32_t* __restri
   return cell_of_tab((uint32_t)x, n, bnd, inv_w);
 }
 
-// the coordinate of the particle shifted into the image an unwrapped cell
-// index u lies in: offsets x_j - that are exact in wrapping 32-bit arithmetic
-__device__ __forceinline__ uint32_t image_ref(uint32_t p, int u, int n, uint32_t L) {
-  return u < 0 ? p + L : (u >= n ? p - L : p);
-}
-
-// the k nearest from the cube of half-width a; true when they are exact
+// the k nearest from the cube of half-width ceil(radius), as keys
+// t[KC-1-k .. KC-2] in order; false when it cannot decide, with the radius to
+// try next
 template <int KC>
-__device__ __forceinline__ bool cube_search(const Rep& R, const uint32_t* __restrict__ bounds, const GridView& G,
-                                            const int4* __restrict__ pos, const int32_t* __restrict__ ids,
-                                            int64_t self, const int32_t* pi, int64_t a, TopK<KC>& T,
+__device__ __forceinline__ bool cube_search(CubeShared<KC>& H, const Rep& R, const uint32_t* __restrict__ bounds,
+                                            const GridView& G, const int4* __restrict__ pos, int32_t self,
+                                            const int32_t* pi, float radius, int k, uint32_t* t, float* r_next,
                                             uint32_t* n_cand, uint32_t* n_runs) {
+  constexpr int B = CubeCfg<KC>::BITS, CAP = CubeCfg<KC>::CAP;
+  const int tid = (int)threadIdx.x;
+  const int32_t a = (int32_t)ceilf(fminf(radius, 1.0e9f));
+  *r_next = (float)a;
   int lo[3], hi[3];
 #pragma unroll
   for (int ax = 0; ax < 3; ++ax) {
     const int64_t L = R.L[ax];
-    if (2 * (2 * a + 1) >= L) return false;
+    if (4ll * a + 2 >= L) return false;
     const uint32_t* bnd = bounds + R.bnd[ax];
     lo[ax] = ucell3((int64_t)pi[ax] - a, R.nc[ax], bnd, R.inv_w[ax], L);
     hi[ax] = ucell3((int64_t)pi[ax] + a, R.nc[ax], bnd, R.inv_w[ax], L);
     if (hi[ax] - lo[ax] + 1 > R.nc[ax]) return false;
   }
-  const uint64_t tau = (uint64_t)(a + 1) * (uint64_t)(a + 1) - 1;
+  const float a1 = (float)a + 1.0f;
+  float tau = a1 * a1 * (1.0f - 9.5367431640625e-07f);
+  const uint32_t edge = __float_as_uint(tau) >> B;
+#pragma unroll
+  for (int e = 0; e < KC; ++e) t[e] = e < KC - 1 - k ? 0u : 0xFFFFFFFFu;
   const int nx = R.nc[0], ny = R.nc[1], nz = R.nc[2];
-  for (int uz = lo[2]; uz <= hi[2]; ++uz) {
-    const int cz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
-    const uint32_t oz = image_ref((uint32_t)pi[2], uz, nz, R.L[2]);
-    for (int uy = lo[1]; uy <= hi[1]; ++uy) {
-      const int cy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy);
-      const uint32_t oy = image_ref((uint32_t)pi[1], uy, ny, R.L[1]);
-      const int64_t row = R.c0 + ((int64_t)cz * ny + cy) * nx;
-      // the x range splits at the period into up to three segments
-      for (int seg = 0; seg < 3; ++seg) {
-        int xs = seg == 0 ? lo[0] : (seg == 1 ? max(lo[0], 0) : max(lo[0], nx));
-        int xe = seg == 0 ? min(hi[0], -1) : (seg == 1 ? min(hi[0], nx - 1) : hi[0]);
-        if (xs > xe) continue;
-        const uint32_t ox = image_ref((uint32_t)pi[0], xs, nx, R.L[0]);
-        const int wxs = xs < 0 ? xs + nx : (xs >= nx ? xs - nx : xs);
-        const uint32_t qb = __ldg(G.off + row + wxs), qe = __ldg(G.off + row + wxs + (xe - xs) + 1);
-        if (n_cand) {
-          *n_cand += qe - qb;
-          *n_runs += 1;
-        }
-        for (uint32_t q = qb; q < qe; ++q) {
-          const int4 pj = __ldg(pos + q);
-          const int32_t dx = (int32_t)((uint32_t)pj.x - ox), dy = (int32_t)((uint32_t)pj.y - oy),
-                        dz = (int32_t)((uint32_t)pj.z - oz);
-          const uint64_t D = (uint64_t)((int64_t)dx * dx) + (uint64_t)((int64_t)dy * dy) +
-                             (uint64_t)((int64_t)dz * dz);
-          if (D <= tau && D <= T.d[KC - 1] && (int64_t)q != self) {
-            const int32_t idj = __ldg(ids + q);
-            if (D < T.d[KC - 1] || idj < T.id[KC - 1]) topk_insert<KC>(T, D, idj, (int32_t)q);
+  int cnt = 0, merged = 0, got = 0;
+  int uy = lo[1], uz = lo[2], seg = 0, nrun = 0, r = 0;
+  uint32_t q = 0, qe = 0, ox = 0, oy = 0, oz = 0;
+  bool more = true, done = false;
+  for (;;) {
+    while (cnt <= CAP - 2) {
+      if (q == qe) {
+        if (r == nrun) {
+          nrun = r = 0;
+          while (more && nrun < kRuns3) {
+            const int cz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
+            const int cy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy);
+            const int64_t row = R.c0 + ((int64_t)cz * ny + cy) * nx;
+            // the x range splits at the period into up to three segments
+            const int xs = seg == 0 ? lo[0] : (seg == 1 ? max(lo[0], 0) : max(lo[0], nx));
+            const int xe = seg == 0 ? min(hi[0], -1) : (seg == 1 ? min(hi[0], nx - 1) : hi[0]);
+            if (xs <= xe) {
+              const int wx = xs < 0 ? xs + nx : (xs >= nx ? xs - nx : xs);
+              const uint32_t qb = __ldg(G.off + row + wx), qf = __ldg(G.off + row + wx + (xe - xs) + 1);
+              // image codes per axis: 0 same, 1 at -L, 2 at +L
+              const uint32_t code = (xs < 0 ? 1u : xs >= nx ? 2u : 0u) | (uy < 0 ? 4u : uy >= ny ? 8u : 0u) |
+                                    (uz < 0 ? 16u : uz >= nz ? 32u : 0u);
+              if (qf > qb) H.run[nrun++][tid] = make_uint2(qb, (qf - qb) << 6 | code);
+            }
+            if (++seg == 3 || (lo[0] >= 0 && hi[0] < nx && seg == 2)) {
+              seg = lo[0] >= 0 && hi[0] < nx ? 1 : 0;
+              if (++uy > hi[1]) {
+                uy = lo[1];
+                if (++uz > hi[2]) more = false;
+              }
+            }
+          }
+          *n_runs += (uint32_t)nrun;
+          if (nrun == 0) {
+            done = true;
+            break;
           }
         }
+        const uint2 e = H.run[r++][tid];
+        q = e.x;
+        qe = e.x + (e.y >> 6);
+        *n_cand += e.y >> 6;
+        // the particle shifted into the run's periodic image: offsets x_j - ox exactly
+        ox = (uint32_t)pi[0] + (e.y & 1u ? R.L[0] : 0u) - (e.y & 2u ? R.L[0] : 0u);
+        oy = (uint32_t)pi[1] + (e.y & 4u ? R.L[1] : 0u) - (e.y & 8u ? R.L[1] : 0u);
+        oz = (uint32_t)pi[2] + (e.y & 16u ? R.L[2] : 0u) - (e.y & 32u ? R.L[2] : 0u);
+      }
+      // two candidates at a time (the second of an odd run's end is masked)
+      const int4 p0 = __ldg(pos + q), p1 = __ldg(pos + min(q + 1, qe - 1));
+      const int4 ps[2] = {p0, p1};
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const float fx = (float)(int32_t)((uint32_t)ps[u].x - ox), fy = (float)(int32_t)((uint32_t)ps[u].y - oy),
+                    fz = (float)(int32_t)((uint32_t)ps[u].z - oz);
+        const float D = __fmaf_rn(fx, fx, __fmaf_rn(fy, fy, __fmul_rn(fz, fz)));
+        H.hit[cnt][tid] = make_uint2(q + (uint32_t)u, __float_as_uint(D));
+        cnt += D <= tau && q + (uint32_t)u < qe ? 1 : 0;
+      }
+      q = min(q + 2, qe);
+      if (q == qe && r == nrun && !more) {
+        done = true;
+        break;
       }
     }
+#pragma unroll 2
+    for (int b = merged; b < cnt; ++b) {
+      const uint2 h = H.hit[b][tid];
+      const bool keep = (int32_t)h.x != self;
+      got += keep ? 1 : 0;
+      uint32_t x = keep ? (h.y & ~((1u << B) - 1u)) | (uint32_t)b : 0xFFFFFFFFu;
+#pragma unroll
+      for (int e = 0; e < KC; ++e) {
+        const uint32_t m = min(t[e], x);
+        x = max(t[e], x);
+        t[e] = m;
+      }
+    }
+    if (done) break;
+    // full column: its KC best move to the front and keep their order
+    merged = 0;
+    uint2 best[KC];
+#pragma unroll
+    for (int e = 0; e < KC; ++e)
+      if (e >= KC - 1 - k && t[e] != 0xFFFFFFFFu) best[e] = H.hit[t[e] & ((1u << B) - 1u)][tid];
+#pragma unroll
+    for (int e = 0; e < KC; ++e)
+      if (e >= KC - 1 - k && t[e] != 0xFFFFFFFFu) {
+        H.hit[merged][tid] = best[e];
+        t[e] = (t[e] & ~((1u << B) - 1u)) | (uint32_t)merged;
+        ++merged;
+      }
+    cnt = merged;
+    if (t[KC - 2] < 0xFF000000u) tau = fminf(tau, __uint_as_float(((t[KC - 2] >> B) + 3u) << B));
   }
-  return T.d[KC - 1] <= tau;
+  if ((t[KC - 2] >> B) + 1u < edge) {
+    bool close = false;  // a pair whose order the keys leave open
+#pragma unroll
+    for (int e = 0; e < KC - 1; ++e) close |= e >= KC - 1 - k && (t[e + 1] >> B) - (t[e] >> B) <= 1u;
+    return !close;
+  }
+  // too few: scale the radius towards about 1.6 k expected hits
+  *r_next = (float)a * (got > 0 ? fminf(cbrtf(1.6f * (float)(k + 1) / (float)got), 2.f) : 2.f);
+  return false;
 }
 
 // search radius without a hint: from the density of the particle's own cell
@@ -191,68 +288,263 @@ __device__ __forceinline__ float cube_radius_estimate(const Rep& R, const uint32
   return 1.3f * cbrtf(3.f * (float)k * vol / (4.f * 3.14159265f * m));
 }
 
-template <int DIM, int KC>
-__global__ void __launch_bounds__(kBlock) knn_step_kernel(
-    const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks,
-    const typename Vec<DIM>::P* __restrict__ S_pos, const typename Vec<DIM>::F* __restrict__ S_dir,
-    const int32_t* __restrict__ S_id, GridView G, typename Vec<DIM>::P* __restrict__ U_pos,
-    typename Vec<DIM>::F* __restrict__ U_dir, int32_t* __restrict__ U_id,
-    uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P,
-    const uint32_t* __restrict__ bounds, const float* __restrict__ S_hint, float* __restrict__ U_hint) {
-  using PV = typename Vec<DIM>::P;
-  using FV = typename Vec<DIM>::F;
-  const BlockTask t = tasks[blockIdx.x];
+// Eq. (2) + Eq. (1) of one particle; at(j) is the slot of list entry j in
+// [KC-1-k, KC-1), in (D, id) order.  Writes the next state and counts the new cell.
+template <int KC, class At>
+__device__ __forceinline__ void knn3_update(const Rep& R, const StepParams& P, int64_t step, int64_t s,
+                                            const int32_t* pi, int32_t id, At at, const float4* __restrict__ S_dir,
+                                            int4* __restrict__ U_pos, float4* __restrict__ U_dir,
+                                            int32_t* __restrict__ U_id, uint32_t* __restrict__ counts,
+                                            const uint32_t* __restrict__ bounds, float* nnew) {
+  float ni[3];
+  unpack(S_dir[s], ni);
+  HeadSum<3> H;
+  H.init();
+  if (P.include_self) H.add(ni, P.sum_mode);
+#pragma unroll
+  for (int c = 0; c < KC - 1; c += 4) {
+    float4 d[4];  // four headings in flight, then summed in order
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c + u < KC - 1 && c + u >= KC - 1 - P.k) d[u] = __ldg(S_dir + at(c + u));
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c + u < KC - 1 && c + u >= KC - 1 - P.k) {
+        const float v[3] = {d[u].x, d[u].y, d[u].z};
+        H.add(v, P.sum_mode);
+      }
+  }
+  int32_t pout[3] = {0, 0, 0};
+  align_advect<3>(R, P, (uint32_t)step, id, ni, H, P.k + (P.include_self ? 1 : 0), pi, pout, nnew);
+  U_pos[s] = make_int4(pout[0], pout[1], pout[2], 0);
+  U_dir[s] = make_float4(nnew[0], nnew[1], nnew[2], 0.f);
+  U_id[s] = id;
+  int64_t lin = 0;
+#pragma unroll
+  for (int ax = 2; ax >= 0; --ax)
+    lin = lin * R.nc[ax] + cell_of_tab((uint32_t)pout[ax], R.nc[ax], bounds + R.bnd[ax], R.inv_w[ax]);
+  atomicAdd(counts + R.c0 + lin, 1u);
+}
+
+// Search + update, one cube per particle.  Particles it cannot serve go on the
+// list (slot, replica), with the radius to try next in U_hint.
+template <int KC>
+__global__ void __launch_bounds__(kBlk3, CubeCfg<KC>::BLOCKS) knn3_step_kernel(
+    const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const int4* __restrict__ S_pos,
+    const float4* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G, int4* __restrict__ U_pos,
+    float4* __restrict__ U_dir, int32_t* __restrict__ U_id, uint32_t* __restrict__ counts,
+    PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P,
+    const uint32_t* __restrict__ bounds, const float* __restrict__ S_hint, float* __restrict__ U_hint,
+    int2* __restrict__ list, int32_t* __restrict__ count) {
+  extern __shared__ __align__(16) unsigned char cube_smem[];
+  CubeShared<KC>& H = *reinterpret_cast<CubeShared<KC>*>(cube_smem);
+  __shared__ PhiShared phs;
+  phi_block_begin(phs);
+  const BlockTask t = tasks[blockIdx.x / kSplit3];
   const Rep R = reps[t.rep];
-  const int li = t.first + (int)threadIdx.x;
+  const int li = t.first + (int)(blockIdx.x % kSplit3) * kBlk3 + (int)threadIdx.x;
   const int64_t step = *d_step;
   float nnew[3] = {0.f, 0.f, 0.f};
   uint32_t n_cand = 0, n_runs = 0;
+  bool served = false;
   if (li < R.n) {
     const int64_t s = R.p0 + li;
-    int32_t pi[3] = {0, 0, 0};
-    float ni[3] = {0.f, 0.f, 0.f};
+    int32_t pi[3];
     unpack(S_pos[s], pi);
-    unpack(S_dir[s], ni);
-    const int32_t id = S_id[s];
-    TopK<KC> T;
-    bool done = false;
-    if (S_hint && P.knn_search == 0) {
-      // radius first: the hinted cube, then one larger
-      const float hint = S_hint[s];
-      float r = hint > 0.f ? P.halo_alpha * hint : cube_radius_estimate(R, bounds, G, pi, P.k);
-      for (int tr = 0; tr < 2 && !done; ++tr) {
-        topk_init<KC>(T, P.k);
-        done = cube_search<KC>(R, bounds, G, S_pos, S_id, s, pi, (int64_t)ceilf(fminf(r, 1.0e9f)), T,
-                               P.stats ? &n_cand : nullptr, &n_runs);
-        r *= 1.6f;
+    const float hint = S_hint[s];
+    const float r = hint > 0.f ? P.halo_alpha * hint : cube_radius_estimate(R, bounds, G, pi, P.k);
+    float r_next = r;
+    if (P.knn_search == 0) {
+      uint32_t key[KC];
+      served = cube_search<KC>(H, R, bounds, G, S_pos, (int32_t)s, pi, r, P.k, key, &r_next, &n_cand, &n_runs);
+      if (served) {
+        knn3_update<KC>(R, P, step, s, pi, S_id[s],
+                        [&](int j) { return H.hit[key[j] & ((1u << CubeCfg<KC>::BITS) - 1u)][threadIdx.x].x; }, S_dir,
+                        U_pos, U_dir, U_id, counts, bounds, nnew);
+        U_hint[s] = sqrtf(__uint_as_float(key[KC - 2])) * 1.0001f + 1.f;
       }
     }
-    if (!done) {
-      topk_init<KC>(T, P.k);
-      if (P.stats) knn_search<DIM, KC>(R, s, pi, S_pos, S_id, G, T, &n_cand, &n_runs);
-      else knn_search<DIM, KC>(R, s, pi, S_pos, S_id, G, T);
-    }
-    if (U_hint) U_hint[s] = sqrtf((float)T.d[KC - 1]) * 1.0001f + 1.f;
-    HeadSum<DIM> H;
-    H.init();
-    if (P.include_self) H.add(ni, P.sum_mode);
-#pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      if (j >= KC - P.k) {
-        float v[3];
-        unpack(S_dir[T.slot[j]], v);
-        H.add(v, P.sum_mode);
-      }
-    }
-    int32_t pout[3] = {0, 0, 0};
-    align_advect<DIM>(R, P, (uint32_t)step, id, ni, H, P.k + (P.include_self ? 1 : 0), pi, pout, nnew);
-    U_pos[s] = make_p(pout, (PV*)nullptr);
-    U_dir[s] = make_f(nnew, (FV*)nullptr);
-    U_id[s] = id;
-    atomicAdd(counts + linear_cell<DIM>(R, pout), 1u);
+    if (!served) U_hint[s] = r_next;
   }
-  record_search_stats(P.stats, li < R.n, n_cand, n_runs);
-  block_phi_accumulate<DIM>(nnew, phi_acc + ((size_t)(step % P.phi_cap) * (size_t)P.n_rep + (size_t)t.rep) * 3);
+  // one atomic per warp: its entries stay neighbors in the list
+  const unsigned m = __ballot_sync(0xffffffffu, li < R.n && !served);
+  if (m) {
+    const int lane = (int)(threadIdx.x & 31);
+    int base = 0;
+    if (lane == 0) base = atomicAdd(count, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (m >> lane & 1u) list[base + __popc(m & ((1u << lane) - 1u))] = make_int2((int)(R.p0 + li), t.rep);
+  }
+  record_search_stats(P.stats, served, n_cand, n_runs);
+  phi_block_end<3>(phs, nnew, phi_acc + ((size_t)(step % P.phi_cap) * (size_t)P.n_rep + (size_t)t.rep) * 3);
+}
+
+// A group of GS lanes searches for one particle, exactly (vk_group.cuh): the
+// lanes look up the rows of a cube's cells and scan them together.
+template <int GS, int CAP>
+struct Group3 : GroupTop<GS, CAP> {
+  using Top = GroupTop<GS, CAP>;
+  using Top::mask;
+  using Top::shift;
+  using Top::gl;
+  using Top::tau;
+  const int4* __restrict__ pos;
+  const uint32_t* __restrict__ bounds;
+  int32_t p[3];
+
+  __device__ __forceinline__ void run(const Rep& R, uint32_t qb, uint32_t qe) {
+    Top::n_cand += qe - qb;
+    for (uint32_t b = qb; b < qe; b += GS) {
+      const uint32_t q = b + (uint32_t)gl;
+      bool hit = false;
+      unsigned long long D = 0;
+      if (q < qe && (int32_t)q != Top::self) {
+        int32_t pj[3];
+        unpack(__ldg(pos + q), pj);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int64_t d = min_image((int64_t)pj[a] - p[a], (int64_t)R.L[a]);
+          D += (unsigned long long)(d * d);
+        }
+        hit = D <= tau;
+      }
+      Top::append(hit, D, q);
+    }
+  }
+
+  // Every candidate of the cube of half-width a (an axis along which it meets
+  // some cell twice is covered whole); true when it is the whole box.  Rows
+  // farther than tau are passed over: a list that has filled up on the way
+  // leaves little to scan.
+  __device__ __forceinline__ bool cube(const Rep& R, const GridView& G, int64_t a) {
+    int lo[3], hi[3];
+    bool all = true;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      const int64_t L = R.L[x];
+      lo[x] = 0;
+      hi[x] = R.nc[x] - 1;
+      if (2 * a + 1 < L) {
+        const int l = ucell3((int64_t)p[x] - a, R.nc[x], bounds + R.bnd[x], R.inv_w[x], L);
+        const int h = ucell3((int64_t)p[x] + a, R.nc[x], bounds + R.bnd[x], R.inv_w[x], L);
+        if (h - l < R.nc[x]) {
+          lo[x] = l;
+          hi[x] = h;
+          all = false;
+        }
+      }
+    }
+    tau = all ? ~0ull : (unsigned long long)(a + 1) * (unsigned long long)(a + 1) - 1;
+    const int nx = R.nc[0], ny = R.nc[1], nz = R.nc[2];
+    const int ry = hi[1] - lo[1] + 1, rows = ry * (hi[2] - lo[2] + 1);
+    for (int xs = lo[0]; xs <= hi[0];) {  // the x range splits at the period
+      const int wx = xs < 0 ? xs + nx : (xs >= nx ? xs - nx : xs);
+      const int xe = min(hi[0], xs < 0 ? -1 : (xs < nx ? nx - 1 : INT_MAX));
+      for (int r0 = 0; r0 < rows; r0 += GS) {
+        const int row = r0 + gl;
+        uint32_t qb = 0, qe = 0;
+        if (row < rows) {
+          const int uy = lo[1] + row % ry, uz = lo[2] + row / ry;
+          const int cy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy), cz = uz < 0 ? uz + nz : (uz >= nz ? uz - nz : uz);
+          const float dy = slab(1, cy, R), dz = slab(2, cz, R);
+          if ((dy * dy + dz * dz) * 0.99999f <= (float)tau) {
+            const int64_t rb = R.c0 + ((int64_t)cz * ny + cy) * nx;
+            qb = __ldg(G.off + rb + wx);
+            qe = __ldg(G.off + rb + wx + (xe - xs) + 1);
+          }
+        }
+        unsigned m = (__ballot_sync(mask, qe > qb) & mask) >> shift;
+        while (m) {
+          const int j = shift + __ffs(m) - 1;
+          m &= m - 1u;
+          run(R, __shfl_sync(mask, qb, j), __shfl_sync(mask, qe, j));
+        }
+      }
+      xs = xe + 1;
+    }
+    return all;
+  }
+
+  // (per lane) distance of cell slab c of axis x from the particle, over both images
+  __device__ __forceinline__ float slab(int x, int c, const Rep& R) const {
+    const uint32_t* bnd = bounds + R.bnd[x];
+    const int64_t l = (int64_t)__ldg(bnd + c) - p[x], h = (int64_t)__ldg(bnd + c + 1) - 1 - p[x], L = R.L[x];
+    if (l > 0) return (float)min(l, L - h);
+    if (h < 0) return (float)min(-h, L + l);
+    return 0.f;
+  }
+};
+
+// The listed particles: 16 lanes each, larger cubes until k hits are in one
+// (one thread each, with the ring walk as its last resort, took 500 us for the
+// few particles of a small system).  A warp takes up to 32 of them, its groups
+// search one after another, and then every lane updates one.
+constexpr int kGS3 = 16, kGroupBlk3 = 128;
+
+template <int KC>
+__global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_kernel(
+    const Rep* __restrict__ reps, const int4* __restrict__ S_pos, const float4* __restrict__ S_dir,
+    const int32_t* __restrict__ S_id, GridView G, int4* __restrict__ U_pos, float4* __restrict__ U_dir,
+    int32_t* __restrict__ U_id, uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc,
+    const int64_t* __restrict__ d_step, StepParams P, const uint32_t* __restrict__ bounds, float* U_hint,
+    const int2* __restrict__ list, const int32_t* __restrict__ count) {
+  constexpr int CAP = GroupCfg<KC>::CAP, NG = 32 / kGS3, NW = kGroupBlk3 / 32;
+  __shared__ GroupList<CAP> lists[kGroupBlk3 / kGS3];
+  __shared__ int32_t res[NW][32][KC - 1];
+  __shared__ float res_d[NW][32];
+  const int total = *count;
+  const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
+  const int nw = (int)gridDim.x * NW, w = (int)blockIdx.x * NW + wid;
+  const int chunk = min(32, (int)(((int64_t)total + (int64_t)nw * NG - 1) / ((int64_t)nw * NG)) * NG);
+  const int64_t step = *d_step;
+  const int k = P.k;
+  for (int64_t base = (int64_t)w * chunk; base < total; base += (int64_t)nw * chunk) {
+    const int todo = (int)min((int64_t)chunk, (int64_t)total - base);
+    for (int i = lane / kGS3; i < todo; i += NG) {
+      const int2 e = list[base + i];
+      const Rep& R = reps[e.y];
+      const int4 p = S_pos[e.x];
+      Group3<kGS3, CAP> g{{lists[threadIdx.x / kGS3], S_id, ((1u << kGS3) - 1u) << (lane / kGS3 * kGS3),
+                           lane / kGS3 * kGS3, lane % kGS3, e.x},
+                          S_pos, bounds, {p.x, p.y, p.z}};
+      g.k = k;
+      g.n_cand = 0;
+      float r = U_hint[e.x];
+      uint32_t tries = 1;
+      for (;; ++tries) {
+        const int64_t a = (int64_t)ceilf(fminf(r, 4.0e9f));
+        g.cnt = 0;
+        if (g.cube(R, G, a) || g.cnt >= k) break;
+        r = (float)a * (g.cnt > 0 ? fminf(cbrtf(1.6f * (float)(k + 1) / (float)g.cnt), 2.f) : 2.f) + 1.f;
+      }
+      __syncwarp(g.mask);
+      g.rank([&](int, int rk, unsigned long long D, int32_t q) {
+        if (rk < k) res[wid][i][rk] = q;
+        if (rk == k - 1) res_d[wid][i] = (float)D;
+      });
+      __syncwarp(g.mask);
+      if (P.stats && g.gl == 0) {
+        atomicAdd(P.stats + 0, (unsigned long long)g.n_cand);
+        atomicAdd(P.stats + 1, (unsigned long long)tries);
+        atomicMax(P.stats + 2, (unsigned long long)g.n_cand);
+        atomicAdd(P.stats + 3, 1ull);
+      }
+    }
+    __syncwarp();
+    int2 e = make_int2(0, 0);
+    float nnew[3] = {0.f, 0.f, 0.f};
+    const bool mine = lane < todo;
+    if (mine) {
+      e = list[base + lane];
+      int32_t pi[3];
+      unpack(S_pos[e.x], pi);
+      knn3_update<KC>(reps[e.y], P, step, e.x, pi, S_id[e.x], [&](int j) { return res[wid][lane][j - (KC - 1 - k)]; },
+                      S_dir, U_pos, U_dir, U_id, counts, bounds, nnew);
+      U_hint[e.x] = sqrtf(res_d[wid][lane]) * 1.0001f + 1.f;
+    }
+    phi_add_warp<3>(phi_acc + (size_t)(step % P.phi_cap) * (size_t)P.n_rep * 3, e.y, nnew, mine);
+    __syncwarp();
+  }
 }
 
 // neighbor lists of the current positions of one replica, written by id
@@ -285,14 +577,24 @@ GridView grid_view(const Buffers& b) {
   return G;
 }
 
-template <int DIM, int KC>
+template <int KC>
 cudaError_t step_dispatch(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
-  using PV = typename Vec<DIM>::P;
-  using FV = typename Vec<DIM>::F;
-  knn_step_kernel<DIM, KC><<<g.n_tasks, kBlock, 0, st>>>(
-      g.reps, g.tasks, (const PV*)b.S_pos, (const FV*)b.S_dir, b.S_id, grid_view(b), (PV*)b.U_pos,
-      (FV*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.S_hint, b.U_hint);
+  const size_t smem = sizeof(CubeShared<KC>);
+  knn3_step_kernel<KC><<<g.n_tasks * kSplit3, kBlk3, smem, st>>>(
+      g.reps, g.tasks, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view(b), (int4*)b.U_pos,
+      (float4*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.S_hint, b.U_hint, b.ovf_list,
+      b.ovf_count);
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((g.n_total + 7) / 8, (int64_t)device_sm_count() * 5));
+  knn3_group_kernel<KC><<<blocks, kGroupBlk3, 0, st>>>(
+      g.reps, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view(b), (int4*)b.U_pos, (float4*)b.U_dir,
+      b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.U_hint, b.ovf_list, b.ovf_count);
   return cudaGetLastError();
+}
+
+template <int KC>
+cudaError_t prepare3() {
+  return cudaFuncSetAttribute(knn3_step_kernel<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)sizeof(CubeShared<KC>));
 }
 
 template <int DIM, int KC>
@@ -307,11 +609,18 @@ cudaError_t export_dispatch(const Geometry& g, const Buffers& b, int k, int rep,
 
 }  // namespace
 
+cudaError_t prepare_knn3() {
+  cudaError_t e = prepare3<8>();
+  if (e == cudaSuccess) e = prepare3<17>();
+  if (e == cudaSuccess) e = prepare3<33>();
+  return e;
+}
+
 cudaError_t launch_knn_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
   if (g.dim != 3) return cudaErrorInvalidValue;  // 2D: launch_knn2_step
-  if (P.k <= 8) return step_dispatch<3, 8>(g, b, P, st);
-  if (P.k <= 16) return step_dispatch<3, 16>(g, b, P, st);
-  return step_dispatch<3, 32>(g, b, P, st);
+  if (P.k <= 7) return step_dispatch<8>(g, b, P, st);
+  if (P.k <= 16) return step_dispatch<17>(g, b, P, st);
+  return step_dispatch<33>(g, b, P, st);
 }
 
 cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out,

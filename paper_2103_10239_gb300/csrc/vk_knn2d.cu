@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "vk_box2d.cuh"
+#include "vk_group.cuh"
 
 namespace vk {
 
@@ -237,104 +238,31 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
   return false;
 }
 
-// ---------------------------------------------------------------------------
-// A group of GS lanes searches for one particle, exactly.  Hits (D <= tau)
-// are appended to the group's list by ballot; a nearly full list keeps its k
-// best, and tau follows.  All lanes of the group call every function here.
-// ---------------------------------------------------------------------------
-template <int CAP>
-struct GroupList {
-  unsigned long long d[CAP];
-  int32_t slot[CAP];
-};
-
-template <int KC> struct GroupCfg { static constexpr int CAP = KC <= 12 ? 64 : KC <= 17 ? 96 : 160; };
-
+// A group of GS lanes searches for one particle, exactly (vk_group.cuh).
 template <int GS, int CAP, bool FOV>
-struct Group {
-  GroupList<CAP>& L;
+struct Group : GroupTop<GS, CAP> {
+  using Top = GroupTop<GS, CAP>;
+  using Top::mask;
+  using Top::shift;
+  using Top::gl;
+  using Top::tau;
   const int2* __restrict__ pos;
-  const int32_t* __restrict__ ids;
-  unsigned mask;      // the group's lanes
-  int shift, gl;      // its first lane, the lane's number in it
-  int32_t self;
   Ctx C;
-  int k, cnt;
-  unsigned long long tau;
-  uint32_t n_cand;
-
-  // the k best of the list by (D, id), in order, through put(rank, D, slot)
-  template <class F>
-  __device__ __forceinline__ void rank(F put) {
-    constexpr int E = (CAP + GS - 1) / GS;
-    __syncwarp(mask);
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int i = gl + e * GS;
-      if (e * GS >= cnt) break;
-      int r = INT_MAX;
-      unsigned long long D = 0;
-      int32_t q = 0;
-      if (i < cnt) {
-        D = L.d[i];
-        q = L.slot[i];
-        r = 0;
-        for (int j = 0; j < cnt; ++j) {
-          const unsigned long long Dj = L.d[j];
-          bool before = Dj < D;
-          if (Dj == D && j != i) before = __ldg(ids + L.slot[j]) < __ldg(ids + q);
-          r += before ? 1 : 0;
-        }
-      }
-      put(e, r, D, q);
-    }
-  }
-
-  __device__ __forceinline__ void compact() {
-    constexpr int E = (CAP + GS - 1) / GS;
-    int rk[E];
-    unsigned long long dk[E];
-    int32_t qk[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) rk[e] = INT_MAX;
-    rank([&](int e, int r, unsigned long long D, int32_t q) {
-      rk[e] = r;
-      dk[e] = D;
-      qk[e] = q;
-    });
-    __syncwarp(mask);
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-      if (rk[e] < k) {
-        L.d[rk[e]] = dk[e];
-        L.slot[rk[e]] = qk[e];
-      }
-    __syncwarp(mask);
-    cnt = min(cnt, k);
-    if (cnt == k) tau = L.d[k - 1];
-  }
 
   // the candidates of slots [qb, qe)
   __device__ __forceinline__ void run(int64_t qb, int64_t qe) {
-    n_cand += (uint32_t)(qe - qb);
+    Top::n_cand += (uint32_t)(qe - qb);
     for (int64_t b = qb; b < qe; b += GS) {
       const int64_t q = b + gl;
       bool hit = false;
       unsigned long long D = 0;
-      if (q < qe && (int32_t)q != self) {
+      if (q < qe && (int32_t)q != Top::self) {
         int32_t dx, dy;
         D = box_offset(C, __ldg(pos + q), dx, dy);
         hit = D <= tau;
         if (FOV) hit = hit && in_view(C.view, dx, dy, D);
       }
-      const unsigned m = (__ballot_sync(mask, hit) & mask) >> shift;
-      if (hit) {
-        const int at = cnt + __popc(m & ((1u << gl) - 1u));
-        L.d[at] = D;
-        L.slot[at] = (int32_t)q;
-      }
-      cnt += __popc(m);
-      if (cnt > CAP - GS) compact();
+      Top::append(hit, D, q);
     }
   }
 
@@ -721,8 +649,9 @@ __global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel
     for (int i = lane / kGS; i < todo; i += NG) {
       const int2 e = list[base + i];
       const Rep& R = reps[e.y];
-      Group<kGS, CAP, FOV> g{lists[threadIdx.x / kGS], S_pos, S_id, ((1u << kGS) - 1u) << (lane / kGS * kGS),
-                             lane / kGS * kGS, lane % kGS, e.x};
+      Group<kGS, CAP, FOV> g{{lists[threadIdx.x / kGS], S_id, ((1u << kGS) - 1u) << (lane / kGS * kGS),
+                              lane / kGS * kGS, lane % kGS, e.x},
+                             S_pos};
       init_ctx(g.C, R, e.x, S_pos[e.x]);
       if (FOV) g.C.view = make_view(out.S_dir[e.x], out.P.fov_cq);
       g.k = k;
