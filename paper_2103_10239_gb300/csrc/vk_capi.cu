@@ -697,10 +697,11 @@ vk_status vk_get_tissue(vk_sim* s, int32_t replica, double KA, double KP, double
   cudaError_t e = cudaSuccess;
   if (!s->tis_out) {
     const bool ok = !((e = dalloc(&w.nb_n, N)) || (e = dalloc(&w.nb_slot, N * kTissueCap)) ||
-                      (e = dalloc(&w.nb_off, N * kTissueCap)) || (e = dalloc(&w.area, N)) ||
+                      (e = dalloc(&w.nb_off, N * kTissueCap)) || (e = dalloc(&w.edge, N * kTissueCap)) ||
+                      (e = dalloc(&w.inv_len, N * kTissueCap)) || (e = dalloc(&w.blocks, kTissueBlocks)) || (e = dalloc(&w.area, N)) ||
                       (e = dalloc(&w.perim, N)) || (e = dalloc(&s->tis_out, 4 * N + 1)));
     if (!ok) {
-      void* part[] = {w.nb_n, w.nb_slot, w.nb_off, w.area, w.perim, s->tis_out};
+      void* part[] = {w.nb_n, w.nb_slot, w.nb_off, w.edge, w.inv_len, w.blocks, w.area, w.perim, s->tis_out};
       for (void* p : part)
         if (p) cudaFree(p);
       w = TissueScratch{};
@@ -716,7 +717,7 @@ vk_status vk_get_tissue(vk_sim* s, int32_t replica, double KA, double KP, double
   e = launch_tissue(s->g, s->b, replica, (int)n, KA, KP, A0, P0, unit, w, area_d, perim_d, force_d, energy_d,
                     s->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-  if (e == cudaSuccess) st = record_end(s, 4, e0, energy ? 3 : 2);
+  if (e == cudaSuccess) st = record_end(s, 4, e0, 1 + (area || perimeter || force) + (energy ? 2 : 0));
   if (e == cudaSuccess && st == VK_OK) st = read_status(s);
   if (e == cudaSuccess && st == VK_OK) {
     if (area) e = cudaMemcpy(area, area_d, sizeof(double) * n, cudaMemcpyDefault);
@@ -862,8 +863,8 @@ void vk_destroy(vk_sim* s) {
                   s->b.ovf_list, s->b.ovf_count, s->reps_d, s->tasks_d, s->b.sub_s, s->b.sub_base,
                   s->b.sub_count, s->b.sub_off, s->b.bsum2, s->d_stats, s->b.bounds,
                   s->st_pos, s->st_dir, s->st_theta, s->b.S_hint, s->b.U_hint, s->b.vor_seed,
-                  s->b.vor_seed_n, s->b.slot_of, s->tis.nb_n, s->tis.nb_slot, s->tis.nb_off, s->tis.area,
-                  s->tis.perim, s->tis_out};
+                  s->b.vor_seed_n, s->b.slot_of, s->tis.nb_n, s->tis.nb_slot, s->tis.nb_off, s->tis.edge,
+                  s->tis.inv_len, s->tis.blocks, s->tis.area, s->tis.perim, s->tis_out};
   for (void* p : bufs)
     if (p) cudaFree(p);
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);

@@ -728,12 +728,16 @@ cudaError_t launch_metric_export(const Geometry& g, const Buffers& b, int rep, i
 
 // vk_tissue.cu (Voronoi tissue model): per-slot scratch of the cells pass
 constexpr int kTissueCap = 32;  // edges per cell kept for the force pass
+constexpr int kTissueBlocks = 608;
 struct TissueScratch {
   int32_t* nb_n;     // edges of every cell (0: failed, status latched)
   int32_t* nb_slot;  // kTissueCap per slot: edge sites, counter-clockwise
   int2* nb_off;      // ... and their exact offsets from the particle
+  double2* edge;     // ... the edges as vectors, length units
+  double* inv_len;   // ... and the inverse of their lengths
   double* area;      // per slot, length units
   double* perim;
+  double* blocks;    // kTissueBlocks partial energies
 };
 // cells, forces (by id) and energy of one replica; any output may be NULL
 cudaError_t launch_tissue(const Geometry& g, const Buffers& b, int rep, int n, double KA, double KP, double A0,

@@ -508,8 +508,8 @@ struct Cell8 {
     }
   }
 
-  // bit a: edge a belongs to another particle and is of positive length, i.e. its two vertices lie apart (group)
-  __device__ __forceinline__ unsigned neighbor_edges() const {
+  // bit a: edge a is of positive length, i.e. its two vertices lie apart (group)
+  __device__ __forceinline__ unsigned positive_edges() const {
     const bool big = __any_sync(kAll, m > 8);
     int2 nq[2];
     next_sites(big, nq);
@@ -533,11 +533,17 @@ struct Cell8 {
           be = he;
         }
       }
-      const bool is = has(i) && slot[i] >= 0 &&
-                      (vertex_cut_fast(bv.x, bv.y, be, nq[i].x, nq[i].y) != 0 ||
-                       vertex_cut_sign(b.x, b.y, q[i].x, q[i].y, nq[i].x, nq[i].y) != 0);
+      const bool is = has(i) && (vertex_cut_fast(bv.x, bv.y, be, nq[i].x, nq[i].y) != 0 ||
+                                 vertex_cut_sign(b.x, b.y, q[i].x, q[i].y, nq[i].x, nq[i].y) != 0);
       kept |= group_bits(is) << (8 * i);
     }
+    return kept;
+  }
+  // ... and belongs to another particle
+  __device__ __forceinline__ unsigned neighbor_edges() const {
+    unsigned kept = positive_edges();
+#pragma unroll
+    for (int i = 0; i < 2; ++i) kept &= ~(group_bits(has(i) && slot[i] < 0) << (8 * i));
     return kept;
   }
 };
