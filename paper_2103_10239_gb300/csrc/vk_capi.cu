@@ -276,7 +276,7 @@ vk_status sort_from_U(vk_sim* s, bool keep_search_state = false) {
   VK_CUDA(s, launch_count(s->g, s->b, s->stream));
   VK_CUDA(s, launch_build(s->g, s->b, s->stream));
   VK_CUDA(s, launch_scatter(s->g, s->b, step_params(s), 0, s->stream));
-  return record_end(s, 3, e0, 9);
+  return record_end(s, 3, e0, build_launches(s->g) + 2);
 }
 
 vk_status read_status(vk_sim* s) {
@@ -297,12 +297,15 @@ vk_status clear_phi(vk_sim* s) {
   return VK_OK;
 }
 
-// kernels of the search+update phase: for 2D kNN the radius-first kernel,
-// the kernel of the particles it hands on and that of the few that need the
-// whole box; two for 3D kNN; one for the metric rule; the Voronoi kernel and
+// kernels of the search+update phase: for kNN the radius-first kernel and
+// those of the particles it hands on (two in 2D, one in 3D), or, in small
+// systems, the last alone; one for the metric rule; the Voronoi kernel and
 // its overflow kernel
 int search_launches(const vk_sim* s) {
-  if (s->prm.rule == VK_RULE_KNN) return s->dim == 2 ? 3 : 2;
+  if (s->prm.rule == VK_RULE_KNN) {
+    const StepParams P = step_params(s);
+    return s->dim == 2 ? (knn2_direct(s->n_total, P) ? 1 : 3) : knn3_launches(s->n_total, P);
+  }
   if (s->prm.rule == VK_RULE_METRIC) return 1;
   return 2;
 }
@@ -317,7 +320,7 @@ vk_status enqueue_step(vk_sim* s) {
   else if (s->prm.rule == VK_RULE_METRIC) VK_CUDA(s, launch_metric_step(s->g, s->b, P, s->stream));
   else if (s->dim == 2) VK_CUDA(s, launch_voronoi_step(s->g, s->b, P, s->stream));
   else VK_CUDA(s, launch_voronoi3_step(s->g, s->b, P, s->stream));
-  const int deferred_launches = (s->prm.rule == VK_RULE_KNN && s->dim == 2) ? 2 : 0;
+  const int deferred_launches = s->prm.rule == VK_RULE_KNN && s->dim == 2 && !knn2_direct(s->n_total, P) ? 2 : 0;
   if ((st = record_end(s, 0, e0, search_launches(s) - deferred_launches))) return st;
   if (deferred_launches) {
     if ((st = record_begin(s, 5, &e0))) return st;
@@ -326,7 +329,7 @@ vk_status enqueue_step(vk_sim* s) {
   }
   if ((st = record_begin(s, 1, &e0))) return st;
   VK_CUDA(s, launch_build(s->g, s->b, s->stream));
-  if ((st = record_end(s, 1, e0, 7))) return st;
+  if ((st = record_end(s, 1, e0, build_launches(s->g)))) return st;
   if ((st = record_begin(s, 2, &e0))) return st;
   VK_CUDA(s, launch_scatter(s->g, s->b, P, 1, s->stream));
   return record_end(s, 2, e0, 1);
@@ -957,7 +960,7 @@ vk_status vk_get_info(vk_sim* s, vk_info* out) {
   out->dim = s->dim;
   out->n_cells = s->n_cells;
   out->step = s->step;
-  out->kernels_per_step = 8 + search_launches(s);
+  out->kernels_per_step = build_launches(s->g) + 1 + search_launches(s);
   out->rule = s->prm.rule;
   out->k = s->prm.k;
   return VK_OK;

@@ -694,6 +694,8 @@ cudaError_t launch_count(const Geometry& g, const Buffers& b, cudaStream_t st);
 // coarse counts -> offsets, sub-grid sides and sub-cell bases; sub-cell
 // histogram of U (ranks); sub-cell scan
 cudaError_t launch_build(const Geometry& g, const Buffers& b, cudaStream_t st);
+int build_launches(const Geometry& g);  // kernels of one launch_build (none in small systems)
+// (in small systems also the work of launch_build)
 cudaError_t launch_scatter(const Geometry& g, const Buffers& b, const StepParams& P, int advance_step,
                            cudaStream_t st);
 cudaError_t launch_export_state(const Geometry& g, const Buffers& b, int rep, int64_t p0, int32_t n,
@@ -705,6 +707,7 @@ cudaError_t launch_import_state(const Geometry& g, const Buffers& b, int rep, in
 
 // vk_knn.cu (3D); one-time kernel attributes first
 cudaError_t prepare_knn3();
+int knn3_launches(int64_t n, const StepParams& P);  // kernels of one launch_knn_step
 cudaError_t launch_knn_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
 cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out,
                               cudaStream_t st);
@@ -713,7 +716,9 @@ cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int k, int re
 // search + update of every particle (those one square each can serve; the
 // rest is listed) ...
 cudaError_t launch_knn2_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
-// ... and of the listed particles (larger squares, then the whole box)
+// ... and of the listed particles (larger squares, then the whole box); not
+// called where the first launch serves every particle
+bool knn2_direct(int64_t n, const StepParams& P);
 cudaError_t launch_knn2_finish(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
 cudaError_t launch_knn2_export(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out, cudaStream_t st,
                                const StepParams& P);

@@ -170,7 +170,7 @@ __device__ __forceinline__ bool cube_search(CubeShared<KC>& H, const Rep& R, con
   int cnt = 0, merged = 0, got = 0;
   int uy = lo[1], uz = lo[2], seg = 0, nrun = 0, r = 0;
   uint32_t q = 0, qe = 0, ox = 0, oy = 0, oz = 0;
-  bool more = true, done = false;
+  bool more = true, done = false, wide = false;
   for (;;) {
     while (cnt <= CAP - 2) {
       if (q == qe) {
@@ -189,6 +189,8 @@ __device__ __forceinline__ bool cube_search(CubeShared<KC>& H, const Rep& R, con
               // image codes per axis: 0 same, 1 at -L, 2 at +L
               const uint32_t code = (xs < 0 ? 1u : xs >= nx ? 2u : 0u) | (uy < 0 ? 4u : uy >= ny ? 8u : 0u) |
                                     (uz < 0 ? 16u : uz >= nz ? 32u : 0u);
+              // longer than a run's length can say (no return from here: the warp's threads have to meet again)
+              wide = wide || qf - qb >= 1u << 26;
               if (qf > qb) H.run[nrun++][tid] = make_uint2(qb, (qf - qb) << 6 | code);
             }
             if (++seg == 3 || (lo[0] >= 0 && hi[0] < nx && seg == 2)) {
@@ -262,7 +264,7 @@ __device__ __forceinline__ bool cube_search(CubeShared<KC>& H, const Rep& R, con
     if (t[KC - 2] < 0xFF000000u) tau = fminf(tau, __uint_as_float(((t[KC - 2] >> B) + 3u) << B));
   }
   if ((t[KC - 2] >> B) + 1u < edge) {
-    bool close = false;  // a pair whose order the keys leave open
+    bool close = wide;  // a pair whose order the keys leave open
 #pragma unroll
     for (int e = 0; e < KC - 1; ++e) close |= e >= KC - 1 - k && (t[e + 1] >> B) - (t[e] >> B) <= 1u;
     return !close;
@@ -286,6 +288,12 @@ __device__ __forceinline__ float cube_radius_estimate(const Rep& R, const uint32
   const int64_t gc = R.c0 + ((int64_t)c[2] * R.nc[1] + c[1]) * R.nc[0] + c[0];
   const float m = (float)max(__ldg(G.off + gc + 1) - __ldg(G.off + gc), 1u);
   return 1.3f * cbrtf(3.f * (float)k * vol / (4.f * 3.14159265f * m));
+}
+
+// the first radius of a particle
+__device__ __forceinline__ float cube_radius(const Rep& R, const uint32_t* __restrict__ bounds, const GridView& G,
+                                             const int32_t* pi, float hint, const StepParams& P) {
+  return hint > 0.f ? P.halo_alpha * hint : cube_radius_estimate(R, bounds, G, pi, P.k);
 }
 
 // Eq. (2) + Eq. (1) of one particle; at(j) is the slot of list entry j in
@@ -351,20 +359,18 @@ __global__ void __launch_bounds__(kBlk3, CubeCfg<KC>::BLOCKS) knn3_step_kernel(
     const int64_t s = R.p0 + li;
     int32_t pi[3];
     unpack(S_pos[s], pi);
-    const float hint = S_hint[s];
-    const float r = hint > 0.f ? P.halo_alpha * hint : cube_radius_estimate(R, bounds, G, pi, P.k);
+    const float r = cube_radius(R, bounds, G, pi, S_hint[s], P);
     float r_next = r;
-    if (P.knn_search == 0) {
-      uint32_t key[KC];
-      served = cube_search<KC>(H, R, bounds, G, S_pos, (int32_t)s, pi, r, P.k, key, &r_next, &n_cand, &n_runs);
-      if (served) {
-        knn3_update<KC>(R, P, step, s, pi, S_id[s],
-                        [&](int j) { return H.hit[key[j] & ((1u << CubeCfg<KC>::BITS) - 1u)][threadIdx.x].x; }, S_dir,
-                        U_pos, U_dir, U_id, counts, bounds, nnew);
-        U_hint[s] = sqrtf(__uint_as_float(key[KC - 2])) * 1.0001f + 1.f;
-      }
+    uint32_t key[KC];
+    served = cube_search<KC>(H, R, bounds, G, S_pos, (int32_t)s, pi, r, P.k, key, &r_next, &n_cand, &n_runs);
+    if (served) {
+      knn3_update<KC>(R, P, step, s, pi, S_id[s],
+                      [&](int j) { return H.hit[key[j] & ((1u << CubeCfg<KC>::BITS) - 1u)][threadIdx.x].x; }, S_dir,
+                      U_pos, U_dir, U_id, counts, bounds, nnew);
+      U_hint[s] = sqrtf(__uint_as_float(key[KC - 2])) * 1.0001f + 1.f;
+    } else {
+      U_hint[s] = r_next;
     }
-    if (!served) U_hint[s] = r_next;
   }
   // one atomic per warp: its entries stay neighbors in the list
   const unsigned m = __ballot_sync(0xffffffffu, li < R.n && !served);
@@ -478,7 +484,9 @@ struct Group3 : GroupTop<GS, CAP> {
 // The listed particles: 16 lanes each, larger cubes until k hits are in one
 // (one thread each, with the ring walk as its last resort, took 500 us for the
 // few particles of a small system).  A warp takes up to 32 of them, its groups
-// search one after another, and then every lane updates one.
+// search one after another, and then every lane updates one.  Small systems
+// (and the general search) come here at once, every particle (n_all of them, by
+// the tasks): the thread kernel's time is one particle's however few there are.
 constexpr int kGS3 = 16, kGroupBlk3 = 128;
 
 template <int KC>
@@ -487,21 +495,31 @@ __global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_kernel
     const int32_t* __restrict__ S_id, GridView G, int4* __restrict__ U_pos, float4* __restrict__ U_dir,
     int32_t* __restrict__ U_id, uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc,
     const int64_t* __restrict__ d_step, StepParams P, const uint32_t* __restrict__ bounds, float* U_hint,
-    const int2* __restrict__ list, const int32_t* __restrict__ count) {
+    const int2* __restrict__ list, const int32_t* __restrict__ count, int64_t n_all,
+    const BlockTask* __restrict__ tasks, const float* __restrict__ S_hint) {
   constexpr int CAP = GroupCfg<KC>::CAP, NG = 32 / kGS3, NW = kGroupBlk3 / 32;
   __shared__ GroupList<CAP> lists[kGroupBlk3 / kGS3];
   __shared__ int32_t res[NW][32][KC - 1];
   __shared__ float res_d[NW][32];
-  const int total = *count;
+  const bool all = n_all > 0;
+  const int64_t total = all ? n_all : *count;
+  // (slot, replica) of entry i; slot -1 where a replica's last task has no particle
+  auto entry = [&](int64_t i) -> int2 {
+    if (!all) return list[i];
+    const BlockTask t = tasks[i / kBlock];
+    const int li = t.first + (int)(i % kBlock);
+    return make_int2(li < reps[t.rep].n ? (int)(reps[t.rep].p0 + li) : -1, t.rep);
+  };
   const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
   const int nw = (int)gridDim.x * NW, w = (int)blockIdx.x * NW + wid;
-  const int chunk = min(32, (int)(((int64_t)total + (int64_t)nw * NG - 1) / ((int64_t)nw * NG)) * NG);
+  const int chunk = (int)min((int64_t)32, (total + (int64_t)nw * NG - 1) / ((int64_t)nw * NG) * NG);
   const int64_t step = *d_step;
   const int k = P.k;
   for (int64_t base = (int64_t)w * chunk; base < total; base += (int64_t)nw * chunk) {
-    const int todo = (int)min((int64_t)chunk, (int64_t)total - base);
+    const int todo = (int)min((int64_t)chunk, total - base);
     for (int i = lane / kGS3; i < todo; i += NG) {
-      const int2 e = list[base + i];
+      const int2 e = entry(base + i);
+      if (e.x < 0) continue;
       const Rep& R = reps[e.y];
       const int4 p = S_pos[e.x];
       Group3<kGS3, CAP> g{{lists[threadIdx.x / kGS3], S_id, ((1u << kGS3) - 1u) << (lane / kGS3 * kGS3),
@@ -509,7 +527,7 @@ __global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_kernel
                           S_pos, bounds, {p.x, p.y, p.z}};
       g.k = k;
       g.n_cand = 0;
-      float r = U_hint[e.x];
+      float r = all ? cube_radius(R, bounds, G, g.p, S_hint[e.x], P) : U_hint[e.x];
       uint32_t tries = 1;
       for (;; ++tries) {
         const int64_t a = (int64_t)ceilf(fminf(r, 4.0e9f));
@@ -533,9 +551,12 @@ __global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_kernel
     __syncwarp();
     int2 e = make_int2(0, 0);
     float nnew[3] = {0.f, 0.f, 0.f};
-    const bool mine = lane < todo;
+    bool mine = lane < todo;
     if (mine) {
-      e = list[base + lane];
+      e = entry(base + lane);
+      mine = e.x >= 0;
+    }
+    if (mine) {
       int32_t pi[3];
       unpack(S_pos[e.x], pi);
       knn3_update<KC>(reps[e.y], P, step, e.x, pi, S_id[e.x], [&](int j) { return res[wid][lane][j - (KC - 1 - k)]; },
@@ -577,17 +598,26 @@ GridView grid_view(const Buffers& b) {
   return G;
 }
 
+// Systems of up to this many particles: the groups alone.  us per step, both
+// kernels / groups: 2048, k = 7 159 / 51; 16384 185 / 121, k = 32 664 / 441;
+// 32768, k = 7 207 / 161, k = 32 752 / 740.
+constexpr int64_t kDirect3 = 32768;
+bool knn3_direct(int64_t n, const StepParams& P) { return P.knn_search == 1 || n <= kDirect3; }
+
 template <int KC>
 cudaError_t step_dispatch(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
   const size_t smem = sizeof(CubeShared<KC>);
-  knn3_step_kernel<KC><<<g.n_tasks * kSplit3, kBlk3, smem, st>>>(
-      g.reps, g.tasks, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view(b), (int4*)b.U_pos,
-      (float4*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.S_hint, b.U_hint, b.ovf_list,
-      b.ovf_count);
+  const bool all = knn3_direct(g.n_total, P);
+  if (!all)
+    knn3_step_kernel<KC><<<g.n_tasks * kSplit3, kBlk3, smem, st>>>(
+        g.reps, g.tasks, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view(b), (int4*)b.U_pos,
+        (float4*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.S_hint, b.U_hint, b.ovf_list,
+        b.ovf_count);
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((g.n_total + 7) / 8, (int64_t)device_sm_count() * 5));
   knn3_group_kernel<KC><<<blocks, kGroupBlk3, 0, st>>>(
       g.reps, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view(b), (int4*)b.U_pos, (float4*)b.U_dir,
-      b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.U_hint, b.ovf_list, b.ovf_count);
+      b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.U_hint, b.ovf_list, b.ovf_count,
+      all ? (int64_t)g.n_tasks * kBlock : 0, g.tasks, b.S_hint);
   return cudaGetLastError();
 }
 
@@ -608,6 +638,8 @@ cudaError_t export_dispatch(const Geometry& g, const Buffers& b, int k, int rep,
 }
 
 }  // namespace
+
+int knn3_launches(int64_t n, const StepParams& P) { return knn3_direct(n, P) ? 1 : 2; }
 
 cudaError_t prepare_knn3() {
   cudaError_t e = prepare3<8>();

@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_box_step_kernel
   if (valid) {
     const int64_t s = R.p0 + li;
     float r = box_radius(R, G, S_pos[s], S_hint[s], out.P);
-    if (out.P.knn_search == 0) served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, step, out, &r, bc, nnew);
+    served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, step, out, &r, bc, nnew);
     if (!served) out.radius()[s] = r;
   }
   warp_append(valid && !served, make_int2((int)(R.p0 + li), t.rep), defer_list, defer_count);
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_box_export_kern
   if (valid) {
     BoxCount bc;
     float r = box_radius(R, G, S_pos[s], S_hint ? S_hint[s] : 0.f, out.P);
-    if (out.P.knn_search == 0) served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, 0, out, &r, bc, nullptr);
+    served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, 0, out, &r, bc, nullptr);
     if (!served) out.radius()[s] = r;
   }
   warp_append(valid && !served, make_int2((int)s, rep), defer_list, defer_count);
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_second_kernel(
   extern __shared__ __align__(16) unsigned char box_smem[];
   BoxShared<KC>& H = *reinterpret_cast<BoxShared<KC>*>(box_smem);
   const int total = *count;
-  if (total < kLongList || out.P.knn_search == 1) return;
+  if (total < kLongList) return;
   int64_t step = 0;
   if constexpr (Out::kStep) step = *out.d_step;
   for (int base = blockIdx.x * kBlk; base < total; base += gridDim.x * kBlk) {
@@ -622,6 +622,10 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_second_kernel(
 // then every lane updates one, so that the update runs on full warps.  Takes
 // the first list where the kernel above left it (its length is read on the
 // device, so that the launch can sit in a CUDA graph).
+//
+// Small systems (and the general search) come here at once, every particle
+// (n_all of them, by the tasks of a step or those of one replica): the thread kernel's time is one particle's, from
+// start to end, however few there are, and the listed ones wait for it.
 constexpr int kGS = 16;
 constexpr int kGroupBlk = 128;
 
@@ -629,33 +633,44 @@ template <int KC, bool FOV, class Out>
 __global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel(
     const Rep* __restrict__ reps, const int2* __restrict__ S_pos, const int32_t* __restrict__ S_id, GridView G,
     Out out, const int2* __restrict__ first_list, const int2* __restrict__ left_list,
-    const int32_t* __restrict__ counts) {
+    const int32_t* __restrict__ counts, int64_t n_all, const BlockTask* __restrict__ tasks, int one_rep,
+    const float* __restrict__ S_hint) {
   constexpr int CAP = GroupCfg<KC>::CAP, NG = 32 / kGS, NW = kGroupBlk / 32;
   __shared__ GroupList<CAP> lists[kGroupBlk / kGS];
   __shared__ int32_t res[NW][32][KC - 1];  // slots of the k nearest of the warp's particles
   __shared__ float res_d[NW][32];          // their k-th squared distance
-  const bool first = counts[0] < kLongList || out.P.knn_search == 1;
+  const bool all = n_all > 0, first = !all && counts[0] < kLongList;
   const int2* __restrict__ list = first ? first_list : left_list;
-  const int total = first ? counts[0] : counts[1];
+  const int64_t total = all ? n_all : first ? counts[0] : counts[1];
+  // (slot, replica) of entry i; slot -1 where a replica's last task has no particle
+  auto entry = [&](int64_t i) -> int2 {
+    if (!all) return list[i];
+    if (!tasks) return make_int2((int)(reps[one_rep].p0 + i), one_rep);
+    const BlockTask t = tasks[i / kBlock];
+    const int li = t.first + (int)(i % kBlock);
+    return make_int2(li < reps[t.rep].n ? (int)(reps[t.rep].p0 + li) : -1, t.rep);
+  };
   const int lane = (int)(threadIdx.x & 31), wid = (int)(threadIdx.x >> 5);
   const int nw = (int)gridDim.x * NW, w = (int)blockIdx.x * NW + wid;
   // short lists are spread over all warps, long ones taken 32 at a time
-  const int chunk = min(32, (int)(((int64_t)total + (int64_t)nw * NG - 1) / ((int64_t)nw * NG)) * NG);
+  const int chunk = (int)min((int64_t)32, (total + (int64_t)nw * NG - 1) / ((int64_t)nw * NG) * NG);
   int64_t step = 0;
   if constexpr (Out::kStep) step = *out.d_step;
   const int k = out.P.k;
   for (int64_t base = (int64_t)w * chunk; base < total; base += (int64_t)nw * chunk) {
-    const int todo = (int)min((int64_t)chunk, (int64_t)total - base);
+    const int todo = (int)min((int64_t)chunk, total - base);
     for (int i = lane / kGS; i < todo; i += NG) {
-      const int2 e = list[base + i];
+      const int2 e = entry(base + i);
+      if (e.x < 0) continue;
       const Rep& R = reps[e.y];
       Group<kGS, CAP, FOV> g{{lists[threadIdx.x / kGS], S_id, ((1u << kGS) - 1u) << (lane / kGS * kGS),
                               lane / kGS * kGS, lane % kGS, e.x},
                              S_pos};
-      init_ctx(g.C, R, e.x, S_pos[e.x]);
+      const int2 p = S_pos[e.x];
+      init_ctx(g.C, R, e.x, p);
       if (FOV) g.C.view = make_view(out.S_dir[e.x], out.P.fov_cq);
       g.k = k;
-      float r = out.radius()[e.x];
+      float r = all ? box_radius(R, G, p, S_hint ? S_hint[e.x] : 0.f, out.P) : out.radius()[e.x];
       uint32_t tries = 1;
       g.n_cand = 0;
       for (;; ++tries) {
@@ -686,9 +701,12 @@ __global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel
     // every lane one particle
     int2 e = make_int2(0, 0);
     float nnew[3] = {0.f, 0.f, 0.f};
-    const bool mine = lane < todo;
+    bool mine = lane < todo;
     if (mine) {
-      e = list[base + lane];
+      e = entry(base + lane);
+      mine = e.x >= 0;
+    }
+    if (mine) {
       out.put(reps[e.y], step, e.x, S_pos[e.x], S_id[e.x],
               [&](int j) { return res[wid][lane][j - (KC - 1 - k)]; }, res_d[wid][lane], nnew);
     }
@@ -717,13 +735,31 @@ int second_blocks(int64_t n) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((n + kBlk - 1) / kBlk, (int64_t)device_sm_count() * BoxCfg<KC>::BLOCKS));
 }
 
+// Systems of up to this many particles: the groups alone.  us per step, all
+// three kernels / groups (up to here the sort also became one launch): 256,
+// k = 7 69 / 23; 2048, k = 7 78 / 31, k = 32 125 / 98; 4096, k = 7 89 / 40, k = 32
+// 142 / 126; 8192, k = 7 97 / 80, k = 16 105 / 114, k = 32 173 / 268.
+constexpr int64_t kDirect2 = 4096;
+
 template <int KC>
 StepOut<KC> step_out(const Buffers& b, const StepParams& P) {
   return {(const float2*)b.S_dir, (int2*)b.U_pos, (float2*)b.U_dir, b.U_id, b.U_hint, b.counts, b.phi_acc, b.d_step, P};
 }
 
+// every particle by the group kernel: those of the tasks (n of them with the
+// tasks' unused places), or of one replica
+template <int KC, bool FOV, class Out>
+cudaError_t group_all(const Geometry& g, const Buffers& b, const Out& out, int64_t n, const BlockTask* tasks, int rep,
+                      cudaStream_t st) {
+  knn2_group_kernel<KC, FOV><<<group_blocks(n), kGroupBlk, 0, st>>>(
+      g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, nullptr, nullptr, nullptr, n, tasks, rep, b.S_hint);
+  return cudaGetLastError();
+}
+
 template <int KC, bool FOV>
 cudaError_t step2(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
+  if (knn2_direct(g.n_total, P))
+    return group_all<KC, FOV>(g, b, step_out<KC>(b, P), (int64_t)g.n_tasks * kBlock, g.tasks, 0, st);
   // the lists are empty here: the previous scatter (or init) cleared them
   knn2_box_step_kernel<KC, FOV><<<g.n_tasks * kSplit, kBlk, sizeof(BoxShared<KC>), st>>>(
       g.reps, g.tasks, (const int2*)b.S_pos, b.S_id, b.S_hint, view_of(b), step_out<KC>(b, P), b.ovf_list,
@@ -739,7 +775,7 @@ void finish_lists(const Geometry& g, const Buffers& b, const Out& out, int64_t n
   knn2_second_kernel<KC, FOV><<<second_blocks<KC>(n), kBlk, sizeof(BoxShared<KC>), st>>>(
         g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, b.ovf_list, b.ovf_count, left, b.ovf_count + 1);
   knn2_group_kernel<KC, FOV><<<group_blocks(n), kGroupBlk, 0, st>>>(
-      g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, b.ovf_list, left, b.ovf_count);
+      g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, b.ovf_list, left, b.ovf_count, 0, nullptr, 0, nullptr);
 }
 
 template <int KC, bool FOV>
@@ -754,6 +790,7 @@ cudaError_t export2(const Geometry& g, const Buffers& b, int rep, int n, int32_t
   if (n == 0) return cudaSuccess;
   // the lists are empty between steps; the export clears what it used
   const RowOut<KC> out{(const float2*)b.S_dir, b.S_id, out_ids, b.U_hint, P};
+  if (knn2_direct(n, P)) return group_all<KC, FOV>(g, b, out, n, nullptr, rep, st);
   knn2_box_export_kernel<KC, FOV><<<(n + kBlk - 1) / kBlk, kBlk, sizeof(BoxShared<KC>), st>>>(
       g.reps, rep, (const int2*)b.S_pos, b.S_id, b.S_hint, view_of(b), out, b.ovf_list, b.ovf_count);
   finish_lists<KC, FOV>(g, b, out, n, st);
@@ -790,6 +827,8 @@ cudaError_t for_k(const StepParams& P, F f) {
 }
 
 }  // namespace
+
+bool knn2_direct(int64_t n, const StepParams& P) { return P.knn_search == 1 || n <= kDirect2; }
 
 cudaError_t prepare_knn2() {
   cudaError_t e = prepare2<8>();
