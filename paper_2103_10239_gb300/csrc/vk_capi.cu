@@ -26,6 +26,7 @@ namespace {
 
 constexpr int kPhases = 6;
 constexpr int kCounters = 14;  // search counters (tracing level 2)
+constexpr int kPhiRows = 4096;  // steps of order-parameter sums read at a time
 const char* kPhaseNames[kPhases] = {"search_update", "build", "scatter", "load_sort", "export", "search_deferred"};
 
 thread_local std::string g_init_error;
@@ -73,6 +74,9 @@ struct vk_sim {
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev[kPhases];
   double prof_ms[kPhases] = {0, 0, 0, 0, 0, 0};
   int64_t prof_launches[kPhases] = {0, 0, 0, 0, 0, 0};
+  int32_t* h_status = nullptr;   // pinned word that the device status is read into
+  long long* h_phi = nullptr;    // pinned: the heading sums of up to kPhiRows steps ...
+  std::mutex h_phi_mu;           // ... (readers of several replicas may be on several threads)
   unsigned long long* d_stats = nullptr;  // search counters, collected while tracing
   std::string err;
 };
@@ -279,10 +283,11 @@ vk_status sort_from_U(vk_sim* s, bool keep_search_state = false) {
   return record_end(s, 3, e0, build_launches(s->g) + 2);
 }
 
+// waits for the sim's stream and reports the latched device status
 vk_status read_status(vk_sim* s) {
-  int32_t h = 0;
-  VK_CUDA(s, cudaMemcpyAsync(&h, s->b.d_status, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
+  VK_CUDA(s, cudaMemcpyAsync(s->h_status, s->b.d_status, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
   VK_CUDA(s, cudaStreamSynchronize(s->stream));
+  const int32_t h = *s->h_status;
   if (h == 0) return VK_OK;
   const char* what = h == VK_ERR_CAPACITY     ? "device: capacity exceeded (Voronoi polygon or buffer)"
                      : h == VK_ERR_DEGENERATE ? "device: coincident particles or a zero-length Voronoi edge"
@@ -481,7 +486,8 @@ vk_status build_sim(int32_t n_rep, const int64_t* n_r, const int32_t* pos_q, con
       (e = dalloc(&s->b.U_id, N)) || (e = dalloc(&s->b.U_rank, N)) ||
       (e = dalloc(&s->b.phi_acc, 3 * (size_t)s->phi_cap * n_rep)) || (e = dalloc(&s->b.d_step, 1)) ||
       (e = dalloc(&s->b.d_status, 1)) || (e = dalloc(&s->reps_d, n_rep)) ||
-      (e = dalloc(&s->b.ovf_list, 2 * N)) || (e = dalloc(&s->b.ovf_count, 2)) ||
+      (e = cudaMallocHost(&s->h_status, sizeof(int32_t))) ||
+      (e = cudaMallocHost(&s->h_phi, 3 * sizeof(long long) * kPhiRows)) || (e = dalloc(&s->b.ovf_list, 2 * N)) || (e = dalloc(&s->b.ovf_count, 2)) ||
       (e = dalloc(&s->d_stats, kCounters)) ||
       (e = dalloc(&s->tasks_d, s->tasks_h.size())))
     return bail(cuda_fail(s, e, "cudaMalloc"));
@@ -592,7 +598,6 @@ vk_status vk_step(vk_sim* s, int64_t nsteps) {
 
 vk_status vk_sync(vk_sim* s) {
   if (!s) return fail(s, VK_ERR_ARG, "sim is NULL");
-  VK_CUDA(s, cudaStreamSynchronize(s->stream));
   return read_status(s);
 }
 
@@ -732,27 +737,45 @@ vk_status vk_get_tissue(vk_sim* s, int32_t replica, double KA, double KP, double
   return st;
 }
 
+// is it ordinary (or pinned) host memory?
+static bool on_host(const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeUnregistered || at.type == cudaMemoryTypeHost;
+}
+
 vk_status vk_get_order_parameter(vk_sim* s, int32_t replica, double* phi, int64_t max_values, int64_t* count) {
   if (!s || replica < 0 || replica >= s->n_rep || (!phi && max_values > 0)) return fail(s, VK_ERR_ARG, "bad arguments");
-  VK_CUDA(s, cudaStreamSynchronize(s->stream));
   // the slot of the upcoming step is already cleared: cap-1 values are kept
   const int64_t have = std::min<int64_t>(s->step - s->phi_first, s->phi_cap - 1);
   const int64_t nout = std::min<int64_t>(have, std::max<int64_t>(0, max_values));
   if (count) *count = nout;
-  if (nout == 0) return VK_OK;
-  std::vector<long long> ring(3 * (size_t)s->phi_cap * s->n_rep);
-  VK_CUDA(s, cudaMemcpy(ring.data(), s->b.phi_acc, sizeof(long long) * ring.size(), cudaMemcpyDeviceToHost));
+  if (nout == 0) {
+    VK_CUDA(s, cudaStreamSynchronize(s->stream));
+    return VK_OK;
+  }
+  // this replica's sums of the asked steps only, written to the host by one
+  // kernel (a copy of the whole ring of 512 replicas is 0.8 MB, 100 us a call)
   std::vector<double> vals(nout);
   const double n = (double)s->reps_h[replica].n;
-  for (int64_t i = 0; i < nout; ++i) {
-    const int64_t t = s->step - nout + i;  // phi after the update from step t to t+1
-    const long long* a = ring.data() + ((size_t)(t % s->phi_cap) * s->n_rep + replica) * 3;
-    // fixed-point sums (2^-32 units) -> FP64
-    const double x = std::ldexp((double)a[0], -32), y = std::ldexp((double)a[1], -32),
-                 z = std::ldexp((double)a[2], -32);
-    vals[i] = std::sqrt(x * x + y * y + z * z) / n;
+  std::lock_guard<std::mutex> lock(s->h_phi_mu);
+  for (int64_t i0 = 0; i0 < nout; i0 += kPhiRows) {
+    const int rows = (int)std::min<int64_t>(nout - i0, kPhiRows);
+    VK_CUDA(s, launch_export_phi(s->b, s->phi_cap, s->n_rep, replica, s->step - nout + i0, rows, s->h_phi, s->stream));
+    VK_CUDA(s, cudaStreamSynchronize(s->stream));
+    for (int i = 0; i < rows; ++i) {
+      const long long* a = s->h_phi + 3 * i;
+      // fixed-point sums (2^-32 units) -> FP64
+      const double x = std::ldexp((double)a[0], -32), y = std::ldexp((double)a[1], -32),
+                   z = std::ldexp((double)a[2], -32);
+      vals[i0 + i] = std::sqrt(x * x + y * y + z * z) / n;
+    }
   }
-  VK_CUDA(s, cudaMemcpy(phi, vals.data(), sizeof(double) * nout, cudaMemcpyDefault));
+  if (on_host(phi)) std::memcpy(phi, vals.data(), sizeof(double) * nout);
+  else VK_CUDA(s, cudaMemcpy(phi, vals.data(), sizeof(double) * nout, cudaMemcpyDefault));
   return VK_OK;
 }
 
@@ -770,23 +793,36 @@ vk_status ensure_staging(vk_sim* s) {
   return VK_OK;
 }
 
+// can a kernel of this device use the caller's array of 4-byte values as it is?
+static bool kernel_reaches(const void* p) {
+  if (!p || ((uintptr_t)p & 3u)) return false;
+  cudaPointerAttributes at;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 vk_status vk_get_state(vk_sim* s, int32_t replica, int32_t* pos_q, float* dir, float* theta, int64_t* step) {
   if (!s || replica < 0 || replica >= s->n_rep) return fail(s, VK_ERR_ARG, "bad arguments");
   cudaStreamSynchronize(cudaStreamLegacy);
   if (vk_status st = ensure_staging(s)) return st;
   const Rep& R = s->reps_h[replica];
   const size_t n = (size_t)R.n, d = (size_t)s->dim;
-  int32_t* pd = s->st_pos;
-  float* dd = s->st_dir;
-  float* td = s->st_theta;
+  if (s->dim != 2) theta = nullptr;
+  // arrays on this device are written by the kernel, others through the staging arrays
+  const bool pin = kernel_reaches(pos_q), din = kernel_reaches(dir), tin = kernel_reaches(theta);
+  int32_t* pd = pin ? pos_q : pos_q ? s->st_pos : nullptr;
+  float* dd = din ? dir : dir ? s->st_dir : nullptr;
+  float* td = tin ? theta : theta ? s->st_theta : nullptr;
   cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess)
-    e = launch_export_state(s->g, s->b, replica, R.p0, R.n, pd, dd, s->dim == 2 ? td : nullptr, s->stream);
-  if (e == cudaSuccess && pos_q) e = cudaMemcpyAsync(pos_q, pd, sizeof(int32_t) * n * d, cudaMemcpyDefault, s->stream);
-  if (e == cudaSuccess && dir) e = cudaMemcpyAsync(dir, dd, sizeof(float) * n * d, cudaMemcpyDefault, s->stream);
-  if (e == cudaSuccess && theta && s->dim == 2)
-    e = cudaMemcpyAsync(theta, td, sizeof(float) * n, cudaMemcpyDefault, s->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+  if (pd || dd || td) e = launch_export_state(s->g, s->b, replica, R.p0, R.n, pd, dd, td, s->stream);
+  if (e == cudaSuccess && pd && !pin)
+    e = cudaMemcpyAsync(pos_q, pd, sizeof(int32_t) * n * d, cudaMemcpyDefault, s->stream);
+  if (e == cudaSuccess && dd && !din) e = cudaMemcpyAsync(dir, dd, sizeof(float) * n * d, cudaMemcpyDefault, s->stream);
+  if (e == cudaSuccess && td && !tin) e = cudaMemcpyAsync(theta, td, sizeof(float) * n, cudaMemcpyDefault, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "get_state");
   if (step) *step = s->step;
   return read_status(s);
@@ -800,10 +836,13 @@ vk_status vk_set_state(vk_sim* s, int32_t replica, const int32_t* pos_q, const f
   const size_t pv = s->dim == 2 ? sizeof(int2) : sizeof(int4);
   const size_t fv = s->dim == 2 ? sizeof(float2) : sizeof(float4);
   if (vk_status st = ensure_staging(s)) return st;
-  int32_t* pd = s->st_pos;
-  float* dd = s->st_dir;
-  cudaError_t e = cudaMemcpyAsync(pd, pos_q, sizeof(int32_t) * n * d, cudaMemcpyDefault, s->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dd, dir, sizeof(float) * n * d, cudaMemcpyDefault, s->stream);
+  // arrays on this device are read where they are, others copied first
+  const int32_t* pd = kernel_reaches(pos_q) ? pos_q : s->st_pos;
+  const float* dd = kernel_reaches(dir) ? dir : s->st_dir;
+  cudaError_t e = cudaSuccess;
+  if (pd != pos_q) e = cudaMemcpyAsync(s->st_pos, pos_q, sizeof(int32_t) * n * d, cudaMemcpyDefault, s->stream);
+  if (e == cudaSuccess && dd != dir)
+    e = cudaMemcpyAsync(s->st_dir, dir, sizeof(float) * n * d, cudaMemcpyDefault, s->stream);
   // the search state follows the particles (by id): a state read with
   // vk_get_state and set again steps as fast as it would have
   if (e == cudaSuccess && s->b.S_hint && s->n_rep > 1)
@@ -828,7 +867,6 @@ vk_status vk_set_state(vk_sim* s, int32_t replica, const int32_t* pos_q, const f
     VK_CUDA(s, cudaMemcpyAsync(s->b.d_step, &s->step, sizeof(int64_t), cudaMemcpyHostToDevice, s->stream));
     if ((st = clear_phi(s))) return st;
   }
-  VK_CUDA(s, cudaStreamSynchronize(s->stream));
   return read_status(s);
 }
 
@@ -870,6 +908,8 @@ void vk_destroy(vk_sim* s) {
                   s->tis.inv_len, s->tis.blocks, s->tis.area, s->tis.perim, s->tis_out};
   for (void* p : bufs)
     if (p) cudaFree(p);
+  if (s->h_status) cudaFreeHost(s->h_status);
+  if (s->h_phi) cudaFreeHost(s->h_phi);
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
   delete s;
 }

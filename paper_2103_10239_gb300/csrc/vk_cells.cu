@@ -547,6 +547,13 @@ __global__ void __launch_bounds__(kBlock) hints_by_id_kernel(const int32_t* __re
   U_hint[p0 + S_id[s]] = S_hint[s];
 }
 
+__global__ void __launch_bounds__(kBlock) export_phi_kernel(const PhiAcc* __restrict__ phi_acc, int phi_cap, int n_rep,
+                                                            int rep, int64_t first, int n, long long* __restrict__ out) {
+  const int i = blockIdx.x * kBlock + (int)threadIdx.x;
+  if (i < 3 * n)
+    out[i] = (long long)phi_acc[((size_t)((first + i / 3) % phi_cap) * (size_t)n_rep + (size_t)rep) * 3 + i % 3];
+}
+
 }  // namespace
 
 cudaError_t launch_load(const Geometry& g, const Buffers& b, const int32_t* pos_in, const float* head_in,
@@ -657,6 +664,12 @@ cudaError_t launch_import_state(const Geometry& g, const Buffers& b, int rep, in
   else
     import_state_kernel<3><<<nb, kBlock, 0, st>>>(pos_in, dir_in, p0, n, L, (int4*)b.U_pos, (float4*)b.U_dir,
                                                    b.U_id, b.d_status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_export_phi(const Buffers& b, int phi_cap, int n_rep, int rep, int64_t first, int n, long long* out,
+                              cudaStream_t st) {
+  export_phi_kernel<<<(3 * n + kBlock - 1) / kBlock, kBlock, 0, st>>>(b.phi_acc, phi_cap, n_rep, rep, first, n, out);
   return cudaGetLastError();
 }
 
