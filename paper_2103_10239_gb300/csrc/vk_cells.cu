@@ -51,13 +51,15 @@ __global__ void __launch_bounds__(kBlock) load_kernel(const Rep* __restrict__ re
   U_id[s] = li;
 }
 
-// coarse histogram of U (the search+update kernel does this for every step)
+// coarse histogram of U, with the ranks in 3D (the search+update kernel does
+// this for every step)
 template <int DIM>
 __global__ void __launch_bounds__(kBlock) count_kernel(const Rep* __restrict__ reps,
                                                        const BlockTask* __restrict__ tasks,
                                                        const typename Vec<DIM>::P* __restrict__ U_pos,
                                                        const uint32_t* __restrict__ bounds,
-                                                       uint32_t* __restrict__ counts) {
+                                                       uint32_t* __restrict__ counts,
+                                                       uint32_t* __restrict__ U_rank) {
   const BlockTask t = tasks[blockIdx.x];
   const Rep R = reps[t.rep];
   const int li = t.first + (int)threadIdx.x;
@@ -73,15 +75,14 @@ __global__ void __launch_bounds__(kBlock) count_kernel(const Rep* __restrict__ r
     for (int a = DIM - 1; a >= 0; --a)
       lin = lin * R.nc[a] + cell_of_tab((uint32_t)p[a], R.nc[a], bounds + R.bnd[a], R.inv_w[a]);
   }
-  atomicAdd(counts + R.c0 + lin, 1u);
+  const uint32_t rank = atomicAdd(counts + R.c0 + lin, 1u);
+  if (DIM == 3) U_rank[s] = rank;
 }
 
-// sub-cell histogram of U: the rank of every particle inside its sub-cell
-template <int DIM>
+// (2D) sub-cell histogram of U: the rank of every particle inside its sub-cell
 __global__ void __launch_bounds__(kBlock) sub_count_kernel(const Rep* __restrict__ reps,
                                                            const BlockTask* __restrict__ tasks,
-                                                           const typename Vec<DIM>::P* __restrict__ U_pos,
-                                                           const uint32_t* __restrict__ bounds, GridView G,
+                                                           const int2* __restrict__ U_pos, GridView G,
                                                            uint32_t* __restrict__ sub_count,
                                                            uint32_t* __restrict__ U_rank) {
   const BlockTask t = tasks[blockIdx.x];
@@ -92,7 +93,7 @@ __global__ void __launch_bounds__(kBlock) sub_count_kernel(const Rep* __restrict
   int32_t p[3];
   unpack(U_pos[s], p);
   int64_t gc, g;
-  locate<DIM>(R, G, bounds, p, &gc, &g);
+  locate<2>(R, G, nullptr, p, &gc, &g);
   U_rank[s] = atomicAdd(sub_count + g, 1u);
 }
 
@@ -189,13 +190,13 @@ __global__ void __launch_bounds__(kBlock) scan_apply_kernel(uint32_t* __restrict
 }
 
 // ---- coarse scan: (count, s^2) pairs -> offsets, sub-grid sides, sub bases
-__device__ __forceinline__ uint32_t sub_cells(uint32_t count, int dim) {
-  const int s = dim == 2 ? sub_side(count) : 1;
+__device__ __forceinline__ uint32_t sub_cells(uint32_t count) {
+  const int s = sub_side(count);
   return (uint32_t)(s * s);
 }
 
 __global__ void __launch_bounds__(kBlock) pair_reduce_kernel(const uint32_t* __restrict__ counts, int64_t n,
-                                                             int dim, uint2* __restrict__ bsum) {
+                                                             uint2* __restrict__ bsum) {
   const int64_t base = (int64_t)blockIdx.x * kScanTile;
   uint32_t v = 0, w = 0;
 #pragma unroll
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kBlock) pair_reduce_kernel(const uint32_t* __r
     if (c < n) {
       const uint32_t m = counts[c];
       v += m;
-      w += sub_cells(m, dim);
+      w += sub_cells(m);
     }
   }
 #pragma unroll
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(kBlock) pair_bsum_kernel(uint2* __restrict__ b
   }
 }
 
-__global__ void __launch_bounds__(kBlock) pair_apply_kernel(uint32_t* __restrict__ counts, int64_t n, int dim,
+__global__ void __launch_bounds__(kBlock) pair_apply_kernel(uint32_t* __restrict__ counts, int64_t n,
                                                             const uint2* __restrict__ bsum,
                                                             uint32_t* __restrict__ offsets,
                                                             uint8_t* __restrict__ sub_s,
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(kBlock) pair_apply_kernel(uint32_t* __restrict
   for (int j = 0; j < kScanItems; ++j) {
     const int64_t c = base + j;
     v[j] = c < n ? counts[c] : 0u;
-    w[j] = c < n ? sub_cells(v[j], dim) : 0u;
+    w[j] = c < n ? sub_cells(v[j]) : 0u;
     tv += v[j];
     tw += w[j];
   }
@@ -270,7 +271,7 @@ __global__ void __launch_bounds__(kBlock) pair_apply_kernel(uint32_t* __restrict
     if (c < n) {
       offsets[c] = rv;
       sub_base[c] = rw;
-      sub_s[c] = (uint8_t)(dim == 2 ? sub_side(v[j]) : 1);
+      sub_s[c] = (uint8_t)sub_side(v[j]);
       counts[c] = 0u;
     }
     rv += v[j];
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(kBlock) scatter_kernel(const Rep* __restrict__
   unpack(pv, p);
   int64_t gc, g;
   locate<DIM>(R, G, bounds, p, &gc, &g);
-  const uint32_t dst = G.sub_off[g] + U_rank[s];
+  const uint32_t dst = (DIM == 2 ? G.sub_off[g] : G.off[gc]) + U_rank[s];
   S_pos[dst] = pv;
   S_dir[dst] = U_dir[s];
   const int32_t id = U_id[s];
@@ -578,28 +579,32 @@ static GridView grid_view(const Buffers& b) {
 
 cudaError_t launch_count(const Geometry& g, const Buffers& b, cudaStream_t st) {
   if (g.dim == 2)
-    count_kernel<2><<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, (const int2*)b.U_pos, b.bounds, b.counts);
+    count_kernel<2><<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, (const int2*)b.U_pos, b.bounds, b.counts, b.U_rank);
   else
-    count_kernel<3><<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, (const int4*)b.U_pos, b.bounds, b.counts);
+    count_kernel<3><<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, (const int4*)b.U_pos, b.bounds, b.counts, b.U_rank);
   return cudaGetLastError();
 }
 
-int build_launches(const Geometry& g) { return small_system(g) ? 0 : 7; }
+int build_launches(const Geometry& g) { return small_system(g) ? 0 : g.dim == 3 ? 3 : 7; }
 
 cudaError_t launch_build(const Geometry& g, const Buffers& b, cudaStream_t st) {
   if (small_system(g)) return cudaSuccess;  // launch_scatter does it all
   const int nb = (int)((g.n_cells + kScanTile - 1) / kScanTile);
-  pair_reduce_kernel<<<nb, kBlock, 0, st>>>(b.counts, g.n_cells, g.dim, (uint2*)b.bsum);
+  if (g.dim == 3) {
+    // cells are never split: the rank in a cell is what its counter said, and
+    // one scan gives the slots (1M particles: 66 us for the seven launches that
+    // split cells take, 21 for these three; 8000: 39, 16)
+    scan_reduce_kernel<<<nb, kBlock, 0, st>>>(b.counts, g.n_cells, b.bsum);
+    scan_bsum_kernel<<<1, kBlock, 0, st>>>(b.bsum, nb, b.offsets, g.n_cells);
+    scan_apply_kernel<<<nb, kBlock, 0, st>>>(b.counts, g.n_cells, b.bsum, b.offsets);
+    return cudaGetLastError();
+  }
+  pair_reduce_kernel<<<nb, kBlock, 0, st>>>(b.counts, g.n_cells, (uint2*)b.bsum);
   pair_bsum_kernel<<<1, kBlock, 0, st>>>((uint2*)b.bsum, nb, b.offsets, b.sub_base, g.n_cells);
-  pair_apply_kernel<<<nb, kBlock, 0, st>>>(b.counts, g.n_cells, g.dim, (const uint2*)b.bsum, b.offsets, b.sub_s,
+  pair_apply_kernel<<<nb, kBlock, 0, st>>>(b.counts, g.n_cells, (const uint2*)b.bsum, b.offsets, b.sub_s,
                                            b.sub_base);
   const GridView G = grid_view(b);
-  if (g.dim == 2)
-    sub_count_kernel<2><<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, (const int2*)b.U_pos, b.bounds, G, b.sub_count,
-                                                       b.U_rank);
-  else
-    sub_count_kernel<3><<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, (const int4*)b.U_pos, b.bounds, G, b.sub_count,
-                                                       b.U_rank);
+  sub_count_kernel<<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, (const int2*)b.U_pos, G, b.sub_count, b.U_rank);
   const int nb2 = (int)((g.n_sub_max + kScanTile - 1) / kScanTile);
   scan_reduce_kernel<<<nb2, kBlock, 0, st>>>(b.sub_count, g.n_sub_max, b.bsum2);
   scan_bsum_kernel<<<1, kBlock, 0, st>>>(b.bsum2, nb2, b.sub_off, g.n_sub_max);

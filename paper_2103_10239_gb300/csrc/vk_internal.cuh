@@ -288,8 +288,7 @@ __device__ __forceinline__ void locate(const Rep& R, const GridView& G, const ui
 #pragma unroll
     for (int a = DIM - 1; a >= 0; --a)
       lin = lin * R.nc[a] + cell_of_tab((uint32_t)p[a], R.nc[a], bounds + R.bnd[a], R.inv_w[a]);
-    *gcell = R.c0 + lin;
-    *gsub = (int64_t)G.sub_base[*gcell];
+    *gsub = *gcell = R.c0 + lin;
   }
 }
 
@@ -640,7 +639,7 @@ struct Buffers {
   void* U_pos;
   void* U_dir;
   int32_t* U_id;
-  uint32_t* U_rank;
+  uint32_t* U_rank;   // (3D: by the search and count kernels; 2D: by the sub-cell histogram)
   uint32_t* counts;   // n_cells
   uint32_t* offsets;  // n_cells + 1
   uint32_t* bsum;     // scan block sums (coarse)

@@ -302,8 +302,9 @@ template <int KC, class At>
 __device__ __forceinline__ void knn3_update(const Rep& R, const StepParams& P, int64_t step, int64_t s,
                                             const int32_t* pi, int32_t id, At at, const float4* __restrict__ S_dir,
                                             int4* __restrict__ U_pos, float4* __restrict__ U_dir,
-                                            int32_t* __restrict__ U_id, uint32_t* __restrict__ counts,
-                                            const uint32_t* __restrict__ bounds, float* nnew) {
+                                            int32_t* __restrict__ U_id, uint32_t* __restrict__ U_rank,
+                                            uint32_t* __restrict__ counts, const uint32_t* __restrict__ bounds,
+                                            float* nnew) {
   float ni[3];
   unpack(S_dir[s], ni);
   HeadSum<3> H;
@@ -331,7 +332,7 @@ __device__ __forceinline__ void knn3_update(const Rep& R, const StepParams& P, i
 #pragma unroll
   for (int ax = 2; ax >= 0; --ax)
     lin = lin * R.nc[ax] + cell_of_tab((uint32_t)pout[ax], R.nc[ax], bounds + R.bnd[ax], R.inv_w[ax]);
-  atomicAdd(counts + R.c0 + lin, 1u);
+  U_rank[s] = atomicAdd(counts + R.c0 + lin, 1u);
 }
 
 // Search + update, one cube per particle.  Particles it cannot serve go on the
@@ -340,8 +341,8 @@ template <int KC>
 __global__ void __launch_bounds__(kBlk3, CubeCfg<KC>::BLOCKS) knn3_step_kernel(
     const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const int4* __restrict__ S_pos,
     const float4* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G, int4* __restrict__ U_pos,
-    float4* __restrict__ U_dir, int32_t* __restrict__ U_id, uint32_t* __restrict__ counts,
-    PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P,
+    float4* __restrict__ U_dir, int32_t* __restrict__ U_id, uint32_t* __restrict__ U_rank,
+    uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P,
     const uint32_t* __restrict__ bounds, const float* __restrict__ S_hint, float* __restrict__ U_hint,
     int2* __restrict__ list, int32_t* __restrict__ count) {
   extern __shared__ __align__(16) unsigned char cube_smem[];
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(kBlk3, CubeCfg<KC>::BLOCKS) knn3_step_kernel(
     if (served) {
       knn3_update<KC>(R, P, step, s, pi, S_id[s],
                       [&](int j) { return H.hit[key[j] & ((1u << CubeCfg<KC>::BITS) - 1u)][threadIdx.x].x; }, S_dir,
-                      U_pos, U_dir, U_id, counts, bounds, nnew);
+                      U_pos, U_dir, U_id, U_rank, counts, bounds, nnew);
       U_hint[s] = sqrtf(__uint_as_float(key[KC - 2])) * 1.0001f + 1.f;
     } else {
       U_hint[s] = r_next;
@@ -493,8 +494,9 @@ template <int KC>
 __global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_kernel(
     const Rep* __restrict__ reps, const int4* __restrict__ S_pos, const float4* __restrict__ S_dir,
     const int32_t* __restrict__ S_id, GridView G, int4* __restrict__ U_pos, float4* __restrict__ U_dir,
-    int32_t* __restrict__ U_id, uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc,
-    const int64_t* __restrict__ d_step, StepParams P, const uint32_t* __restrict__ bounds, float* U_hint,
+    int32_t* __restrict__ U_id, uint32_t* __restrict__ U_rank, uint32_t* __restrict__ counts,
+    PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P,
+    const uint32_t* __restrict__ bounds, float* U_hint,
     const int2* __restrict__ list, const int32_t* __restrict__ count, int64_t n_all,
     const BlockTask* __restrict__ tasks, const float* __restrict__ S_hint) {
   constexpr int CAP = GroupCfg<KC>::CAP, NG = 32 / kGS3, NW = kGroupBlk3 / 32;
@@ -560,7 +562,7 @@ __global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_kernel
       int32_t pi[3];
       unpack(S_pos[e.x], pi);
       knn3_update<KC>(reps[e.y], P, step, e.x, pi, S_id[e.x], [&](int j) { return res[wid][lane][j - (KC - 1 - k)]; },
-                      S_dir, U_pos, U_dir, U_id, counts, bounds, nnew);
+                      S_dir, U_pos, U_dir, U_id, U_rank, counts, bounds, nnew);
       U_hint[e.x] = sqrtf(res_d[wid][lane]) * 1.0001f + 1.f;
     }
     phi_add_warp<3>(phi_acc + (size_t)(step % P.phi_cap) * (size_t)P.n_rep * 3, e.y, nnew, mine);
@@ -611,12 +613,12 @@ cudaError_t step_dispatch(const Geometry& g, const Buffers& b, const StepParams&
   if (!all)
     knn3_step_kernel<KC><<<g.n_tasks * kSplit3, kBlk3, smem, st>>>(
         g.reps, g.tasks, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view(b), (int4*)b.U_pos,
-        (float4*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.S_hint, b.U_hint, b.ovf_list,
+        (float4*)b.U_dir, b.U_id, b.U_rank, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.S_hint, b.U_hint, b.ovf_list,
         b.ovf_count);
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((g.n_total + 7) / 8, (int64_t)device_sm_count() * 5));
   knn3_group_kernel<KC><<<blocks, kGroupBlk3, 0, st>>>(
       g.reps, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view(b), (int4*)b.U_pos, (float4*)b.U_dir,
-      b.U_id, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.U_hint, b.ovf_list, b.ovf_count,
+      b.U_id, b.U_rank, b.counts, b.phi_acc, b.d_step, P, b.bounds, b.U_hint, b.ovf_list, b.ovf_count,
       all ? (int64_t)g.n_tasks * kBlock : 0, g.tasks, b.S_hint);
   return cudaGetLastError();
 }

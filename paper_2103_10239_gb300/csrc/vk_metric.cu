@@ -330,7 +330,7 @@ __device__ __forceinline__ void metric_walk3(const Rep& R, int64_t self, const i
 __global__ void __launch_bounds__(kBlock) metric3_step_kernel(
     const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const uint32_t* __restrict__ bounds, const int4* __restrict__ S_pos,
     const float4* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G, int4* __restrict__ U_pos,
-    float4* __restrict__ U_dir, int32_t* __restrict__ U_id, uint32_t* __restrict__ counts,
+    float4* __restrict__ U_dir, int32_t* __restrict__ U_id, uint32_t* __restrict__ U_rank, uint32_t* __restrict__ counts,
     PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams P) {
   const BlockTask t = tasks[blockIdx.x];
   const Rep R = reps[t.rep];
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kBlock) metric3_step_kernel(
 #pragma unroll
     for (int a = 2; a >= 0; --a)
       lin = lin * R.nc[a] + cell_of_tab((uint32_t)pout[a], R.nc[a], bounds + R.bnd[a], R.inv_w[a]);
-    atomicAdd(counts + R.c0 + lin, 1u);
+    U_rank[s] = atomicAdd(counts + R.c0 + lin, 1u);
   }
   record_search_stats(P.stats, li < R.n, n_cand, n_runs);
   block_phi_accumulate<3>(nnew, phi_acc + ((size_t)(step % P.phi_cap) * (size_t)P.n_rep + (size_t)t.rep) * 3);
@@ -462,7 +462,7 @@ cudaError_t launch_metric_step(const Geometry& g, const Buffers& b, const StepPa
   } else {
     metric3_step_kernel<<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, b.bounds, (const int4*)b.S_pos,
                                                       (const float4*)b.S_dir, b.S_id, metric_view(b),
-                                                      (int4*)b.U_pos, (float4*)b.U_dir, b.U_id, b.counts,
+                                                      (int4*)b.U_pos, (float4*)b.U_dir, b.U_id, b.U_rank, b.counts,
                                                       b.phi_acc, b.d_step, P);
   }
   return cudaGetLastError();

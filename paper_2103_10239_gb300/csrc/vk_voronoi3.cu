@@ -610,7 +610,8 @@ __global__ void __launch_bounds__(32 * kV3Warps, VK_V3_BLOCKS) voronoi3_step_ker
     const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, int n_items, int chunk,
     const uint32_t* __restrict__ bounds, const int4* __restrict__ S_pos, const float4* __restrict__ S_dir,
     const int32_t* __restrict__ S_id, GridView G, int4* __restrict__ U_pos, float4* __restrict__ U_dir,
-    int32_t* __restrict__ U_id, uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc,
+    int32_t* __restrict__ U_id, uint32_t* __restrict__ U_rank, uint32_t* __restrict__ counts,
+    PhiAcc* __restrict__ phi_acc,
     const int64_t* __restrict__ d_step, StepParams Pm, int32_t* status, int2* __restrict__ ovf_list,
     int32_t* __restrict__ ovf_count) {
   extern __shared__ __align__(16) unsigned char v3_smem[];
@@ -713,7 +714,7 @@ __global__ void __launch_bounds__(32 * kV3Warps, VK_V3_BLOCKS) voronoi3_step_ker
       U_pos[s] = make_int4(pout[0], pout[1], pout[2], 0);
       U_dir[s] = make_float4(nnew[0], nnew[1], nnew[2], 0.f);
       U_id[s] = id;
-      atomicAdd(counts + linear_cell<3>(R, pout), 1u);
+      U_rank[s] = atomicAdd(counts + linear_cell<3>(R, pout), 1u);
     }
     phi_add_warp<3>(phi_acc + (size_t)(step % Pm.phi_cap) * (size_t)Pm.n_rep * 3, rep, nnew, m > -2);
     __syncwarp();
@@ -787,11 +788,11 @@ cudaError_t launch_voronoi3_step(const Geometry& g, const Buffers& b, const Step
   const int chunk = std::max(1, std::min(kPend, n_items / (blocks * kV3Warps * 4)));
   voronoi3_step_kernel<CellS, false><<<blocks, 32 * kV3Warps, sizeof(Warp3<CellS>) * kV3Warps, st>>>(
       g.reps, g.tasks, n_items, chunk, b.bounds, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view3(b),
-      (int4*)b.U_pos, (float4*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P, b.d_status, b.ovf_list,
+      (int4*)b.U_pos, (float4*)b.U_dir, b.U_id, b.U_rank, b.counts, b.phi_acc, b.d_step, P, b.d_status, b.ovf_list,
       b.ovf_count);
   voronoi3_step_kernel<CellL, true><<<sms, 32 * kV3Warps, sizeof(Warp3<CellL>) * kV3Warps, st>>>(
       g.reps, g.tasks, 0, 1, b.bounds, (const int4*)b.S_pos, (const float4*)b.S_dir, b.S_id, grid_view3(b),
-      (int4*)b.U_pos, (float4*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P, b.d_status, b.ovf_list,
+      (int4*)b.U_pos, (float4*)b.U_dir, b.U_id, b.U_rank, b.counts, b.phi_acc, b.d_step, P, b.d_status, b.ovf_list,
       b.ovf_count);
   return cudaGetLastError();
 }
