@@ -112,14 +112,17 @@ typedef struct {
   int32_t advect_new;   /* 1: advect with n_i(t+dt) instead of n_i(t) (default 0) */
   int32_t sum_mode;     /* vk_sum_mode for the heading sums (default compensated) */
   float cell_occupancy; /* target particles per coarse cell of the search grid at the mean
-                           density; 0 = default (256 in 2D, 2 for Voronoi, 1.5 in 3D).
+                           density; 0 = default (2D: 256, kNN in large systems 64,
+                           Voronoi 2; 3D: kNN 3.5, metric 1.5, Voronoi 1).
                            Dense coarse cells get sub-grids of about 2 particles per sub-cell.
                            Results never depend on it; only the speed does. */
   int32_t phi_capacity; /* order-parameter history kept per replica; 0 = 4096 steps */
   int32_t knn_search;   /* kNN search: 0 = radius first (default; a square in 2D, a cube in 3D),
-                           1 = the ring walk only.  Results never depend on it; only the speed does. */
+                           1 = the general search only (a group of lanes per particle, larger squares
+                           or cubes until k neighbors are in one).  Results never depend on it; only
+                           the speed does. */
   float search_halo;    /* radius first: half-width of a particle's search square (cube), as a multiple
-                           of its k-th neighbor distance at the previous step; 0 = default (1.15 in 2D, 1.3 in 3D).
+                           of its k-th neighbor distance at the previous step; 0 = default (1.15; 1.2 in 3D for k <= 10).
                            Results never depend on it; only the speed does. */
   float search_halo_step; /* radius first: plus this multiple of the distance a particle moves
                            in one step (v0 dt); < 0 = default (0).  Speed only. */
@@ -259,7 +262,8 @@ vk_status vk_set_graph_steps(vk_sim* sim, int32_t steps_per_graph);
  * 0 search_update (the search + update kernel of every particle), 1 build
  * (grid scans), 2 scatter, 3 load_sort (init / set_state), 4 export
  * (vk_get_neighbors), 5 search_deferred (2D kNN radius first: the particles
- * the first kernel listed for larger squares or the walk). */
+ * the first kernel listed for larger squares; nothing in small systems, whose
+ * only search kernel is phase 0; their build is part of phase 2). */
 vk_status vk_set_profiling(vk_sim* sim, int32_t enable);
 vk_status vk_get_profile(vk_sim* sim, double* ms, int64_t* launches, int32_t max_phases,
                          int32_t* n_phases);
@@ -269,22 +273,21 @@ const char* vk_phase_name(int32_t phase);
  * mean candidates examined per particle update, mean contiguous slot runs
  * read per particle update (2D kNN radius first: mean squares scanned), the
  * largest candidate count of one particle, and the fraction of particle
- * updates whose own coarse cell was split into sub-cells (2D kNN radius
- * first: that fell back to the per-particle walk).  Any output may be NULL. */
+ * updates that the general code finished (2D kNN: groups of lanes; 2D Voronoi:
+ * the warp kernel).  Any output may be NULL. */
 vk_status vk_get_search_stats(vk_sim* sim, double* mean_candidates, double* mean_runs,
                               int64_t* max_candidates, double* split_fraction);
 
 /* Raw totals of the search counters collected while tracing at level 2, in
  * this order: 0 candidates examined (summed over particle updates), 1 slot
- * runs (walk) or squares scanned (radius first), 2 largest candidate count
- * of one particle update, 3 particle updates, 4 updates whose own coarse
- * cell was split (walk) or that fell back to the walk (radius first); radius
- * first only, over the particles it served or handed on: 5 squares scanned,
- * 6 slot runs, 7 candidates, 8 coarse cells visited, 9 hits merged, and the
- * particles the step kernel deferred because 10 the square was too wide for
- * the box or listed too many slot runs (these go straight to the walk),
- * 11 the square held fewer than k hits (a larger square follows), 12 two
- * candidates were at the same distance (walk), 13 (unused, 0).  Writes
+ * runs or squares scanned, 2 largest candidate count of one particle update,
+ * 3 particle updates, 4 updates that the general code finished (2D kNN: groups
+ * of lanes; 2D Voronoi: the warp kernel); 2D kNN's first squares only, over the
+ * particles they served or handed on: 5 squares scanned, 6 slot runs, 7
+ * candidates, 8 coarse cells visited, 9 hits merged, and the particles handed
+ * on because 10 the square was too wide for the box, 11 it held fewer than k
+ * hits (a larger square follows), 12 two candidates' distances were too close
+ * to order in 32 bits, 13 (unused, 0).  Writes
  * min(max_values, 14) values; *n (may be NULL) receives 14. */
 vk_status vk_get_search_counters(vk_sim* sim, int64_t* values, int32_t max_values, int32_t* n);
 

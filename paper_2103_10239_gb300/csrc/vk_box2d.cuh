@@ -1,9 +1,8 @@
-// vk_box2d.cuh -- the square walk of the 2D two-level search grid, shared
-// by the radius-first k-nearest search (vk_knn2d.cu) and the metric rule
-// (vk_metric.cu): every particle of the square [p - a, p + a] around a
-// particle, listed as contiguous runs of the cell-sorted arrays, with exact
-// minimum-image offsets.  Also the particle's search context and the exact
-// field-of-view test of the kNN rule.
+// vk_box2d.cuh -- a particle's search context and the exact field-of-view test
+// of the 2D kNN rule (vk_knn2d.cu), and the square walk of the two-level grid
+// that exports the metric rule's lists (vk_metric.cu): every particle of the
+// square [p - a, p + a] around a particle, as contiguous runs of the
+// cell-sorted arrays, with exact minimum-image offsets.
 #pragma once
 #include <climits>
 
@@ -91,11 +90,6 @@ __device__ __forceinline__ uint64_t box_offset(const Ctx& C, int2 pj, int32_t& d
   if (dy > C.hiy) dy = (int32_t)((uint32_t)dy - C.Ly);
   else if (dy <= C.loy) dy = (int32_t)((uint32_t)dy + C.Ly);
   return (uint64_t)((int64_t)dx * dx) + (uint64_t)((int64_t)dy * dy);
-}
-
-__device__ __forceinline__ uint64_t box_dist2(const Ctx& C, int2 pj) {
-  int32_t dx, dy;
-  return box_offset(C, pj, dx, dy);
 }
 
 // Walk the slot runs of the square [p - a, p + a] (the sub-cell rows of the

@@ -125,8 +125,10 @@ StepParams step_params(const vk_sim* s) {
   P.n_rep = s->n_rep;
   P.phi_cap = s->phi_cap;
   P.knn_search = s->prm.knn_search;
-  // measured defaults: squares 1.15 x the last k-th distance (2D), cubes 1.3 x (3D)
-  P.halo_alpha = s->prm.search_halo > 0.f ? s->prm.search_halo : (s->dim == 3 ? 1.3f : 1.15f);
+  // measured defaults: squares 1.15 x the last k-th distance (2D), cubes 1.2 x (3D;
+  // 1.15 x for many neighbors, whose k-th distance varies less: 262,144 particles,
+  // k = 32 1484 against 1313 us per step, but 1M, k = 7 936 against 1039)
+  P.halo_alpha = s->prm.search_halo > 0.f ? s->prm.search_halo : (s->dim == 3 && s->prm.k <= 10 ? 1.2f : 1.15f);
   P.halo_beta = s->prm.search_halo_step >= 0.f ? s->prm.search_halo_step : 0.f;
   P.fov_cq = fov_cq(s->prm);
   P.stats = (s->prof && s->prof_counters) ? s->d_stats : nullptr;
@@ -158,9 +160,17 @@ float default_occupancy(const vk_params& p, int dim, int64_t n_total, int n_rep)
   // Voronoi: 2 particles per cell in 2D; 1 in 3D (a sweep of 1, 1.5, 2 and 3
   // at N = 2^18 uniform: 83, 89, 96, 109 ms per step)
   if (p.rule == VK_RULE_VORONOI) return dim == 2 ? 2.0f : 1.0f;
-  // 2D kNN and metric: coarse cells of a few hundred particles split into
-  // sub-grids (the radius-first search measured fastest at 256 on uniform
-  // and clustered flocks); 3D: cells of about 1.5 particles (the cube search)
+  // 2D kNN: coarse cells of 256 particles split into sub-grids, of 64 in large
+  // systems (ms per pass of 10 steps, 64 / 128 / 256 per cell: 4M clustered 17.9,
+  // 19.8, 19.7; 1M uniform 4.22, 4.64, 4.64; 300,000 2.03, 2.04, 2.18; 50,000 1.17,
+  // 1.18, 1.17; 512 replicas, 8M in all, 20 steps 46, 47, 50); not in a field of
+  // view, whose squares meet many empty cells (1M: 4.38, 4.18, 4.13).  3D kNN: cells
+  // of 3.5 particles (us per step, 1.5 / 2.5 / 3.5 / 5 per cell: 1M, k = 7 1017, 946,
+  // 936, 938; 262,144, k = 32 1717, 1551, 1484, 1428; 16,384 100, 94, 93, 92).
+  // Metric rule, whose rectangles are of one cell: 256 in 2D; 1.5 in 3D (the best
+  // lies between 1 and 4 as r0 goes)
+  if (p.rule == VK_RULE_KNN && dim == 3) return 3.5f;
+  if (p.rule == VK_RULE_KNN && !p.fov && n_total >= 1 << 17) return 64.0f;
   return dim == 2 ? 256.0f : 1.5f;
 }
 
