@@ -109,8 +109,8 @@ __device__ __forceinline__ void knn_search(const Rep& R, int64_t self, const int
 // closer than a + 1.  As in 2D (vk_knn2d.cu) the selection runs on 32-bit
 // keys, the FP32 squared distance with the hit's number in its low bits: a
 // 64-bit list with ids cost eight compares and moves per hit, run by the few
-// lanes that had one: 1943 us per step at 1M particles; this takes 1058, and 86
-// for the particles handed on.
+// lanes that had one: 1943 us per step at 1M particles; this takes 906 with the
+// particles handed on (1144 in cells of 1.5 particles and cubes of 1.3).
 // Candidates within the cube's inscribed ball are buffered and merged after
 // the scan by min / max; a list whose order the keys leave open, or with too
 // few hits, is handed on.

@@ -25,9 +25,10 @@
 //     (int64 squared distance, id).
 //
 // Measured (GB300, us per step, 64-bit list / 32-bit keys and power-of-two
-// cells): 4M clustered, k = 7: first square 2372 / 1175, listed particles
-// 1232 / 594; 50,021 uniform, k = 16, vectorial noise: 178 / 35, 183 / 36;
-// 2048 uniform: 45 / 26, 48 / 26.
+// cells): 4M clustered, k = 7, ten steps from a set state: first square 2372 /
+// 1175, listed particles 1232 / 594 (thirty steps on, with cells of 64 particles,
+// 905 and 332); 50,021 uniform, k = 16, vectorial noise: 178 / 35, 183 / 36.  2048
+// uniform: 45 + 48 / 26 + 26, and 27 by the groups alone.
 #include <algorithm>
 #include <climits>
 #include <type_traits>
@@ -44,18 +45,20 @@ constexpr int kSplit = kBlock / kBlk;
 
 // KC keys per thread: room for k <= KC - 1 neighbors and the one after them.
 // CAP hits buffered per thread (about 1.3 k + 1 are expected), numbered in
-// BITS bits.
+// BITS bits, and RUNS slot runs listed before they are scanned.  What they do not
+// take of shared memory caches positions: for k <= 7, 24 hits and 8 runs / 20 and
+// 6: 512 replicas 1634 / 1563 us per step, 4M clustered 943 / 905; 16 hits (956)
+// fill too often, and 6 runs for k = 16 (448 against 431 at 1M) are too few.
 template <int KC> struct BoxCfg;
-template <> struct BoxCfg<8> { static constexpr int CAP = 24, BITS = 5, BLOCKS = 6; };
-template <> struct BoxCfg<12> { static constexpr int CAP = 32, BITS = 5, BLOCKS = 5; };
-template <> struct BoxCfg<17> { static constexpr int CAP = 48, BITS = 6, BLOCKS = 3; };
-template <> struct BoxCfg<33> { static constexpr int CAP = 64, BITS = 6, BLOCKS = 2; };
-constexpr int kRuns = 8;  // slot runs listed before they are scanned
+template <> struct BoxCfg<8> { static constexpr int CAP = 20, BITS = 5, BLOCKS = 6, RUNS = 6; };
+template <> struct BoxCfg<12> { static constexpr int CAP = 32, BITS = 5, BLOCKS = 5, RUNS = 8; };
+template <> struct BoxCfg<17> { static constexpr int CAP = 48, BITS = 6, BLOCKS = 3, RUNS = 8; };
+template <> struct BoxCfg<33> { static constexpr int CAP = 64, BITS = 6, BLOCKS = 2, RUNS = 8; };
 
 template <int KC>
 struct BoxShared {
   uint2 hit[BoxCfg<KC>::CAP][kBlk];  // (slot, bits of the FP32 squared distance), one column per thread
-  uint2 run[kRuns][kBlk];            // (first slot, length << 4 | image shift codes)
+  uint2 run[BoxCfg<KC>::RUNS][kBlk];  // (first slot, length << 4 | image shift codes)
 };
 
 // the slot behind a key of the list
@@ -114,10 +117,10 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
     while (cnt <= CAP - 4) {
       if (q - qb >= len) {  // next run
         if (r == nrun) {
-          // list up to kRuns runs, so that one flat loop scans them and the
+          // list up to RUNS runs, so that one flat loop scans them and the
           // threads of a warp scan candidates together however their squares split
           nrun = r = 0;
-          while (more && nrun <= kRuns - 2) {
+          while (more && nrun <= BoxCfg<KC>::RUNS - 2) {
             if (row > row_end) {  // next coarse cell
               if (ucx > ucx1) {
                 ucx = ucx0;
