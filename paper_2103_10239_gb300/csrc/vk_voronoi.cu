@@ -18,7 +18,7 @@
 //     points closer to V than the particle is); its bounding box, the
 //     relevance box, only shrinks;
 //   * ordinary cells: vk_voronoi_fast.cuh.  A cell that outgrows 16 edges, meets
-//     more than kHeavy candidates (a particle bordering a void), reaches half a
+//     too many candidates (a particle bordering a void), reaches half a
 //     period or has coincident particles is finished by the overflow kernel,
 //     one warp per cell: the lanes test 32 candidates at a time against the
 //     current cell and one lane applies the few that cut it;
@@ -65,15 +65,11 @@ __device__ __forceinline__ void voronoi_update(const Rep& R, const StepParams& P
   atomicAdd(counts + linear_cell<2>(R, pout), 1u);
 }
 
-// Heavy-cell hint: a cell that needed more than kHeavyHint candidates in the
-// main kernel, or more than kHeavyKeep in the warp kernel, is flagged in its
-// seed word, and the next step sends it to the warp kernel at once (particles
-// on the rim of a void stay there for many steps).  Speed only.
-#ifndef VK_VOR_HEAVY_HINT
-#define VK_VOR_HEAVY_HINT 320
-#endif
-constexpr uint32_t kHeavyHint = VK_VOR_HEAVY_HINT > 0 ? VK_VOR_HEAVY_HINT : 0xFFFFFFFFu;
-constexpr uint32_t kHeavyKeep = VK_VOR_HEAVY_HINT > 0 ? VK_VOR_HEAVY_HINT / 2 : 0xFFFFFFFFu;
+// Heavy-cell hint: a cell that needed more than heavy_hint candidates in the
+// main kernel, or half as many in the warp kernel, is flagged in its seed word,
+// and the next step sends it to the warp kernel at once (particles on the rim of
+// a void stay there for many steps).  Speed only.
+__device__ __forceinline__ uint32_t heavy_hint(uint32_t heavy) { return heavy / 6u * 5u; }
 
 // Main kernel: the ordinary cells, eight lanes each (vk_voronoi_fast.cuh).
 // The others go on the overflow list.  A warp builds the cells of 4 x ROUNDS
@@ -96,7 +92,7 @@ __global__ void __launch_bounds__(kCellBlk, VK_VOR_MIN_BLOCKS) voronoi_step_kern
     int2* __restrict__ U_pos, float2* __restrict__ U_dir, int32_t* __restrict__ U_id,
     uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams Pm,
     int2* __restrict__ ovf_list, int32_t* __restrict__ ovf_count, int32_t* __restrict__ vor_seed,
-    int32_t* __restrict__ vor_seed_n, const int32_t* __restrict__ slot_of) {
+    int32_t* __restrict__ vor_seed_n, const int32_t* __restrict__ slot_of, uint32_t heavy) {
   __shared__ PhiShared phs;
   phi_block_begin(phs);
   constexpr int kPerBlock = kCellBlk / kCG * ROUNDS, kPerWarp = 4 * ROUNDS, kBlocks = kBlock / kPerBlock;
@@ -126,7 +122,7 @@ __global__ void __launch_bounds__(kCellBlk, VK_VOR_MIN_BLOCKS) voronoi_step_kern
     const Seeds sd{vor_seed ? vor_seed + gi * kVorSeed : nullptr, min(sw & kSeedCount, kVorSeed), slot_of};
     // a cell that was heavy at the last step goes straight to the warp kernel
     const bool mine = on && !(sw & kSeedHeavy);
-    c.build(mine, R, s, p, S_pos, G, sd, kHeavy);
+    c.build(mine, R, s, p, S_pos, G, sd, heavy);
     const bool ok = mine && !c.other;
     if (on && !ok && c.gl == 0) ovf_list[atomicAdd(ovf_count, 1)] = make_int2((int)s, t.rep);
     // neighbors: the sites of edges of positive length, ordered by id
@@ -180,7 +176,7 @@ __global__ void __launch_bounds__(kCellBlk, VK_VOR_MIN_BLOCKS) voronoi_step_kern
 #pragma unroll
       for (int i = 0; i < 2; ++i)
         if (keep && rank[i] >= 0 && rank[i] < kVorSeed) vor_seed[gi * kVorSeed + rank[i]] = nid[i];
-      if (c.gl == 0) vor_seed_n[gi] = keep ? min(cnt, kVorSeed) | (c.n_seen > kHeavyHint ? kSeedHeavy : 0) : 0;
+      if (c.gl == 0) vor_seed_n[gi] = keep ? min(cnt, kVorSeed) | (c.n_seen > heavy_hint(heavy) ? kSeedHeavy : 0) : 0;
     }
     // hand the sums to the lanes of these four particles
     const int from = (lane & 3) * kCG;
@@ -224,7 +220,7 @@ __global__ void __launch_bounds__(kCellBlk, VK_VOR_MIN_BLOCKS) voronoi_step_kern
 
 // Overflow kernel: the few particles whose cell outgrew the main kernel's
 // polygon (a particle bordering a void can have dozens of Voronoi
-// neighbors) or needed more than kHeavy candidates; one warp per particle.
+// neighbors) or needed too many candidates; one warp per particle.
 constexpr int kOvfWarps = 4;
 
 __global__ void __launch_bounds__(32 * kOvfWarps) voronoi_overflow_kernel(
@@ -233,7 +229,8 @@ __global__ void __launch_bounds__(32 * kOvfWarps) voronoi_overflow_kernel(
     float2* __restrict__ U_dir, int32_t* __restrict__ U_id,
     uint32_t* __restrict__ counts, PhiAcc* __restrict__ phi_acc, const int64_t* __restrict__ d_step, StepParams Pm,
     const int2* __restrict__ ovf_list, const int32_t* __restrict__ ovf_count, int32_t* status,
-    int32_t* __restrict__ vor_seed, int32_t* __restrict__ vor_seed_n, const int32_t* __restrict__ slot_of) {
+    int32_t* __restrict__ vor_seed, int32_t* __restrict__ vor_seed_n, const int32_t* __restrict__ slot_of,
+    uint32_t heavy) {
   __shared__ Poly<kSlowCap> poly[kOvfWarps];
   Poly<kSlowCap>& P = poly[threadIdx.x >> 5];
   const int total = *ovf_count;
@@ -259,7 +256,7 @@ __global__ void __launch_bounds__(32 * kOvfWarps) voronoi_overflow_kernel(
         const float ni[3] = {nv.x, nv.y, 0.f};
         float nnew[3] = {0.f, 0.f, 0.f};
         voronoi_update(R, Pm, step, s, P, pi, ni, id, S_dir, U_pos, U_dir, U_id, counts, nnew,
-                       vor_seed ? vor_seed + gi * kVorSeed : nullptr, vor_seed_n + gi, seen > kHeavyKeep);
+                       vor_seed ? vor_seed + gi * kVorSeed : nullptr, vor_seed_n + gi, seen > heavy_hint(heavy) / 2u);
         PhiAcc* acc = phi_acc + ((size_t)(step % Pm.phi_cap) * (size_t)Pm.n_rep + (size_t)e.y) * 3;
         atomicAdd(acc + 0, (PhiAcc)phi_fixed(nnew[0]));
         atomicAdd(acc + 1, (PhiAcc)phi_fixed(nnew[1]));
@@ -320,11 +317,13 @@ static GridView grid_view(const Buffers& b) {
 
 cudaError_t launch_voronoi_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
   const GridView G = grid_view(b);
+  const uint32_t heavy = g.n_total < kHeavyLine ? kHeavySmall : kHeavy;
   // 32 cells per warp (one full update) where that still fills the chip, 4 in small systems
   auto step = [&](auto kernel, int rounds) {
     kernel<<<g.n_tasks * (kBlock / (kCellBlk / kCG * rounds)), kCellBlk, 0, st>>>(
         g.reps, g.tasks, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id, G, (int2*)b.U_pos, (float2*)b.U_dir,
-        b.U_id, b.counts, b.phi_acc, b.d_step, P, b.ovf_list, b.ovf_count, b.vor_seed, b.vor_seed_n, b.slot_of);
+        b.U_id, b.counts, b.phi_acc, b.d_step, P, b.ovf_list, b.ovf_count, b.vor_seed, b.vor_seed_n, b.slot_of,
+        heavy);
   };
   const int64_t fill = (int64_t)device_sm_count() * VK_VOR_MIN_BLOCKS * (kCellBlk / kCG) * 3;
   if (g.n_total >= 8 * fill) step(voronoi_step_kernel<8>, 8);
@@ -333,7 +332,7 @@ cudaError_t launch_voronoi_step(const Geometry& g, const Buffers& b, const StepP
   voronoi_overflow_kernel<<<device_sm_count() * 4, 32 * kOvfWarps, 0, st>>>(g.reps, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id,
                                               G, (int2*)b.U_pos, (float2*)b.U_dir, b.U_id,
                                               b.counts, b.phi_acc, b.d_step, P, b.ovf_list, b.ovf_count,
-                                              b.d_status, b.vor_seed, b.vor_seed_n, b.slot_of);
+                                              b.d_status, b.vor_seed, b.vor_seed_n, b.slot_of, heavy);
   return cudaGetLastError();
 }
 

@@ -16,7 +16,13 @@ namespace {
 
 constexpr int kFastCap = 32;    // polygon capacity of the main kernel
 constexpr int kSlowCap = kVoronoiMaxDeg;  // capacity of the overflow kernel and the export
-constexpr uint32_t kHeavy = 384;  // candidates after which the main kernel hands a cell to the overflow kernel
+// candidates after which the main kernel hands a cell to the overflow kernel.
+// Large systems: the groups' throughput counts (us per step, 384 / 512 / 768 /
+// 1024: 512k with grown voids 7867, 6520, 5579, 5370; 65,536 beside a lattice, steps
+// 80 on, 2192, 1939, 1871, 1878).  Small ones: the time of the longest cell (20
+// steps, us: 6000 particles 5562, 5406, 5707, 5763; 2000 3736, 3551, 3473, 3492).
+constexpr uint32_t kHeavy = 768, kHeavySmall = 512;
+constexpr int64_t kHeavyLine = 16384;  // particles
 
 __device__ __noinline__ int vertex_cut_exact(int32_t ax, int32_t ay, int32_t bx, int32_t by, int32_t mx,
                                              int32_t my);
