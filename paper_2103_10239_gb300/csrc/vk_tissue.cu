@@ -123,8 +123,7 @@ __global__ void __launch_bounds__(kTissueBlk, 4) tissue_cells_kernel(
     const int2 p = S_pos[s];
     // a Voronoi-rule sim's last neighbors seed the cell (any seeds give the same cell)
     const int64_t gi = R.p0 + S_id[s];
-    const Seeds sd{vor_seed ? vor_seed + gi * kVorSeed : nullptr,
-                   vor_seed ? min(vor_seed_n[gi] & kSeedCount, kVorSeed) : 0, slot_of};
+    const Seeds sd = seeds_of(vor_seed, vor_seed ? vor_seed_n[gi] : 0, gi, slot_of);
     c.build(on, R, s, p, S_pos, G, sd, 2 * kHeavy);
     const bool ok = on && !c.other;
     // an edge of zero length (four cocircular particles): no derivative

@@ -47,7 +47,7 @@ __device__ __forceinline__ void voronoi_update(const Rep& R, const StepParams& P
     // the next step's seeds (any subset of sites would do)
     const int ns = min(cnt, kVorSeed);
     for (int j = 0; j < ns; ++j) seed_out[j] = nid[j];
-    *seed_n_out = ns | (heavy_next ? kSeedHeavy : 0);
+    *seed_n_out = seed_word(ns, heavy_next, 2.0f * sqrtf(P.max_r2));
   }
   HeadSum<2> H;
   H.init();
@@ -75,9 +75,14 @@ __device__ __forceinline__ uint32_t heavy_hint(uint32_t heavy) { return heavy / 
 // The others go on the overflow list.  A warp builds the cells of 4 x ROUNDS
 // consecutive particles, four at a time, and then updates them, one per lane.
 // A cell that met more than kSeedMin candidates keeps its neighbors as the
-// next step's seeds: a particle beside a void has a wide box until its own
-// neighbors bound the cell, while the nearest particles bound an ordinary one
-// as well.
+// next step's seeds, until it has shrunk to half the reach it had then: a
+// particle beside a void has a wide box until its own neighbors bound the cell,
+// while the nearest particles bound an ordinary one as well, and are one load
+// away instead of three.  Measured (us per step, no seeds / these / seeds for
+// every cell): 65,536 particles beside a lattice, steps 100 on, 1645 / 1534 / 1493,
+// 1000 particles with voids 186 / 138 / 121, 512k 4682 / 3980 / 3435, but 20,000 in a
+// random state 171 / 169 / 263 and the first ten steps beside the lattice 344 / 343 /
+// 540.  (kSeedMin of 96 and 256: 512k 3863 and 4318, beside the lattice 352 and 375.)
 constexpr uint32_t kSeedMin = 160;
 constexpr int kCellBlk = 128;
 // resident blocks per SM the main kernel is compiled for
@@ -119,7 +124,7 @@ __global__ void __launch_bounds__(kCellBlk, VK_VOR_MIN_BLOCKS) voronoi_step_kern
     const int32_t id = S_id[s];
     const int64_t gi = R.p0 + id;
     const int32_t sw = vor_seed && on ? vor_seed_n[gi] : 0;
-    const Seeds sd{vor_seed ? vor_seed + gi * kVorSeed : nullptr, min(sw & kSeedCount, kVorSeed), slot_of};
+    const Seeds sd = seeds_of(vor_seed, sw, gi, slot_of);
     // a cell that was heavy at the last step goes straight to the warp kernel
     const bool mine = on && !(sw & kSeedHeavy);
     c.build(mine, R, s, p, S_pos, G, sd, heavy);
@@ -172,11 +177,13 @@ __global__ void __launch_bounds__(kCellBlk, VK_VOR_MIN_BLOCKS) voronoi_step_kern
       if (who) H.add(v, Pm.sum_mode);
     }
     if (vor_seed && ok) {
-      const bool keep = c.n_seen > kSeedMin;
+      const bool far = c.n_seen > kSeedMin, keep = far || (sd.n > 0 && c.reach() > 0.5f * sd.reach);
 #pragma unroll
       for (int i = 0; i < 2; ++i)
         if (keep && rank[i] >= 0 && rank[i] < kVorSeed) vor_seed[gi * kVorSeed + rank[i]] = nid[i];
-      if (c.gl == 0) vor_seed_n[gi] = keep ? min(cnt, kVorSeed) | (c.n_seen > heavy_hint(heavy) ? kSeedHeavy : 0) : 0;
+      if (c.gl == 0)
+        vor_seed_n[gi] =
+            keep ? seed_word(min(cnt, kVorSeed), c.n_seen > heavy_hint(heavy), far ? c.reach() : sd.reach) : 0;
     }
     // hand the sums to the lanes of these four particles
     const int from = (lane & 3) * kCG;
@@ -244,8 +251,7 @@ __global__ void __launch_bounds__(32 * kOvfWarps) voronoi_overflow_kernel(
     const int32_t pi[3] = {p.x, p.y, 0};
     const int32_t id = S_id[s];
     const int64_t gi = R.p0 + id;
-    const Seeds sd{vor_seed ? vor_seed + gi * kVorSeed : nullptr, vor_seed ? vor_seed_n[gi] & kSeedCount : 0,
-                   slot_of};
+    const Seeds sd = seeds_of(vor_seed, vor_seed ? vor_seed_n[gi] : 0, gi, slot_of);
     uint32_t seen = 0;
     const bool ok = voronoi_cell_warp(R, s, pi, id, S_pos, S_id, G, P, status, sd, &seen);
     if ((threadIdx.x & 31) == 0) {
@@ -285,8 +291,7 @@ __global__ void __launch_bounds__(64) voronoi_export_kernel(const Rep* __restric
     const int32_t pi[3] = {p.x, p.y, 0};
     const int32_t id = S_id[s];
     const int64_t gi = R.p0 + id;
-    const Seeds sd{vor_seed ? vor_seed + gi * kVorSeed : nullptr, vor_seed ? vor_seed_n[gi] & kSeedCount : 0,
-                   slot_of};
+    const Seeds sd = seeds_of(vor_seed, vor_seed ? vor_seed_n[gi] : 0, gi, slot_of);
     Poly<kSlowCap> P;
     if (!voronoi_cell(R, s, pi, id, S_pos, S_id, G, P, status, 0u, sd, nullptr)) {
       set_status(status, kStCapacity);

@@ -17,10 +17,11 @@ namespace {
 constexpr int kFastCap = 32;    // polygon capacity of the main kernel
 constexpr int kSlowCap = kVoronoiMaxDeg;  // capacity of the overflow kernel and the export
 // candidates after which the main kernel hands a cell to the overflow kernel.
-// Large systems: the groups' throughput counts (us per step, 384 / 512 / 768 /
-// 1024: 512k with grown voids 7867, 6520, 5579, 5370; 65,536 beside a lattice, steps
-// 80 on, 2192, 1939, 1871, 1878).  Small ones: the time of the longest cell (20
-// steps, us: 6000 particles 5562, 5406, 5707, 5763; 2000 3736, 3551, 3473, 3492).
+// Large systems: the groups' throughput counts (us per step, 512 / 768 / 1024 / 1536:
+// 512k with grown voids 4095, 3980, 3975, 4024; 65,536 beside a lattice, steps 100 on,
+// 1552, 1533, 1564, 1634; 100,000 1420, 1407, 1446, 1514).  Small ones: the time of the
+// longest cell (384 / 512 / 768 / 1024: 6000 particles 739, 746, 786, 816; 2000 774, 785,
+// 811, 838, but 20 steps from a random state 3049, 2755, 2754, 2754).
 constexpr uint32_t kHeavy = 768, kHeavySmall = 512;
 constexpr int64_t kHeavyLine = 16384;  // particles
 
@@ -530,14 +531,27 @@ __device__ __noinline__ void far_images(const Rep& R, int64_t self, const int32_
 struct Seeds {
   const int32_t* ids;      // replica-local ids of last step's neighbors (NULL: none)
   int n;
+  float reach;             // of the cell they come from
   const int32_t* slot_of;  // sorted slot by (replica's first slot + id)
 };
 
-// a particle's seed word: the number of seeds in the low byte, and a flag
-// for a cell that needed many candidates at the last step (a particle on the
-// rim of a void), which goes straight to the warp-cooperative kernel
+// a particle's seed word: the number of seeds in the low byte, a flag for a
+// cell that needed many candidates at the last step (a particle on the rim of
+// a void), which goes straight to the warp-cooperative kernel, and in the high
+// half that of a float: the reach (twice the largest vertex distance) of the
+// cell when it was found to be worth seeding
 constexpr int32_t kSeedCount = 0xFF;
 constexpr int32_t kSeedHeavy = 0x100;
+__device__ __forceinline__ float seed_reach(int32_t word) { return __uint_as_float((uint32_t)word & 0xFFFF0000u); }
+__device__ __forceinline__ int32_t seed_word(int n, bool heavy, float reach) {
+  return n | (heavy ? kSeedHeavy : 0) | (int32_t)(__float_as_uint(reach) & 0xFFFF0000u);
+}
+
+// the seeds of the particle with index gi (replica's first slot + id)
+__device__ __forceinline__ Seeds seeds_of(const int32_t* __restrict__ vor_seed, int32_t word, int64_t gi,
+                                          const int32_t* __restrict__ slot_of) {
+  return {vor_seed ? vor_seed + gi * kVorSeed : nullptr, min(word & kSeedCount, kVorSeed), seed_reach(word), slot_of};
+}
 
 // flags of one cell build
 struct CellFlags {

@@ -22,7 +22,7 @@
 // lanes clip at different times and run loops of different lengths; eight
 // lanes per cell keep 24 busy.  Measured (GB300, us per step, one thread per
 // cell with the polygon in thread-local memory / this): 65,536 particles beside
-// a lattice 889 / 306, 1M uniform 10751 / 3498.
+// a lattice 889 / 306, 1M uniform 10751 / 3176.
 #pragma once
 #include "vk_voronoi.cuh"
 
@@ -36,6 +36,12 @@ namespace {
 #define VK_VOR_SQUARE 1.0f
 #endif
 // a cell that reaches farther than this many half-widths gets a larger square first
+// seeds that leave a cell this many times as wide as the one they come from are
+// followed by the squares (1.25, 2, 4: 65,536 particles 3717, 3727, 3733 us, 150 to
+// 8000 within 4 %)
+#ifndef VK_VOR_STALE
+#define VK_VOR_STALE 2.0f
+#endif
 #ifndef VK_VOR_REACH
 #define VK_VOR_REACH 4.0f
 #endif
@@ -274,6 +280,9 @@ struct Cell8 {
       open |= __ballot_sync(kAll, f[i] == 0);
     }
     if (open) {  // vertices that the estimate leaves undecided: exactly
+      // (no work for a site that is an edge already: a seed that comes round again)
+      const bool edge = group_bits((has(0) && slot[0] == sl) || (has(1) && slot[1] == sl)) != 0;
+      if (edge) f[0] = f[1] = -1;
       int2 nq[2];
       next_sites(big, nq);
       bool touch = false;
@@ -408,11 +417,12 @@ struct Cell8 {
               if (stage == kSeeds) {
                 left = seeds_left;
                 seeds_left = false;
-                qe = left ? (uint32_t)sd.n : 0u;
+                qb = 0;
+                qe = (uint32_t)sd.n;
               } else {
                 left = rc.next(R, G, &qb, &qe);
-                if (!left) qb = qe = 0;
               }
+              if (!left) qb = qe = 0;
               n_seen += qe - qb;
             }
             const int take = min((int)(qe - qb), kCG * kPer - n);
@@ -495,18 +505,20 @@ struct Cell8 {
       }
       if (other || stage == kBox) going = false;
       // a cell still much wider than the square: the box would hold far more
-      // particles than a larger square needs to close the cell.  (Seeds may
-      // leave a wide cell beside a void, but not an open one.)
-      const float reach = 2.0f * sqrtf(r2max);
-      if (stage == kSeeds && reach > 16.0f * w && w < wmax) {
+      // particles than a larger square needs to close the cell.  (Seeds leave a
+      // cell about as wide as it was, unless they are of a state long past.)
+      if (stage == kSeeds && reach() > VK_VOR_STALE * sd.reach && w < wmax) {
         stage = kSquare;
-      } else if (stage == kSquare && reach > VK_VOR_REACH * w && 2.0f * w < wmax) {
+      } else if (stage == kSquare && reach() > VK_VOR_REACH * w && 2.0f * w < wmax) {
         w *= 2.0f;
       } else {
         stage = kBox;
       }
     }
   }
+
+  // twice the largest distance of a vertex: no site farther away can cut the cell (group)
+  __device__ __forceinline__ float reach() const { return 2.0f * sqrtf(r2max); }
 
   // bit a: edge a is of positive length, i.e. its two vertices lie apart (group)
   __device__ __forceinline__ unsigned positive_edges() const {
