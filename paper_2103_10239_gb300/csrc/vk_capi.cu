@@ -714,12 +714,14 @@ vk_status vk_get_tissue(vk_sim* s, int32_t replica, double KA, double KP, double
   TissueScratch& w = s->tis;
   cudaError_t e = cudaSuccess;
   if (!s->tis_out) {
-    const bool ok = !((e = dalloc(&w.nb_n, N)) || (e = dalloc(&w.nb_slot, N * kTissueCap)) ||
-                      (e = dalloc(&w.nb_off, N * kTissueCap)) || (e = dalloc(&w.edge, N * kTissueCap)) ||
-                      (e = dalloc(&w.inv_len, N * kTissueCap)) || (e = dalloc(&w.blocks, kTissueBlocks)) || (e = dalloc(&w.area, N)) ||
+    w.cap = (int64_t)N * kTissueMean;
+    const size_t E = (size_t)w.cap;
+    const bool ok = !((e = dalloc(&w.used, 1)) || (e = dalloc(&w.row, N)) || (e = dalloc(&w.nb_slot, E)) ||
+                      (e = dalloc(&w.nb_off, E)) || (e = dalloc(&w.edge, E)) || (e = dalloc(&w.inv_len, E)) ||
+                      (e = dalloc(&w.blocks, kTissueBlocks)) || (e = dalloc(&w.area, N)) ||
                       (e = dalloc(&w.perim, N)) || (e = dalloc(&s->tis_out, 4 * N + 1)));
     if (!ok) {
-      void* part[] = {w.nb_n, w.nb_slot, w.nb_off, w.edge, w.inv_len, w.blocks, w.area, w.perim, s->tis_out};
+      void* part[] = {w.used, w.row, w.nb_slot, w.nb_off, w.edge, w.inv_len, w.blocks, w.area, w.perim, s->tis_out};
       for (void* p : part)
         if (p) cudaFree(p);
       w = TissueScratch{};
@@ -914,7 +916,7 @@ void vk_destroy(vk_sim* s) {
                   s->b.ovf_list, s->b.ovf_count, s->reps_d, s->tasks_d, s->b.sub_s, s->b.sub_base,
                   s->b.sub_count, s->b.sub_off, s->b.bsum2, s->d_stats, s->b.bounds,
                   s->st_pos, s->st_dir, s->st_theta, s->b.S_hint, s->b.U_hint, s->b.vor_seed,
-                  s->b.vor_seed_n, s->b.slot_of, s->tis.nb_n, s->tis.nb_slot, s->tis.nb_off, s->tis.edge,
+                  s->b.vor_seed_n, s->b.slot_of, s->tis.used, s->tis.row, s->tis.nb_slot, s->tis.nb_off, s->tis.edge,
                   s->tis.inv_len, s->tis.blocks, s->tis.area, s->tis.perim, s->tis_out};
   for (void* p : bufs)
     if (p) cudaFree(p);

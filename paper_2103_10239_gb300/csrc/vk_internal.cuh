@@ -733,19 +733,28 @@ cudaError_t launch_metric_step(const Geometry& g, const Buffers& b, const StepPa
 cudaError_t launch_metric_export(const Geometry& g, const Buffers& b, int rep, int n, int pass, int32_t* deg,
                                  const int64_t* out_off, int32_t* out_ids, cudaStream_t st);
 
-// vk_tissue.cu (Voronoi tissue model): per-slot scratch of the cells pass
-constexpr int kTissueCap = 32;  // edges per cell kept for the force pass
+// vk_tissue.cu (Voronoi tissue model): scratch of the cells pass.  The edges of
+// a cell are consecutive entries of the edge arrays, taken from a counter: a
+// periodic Voronoi diagram of N particles has at most 3 N edges, each an edge of
+// two cells, so 6 N entries hold all.
+constexpr int kTissueCap = 32;  // edges of one cell
+constexpr int kTissueMean = 6;  // entries per particle
 constexpr int kTissueBlocks = 608;
 struct TissueScratch {
-  int32_t* nb_n;     // edges of every cell (0: failed, status latched)
-  int32_t* nb_slot;  // kTissueCap per slot: edge sites, counter-clockwise
+  int64_t cap;       // entries of the edge arrays
+  unsigned long long* used;  // ... taken so far
+  // per slot
+  int64_t* row;      // first entry << kRowShift | edges (0: failed, status latched)
+  double* area;      // length units
+  double* perim;
+  // per entry
+  int32_t* nb_slot;  // edge sites, counter-clockwise
   int2* nb_off;      // ... and their exact offsets from the particle
   double2* edge;     // ... the edges as vectors, length units
   double* inv_len;   // ... and the inverse of their lengths
-  double* area;      // per slot, length units
-  double* perim;
   double* blocks;    // kTissueBlocks partial energies
 };
+constexpr int kRowShift = 6;
 // cells, forces (by id) and energy of one replica; any output may be NULL
 cudaError_t launch_tissue(const Geometry& g, const Buffers& b, int rep, int n, double KA, double KP, double A0,
                           double P0, double unit, TissueScratch w, double* area_out, double* perim_out,

@@ -10,7 +10,8 @@
 //      (vk_voronoi_fast.cuh, eight lanes each; vk_voronoi.cuh where that one
 //      cannot) and stores its edge sites in counter-clockwise order (sorted
 //      slot and exact offset), its edges as vectors with their inverse lengths,
-//      its area and its perimeter;
+//      its area and its perimeter; the edges of all cells are packed (36 bytes
+//      each, 6 a cell on average);
 //   2. forces, eight lanes per particle: for every vertex h of cell i (edge
 //      sites a, b) the three cells i, a, b that share h contribute dE_c/dh; the
 //      vertex's place in cells a and b comes from their stored edge lists
@@ -22,8 +23,9 @@
 // The FP64 units are few (about 0.6 Tops/s): recomputing circumcenters, edge
 // lengths and quotients at every vertex took 780 FP64 operations per vertex and
 // cell; with the stored edges it is about 110.  Measured (GB300, 1M uniform
-// particles, ms, before / after): cells 13.6 / 4.05, forces 11.1 / 2.31, energy
-// 3.1 / 0.03.
+// particles, ms, recomputed by one thread per cell / stored): cells 13.6 / 4.05,
+// forces 11.1 / 2.31, energy 3.1 / 0.03.  Packed rows in place of 32 entries per
+// cell: 273 instead of 1185 bytes a particle, and 6.45 / 6.11 ms for all three.
 #include "vk_voronoi_fast.cuh"
 
 namespace vk {
@@ -45,6 +47,10 @@ __device__ __forceinline__ double2 circum64(double ax, double ay, double bx, dou
 __device__ __forceinline__ double2 circum_off(int2 a, int2 b, double u) {
   return circum64((double)a.x * u, (double)a.y * u, (double)b.x * u, (double)b.y * u);
 }
+
+// first entry and edges of a stored cell
+__device__ __forceinline__ int64_t row_first(int64_t row) { return row >> kRowShift; }
+__device__ __forceinline__ int row_edges(int64_t row) { return (int)(row & ((1 << kRowShift) - 1)); }
 
 // Store edge a of a cell, from the vertex of sites (a - 1, a) to that of (a, a + 1).
 __device__ __forceinline__ void put_edge(const TissueScratch& w, int64_t at, int32_t slot, int2 off, double2 h0,
@@ -68,10 +74,13 @@ __device__ __noinline__ void tissue_cell_general(const Rep& R, int64_t s, const 
   Poly<kFastCap> P;
   int m = 0;
   double A = 0.0, Pm = 0.0;
+  int64_t first = 0;
   if (!voronoi_cell(R, s, pi, S_id[s], S_pos, S_id, G, P, status, 0u, sd, nullptr) || P.m > kTissueCap) {
     set_status(status, kStCapacity);
   } else if (P.nt > 0) {
     set_status(status, kStDegenerate);  // coincident particles: one site, no cell each
+  } else if ((first = (int64_t)atomicAdd(w.used, (unsigned long long)P.m)) + P.m > w.cap) {
+    set_status(status, kStDegenerate);  // more than 6 N edges: some are of zero length
   } else {
     m = P.m;
     double2 h0 = circum_off(make_int2(P.qx[m - 1], P.qy[m - 1]), make_int2(P.qx[0], P.qy[0]), unit);
@@ -83,12 +92,12 @@ __device__ __noinline__ void tissue_cell_general(const Rep& R, int64_t s, const 
       const double2 h1 = circum_off(make_int2(P.qx[a], P.qy[a]), make_int2(P.qx[na], P.qy[na]), unit);
       // an edge to an image of the particle itself (tiny boxes) is kept with
       // the particle's own slot and the image's offset
-      put_edge(w, s * kTissueCap + a, P.slot[a] >= 0 ? P.slot[a] : (int32_t)s, make_int2(P.qx[a], P.qy[a]), h0, h1, &A,
+      put_edge(w, first + a, P.slot[a] >= 0 ? P.slot[a] : (int32_t)s, make_int2(P.qx[a], P.qy[a]), h0, h1, &A,
                &Pm);
       h0 = h1;
     }
   }
-  w.nb_n[s] = m;
+  w.row[s] = m ? first << kRowShift | m : 0;
   w.area[s] = A;
   w.perim[s] = Pm;
 }
@@ -125,10 +134,24 @@ __global__ void __launch_bounds__(kTissueBlk, 4) tissue_cells_kernel(
     const int64_t gi = R.p0 + S_id[s];
     const Seeds sd = seeds_of(vor_seed, vor_seed ? vor_seed_n[gi] : 0, gi, slot_of);
     c.build(on, R, s, p, S_pos, G, sd, 2 * kHeavy);
-    const bool ok = on && !c.other;
+    bool ok = on && !c.other;
+    // entries for the four cells' edges
+    const int mine = ok ? c.m : 0;
+    int before = 0, all = 0;
+#pragma unroll
+    for (int g = 0; g < 32; g += kCG) {
+      const int v = __shfl_sync(kAll, mine, g);
+      before += g < c.base ? v : 0;
+      all += v;
+    }
+    unsigned long long taken = 0;
+    if (lane == 0) taken = atomicAdd(w.used, (unsigned long long)all);
+    const int64_t first = (int64_t)__shfl_sync(kAll, taken, 0) + before;
+    const bool fits = first + mine <= w.cap;  // if not, some edges are of zero length
+    if (ok && !fits) ok = false;
     // an edge of zero length (four cocircular particles): no derivative
     const unsigned positive = c.positive_edges();
-    if (ok && c.gl == 0 && positive != (1u << c.m) - 1u) set_status(status, kStDegenerate);
+    if (on && !c.other && c.gl == 0 && (!fits || positive != (1u << c.m) - 1u)) set_status(status, kStDegenerate);
     // vertex after each of the lane's edges, and the one before
     const bool big = __any_sync(kAll, c.m > 8);
     int2 nq[2];
@@ -148,13 +171,13 @@ __global__ void __launch_bounds__(kTissueBlk, 4) tissue_cells_kernel(
         if (j >= 8) h0 = h8;
       }
       if (ok && c.has(i))
-        put_edge(w, s * kTissueCap + a, c.slot[i] >= 0 ? c.slot[i] : (int32_t)s, c.q[i], h0, h[i], &A, &Pm);
+        put_edge(w, first + a, c.slot[i] >= 0 ? c.slot[i] : (int32_t)s, c.q[i], h0, h[i], &A, &Pm);
     }
     A = group_sum(A);
     Pm = group_sum(Pm);
     if (on && c.gl == 0) {
-      if (ok) {
-        w.nb_n[s] = c.m;
+      if (!c.other) {
+        w.row[s] = ok ? first << kRowShift | c.m : 0;
         w.area[s] = A;
         w.perim[s] = Pm;
       } else {
@@ -202,16 +225,16 @@ __global__ void __launch_bounds__(kTissueBlk) tissue_force_kernel(
     const bool on = li < R.n;
     const int64_t s = R.p0 + (on ? li : 0);
     const int32_t id = S_id[s];
-    const int m = on ? w.nb_n[s] : 0;
+    const int64_t own = on ? w.row[s] : 0, row = row_first(own);
+    const int m = row_edges(own);
     const double area = w.area[s], perim = w.perim[s];
     if (on && gl == 0 && area_out) area_out[id] = area;
     if (on && gl == 0 && perim_out) perim_out[id] = perim;
     if (!force_out) continue;
-    const int64_t row = s * kTissueCap;
     for (int k = gl; k < m; k += kCG) {
-      const int64_t ra = (int64_t)w.nb_slot[row + k] * kTissueCap;
+      const int64_t wa = w.row[w.nb_slot[row + k]], ra = row_first(wa);
       const int2 d = w.nb_off[row + k];
-      place[grp][k] = (int8_t)find_entry(w.nb_slot + ra, w.nb_off + ra, w.nb_n[w.nb_slot[row + k]], (int32_t)s,
+      place[grp][k] = (int8_t)find_entry(w.nb_slot + ra, w.nb_off + ra, row_edges(wa), (int32_t)s,
                                          make_int2(-d.x, -d.y));
     }
     __syncwarp();
@@ -222,9 +245,9 @@ __global__ void __launch_bounds__(kTissueBlk) tissue_force_kernel(
       const int kn = k + 1 == m ? 0 : k + 1;
       const int32_t sa = w.nb_slot[row + k], sb = w.nb_slot[row + kn];
       const int2 da = w.nb_off[row + k], db = w.nb_off[row + kn];
-      const int64_t ra = (int64_t)sa * kTissueCap, rb = (int64_t)sb * kTissueCap;
+      const int64_t wa = w.row[sa], wb = w.row[sb], ra = row_first(wa), rb = row_first(wb);
       // cell a: around a the sites run ... b, i ...; cell b: ... i, a ...
-      const int ma = w.nb_n[sa], mb = w.nb_n[sb], ta = place[grp][k], tb = place[grp][kn];
+      const int ma = row_edges(wa), mb = row_edges(wb), ta = place[grp][k], tb = place[grp][kn];
       const int tp = ta <= 0 ? ma - 1 : ta - 1, tn = tb < 0 || tb + 1 == mb ? 0 : tb + 1;
       ok = ta >= 0 && tb >= 0;
       if (ok) {
@@ -335,6 +358,8 @@ cudaError_t launch_tissue(const Geometry& g, const Buffers& b, int rep, int n, d
   if (n == 0) return cudaSuccess;
   const TissueParams T{KA, KP, A0, P0, unit};
   const int sms = device_sm_count(), per = kTissueBlk / kCG;
+  const cudaError_t e = cudaMemsetAsync(w.used, 0, sizeof(*w.used), st);
+  if (e != cudaSuccess) return e;
   tissue_cells_kernel<<<std::min((n + per - 1) / per, sms * 16), kTissueBlk, 0, st>>>(
       g.reps, rep, (const int2*)b.S_pos, b.S_id, tissue_view(b), unit, w, b.d_status, b.vor_seed, b.vor_seed_n,
       b.slot_of);
