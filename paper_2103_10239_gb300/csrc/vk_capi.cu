@@ -259,6 +259,9 @@ void refresh_geometry(vk_sim* s) {
   s->g.n_tasks = (int)s->tasks_h.size();
   s->g.reps = s->reps_d;
   s->g.tasks = s->tasks_d;
+  s->g.metric_wide = false;
+  if (s->prm.rule == VK_RULE_METRIC && s->dim == 2)
+    for (const Rep& R : s->reps_h) s->g.metric_wide = s->g.metric_wide || metric_wide(R);
 }
 
 vk_status upload_reps(vk_sim* s) {

@@ -617,6 +617,18 @@ inline void plan_grid2(Rep& R, double side) {
   R.nc[2] = 1;
 }
 
+// Metric rule, 2D: may the rectangle of the particles of one coarse cell (at
+// most 2^sh + 2 r0q wide) reach half a period, or meet a coarse cell twice?  (It
+// meets at most one cell more than its width says, and one for the last cell of
+// the axis, which may be narrower.)
+inline bool metric_wide(const Rep& R) {
+  for (int a = 0; a < 2; ++a) {
+    const int64_t w = (1ll << R.sh[a]) + 2 * (int64_t)R.r0q;
+    if (2 * w >= (int64_t)R.L[a] || (w >> R.sh[a]) + 2 >= R.nc[a]) return true;
+  }
+  return false;
+}
+
 // streaming multiprocessors of the current device (for fixed-size grids)
 inline int device_sm_count() {
   int dev = 0, sms = 0;
@@ -682,6 +694,7 @@ struct Geometry {
   int64_t n_cells;
   int64_t n_sub_max;  // bound of the number of sub-cells: n_cells + n_total / kSubTarget
   int n_tasks;
+  bool metric_wide;   // metric rule, 2D: of some replica (see metric_wide)
   const Rep* reps;
   const BlockTask* tasks;
 };

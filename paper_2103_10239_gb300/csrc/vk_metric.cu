@@ -108,6 +108,13 @@ struct MetricStage {
 
 constexpr int kMetricBlk = 128;
 
+// WIDE: some rectangle of some replica may reach half a period or meet a coarse
+// cell twice (metric_wide).  The rectangle is then cut per axis, and minimum
+// images are taken one by one (20,000 particles, r0 a fifth and a quarter of the
+// box: 464 and 682 us per step; the whole box for such rectangles 2148 and 3424, one
+// thread per square 1179 and 1459).  The narrow kernel has no code for that: with
+// it, it loses 5 to 10 %.
+template <bool WIDE>
 __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
     const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const int2* __restrict__ S_pos,
     const float2* __restrict__ S_dir, const int32_t* __restrict__ S_id, GridView G, int2* __restrict__ U_pos,
@@ -143,22 +150,29 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
     left &= ~__ballot_sync(0xffffffffu, on);
     const int32_t x0 = __reduce_min_sync(0xffffffffu, on ? p.x : INT_MAX), x1 = __reduce_max_sync(0xffffffffu, on ? p.x : -1);
     const int32_t y0 = __reduce_min_sync(0xffffffffu, on ? p.y : INT_MAX), y1 = __reduce_max_sync(0xffffffffu, on ? p.y : -1);
-    // their rectangle; offsets within it are exact in one image while it is
-    // narrower than half a period and meets no coarse cell twice
+    // their rectangle.  Offsets within it are exact in one image while it is
+    // narrower than half a period; otherwise minimum images are taken one by
+    // one.  An axis that it covers, or on which it meets a coarse cell twice, is
+    // covered whole.
     const int64_t ax = x0 - r, bx = x1 + r, ay = y0 - r, by = y1 + r;
     const long long lim = on ? r2 : -1;  // squared distances are >= 0: the other lanes find nothing
-    bool whole = 2 * (bx - ax + 1) >= Lx || 2 * (by - ay + 1) >= Ly;
-    int ux0 = 0, ux1 = 0, uy0 = 0, uy1 = 0;
-    if (!whole) {
+    bool fullx = WIDE && bx - ax + 1 >= Lx, fully = WIDE && by - ay + 1 >= Ly;
+    int ux0 = 0, ux1 = nx - 1, uy0 = 0, uy1 = ny - 1;
+    if (!fullx) {
       ux0 = ucell2(ax, nx, shx, Lx);
       ux1 = ucell2(bx, nx, shx, Lx);
+      fullx = WIDE && ux1 - ux0 >= nx;
+      if (fullx) ux0 = 0, ux1 = nx - 1;
+    }
+    if (!fully) {
       uy0 = ucell2(ay, ny, shy, Ly);
       uy1 = ucell2(by, ny, shy, Ly);
-      whole = ux1 - ux0 >= nx || uy1 - uy0 >= ny;
+      fully = WIDE && uy1 - uy0 >= ny;
+      if (fully) uy0 = 0, uy1 = ny - 1;
     }
-    // candidates [qb, qe); (ox, oy): the period added to their coordinates, or
-    // (all) minimum images taken one by one
-    auto scan = [&](int64_t qb, int64_t qe, uint32_t ox, uint32_t oy, bool all) {
+    const bool image = WIDE && (fullx || fully || 2 * (bx - ax + 1) >= Lx || 2 * (by - ay + 1) >= Ly);
+    // candidates [qb, qe); (ox, oy): the period added to their coordinates (unless `image`)
+    auto scan = [&](int64_t qb, int64_t qe, uint32_t ox, uint32_t oy) {
       n_cand += on ? (uint32_t)(qe - qb) : 0u;
       for (int64_t q0 = qb; q0 < qe; q0 += 32) {
         const int n = (int)min(qe - q0, (int64_t)32);
@@ -170,12 +184,12 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
           M.head[lane] = make_longlong2(phi_fixed(d.x), phi_fixed(d.y));
         }
         __syncwarp();
-        auto test = [&](int j, bool image) {
+        auto test = [&](int j, bool wrap) {
           const int2 pj = M.pos[j];
           int32_t dx = (int32_t)((uint32_t)pj.x - (uint32_t)p.x), dy = (int32_t)((uint32_t)pj.y - (uint32_t)p.y);
-          if (image) {
-            dx = (int32_t)min_image((int64_t)pj.x - p.x, Lx);
-            dy = (int32_t)min_image((int64_t)pj.y - p.y, Ly);
+          if (wrap) {  // a distance of half a period is the same in both images
+            dx = (uint32_t)abs(dx) > R.L[0] / 2 ? (int32_t)(R.L[0] - (uint32_t)abs(dx)) : dx;
+            dy = (uint32_t)abs(dy) > R.L[1] / 2 ? (int32_t)(R.L[1] - (uint32_t)abs(dy)) : dy;
           }
           if ((int64_t)dx * dx + (int64_t)dy * dy <= lim) {
             const longlong2 h = M.head[j];
@@ -184,7 +198,8 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
             ++S.m;
           }
         };
-        if (all) {
+        if (image) {
+#pragma unroll 4
           for (int j = 0; j < n; ++j) test(j, true);
         } else {
 #pragma unroll 4
@@ -192,8 +207,8 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
         }
       }
     };
-    if (whole) {
-      scan(R.p0, R.p0 + R.n, 0u, 0u, true);
+    if (fullx && fully) {
+      scan(R.p0, R.p0 + R.n, 0u, 0u);
       continue;
     }
     const uint32_t fx0 = cell_frac((uint32_t)(ax < 0 ? ax + Lx : ax), shx);
@@ -204,15 +219,15 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
       for (int ux = ux0; ux <= ux1; ++ux) {
         const int wy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy);
         const int wx = ux < 0 ? ux + nx : (ux >= nx ? ux - nx : ux);
-        const uint32_t ox = ux < 0 ? 0u - R.L[0] : (ux >= nx ? R.L[0] : 0u);
-        const uint32_t oy = uy < 0 ? 0u - R.L[1] : (uy >= ny ? R.L[1] : 0u);
+        const uint32_t ox = image ? 0u : ux < 0 ? 0u - R.L[0] : (ux >= nx ? R.L[0] : 0u);
+        const uint32_t oy = image ? 0u : uy < 0 ? 0u - R.L[1] : (uy >= ny ? R.L[1] : 0u);
         const int64_t gc = R.c0 + (int64_t)wy * nx + wx;
         const uint32_t base = __ldg(G.sub_base + gc);
         const int sd = __ldg(G.sub_s + gc);
-        const int c0 = ux == ux0 ? sub_of(fx0, sd) : 0, c1 = ux == ux1 ? sub_of(fx1, sd) : sd - 1;
-        const int r0 = uy == uy0 ? sub_of(fy0, sd) : 0, r1 = uy == uy1 ? sub_of(fy1, sd) : sd - 1;
+        const int c0 = ux == ux0 && !fullx ? sub_of(fx0, sd) : 0, c1 = ux == ux1 && !fullx ? sub_of(fx1, sd) : sd - 1;
+        const int r0 = uy == uy0 && !fully ? sub_of(fy0, sd) : 0, r1 = uy == uy1 && !fully ? sub_of(fy1, sd) : sd - 1;
         if (c0 == 0 && c1 == sd - 1) {  // whole rows follow one another
-          scan(__ldg(G.sub_off + base + r0 * sd), __ldg(G.sub_off + base + (r1 + 1) * sd), ox, oy, false);
+          scan(__ldg(G.sub_off + base + r0 * sd), __ldg(G.sub_off + base + (r1 + 1) * sd), ox, oy);
           continue;
         }
         for (int rr = r0; rr <= r1; rr += 32) {
@@ -226,7 +241,7 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
           while (rows) {
             const int j = __ffs(rows) - 1;
             rows &= rows - 1u;
-            scan(__shfl_sync(0xffffffffu, qb, j), __shfl_sync(0xffffffffu, qe, j), ox, oy, false);
+            scan(__shfl_sync(0xffffffffu, qb, j), __shfl_sync(0xffffffffu, qe, j), ox, oy);
           }
         }
       }
@@ -455,10 +470,10 @@ GridView metric_view(const Buffers& b) {
 
 cudaError_t launch_metric_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {
   if (g.dim == 2) {
-    metric2_step_kernel<<<g.n_tasks * (kBlock / kMetricBlk), kMetricBlk, 0, st>>>(g.reps, g.tasks, (const int2*)b.S_pos,
-                                                      (const float2*)b.S_dir, b.S_id, metric_view(b),
-                                                      (int2*)b.U_pos, (float2*)b.U_dir, b.U_id, b.counts,
-                                                      b.phi_acc, b.d_step, P);
+    auto kernel = g.metric_wide ? metric2_step_kernel<true> : metric2_step_kernel<false>;
+    kernel<<<g.n_tasks * (kBlock / kMetricBlk), kMetricBlk, 0, st>>>(
+        g.reps, g.tasks, (const int2*)b.S_pos, (const float2*)b.S_dir, b.S_id, metric_view(b), (int2*)b.U_pos,
+        (float2*)b.U_dir, b.U_id, b.counts, b.phi_acc, b.d_step, P);
   } else {
     metric3_step_kernel<<<g.n_tasks, kBlock, 0, st>>>(g.reps, g.tasks, b.bounds, (const int4*)b.S_pos,
                                                       (const float4*)b.S_dir, b.S_id, metric_view(b),
