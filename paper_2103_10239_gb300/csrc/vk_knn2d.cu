@@ -61,6 +61,20 @@ struct BoxShared {
   uint2 run[BoxCfg<KC>::RUNS][kBlk];  // (first slot, length << 4 | image shift codes)
 };
 
+// A thread does not take a square of more coarse cells or more candidates than
+// these: a particle outside a cluster has a wide square, most of it empty cells,
+// and a first radius, guessed from the density around it, that may hold the whole
+// cluster, and the whole launch waits for it.  The groups look at 16 cells and 16
+// candidates at a time.  Ordinary squares meet one to four cells and 30 to 180
+// candidates.  Measured (us; no limits / 144 and 1024 / 64 and 1024 / 25 and 512 / 25
+// and 256): 65,536 particles around one point, all lists, k = 7 2896, 460, 460, 289,
+// 259, k = 32 11,680, 617, 634, 544, 501; 200,000 in a wide cluster, a step 210, 231,
+// 203, 189, 190, and around one point 329, 326, 326, 336, 349.  Not in a field of
+// view, whose squares are wider for every particle that faces a void (1M 4.1 ms a
+// pass without, 4.5 with).
+constexpr int kMaxCells = 25;
+constexpr uint32_t kMaxCand = 512;
+
 // the slot behind a key of the list
 template <int KC>
 __device__ __forceinline__ int32_t key_slot(const BoxShared<KC>& H, uint32_t key) {
@@ -86,7 +100,7 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
   const int32_t a = (int32_t)ceilf(fminf(radius, 1.0e9f));
   *r_next = (float)a;
   const uint32_t Lx = R.L[0], Ly = R.L[1];
-  bc.why = 1u;  // too wide for the minimum image, or a coarse cell met through two periodic images
+  bc.why = 1u;  // too wide for the minimum image, a coarse cell met through two periodic images, or too many cells
   if (4ll * a + 2 >= (int64_t)Lx || 4ll * a + 2 >= (int64_t)Ly) return false;
   const int nx = R.nc[0], ny = R.nc[1], shx = R.sh[0], shy = R.sh[1];
   const int tid = (int)threadIdx.x;
@@ -98,9 +112,11 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
   const int ucx0 = (int)(x0 >> shx) - (wx0 ? nx : 0), ucx1 = (int)(x1 >> shx) + (wx1 ? nx : 0);
   const int ucy0 = (int)(y0 >> shy) - (wy0 ? ny : 0), ucy1 = (int)(y1 >> shy) + (wy1 ? ny : 0);
   if (ucx1 - ucx0 >= nx || ucy1 - ucy0 >= ny) return false;
+  if (!FOV && (ucx1 - ucx0 + 1) * (ucy1 - ucy0 + 1) > kMaxCells) return false;
   const uint32_t fx0 = cell_frac(x0, shx), fx1 = cell_frac(x1, shx);
   const uint32_t fy0 = cell_frac(y0, shy), fy1 = cell_frac(y1, shy);
   bc.tries += 1;
+  const uint32_t cand0 = bc.cand;
   // below (a + 1)^2 by more than the rounding of the distances
   const float a1 = (float)a + 1.0f;
   float tau = a1 * a1 * (1.0f - 9.5367431640625e-07f);
@@ -112,15 +128,17 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
   int ucx = ucx0, ucy = ucy0, row = 0, row_end = -1, s = 1, nrun = 0, r = 0;
   uint32_t lo = 0, hi = 0, code = 0;  // first and one-past-last sub-cell of the row
   uint32_t q = 0, qb = 0, len = 0, ox = 0, oy = 0;
-  bool more = true, done = false;
+  bool more = true, done = false, heavy = false;
   for (;;) {
     while (cnt <= CAP - 4) {
       if (q - qb >= len) {  // next run
         if (r == nrun) {
           // list up to RUNS runs, so that one flat loop scans them and the
           // threads of a warp scan candidates together however their squares split
+          // (no return from here: the warp's threads have to meet again)
+          heavy = !FOV && bc.cand - cand0 > kMaxCand;
           nrun = r = 0;
-          while (more && nrun <= BoxCfg<KC>::RUNS - 2) {
+          while (more && !heavy && nrun <= BoxCfg<KC>::RUNS - 2) {
             if (row > row_end) {  // next coarse cell
               if (ucx > ucx1) {
                 ucx = ucx0;
@@ -227,6 +245,11 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
     if (t[KC - 2] < 0xFF000000u) tau = fminf(tau, __uint_as_float(((t[KC - 2] >> B) + 3u) << B));
   }
   bc.hits += (uint32_t)got;
+  if (heavy) {  // only a part was scanned: as wide next as it says that about 1.5 k hits need
+    *r_next = (float)a * sqrtf((1.5f * (float)k + 1.f) / (float)(bc.cand - cand0));
+    bc.why = 4u;
+    return false;
+  }
   if ((t[KC - 2] >> B) + 1u < edge) {
     bool close = false;  // a pair whose order the keys leave open
 #pragma unroll
@@ -288,8 +311,10 @@ struct Group : GroupTop<GS, CAP> {
   // covered whole).  The lanes look at GS coarse cells at a time, so that
   // empty ones cost little; a non-empty one is scanned by rows of the
   // sub-cells that meet the square of half-width min(a, sqrt(tau)): a list
-  // that has filled up on the way leaves little to scan.  True when the
-  // square is the whole box.
+  // that has filled up on the way leaves little to scan.  Near cells and rows
+  // go first: of a cluster that the square reaches from outside, met from its far
+  // side, every particle would be nearer than the last (65,536 particles around one
+  // point, k = 32: 7890 / 634 us for all lists).  True when the square is the whole box.
   __device__ __forceinline__ bool square(const Rep& R, const GridView& G, int64_t a) {
     const int64_t Lx = C.Lx, Ly = C.Ly;
     const int nx = R.nc[0], ny = R.nc[1], shx = R.sh[0], shy = R.sh[1];
@@ -301,7 +326,10 @@ struct Group : GroupTop<GS, CAP> {
     tau = fullx && fully ? ~0ull : (unsigned long long)(a + 1) * (unsigned long long)(a + 1) - 1;
     unsigned long long at = ~0ull;  // the tau that w was taken for
     int64_t w = a;
-    for (int uy = uy0; uy <= uy1; ++uy) {
+    const int ownx = (int)(C.px >> shx), owny = (int)(C.py >> shy);
+    for (int iy = uy0; iy <= uy1; ++iy) {
+      const int uy = iy <= owny ? owny + uy0 - iy : iy;  // down from the particle's own, then up
+      const bool below = uy < owny;
       const int cy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy);
       const int64_t rb = R.c0 + (int64_t)cy * nx;
       for (int uc = ux0; uc <= ux1; uc += GS) {
@@ -309,9 +337,11 @@ struct Group : GroupTop<GS, CAP> {
         const int64_t lc = rb + (lx < 0 ? lx + nx : (lx >= nx ? lx - nx : lx));
         const bool some = lx <= ux1 && __ldg(G.off + lc) != __ldg(G.off + lc + 1);
         unsigned cells = (__ballot_sync(mask, some) & mask) >> shift;
+        const unsigned left = ownx < uc ? 0u : ownx - uc >= GS ? ~0u : (2u << (ownx - uc)) - 1u;
         while (cells) {
-          const int ux = uc + __ffs(cells) - 1;
-          cells &= cells - 1u;
+          const int bit = cells & left ? 31 - __clz(cells & left) : __ffs(cells) - 1;
+          const int ux = uc + bit;
+          cells &= ~(1u << bit);
           const int64_t gc = rb + (ux < 0 ? ux + nx : (ux >= nx ? ux - nx : ux));
           const uint32_t base = __ldg(G.sub_base + gc);
           const int s = __ldg(G.sub_s + gc);
@@ -327,7 +357,7 @@ struct Group : GroupTop<GS, CAP> {
             // each lane looks up one row of sub-cells
             uint32_t qb = 0, qe = 0;
             if (rr + gl <= r1) {
-              const uint32_t lo = base + (uint32_t)((rr + gl) * s);
+              const uint32_t lo = base + (uint32_t)((below ? r0 + r1 - rr - gl : rr + gl) * s);
               qb = __ldg(G.sub_off + lo + sx0);
               qe = __ldg(G.sub_off + lo + sx1 + 1);
             }
