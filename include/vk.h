@@ -281,9 +281,10 @@ vk_status vk_get_search_stats(vk_sim* sim, double* mean_candidates, double* mean
 
 /* Raw totals of the search counters collected while tracing at level 2, in
  * this order: 0 candidates examined (summed over particle updates), 1 slot
- * runs or squares scanned, 2 largest candidate count of one particle update,
- * 3 particle updates, 4 updates that the general code finished (2D kNN: groups
- * of lanes; 2D Voronoi: the warp kernel); 2D kNN's first squares only, over the
+ * runs or squares scanned (2D kNN: also for particles then handed on), 2 largest
+ * candidate count of one particle update, 3 particle updates, 4 updates that the
+ * general code finished (2D kNN: groups of lanes; 2D Voronoi: the warp kernel);
+ * 2D kNN's first squares only, over the
  * particles they served or handed on: 5 squares scanned, 6 slot runs, 7
  * candidates, 8 coarse cells visited, 9 hits merged, and the particles handed
  * on because 10 the square was too wide for the box or met too many coarse

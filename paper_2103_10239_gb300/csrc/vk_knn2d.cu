@@ -464,7 +464,8 @@ __device__ __forceinline__ float box_radius_estimate(const Rep& R, const GridVie
   return 1.6f * sqrtf((float)k * area / (3.14159265f * (float)max(cnt, 1u)));
 }
 
-// Tracing: totals of the radius-first counters (stats[5..13]).
+// Tracing: totals of the radius-first counters (stats[5..13]; the squares also count
+// in stats[1]).
 __device__ __forceinline__ void record_box_stats(unsigned long long* stats, const BoxCount& bc) {
   if (!stats) return;
   unsigned long long v[9] = {bc.tries, bc.runs, bc.cand, bc.cells, bc.hits, bc.why == 1u, bc.why == 2u,
@@ -473,9 +474,11 @@ __device__ __forceinline__ void record_box_stats(unsigned long long* stats, cons
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
     for (int i = 0; i < 9; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-  if ((threadIdx.x & 31) == 0)
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(stats + 1, v[0]);
 #pragma unroll
     for (int i = 0; i < 9; ++i) atomicAdd(stats + 5 + i, v[i]);
+  }
 }
 
 // Append (slot, replica) to a device list, one atomic per warp: the
@@ -505,7 +508,8 @@ struct StepOut {
   const int64_t* __restrict__ d_step;
   StepParams P;
   static constexpr bool kStep = true;
-  // by slot: the radius a handed-on particle tries next (its hint replaces it in the end)
+  // by slot: the radius a handed-on particle tries next, negative where only a
+  // group can serve it (its hint replaces it in the end)
   __device__ __forceinline__ float* radius() const { return U_hint; }
   template <class At>
   __device__ __forceinline__ void put(const Rep& R, int64_t step, int64_t s, int2 p, int32_t id, At at, float dk,
@@ -534,6 +538,12 @@ struct RowOut {
       }
   }
 };
+
+// what a particle that a thread could not serve is left with: close distances
+// and squares too wide stay what they are, so that another thread would fail too
+__device__ __forceinline__ float left_radius(float r, const BoxCount& bc) {
+  return bc.why == 1u || bc.why == 3u ? -r : r;
+}
 
 // the first radius of a particle
 __device__ __forceinline__ float box_radius(const Rep& R, const GridView& G, int2 p, float hint, const StepParams& P) {
@@ -578,10 +588,10 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_box_step_kernel
     const int64_t s = R.p0 + li;
     float r = box_radius(R, G, S_pos[s], S_hint[s], out.P);
     served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, step, out, &r, bc, nnew);
-    if (!served) out.radius()[s] = r;
+    if (!served) out.radius()[s] = left_radius(r, bc);
   }
   warp_append(valid && !served, make_int2((int)(R.p0 + li), t.rep), defer_list, defer_count);
-  record_search_stats(out.P.stats, served, bc.cand, bc.tries, false);
+  record_search_stats(out.P.stats, served, bc.cand, 0u, false);
   record_box_stats(out.P.stats, bc);
   phi_block_end<2>(phs, nnew,
                    out.phi_acc + ((size_t)(step % out.P.phi_cap) * (size_t)out.P.n_rep + (size_t)t.rep) * 3);
@@ -603,7 +613,7 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_box_export_kern
     BoxCount bc;
     float r = box_radius(R, G, S_pos[s], S_hint ? S_hint[s] : 0.f, out.P);
     served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, 0, out, &r, bc, nullptr);
-    if (!served) out.radius()[s] = r;
+    if (!served) out.radius()[s] = left_radius(r, bc);
   }
   warp_append(valid && !served, make_int2((int)s, rep), defer_list, defer_count);
 }
@@ -638,14 +648,17 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_second_kernel(
       e = list[i];
       const Rep R = reps[e.y];
       float r = out.radius()[e.x];
-      for (int tr = 0; tr < kSecondTries && !served; ++tr)
+      for (int tr = 0; tr < kSecondTries && !served && r > 0.f; ++tr) {
         served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, e.x, step, out, &r, bc, nnew);
+        if (!served) r = left_radius(r, bc);
+      }
       if (!served) out.radius()[e.x] = r;
     }
     warp_append(valid && !served, e, left_list, left_count);
     if constexpr (Out::kStep) {
       phi_add_warp<2>(out.phi_acc + (size_t)(step % out.P.phi_cap) * (size_t)out.P.n_rep * 3, e.y, nnew, served);
-      record_search_stats(out.P.stats, served, bc.cand, bc.tries, false);
+      record_search_stats(out.P.stats, served, bc.cand, 0u, false);
+      if (out.P.stats && bc.tries) atomicAdd(out.P.stats + 1, (unsigned long long)bc.tries);
     }
   }
 }
@@ -703,7 +716,7 @@ __global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel
       init_ctx(g.C, R, e.x, p);
       if (FOV) g.C.view = make_view(out.S_dir[e.x], out.P.fov_cq);
       g.k = k;
-      float r = all ? box_radius(R, G, p, S_hint ? S_hint[e.x] : 0.f, out.P) : out.radius()[e.x];
+      float r = all ? box_radius(R, G, p, S_hint ? S_hint[e.x] : 0.f, out.P) : fabsf(out.radius()[e.x]);
       uint32_t tries = 1;
       g.n_cand = 0;
       for (;; ++tries) {
