@@ -674,6 +674,7 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_second_kernel(
 // start to end, however few there are, and the listed ones wait for it.
 constexpr int kGS = 16;
 constexpr int kGroupBlk = 128;
+constexpr float kWholeBox = 4.6e18f;  // squared distance beyond every box's
 
 template <int KC, bool FOV, class Out>
 __global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel(
@@ -727,7 +728,8 @@ __global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel
         r = (float)a * (g.cnt > 0 ? fminf(sqrtf(want / (float)g.cnt), 2.f) : 2.f) + 1.f;
       }
       for (int j = g.cnt + g.gl; j < k; j += kGS) res[wid][i][j] = -1;
-      if (g.gl == 0) res_d[wid][i] = 0.f;
+      // (a view that holds fewer than k: the next search begins with the whole box)
+      if (g.gl == 0) res_d[wid][i] = FOV && g.cnt < k ? kWholeBox : 0.f;
       __syncwarp(g.mask);
       g.rank([&](int, int rk, unsigned long long D, int32_t q) {
         if (rk < k) res[wid][i][rk] = q;
