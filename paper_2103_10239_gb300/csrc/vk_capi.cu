@@ -135,11 +135,14 @@ StepParams step_params(const vk_sim* s) {
   return P;
 }
 
-// Occupancies chosen by vk_autotune, keyed by (dimension, rule, k, size
-// bucket = floor(log2(mean particles per replica))): a later sim of the same
+constexpr int64_t kLargeFlock = 1 << 17;  // particles in all, from which 2D kNN cells are smaller
+
+// Occupancies chosen by vk_autotune, keyed by what the default depends on
+// (dimension, rule, field of view or not, large in all or not), k, and a size
+// bucket = floor(log2(mean particles per replica)): a later sim of the same
 // kind whose caller leaves cell_occupancy at 0 starts from the tuned value.
 // Process-wide; speed only.
-using TuneKey = std::tuple<int, int, int, int>;
+using TuneKey = std::tuple<int, int, int, bool, bool, int>;
 std::map<TuneKey, float> g_tuned;
 std::mutex g_tuned_mu;
 
@@ -147,7 +150,8 @@ TuneKey tune_key(const vk_params& p, int dim, int64_t n_total, int n_rep) {
   const int64_t mean = std::max<int64_t>(1, n_total / std::max(1, n_rep));
   int bucket = 0;
   while ((int64_t)1 << (bucket + 1) <= mean) ++bucket;
-  return TuneKey(dim, p.rule, p.rule == VK_RULE_KNN ? p.k : 0, bucket);
+  const bool knn = p.rule == VK_RULE_KNN;
+  return TuneKey(dim, p.rule, knn ? p.k : 0, knn && p.fov, n_total >= kLargeFlock, bucket);
 }
 
 float default_occupancy(const vk_params& p, int dim, int64_t n_total, int n_rep) {
@@ -170,7 +174,7 @@ float default_occupancy(const vk_params& p, int dim, int64_t n_total, int n_rep)
   // Metric rule, whose rectangles are of one cell: 256 in 2D; 1.5 in 3D (the best
   // lies between 1 and 4 as r0 goes)
   if (p.rule == VK_RULE_KNN && dim == 3) return 3.5f;
-  if (p.rule == VK_RULE_KNN && !p.fov && n_total >= 1 << 17) return 64.0f;
+  if (p.rule == VK_RULE_KNN && !p.fov && n_total >= kLargeFlock) return 64.0f;
   return dim == 2 ? 256.0f : 1.5f;
 }
 
