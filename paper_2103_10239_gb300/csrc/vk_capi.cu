@@ -31,6 +31,48 @@ const char* kPhaseNames[kPhases] = {"search_update", "build", "scatter", "load_s
 
 thread_local std::string g_init_error;
 
+// Pinned host memory of a sim, read by the host after a wait for its stream.
+// Allocating and freeing it takes 120 and 180 us, more than the rest of a small
+// sim, so up to kHostKeep blocks of closed sims wait for the next ones (a block
+// serves a sim on any device; one that a reset of the device has taken is dropped).
+struct HostBlock {
+  int32_t status;                // the device status
+  long long phi[3 * kPhiRows];   // heading sums of some steps
+};
+constexpr size_t kHostKeep = 16;
+std::mutex g_host_mu;
+std::vector<HostBlock*> g_host_blocks;
+
+cudaError_t take_host_block(HostBlock** out) {
+  {
+    std::lock_guard<std::mutex> lock(g_host_mu);
+    while (!g_host_blocks.empty()) {
+      HostBlock* b = g_host_blocks.back();
+      g_host_blocks.pop_back();
+      cudaPointerAttributes at;
+      if (cudaPointerGetAttributes(&at, b) == cudaSuccess && at.type == cudaMemoryTypeHost) {
+        *out = b;
+        return cudaSuccess;
+      }
+      cudaGetLastError();
+    }
+  }
+  return cudaHostAlloc((void**)out, sizeof(HostBlock), cudaHostAllocPortable);
+}
+
+// (after a wait for the work that writes it)
+void give_host_block(HostBlock* b) {
+  if (!b) return;
+  {
+    std::lock_guard<std::mutex> lock(g_host_mu);
+    if (g_host_blocks.size() < kHostKeep) {
+      g_host_blocks.push_back(b);
+      return;
+    }
+  }
+  cudaFreeHost(b);
+}
+
 }  // namespace
 
 struct vk_sim {
@@ -74,9 +116,8 @@ struct vk_sim {
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev[kPhases];
   double prof_ms[kPhases] = {0, 0, 0, 0, 0, 0};
   int64_t prof_launches[kPhases] = {0, 0, 0, 0, 0, 0};
-  int32_t* h_status = nullptr;   // pinned word that the device status is read into
-  long long* h_phi = nullptr;    // pinned: the heading sums of up to kPhiRows steps ...
-  std::mutex h_phi_mu;           // ... (readers of several replicas may be on several threads)
+  HostBlock* host = nullptr;
+  std::mutex host_phi_mu;  // of host->phi: readers of several replicas may be on several threads
   unsigned long long* d_stats = nullptr;  // search counters, collected while tracing
   std::string err;
 };
@@ -302,9 +343,9 @@ vk_status sort_from_U(vk_sim* s, bool keep_search_state = false) {
 
 // waits for the sim's stream and reports the latched device status
 vk_status read_status(vk_sim* s) {
-  VK_CUDA(s, cudaMemcpyAsync(s->h_status, s->b.d_status, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
+  VK_CUDA(s, cudaMemcpyAsync(&s->host->status, s->b.d_status, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
   VK_CUDA(s, cudaStreamSynchronize(s->stream));
-  const int32_t h = *s->h_status;
+  const int32_t h = s->host->status;
   if (h == 0) return VK_OK;
   const char* what = h == VK_ERR_CAPACITY     ? "device: capacity exceeded (Voronoi polygon or buffer)"
                      : h == VK_ERR_DEGENERATE ? "device: coincident particles or a zero-length Voronoi edge"
@@ -503,13 +544,12 @@ vk_status build_sim(int32_t n_rep, const int64_t* n_r, const int32_t* pos_q, con
       (e = dalloc(&s->b.U_id, N)) || (e = dalloc(&s->b.U_rank, N)) ||
       (e = dalloc(&s->b.phi_acc, 3 * (size_t)s->phi_cap * n_rep)) || (e = dalloc(&s->b.d_step, 1)) ||
       (e = dalloc(&s->b.d_status, 1)) || (e = dalloc(&s->reps_d, n_rep)) ||
-      (e = cudaMallocHost(&s->h_status, sizeof(int32_t))) ||
-      (e = cudaMallocHost(&s->h_phi, 3 * sizeof(long long) * kPhiRows)) || (e = dalloc(&s->b.ovf_list, 2 * N)) || (e = dalloc(&s->b.ovf_count, 2)) ||
+      (e = take_host_block(&s->host)) || (e = dalloc(&s->b.ovf_list, 2 * N)) || (e = dalloc(&s->b.ovf_count, 2)) ||
       (e = dalloc(&s->d_stats, kCounters)) ||
       (e = dalloc(&s->tasks_d, s->tasks_h.size())))
     return bail(cuda_fail(s, e, "cudaMalloc"));
   if (params->rule == VK_RULE_KNN) {
-    if ((e = dalloc(&s->b.S_hint, N)) || (e = dalloc(&s->b.U_hint, N)) || (e = dim == 2 ? prepare_knn2() : prepare_knn3()))
+    if ((e = dalloc(&s->b.S_hint, N)) || (e = dalloc(&s->b.U_hint, N)) || (e = dim == 2 ? prepare_knn2(params->k) : prepare_knn3()))
       return bail(cuda_fail(s, e, "kNN search buffers"));
   }
   if (params->rule == VK_RULE_VORONOI && dim == 2 && !params->voronoi_rebuild) {
@@ -780,13 +820,13 @@ vk_status vk_get_order_parameter(vk_sim* s, int32_t replica, double* phi, int64_
   // kernel (a copy of the whole ring of 512 replicas is 0.8 MB, 100 us a call)
   std::vector<double> vals(nout);
   const double n = (double)s->reps_h[replica].n;
-  std::lock_guard<std::mutex> lock(s->h_phi_mu);
+  std::lock_guard<std::mutex> lock(s->host_phi_mu);
   for (int64_t i0 = 0; i0 < nout; i0 += kPhiRows) {
     const int rows = (int)std::min<int64_t>(nout - i0, kPhiRows);
-    VK_CUDA(s, launch_export_phi(s->b, s->phi_cap, s->n_rep, replica, s->step - nout + i0, rows, s->h_phi, s->stream));
+    VK_CUDA(s, launch_export_phi(s->b, s->phi_cap, s->n_rep, replica, s->step - nout + i0, rows, s->host->phi, s->stream));
     VK_CUDA(s, cudaStreamSynchronize(s->stream));
     for (int i = 0; i < rows; ++i) {
-      const long long* a = s->h_phi + 3 * i;
+      const long long* a = s->host->phi + 3 * i;
       // fixed-point sums (2^-32 units) -> FP64
       const double x = std::ldexp((double)a[0], -32), y = std::ldexp((double)a[1], -32),
                    z = std::ldexp((double)a[2], -32);
@@ -927,8 +967,7 @@ void vk_destroy(vk_sim* s) {
                   s->tis.inv_len, s->tis.blocks, s->tis.area, s->tis.perim, s->tis_out};
   for (void* p : bufs)
     if (p) cudaFree(p);
-  if (s->h_status) cudaFreeHost(s->h_status);
-  if (s->h_phi) cudaFreeHost(s->h_phi);
+  give_host_block(s->host);
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
   delete s;
 }

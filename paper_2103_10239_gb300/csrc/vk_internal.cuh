@@ -737,8 +737,8 @@ bool knn2_direct(int64_t n, const StepParams& P);
 cudaError_t launch_knn2_finish(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
 cudaError_t launch_knn2_export(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out, cudaStream_t st,
                                const StepParams& P);
-// one-time kernel attributes (shared memory of the radius-first search)
-cudaError_t prepare_knn2();
+// one-time kernel attributes for k neighbors (shared memory of the radius-first search)
+cudaError_t prepare_knn2(int k);
 
 // vk_metric.cu (metric rule, 2D and 3D)
 cudaError_t launch_metric_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);

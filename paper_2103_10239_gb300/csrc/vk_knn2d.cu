@@ -878,12 +878,11 @@ cudaError_t for_k(const StepParams& P, F f) {
 
 bool knn2_direct(int64_t n, const StepParams& P) { return P.knn_search == 1 || n <= kDirect2; }
 
-cudaError_t prepare_knn2() {
-  cudaError_t e = prepare2<8>();
-  if (e == cudaSuccess) e = prepare2<12>();
-  if (e == cudaSuccess) e = prepare2<17>();
-  if (e == cudaSuccess) e = prepare2<33>();
-  return e;
+cudaError_t prepare_knn2(int k) {
+  if (k <= 7) return prepare2<8>();
+  if (k <= 11) return prepare2<12>();
+  if (k <= 16) return prepare2<17>();
+  return prepare2<33>();
 }
 
 cudaError_t launch_knn2_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st) {

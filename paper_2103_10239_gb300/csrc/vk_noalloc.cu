@@ -51,7 +51,8 @@ cudaError_t scratch_ptr(void** out) {
   if (!g_ptr[dev]) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-    if (e == cudaSuccess) e = prepare_knn2();
+    for (int k : {7, 11, 16, 32})  // each of the list sizes that the kernels are compiled for
+      if (e == cudaSuccess) e = prepare_knn2(k);
     if (e != cudaSuccess) return e;
     g_ptr[dev] = p;
   }
