@@ -558,6 +558,36 @@ struct Cell8 {
     for (int i = 0; i < 2; ++i) kept &= ~(group_bits(has(i) && slot[i] < 0) << (8 * i));
     return kept;
   }
+
+  // Neighbors, the sites of edges of positive length, ordered by id: of each of
+  // the lane's edges the id (INT_MAX: none) and its place in the order (-1).
+  // Returns their number (group).
+  __device__ __forceinline__ int neighbors(bool ok, const int32_t* __restrict__ ids, int32_t* nid, int* rank) const {
+    const unsigned kept = neighbor_edges();
+    const bool big = __any_sync(kAll, m > 8);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      rank[i] = 0;
+      nid[i] = ok && (kept >> (gl + 8 * i) & 1u) ? __ldg(ids + slot[i]) : INT_MAX;
+    }
+#pragma unroll
+    for (int j = 0; j < kCG; ++j) {
+      const int32_t o = __shfl_sync(kAll, nid[0], base + j);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) rank[i] += o < nid[i] ? 1 : 0;
+    }
+    if (big)
+#pragma unroll
+      for (int j = 0; j < kCG; ++j) {
+        const int32_t o = __shfl_sync(kAll, nid[1], base + j);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) rank[i] += o < nid[i] ? 1 : 0;
+      }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (nid[i] == INT_MAX) rank[i] = -1;
+    return __popc(kept);
+  }
 };
 
 }  // namespace
