@@ -673,8 +673,8 @@ vk_status vk_get_neighbors(vk_sim* s, int32_t replica, int64_t* offsets, int32_t
     const int k = s->prm.k;
     int32_t* out_d = nullptr;
     VK_CUDA(s, dalloc(&out_d, (size_t)n * k));
-    cudaError_t e = s->dim == 2 ? launch_knn2_export(s->g, s->b, replica, (int)n, out_d, s->stream, step_params(s))
-                                : launch_knn_export(s->g, s->b, k, replica, (int)n, out_d, s->stream);
+    auto exporter = s->dim == 2 ? launch_knn2_export : launch_knn_export;
+    cudaError_t e = exporter(s->g, s->b, replica, (int)n, out_d, s->stream, step_params(s));
     if (e == cudaSuccess) {
       ids_h.resize((size_t)n * k);
       e = cudaMemcpyAsync(ids_h.data(), out_d, sizeof(int32_t) * n * k, cudaMemcpyDeviceToHost, s->stream);

@@ -724,8 +724,8 @@ cudaError_t launch_import_state(const Geometry& g, const Buffers& b, int rep, in
 cudaError_t prepare_knn3();
 int knn3_launches(int64_t n, const StepParams& P);  // kernels of one launch_knn_step
 cudaError_t launch_knn_step(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
-cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out,
-                              cudaStream_t st);
+cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out, cudaStream_t st,
+                              const StepParams& P);
 
 // vk_knn2d.cu (the 2D kNN hot path)
 // search + update of every particle (those one square each can serve; the

@@ -5,12 +5,10 @@
 //
 // One thread per particle, in cell-sorted order, radius first: the cube around
 // the particle a little wider than its k-th distance at the last step; 16 lanes
-// each for the particles that this cube cannot serve.  The lists are exported by
-// a ring walk: it walks rings of cells around the particle's cell (each row
-// segment of a ring is one contiguous run of the sorted arrays), keeps the k
-// best (exact int64 squared distance, id) pairs in registers, and stops once
-// the k-th best distance is below the exact integer distance from the particle
-// to the boundary of the scanned (2r+1)^d block.
+// each for the particles that this cube cannot serve.  Lists are exported by the
+// same searches (a ring walk by one thread with a 64-bit list took 326 us for 5000
+// particles, k = 7, 3.9 ms for 200,000, k = 32, and 28.4 ms for 60,000 in a cluster; this
+// 67 us, 1.4 and 14.5 ms, with the copies).
 #include <algorithm>
 #include <climits>
 
@@ -20,86 +18,6 @@
 namespace vk {
 
 namespace {
-
-// Top-k list of KC register slots.  For k < KC the first KC-k slots hold
-// sentinels that order before every real candidate, so the threshold is
-// always slot KC-1 and no register array is indexed dynamically.
-template <int KC>
-struct TopK {
-  uint64_t d[KC];
-  int32_t id[KC];
-  int32_t slot[KC];
-};
-
-template <int KC>
-__device__ __forceinline__ void topk_init(TopK<KC>& T, int k) {
-#pragma unroll
-  for (int s = 0; s < KC; ++s) {
-    const bool sentinel = s < KC - k;
-    T.d[s] = sentinel ? 0ull : ~0ull;
-    T.id[s] = sentinel ? INT_MIN : INT_MAX;
-    T.slot[s] = -1;
-  }
-}
-
-template <int KC>
-__device__ __forceinline__ void topk_insert(TopK<KC>& T, uint64_t D, int32_t idj, int32_t q) {
-  bool placed = false;
-#pragma unroll
-  for (int s = KC - 1; s > 0; --s) {
-    const bool before = (D < T.d[s - 1]) || (D == T.d[s - 1] && idj < T.id[s - 1]);
-    if (!placed) {
-      if (before) {
-        T.d[s] = T.d[s - 1];
-        T.id[s] = T.id[s - 1];
-        T.slot[s] = T.slot[s - 1];
-      } else {
-        T.d[s] = D;
-        T.id[s] = idj;
-        T.slot[s] = q;
-        placed = true;
-      }
-    }
-  }
-  if (!placed) {
-    T.d[0] = D;
-    T.id[0] = idj;
-    T.slot[0] = q;
-  }
-}
-
-template <int DIM, int KC>
-__device__ __forceinline__ void knn_search(const Rep& R, int64_t self, const int32_t* pi,
-                                           const typename Vec<DIM>::P* __restrict__ pos,
-                                           const int32_t* __restrict__ ids, const GridView& G, TopK<KC>& T,
-                                           uint32_t* n_cand = nullptr, uint32_t* n_runs = nullptr) {
-  auto run = [&](uint32_t qb, uint32_t qe) {
-    if (n_cand) {
-      *n_cand += qe - qb;
-      *n_runs += 1;
-    }
-    for (uint32_t q = qb; q < qe; ++q) {
-      if ((int64_t)q == self) continue;
-      int32_t pj[3];
-      unpack(pos[q], pj);
-      uint64_t D = 0;
-#pragma unroll
-      for (int a = 0; a < DIM; ++a) {
-        const int64_t d = min_image((int64_t)pj[a] - (int64_t)pi[a], (int64_t)R.L[a]);
-        D += (uint64_t)(d * d);
-      }
-      if (D <= T.d[KC - 1]) {
-        const int32_t idj = ids[q];
-        if (D < T.d[KC - 1] || idj < T.id[KC - 1]) topk_insert<KC>(T, D, idj, (int32_t)q);
-      }
-    }
-  };
-  // every unscanned particle is at squared distance >= B2: stop once the
-  // k-th best is strictly closer (an equal distance could still win on id)
-  auto stop = [&](uint64_t B2) { return T.d[KC - 1] < B2; };
-  static_assert(DIM == 3, "the 2D rule is vk_knn2d.cu");
-  grid_walk3(R, pi, G, run, stop);
-}
 
 // ---------------------------------------------------------------------------
 // Radius first (3D): each particle scans the cube [p - a, p + a]^3, a a
@@ -472,6 +390,16 @@ struct Group3 : GroupTop<GS, CAP> {
     return all;
   }
 
+  // larger cubes, from half-width r, until k hits are in one; the number of cubes
+  __device__ __forceinline__ uint32_t search(const Rep& R, const GridView& G, float r) {
+    for (uint32_t tries = 1;; ++tries) {
+      const int64_t a = (int64_t)ceilf(fminf(r, 4.0e9f));
+      Top::cnt = 0;
+      if (cube(R, G, a) || Top::cnt >= Top::k) return tries;
+      r = (float)a * (Top::cnt > 0 ? fminf(cbrtf(1.6f * (float)(Top::k + 1) / (float)Top::cnt), 2.f) : 2.f) + 1.f;
+    }
+  }
+
   // (per lane) distance of cell slab c of axis x from the particle, over both images
   __device__ __forceinline__ float slab(int x, int c, const Rep& R) const {
     const uint32_t* bnd = bounds + R.bnd[x];
@@ -529,14 +457,7 @@ __global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_kernel
                           S_pos, bounds, {p.x, p.y, p.z}};
       g.k = k;
       g.n_cand = 0;
-      float r = all ? cube_radius(R, bounds, G, g.p, S_hint[e.x], P) : U_hint[e.x];
-      uint32_t tries = 1;
-      for (;; ++tries) {
-        const int64_t a = (int64_t)ceilf(fminf(r, 4.0e9f));
-        g.cnt = 0;
-        if (g.cube(R, G, a) || g.cnt >= k) break;
-        r = (float)a * (g.cnt > 0 ? fminf(cbrtf(1.6f * (float)(k + 1) / (float)g.cnt), 2.f) : 2.f) + 1.f;
-      }
+      const uint32_t tries = g.search(R, G, all ? cube_radius(R, bounds, G, g.p, S_hint[e.x], P) : U_hint[e.x]);
       __syncwarp(g.mask);
       g.rank([&](int, int rk, unsigned long long D, int32_t q) {
         if (rk < k) res[wid][i][rk] = q;
@@ -570,25 +491,62 @@ __global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_kernel
   }
 }
 
-// neighbor lists of the current positions of one replica, written by id
-template <int DIM, int KC>
-__global__ void __launch_bounds__(kBlock) knn_export_kernel(const Rep* __restrict__ reps, int rep,
-                                                            const typename Vec<DIM>::P* __restrict__ S_pos,
-                                                            const int32_t* __restrict__ S_id, GridView G,
-                                                            int k, int32_t* __restrict__ out) {
+// Neighbor lists of one replica, written by id: one cube per particle, as in a
+// step; those that it cannot serve go on the list ...
+template <int KC>
+__global__ void __launch_bounds__(kBlk3, CubeCfg<KC>::BLOCKS) knn3_cube_export_kernel(
+    const Rep* __restrict__ reps, int rep, const int4* __restrict__ S_pos, const int32_t* __restrict__ S_id, GridView G,
+    StepParams P, const uint32_t* __restrict__ bounds, const float* __restrict__ S_hint, float* __restrict__ radius,
+    int32_t* __restrict__ out, int2* __restrict__ list, int32_t* __restrict__ count) {
+  extern __shared__ __align__(16) unsigned char cube_smem[];
+  CubeShared<KC>& H = *reinterpret_cast<CubeShared<KC>*>(cube_smem);
   const Rep R = reps[rep];
-  const int li = blockIdx.x * kBlock + (int)threadIdx.x;
+  const int li = blockIdx.x * kBlk3 + (int)threadIdx.x;
   if (li >= R.n) return;
   const int64_t s = R.p0 + li;
-  int32_t pi[3] = {0, 0, 0};
+  int32_t pi[3];
   unpack(S_pos[s], pi);
-  const int32_t id = S_id[s];
-  TopK<KC> T;
-  topk_init<KC>(T, k);
-  knn_search<DIM, KC>(R, s, pi, S_pos, S_id, G, T);
+  float r_next;
+  uint32_t key[KC], n_cand = 0, n_runs = 0;
+  const float r = cube_radius(R, bounds, G, pi, S_hint[s], P);
+  if (cube_search<KC>(H, R, bounds, G, S_pos, (int32_t)s, pi, r, P.k, key, &r_next, &n_cand, &n_runs)) {
+    int32_t* row = out + (int64_t)S_id[s] * P.k;
 #pragma unroll
-  for (int j = 0; j < KC; ++j)
-    if (j >= KC - k) out[(int64_t)id * k + (j - (KC - k))] = T.id[j];
+    for (int j = 0; j < KC - 1; ++j)
+      if (j >= KC - 1 - P.k)
+        row[j - (KC - 1 - P.k)] = __ldg(S_id + H.hit[key[j] & ((1u << CubeCfg<KC>::BITS) - 1u)][threadIdx.x].x);
+  } else {
+    radius[s] = r_next;
+    list[atomicAdd(count, 1)] = make_int2((int)s, rep);
+  }
+}
+
+// ... of the groups (n_all > 0: every particle, small systems)
+template <int KC>
+__global__ void __launch_bounds__(kGroupBlk3, KC <= 8 ? 5 : 3) knn3_group_export_kernel(
+    const Rep* __restrict__ reps, int rep, const int4* __restrict__ S_pos, const int32_t* __restrict__ S_id, GridView G,
+    StepParams P, const uint32_t* __restrict__ bounds, const float* __restrict__ S_hint,
+    const float* __restrict__ radius, int32_t* __restrict__ out, const int2* __restrict__ list,
+    const int32_t* __restrict__ count, int n_all) {
+  constexpr int CAP = GroupCfg<KC>::CAP, kGroups = kGroupBlk3 / kGS3;
+  __shared__ GroupList<CAP> lists[kGroups];
+  const int lane = (int)(threadIdx.x & 31), total = n_all > 0 ? n_all : *count, k = P.k;
+  const Rep& R = reps[rep];
+  for (int i = blockIdx.x * kGroups + (int)threadIdx.x / kGS3; i < total; i += gridDim.x * kGroups) {
+    const int32_t s = n_all > 0 ? (int32_t)(R.p0 + i) : list[i].x;
+    const int4 p = S_pos[s];
+    Group3<kGS3, CAP> g{{lists[threadIdx.x / kGS3], S_id, ((1u << kGS3) - 1u) << (lane / kGS3 * kGS3),
+                         lane / kGS3 * kGS3, lane % kGS3, s},
+                        S_pos, bounds, {p.x, p.y, p.z}};
+    g.k = k;
+    g.n_cand = 0;
+    g.search(R, G, n_all > 0 ? cube_radius(R, bounds, G, g.p, S_hint[s], P) : radius[s]);
+    int32_t* row = out + (int64_t)S_id[s] * k;
+    g.rank([&](int, int rk, unsigned long long, int32_t q) {
+      if (rk < k) row[rk] = __ldg(S_id + q);
+    });
+    __syncwarp(g.mask);
+  }
 }
 
 GridView grid_view(const Buffers& b) {
@@ -625,18 +583,30 @@ cudaError_t step_dispatch(const Geometry& g, const Buffers& b, const StepParams&
 
 template <int KC>
 cudaError_t prepare3() {
-  return cudaFuncSetAttribute(knn3_step_kernel<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(CubeShared<KC>));
+  cudaError_t e = cudaFuncSetAttribute(knn3_step_kernel<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(CubeShared<KC>));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(knn3_cube_export_kernel<KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(CubeShared<KC>));
+  return e;
 }
 
-template <int DIM, int KC>
-cudaError_t export_dispatch(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out,
-                            cudaStream_t st) {
-  using PV = typename Vec<DIM>::P;
-  const int nb = (n + kBlock - 1) / kBlock;
-  if (nb == 0) return cudaSuccess;
-  knn_export_kernel<DIM, KC><<<nb, kBlock, 0, st>>>(g.reps, rep, (const PV*)b.S_pos, b.S_id, grid_view(b), k, out);
-  return cudaGetLastError();
+template <int KC>
+cudaError_t export_dispatch(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out, cudaStream_t st,
+                            const StepParams& P) {
+  if (n == 0) return cudaSuccess;
+  // the list is empty between steps; the export clears what it used
+  const bool all = knn3_direct(n, P);
+  if (!all)
+    knn3_cube_export_kernel<KC><<<(n + kBlk3 - 1) / kBlk3, kBlk3, sizeof(CubeShared<KC>), st>>>(
+        g.reps, rep, (const int4*)b.S_pos, b.S_id, grid_view(b), P, b.bounds, b.S_hint, b.U_hint, out, b.ovf_list,
+        b.ovf_count);
+  const int blocks = std::max(1, std::min((n + 7) / 8, device_sm_count() * 5));
+  knn3_group_export_kernel<KC><<<blocks, kGroupBlk3, 0, st>>>(g.reps, rep, (const int4*)b.S_pos, b.S_id, grid_view(b), P,
+                                                              b.bounds, b.S_hint, b.U_hint, out, b.ovf_list,
+                                                              b.ovf_count, all ? n : 0);
+  const cudaError_t e = all ? cudaSuccess : cudaMemsetAsync(b.ovf_count, 0, sizeof(int32_t), st);
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 }  // namespace
@@ -657,12 +627,12 @@ cudaError_t launch_knn_step(const Geometry& g, const Buffers& b, const StepParam
   return step_dispatch<33>(g, b, P, st);
 }
 
-cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int k, int rep, int n, int32_t* out,
-                              cudaStream_t st) {
+cudaError_t launch_knn_export(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out, cudaStream_t st,
+                              const StepParams& P) {
   if (g.dim != 3) return cudaErrorInvalidValue;  // 2D: launch_knn2_export
-  if (k <= 8) return export_dispatch<3, 8>(g, b, k, rep, n, out, st);
-  if (k <= 16) return export_dispatch<3, 16>(g, b, k, rep, n, out, st);
-  return export_dispatch<3, 32>(g, b, k, rep, n, out, st);
+  if (P.k <= 7) return export_dispatch<8>(g, b, rep, n, out, st, P);
+  if (P.k <= 16) return export_dispatch<17>(g, b, rep, n, out, st, P);
+  return export_dispatch<33>(g, b, rep, n, out, st, P);
 }
 
 }  // namespace vk

@@ -23,7 +23,8 @@ def _cost(sim):
 
 
 # every pass searches once; 0.1 ms for the copies to the host and the waits between
-@pytest.mark.parametrize("dim,n,rule,passes", [(2, 1000, "voronoi", 2), (2, 10000, "voronoi", 2)])
+@pytest.mark.parametrize("dim,n,rule,passes", [(2, 1000, "voronoi", 2), (2, 10000, "voronoi", 2), (3, 5000, "knn", 1),
+                                               (3, 1000, "knn", 1)])
 def test_export_costs_its_searches(dim, n, rule, passes):
     w = W.uniform_system(n, n ** (1.0 / dim), 15, dim, input_seed=n, rule=rule, k=7, v0=0.3, eta=0.3,
                          noise="vectorial" if dim == 3 else "angular")
@@ -49,3 +50,26 @@ def test_voronoi_lists_of_every_route(n):
             got = sim.neighbors()
             assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
             sim.step(4)
+
+
+# 3D: groups alone (small systems), cubes by threads and the groups for what they leave: ordinary, close distances, a
+# cluster whose first radii are far off; before steps and after
+@pytest.mark.parametrize("kind", ["uniform", "lattice", "cluster"])
+@pytest.mark.parametrize("m,k", [(6, 7), (33, 7), (33, 13), (33, 32)])
+def test_knn3_lists_of_every_route(kind, m, k):
+    rng = np.random.default_rng(m + k)
+    n, L = m ** 3, m << 14
+    if kind == "lattice":
+        pos = W.cubic_lattice("sc", m, 1 << 14)[0]
+    elif kind == "cluster":
+        pos = rng.normal(L / 2, L / 100, (n, 3)).astype(np.int64) % L
+    else:
+        pos = rng.integers(0, L, (n, 3))
+    w = W.Workload(name="export3", dim=3, pos_q=np.ascontiguousarray(pos, np.int32), dir=W.random_dirs(n, dim=3), theta=None,
+                   box_q=(L,) * 3, frac_bits=14, rule="knn", k=k, v0=0.02, eta=0.3, noise="vectorial")
+    query = np.sort(rng.choice(n, min(n, 400), replace=False))
+    with vk.from_workload(w) as sim:
+        for steps in (0, 2):
+            sim.step(steps)
+            ids = sim.neighbors()[1].reshape(-1, k)
+            assert np.array_equal(ids[query], oracle.knn(sim.state()[0], w.box_q, k, query=query))
