@@ -33,8 +33,10 @@
 // to 2^23 grid units.
 //
 // The predicates are plain C++ for the host and the device.  The kernels
-// (vk_voronoi3.cu) clip with a whole warp; cell_init, cell_clip and
-// face_positive below are the same steps written serially, for the host.
+// (vk_voronoi3.cu) have a builder of their own, a warp per cell; cell_init,
+// cell_clip and face_positive below are the same steps written serially, which
+// only the host test runs: it pins the predicates, and the warp's clipping,
+// linking and face walk are pinned on the GPU.
 #pragma once
 #include <cmath>
 #include <cstdint>
