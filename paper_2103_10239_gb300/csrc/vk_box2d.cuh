@@ -48,8 +48,6 @@ struct Ctx {
   uint32_t px, py;
   uint32_t Lx, Ly;
   int32_t hix, lox, hiy, loy;  // minimum image: d > hi -> d - L, d <= lo -> d + L
-  uint32_t n_cand, n_runs;
-  bool split;  // the particle's own coarse cell is split (tracing)
   View view;  // field of view of the kNN rule (everything when view.cq <= -2^24)
 };
 
@@ -63,9 +61,6 @@ __device__ __forceinline__ void init_ctx(Ctx& C, const Rep& R, int64_t self, int
   C.lox = -(int32_t)((R.L[0] + 1) / 2);
   C.hiy = (int32_t)(R.L[1] / 2);
   C.loy = -(int32_t)((R.L[1] + 1) / 2);
-  C.n_cand = 0;
-  C.n_runs = 0;
-  C.split = false;
   C.view.nxq = 0;
   C.view.nyq = 0;
   C.view.cq = kViewAll;

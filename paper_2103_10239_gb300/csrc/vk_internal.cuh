@@ -63,7 +63,7 @@ struct StepParams {
   int32_t n_rep;
   int32_t phi_cap;
   // kNN search: 0 = radius first, one thread per particle; 1 = the general
-  // search only (2D: groups of lanes and larger squares; 3D: the ring walk)
+  // search only (groups of lanes and larger squares or cubes)
   int32_t knn_search;
   // radius-first search square: halo_alpha * (the particle's k-th distance at
   // the previous step) + halo_beta * (grid step per unit heading)
@@ -71,10 +71,7 @@ struct StepParams {
   // 2D kNN field of view: the cosine of the half-angle in 2^-24 units, or
   // INT_MIN for the full circle (the plain rule)
   int32_t fov_cq;
-  // tracing only (NULL = off): [candidates, runs or squares, max candidates,
-  // particles, particles whose own coarse cell is split (walk) or that fell
-  // back to the walk (radius first), then radius first only: squares, runs,
-  // candidates, coarse cells, hits]
+  // tracing only (NULL = off): the counters that vk.h lists
   unsigned long long* stats;
 };
 

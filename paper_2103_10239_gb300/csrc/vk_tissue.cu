@@ -75,7 +75,7 @@ __device__ __noinline__ void tissue_cell_general(const Rep& R, int64_t s, const 
   int m = 0;
   double A = 0.0, Pm = 0.0;
   int64_t first = 0;
-  if (!voronoi_cell(R, s, pi, S_id[s], S_pos, S_id, G, P, status, 0u, sd, nullptr) || P.m > kTissueCap) {
+  if (!voronoi_cell(R, s, pi, S_id[s], S_pos, S_id, G, P, status, sd) || P.m > kTissueCap) {
     set_status(status, kStCapacity);
   } else if (P.nt > 0) {
     set_status(status, kStDegenerate);  // coincident particles: one site, no cell each

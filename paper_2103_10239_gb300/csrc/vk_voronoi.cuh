@@ -14,8 +14,8 @@ namespace vk {
 
 namespace {
 
-constexpr int kFastCap = 32;    // polygon capacity of the main kernel
-constexpr int kSlowCap = kVoronoiMaxDeg;  // capacity of the overflow kernel and the export
+constexpr int kFastCap = 32;    // polygon capacity of the tissue model's cells
+constexpr int kSlowCap = kVoronoiMaxDeg;  // of the warp kernels
 // candidates after which the main kernel hands a cell to the overflow kernel.
 // Large systems: the groups' throughput counts (us per step, 512 / 768 / 1024 / 1536:
 // 512k with grown voids 4095, 3980, 3975, 4024; 65,536 beside a lattice, steps 100 on,
@@ -629,10 +629,8 @@ __device__ __noinline__ void cell_visit_one(Poly<CAP>& P, CellFlags& F, int32_t 
 template <int CAP>
 __device__ bool voronoi_cell(const Rep& R, int64_t self, const int32_t* pi, int32_t self_id,
                              const int2* __restrict__ pos, const int32_t* __restrict__ ids,
-                             const GridView& G, Poly<CAP>& P, int32_t* status, uint32_t budget, const Seeds& sd,
-                             uint32_t* seen_out, uint32_t* n_cand = nullptr, uint32_t* n_runs = nullptr) {
+                             const GridView& G, Poly<CAP>& P, int32_t* status, const Seeds& sd) {
   CellFlags F{false, false};
-  uint32_t seen = 0;
   poly_init(P, self_id, R.L[0], R.L[1], &F.bad);
   const int64_t Lx = R.L[0], Ly = R.L[1];
   // the seeds first: their slots, then one pass of the candidate loop
@@ -643,12 +641,6 @@ __device__ bool voronoi_cell(const Rep& R, int64_t self, const int32_t* pi, int3
     cell_visit_slots(P, F, pos, ids, self, pi[0], pi[1], Lx, Ly, ss, 0u, (uint32_t)n);
   }
   auto run = [&](uint32_t qb, uint32_t qe) {
-    if (n_cand) {
-      *n_cand += qe - qb;
-      *n_runs += 1;
-    }
-    seen += qe - qb;
-    if (budget && seen > budget) F.overflow = true;  // a heavy cell: left to the warp-cooperative kernel
     if (!F.overflow) cell_visit_slots(P, F, pos, ids, self, pi[0], pi[1], Lx, Ly, nullptr, qb, qe);
   };
   auto box = [&](int64_t* b) {
@@ -669,7 +661,6 @@ __device__ bool voronoi_cell(const Rep& R, int64_t self, const int32_t* pi, int3
     if (!within_half(b, Lx, Ly)) far_images(R, self, pi, pos, ids, visit);
   }
   if (F.bad) set_status(status, kStRange);
-  if (seen_out) *seen_out = seen;
   return !F.overflow;
 }
 
