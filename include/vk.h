@@ -289,8 +289,7 @@ vk_status vk_get_search_stats(vk_sim* sim, double* mean_candidates, double* mean
  * candidates, 8 coarse cells visited, 9 hits merged, and the particles handed
  * on because 10 the square was too wide for the box or met too many coarse
  * cells, 11 it held fewer than k hits (a larger square follows), 12 two
- * candidates' distances were too close to order in 32 bits, 13 it held too many
- * candidates for one thread.  Writes
+ * candidates' distances were too close to order in 32 bits, 13 (unused, 0).  Writes
  * min(max_values, 14) values; *n (may be NULL) receives 14. */
 vk_status vk_get_search_counters(vk_sim* sim, int64_t* values, int32_t max_values, int32_t* n);
 

@@ -73,7 +73,7 @@ struct BoxCount {
   uint32_t runs = 0;   // contiguous slot runs read
   uint32_t hits = 0;   // hits merged
   uint32_t cells = 0;  // coarse cells visited
-  uint32_t why = 0;    // fallback reason: 0 none, 1 square too wide, 2 too few hits, 3 close distances, 4 too many candidates
+  uint32_t why = 0;    // fallback reason: 0 none, 1 square too wide, 2 too few hits, 3 close distances
 };
 
 // exact minimum-image offset and squared distance of pj from the particle

@@ -61,19 +61,13 @@ struct BoxShared {
   uint2 run[BoxCfg<KC>::RUNS][kBlk];  // (first slot, length << 4 | image shift codes)
 };
 
-// A thread does not take a square of more coarse cells or more candidates than
-// these: a particle outside a cluster has a wide square, most of it empty cells,
-// and a first radius, guessed from the density around it, that may hold the whole
-// cluster, and the whole launch waits for it.  The groups look at 16 cells and 16
-// candidates at a time.  Ordinary squares meet one to four cells and 30 to 180
-// candidates.  Measured (us; no limits / 144 and 1024 / 64 and 1024 / 25 and 512 / 25
-// and 256): 65,536 particles around one point, all lists, k = 7 2896, 460, 460, 289,
-// 259, k = 32 11,680, 617, 634, 544, 501; 200,000 in a wide cluster, a step 210, 231,
-// 203, 189, 190, and around one point 329, 326, 326, 336, 349.  Not in a field of
-// view, whose squares are wider for every particle that faces a void (1M 4.1 ms a
-// pass without, 4.5 with).
-constexpr int kMaxCells = 25;
-constexpr uint32_t kMaxCand = 512;
+// A thread does not take a square of more coarse cells than these (per axis): a
+// particle outside a cluster has a wide square, most of it empty cells, and the whole
+// launch waits for it.  The groups look at 16 cells at a time.  Ordinary squares meet
+// one to four.  Measured (us per step, 200,000 particles in a wide cluster; no limit /
+// 12 / 8 / 5): 210, 231, 203, 189.  Not in a field of view, whose squares are wider for
+// every particle that faces a void (1M 4.1 ms a pass without, 4.5 with).
+constexpr int kMaxCells = 5;
 
 // the slot behind a key of the list
 template <int KC>
@@ -111,12 +105,10 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
   const uint32_t y0 = (uint32_t)p.y - (uint32_t)a + (wy0 ? Ly : 0u), y1 = (uint32_t)p.y + (uint32_t)a - (wy1 ? Ly : 0u);
   const int ucx0 = (int)(x0 >> shx) - (wx0 ? nx : 0), ucx1 = (int)(x1 >> shx) + (wx1 ? nx : 0);
   const int ucy0 = (int)(y0 >> shy) - (wy0 ? ny : 0), ucy1 = (int)(y1 >> shy) + (wy1 ? ny : 0);
-  if (ucx1 - ucx0 >= nx || ucy1 - ucy0 >= ny) return false;
-  if (!FOV && (ucx1 - ucx0 + 1) * (ucy1 - ucy0 + 1) > kMaxCells) return false;
+  if (ucx1 - ucx0 >= (FOV ? nx : min(nx, kMaxCells)) || ucy1 - ucy0 >= (FOV ? ny : min(ny, kMaxCells))) return false;
   const uint32_t fx0 = cell_frac(x0, shx), fx1 = cell_frac(x1, shx);
   const uint32_t fy0 = cell_frac(y0, shy), fy1 = cell_frac(y1, shy);
   bc.tries += 1;
-  const uint32_t cand0 = bc.cand;
   // below (a + 1)^2 by more than the rounding of the distances
   const float a1 = (float)a + 1.0f;
   float tau = a1 * a1 * (1.0f - 9.5367431640625e-07f);
@@ -128,17 +120,15 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
   int ucx = ucx0, ucy = ucy0, row = 0, row_end = -1, s = 1, nrun = 0, r = 0;
   uint32_t lo = 0, hi = 0, code = 0;  // first and one-past-last sub-cell of the row
   uint32_t q = 0, qb = 0, len = 0, ox = 0, oy = 0;
-  bool more = true, done = false, heavy = false;
+  bool more = true, done = false;
   for (;;) {
     while (cnt <= CAP - 4) {
       if (q - qb >= len) {  // next run
         if (r == nrun) {
           // list up to RUNS runs, so that one flat loop scans them and the
           // threads of a warp scan candidates together however their squares split
-          // (no return from here: the warp's threads have to meet again)
-          heavy = !FOV && bc.cand - cand0 > kMaxCand;
           nrun = r = 0;
-          while (more && !heavy && nrun <= BoxCfg<KC>::RUNS - 2) {
+          while (more && nrun <= BoxCfg<KC>::RUNS - 2) {
             if (row > row_end) {  // next coarse cell
               if (ucx > ucx1) {
                 ucx = ucx0;
@@ -245,11 +235,6 @@ __device__ __forceinline__ bool box_search(BoxShared<KC>& H, const Rep& R, const
     if (t[KC - 2] < 0xFF000000u) tau = fminf(tau, __uint_as_float(((t[KC - 2] >> B) + 3u) << B));
   }
   bc.hits += (uint32_t)got;
-  if (heavy) {  // only a part was scanned: as wide next as it says that about 1.5 k hits need
-    *r_next = (float)a * sqrtf((1.5f * (float)k + 1.f) / (float)(bc.cand - cand0));
-    bc.why = 4u;
-    return false;
-  }
   if ((t[KC - 2] >> B) + 1u < edge) {
     bool close = false;  // a pair whose order the keys leave open
 #pragma unroll
@@ -314,7 +299,7 @@ struct Group : GroupTop<GS, CAP> {
   // that has filled up on the way leaves little to scan.  Near cells and rows
   // go first: of a cluster that the square reaches from outside, met from its far
   // side, every particle would be nearer than the last (65,536 particles around one
-  // point, k = 32: 7890 / 634 us for all lists).  True when the square is the whole box.
+  // point, k = 32: 7890 / 634 us for all lists, with kMaxCand below 1024).  True when the square is the whole box.
   __device__ __forceinline__ bool square(const Rep& R, const GridView& G, int64_t a) {
     const int64_t Lx = C.Lx, Ly = C.Ly;
     const int nx = R.nc[0], ny = R.nc[1], shx = R.sh[0], shy = R.sh[1];
@@ -452,32 +437,62 @@ __device__ __forceinline__ void knn2_update(const Rep& R, const StepParams& P, i
   atomicAdd(counts + linear_cell<2>(R, pout), 1u);
 }
 
-// search radius without a hint: a multiple of the k-th distance expected
-// from the density of the particle's own sub-cell
-__device__ __forceinline__ float box_radius_estimate(const Rep& R, const GridView& G, int2 p, int k) {
+// Search radius without a hint: a multiple of the k-th distance expected from
+// the density of the particle's own sub-cell.  Outside a cluster that is the
+// density of a nearly empty cell, and the square may hold the whole cluster, for
+// which one thread needs milliseconds: a square of more than kMaxCand particles, by
+// the counts of the coarse cells that it meets, shrinks to about 1.5 k of them.
+// Measured (all lists of 65,536 particles around one point, k = 7 and 32): 2896 and
+// 11,680 us without, 195 and 413 with it; with a limit on the thread's scan instead, which
+// every particle has to check, 289 and 534, and 0.5 % on all steps.  Out of line: inlined it
+// takes registers from the search (4M clustered 17.9 ms a pass, 17.1 so).
+constexpr float kMaxCand = 512.f;
+
+__device__ __forceinline__ float axis_share(int64_t p, int64_t a, int u, int n, int sh, int64_t L) {
+  const int64_t lo = cell_lo2(u, n, sh, L) - p, hi = lo + ((int64_t)1 << sh);
+  return (float)(min(a + 1, hi) - max(-a, lo)) / (float)((int64_t)1 << sh);
+}
+
+__device__ __noinline__ float box_radius_estimate(const Rep* __restrict__ rep, GridView G, int2 p, int k) {
+  const Rep& R = *rep;
   const int32_t pi[2] = {p.x, p.y};
   int64_t gc, gs;
   locate<2>(R, G, nullptr, pi, &gc, &gs);
   const float s = (float)__ldg(G.sub_s + gc);
   const uint32_t cnt = __ldg(G.sub_off + gs + 1) - __ldg(G.sub_off + gs);
   const float area = (float)(1ull << R.sh[0]) * (float)(1ull << R.sh[1]) / (s * s);
-  return 1.6f * sqrtf((float)k * area / (3.14159265f * (float)max(cnt, 1u)));
+  const float r = 1.6f * sqrtf((float)k * area / (3.14159265f * (float)max(cnt, 1u)));
+  const int64_t a = (int64_t)ceilf(fminf(r, 1.0e9f)), Lx = R.L[0], Ly = R.L[1];
+  if (4 * a + 2 >= Lx || 4 * a + 2 >= Ly) return r;
+  const int nx = R.nc[0], ny = R.nc[1];
+  const int ux0 = ucell2(p.x - a, nx, R.sh[0], Lx), ux1 = ucell2(p.x + a, nx, R.sh[0], Lx);
+  const int uy0 = ucell2(p.y - a, ny, R.sh[1], Ly), uy1 = ucell2(p.y + a, ny, R.sh[1], Ly);
+  if (ux1 - ux0 > kMaxCells || uy1 - uy0 > kMaxCells) return r;
+  float n = 0.f;
+  for (int uy = uy0; uy <= uy1; ++uy)
+    for (int ux = ux0; ux <= ux1; ++ux) {
+      const int64_t c = R.c0 + (int64_t)(uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy)) * nx +
+                        (ux < 0 ? ux + nx : (ux >= nx ? ux - nx : ux));
+      const uint32_t m = __ldg(G.off + c + 1) - __ldg(G.off + c);
+      if (m > 0)
+        n += (float)m * axis_share(p.x, a, ux, nx, R.sh[0], Lx) * axis_share(p.y, a, uy, ny, R.sh[1], Ly);
+    }
+  return n > kMaxCand ? r * sqrtf((1.5f * (float)k + 1.f) / n) : r;
 }
 
-// Tracing: totals of the radius-first counters (stats[5..13]; the squares also count
+// Tracing: totals of the radius-first counters (stats[5..12]; the squares also count
 // in stats[1]).
 __device__ __forceinline__ void record_box_stats(unsigned long long* stats, const BoxCount& bc) {
   if (!stats) return;
-  unsigned long long v[9] = {bc.tries, bc.runs, bc.cand, bc.cells, bc.hits, bc.why == 1u, bc.why == 2u,
-                              bc.why == 3u, bc.why == 4u};
+  unsigned long long v[8] = {bc.tries, bc.runs, bc.cand, bc.cells, bc.hits, bc.why == 1u, bc.why == 2u, bc.why == 3u};
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-    for (int i = 0; i < 9; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    for (int i = 0; i < 8; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
   if ((threadIdx.x & 31) == 0) {
     atomicAdd(stats + 1, v[0]);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) atomicAdd(stats + 5 + i, v[i]);
+    for (int i = 0; i < 8; ++i) atomicAdd(stats + 5 + i, v[i]);
   }
 }
 
@@ -546,8 +561,9 @@ __device__ __forceinline__ float left_radius(float r, const BoxCount& bc) {
 }
 
 // the first radius of a particle
-__device__ __forceinline__ float box_radius(const Rep& R, const GridView& G, int2 p, float hint, const StepParams& P) {
-  return hint > 0.f ? P.halo_alpha * hint + P.halo_beta * fabsf(R.s) : box_radius_estimate(R, G, p, P.k);
+__device__ __forceinline__ float box_radius(const Rep* __restrict__ rep, const GridView& G, int2 p, float hint,
+                                            const StepParams& P) {
+  return hint > 0.f ? P.halo_alpha * hint + P.halo_beta * fabsf(rep->s) : box_radius_estimate(rep, G, p, P.k);
 }
 
 // the search of one thread's particle with the square of half-width ceil(r)
@@ -586,7 +602,7 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_box_step_kernel
   bool served = false;
   if (valid) {
     const int64_t s = R.p0 + li;
-    float r = box_radius(R, G, S_pos[s], S_hint[s], out.P);
+    float r = box_radius(reps + t.rep, G, S_pos[s], S_hint[s], out.P);
     served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, step, out, &r, bc, nnew);
     if (!served) out.radius()[s] = left_radius(r, bc);
   }
@@ -611,7 +627,7 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_box_export_kern
   bool served = false;
   if (valid) {
     BoxCount bc;
-    float r = box_radius(R, G, S_pos[s], S_hint ? S_hint[s] : 0.f, out.P);
+    float r = box_radius(reps + rep, G, S_pos[s], S_hint ? S_hint[s] : 0.f, out.P);
     served = box_particle<KC, FOV>(H, R, G, S_pos, S_id, r, s, 0, out, &r, bc, nullptr);
     if (!served) out.radius()[s] = left_radius(r, bc);
   }
@@ -669,15 +685,19 @@ __global__ void __launch_bounds__(kBlk, BoxCfg<KC>::BLOCKS) knn2_second_kernel(
 // the first list where the kernel above left it (its length is read on the
 // device, so that the launch can sit in a CUDA graph).
 //
-// Small systems (and the general search) come here at once, every particle
-// (n_all of them, by the tasks of a step or those of one replica): the thread kernel's time is one particle's, from
-// start to end, however few there are, and the listed ones wait for it.
+// ALL: small systems (and the general search) come here at once, every particle
+// (n_all of them, by the tasks of a step or those of one replica): the thread
+// kernel's time is one particle's, from start to end, however few there are, and
+// the listed ones wait for it.
 constexpr int kGS = 16;
 constexpr int kGroupBlk = 128;
+// resident blocks per SM that the kernel is compiled for, for long lists and for small systems
+template <int KC> constexpr int kListBlocks = KC <= 12 ? 6 : 3;
+template <int KC> constexpr int kSmallBlocks = KC <= 12 ? 4 : 3;
 constexpr float kWholeBox = 4.6e18f;  // squared distance beyond every box's
 
-template <int KC, bool FOV, class Out>
-__global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel(
+template <int KC, bool FOV, bool ALL, int BLOCKS, class Out>
+__global__ void __launch_bounds__(kGroupBlk, BLOCKS) knn2_group_kernel(
     const Rep* __restrict__ reps, const int2* __restrict__ S_pos, const int32_t* __restrict__ S_id, GridView G,
     Out out, const int2* __restrict__ first_list, const int2* __restrict__ left_list,
     const int32_t* __restrict__ counts, int64_t n_all, const BlockTask* __restrict__ tasks, int one_rep,
@@ -686,12 +706,12 @@ __global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel
   __shared__ GroupList<CAP> lists[kGroupBlk / kGS];
   __shared__ int32_t res[NW][32][KC - 1];  // slots of the k nearest of the warp's particles
   __shared__ float res_d[NW][32];          // their k-th squared distance
-  const bool all = n_all > 0, first = !all && counts[0] < kLongList;
+  const bool first = !ALL && counts[0] < kLongList;
   const int2* __restrict__ list = first ? first_list : left_list;
-  const int64_t total = all ? n_all : first ? counts[0] : counts[1];
+  const int64_t total = ALL ? n_all : first ? counts[0] : counts[1];
   // (slot, replica) of entry i; slot -1 where a replica's last task has no particle
   auto entry = [&](int64_t i) -> int2 {
-    if (!all) return list[i];
+    if (!ALL) return list[i];
     if (!tasks) return make_int2((int)(reps[one_rep].p0 + i), one_rep);
     const BlockTask t = tasks[i / kBlock];
     const int li = t.first + (int)(i % kBlock);
@@ -717,7 +737,7 @@ __global__ void __launch_bounds__(kGroupBlk, KC <= 12 ? 6 : 3) knn2_group_kernel
       init_ctx(g.C, R, e.x, p);
       if (FOV) g.C.view = make_view(out.S_dir[e.x], out.P.fov_cq);
       g.k = k;
-      float r = all ? box_radius(R, G, p, S_hint ? S_hint[e.x] : 0.f, out.P) : fabsf(out.radius()[e.x]);
+      float r = ALL ? box_radius(reps + e.y, G, p, S_hint ? S_hint[e.x] : 0.f, out.P) : fabsf(out.radius()[e.x]);
       uint32_t tries = 1;
       g.n_cand = 0;
       for (;; ++tries) {
@@ -799,8 +819,13 @@ StepOut<KC> step_out(const Buffers& b, const StepParams& P) {
 template <int KC, bool FOV, class Out>
 cudaError_t group_all(const Geometry& g, const Buffers& b, const Out& out, int64_t n, const BlockTask* tasks, int rep,
                       cudaStream_t st) {
-  knn2_group_kernel<KC, FOV><<<group_blocks(n), kGroupBlk, 0, st>>>(
-      g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, nullptr, nullptr, nullptr, n, tasks, rep, b.S_hint);
+  // a launch that four blocks per SM hold takes more registers (2048 particles, k = 7: 36.0 us
+  // per step with room for six, 34.3 for four; 100,000 by the general search 191 and 213)
+  const int blocks = group_blocks(n);
+  auto kernel = KC <= 12 && blocks > 4 * device_sm_count() ? knn2_group_kernel<KC, FOV, true, kListBlocks<KC>, Out>
+                                                           : knn2_group_kernel<KC, FOV, true, kSmallBlocks<KC>, Out>;
+  kernel<<<blocks, kGroupBlk, 0, st>>>(g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, nullptr, nullptr, nullptr, n,
+                                       tasks, rep, b.S_hint);
   return cudaGetLastError();
 }
 
@@ -822,7 +847,7 @@ void finish_lists(const Geometry& g, const Buffers& b, const Out& out, int64_t n
   int2* left = b.ovf_list + g.n_total;
   knn2_second_kernel<KC, FOV><<<second_blocks<KC>(n), kBlk, sizeof(BoxShared<KC>), st>>>(
         g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, b.ovf_list, b.ovf_count, left, b.ovf_count + 1);
-  knn2_group_kernel<KC, FOV><<<group_blocks(n), kGroupBlk, 0, st>>>(
+  knn2_group_kernel<KC, FOV, false, kListBlocks<KC>><<<group_blocks(n), kGroupBlk, 0, st>>>(
       g.reps, (const int2*)b.S_pos, b.S_id, view_of(b), out, b.ovf_list, left, b.ovf_count, 0, nullptr, 0, nullptr);
 }
 

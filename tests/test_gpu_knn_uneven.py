@@ -38,7 +38,7 @@ def _time(pos, L, k):
 
 # first radii are guessed from the density around a particle: outside a cluster they may hold all of it.  One
 # thread needs 20 times as long for such a square as all lists of a uniform system take; with its share limited (40 us
-# of about 130) and the rest left to groups, no system takes many times as long as another
+# of about 130 at 1024 particles) and the rest left to groups, no system takes many times as long as another
 @pytest.mark.parametrize("k", [7, 32])
 def test_no_particle_holds_up_all_others(k):
     n, L = 65536, 1 << 24
