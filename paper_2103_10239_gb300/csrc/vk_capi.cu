@@ -675,6 +675,9 @@ vk_status vk_get_neighbors(vk_sim* s, int32_t replica, int64_t* offsets, int32_t
     VK_CUDA(s, dalloc(&out_d, (size_t)n * k));
     auto exporter = s->dim == 2 ? launch_knn2_export : launch_knn_export;
     cudaError_t e = exporter(s->g, s->b, replica, (int)n, out_d, s->stream, step_params(s));
+    // (the lists have to be empty before the next step)
+    if (e == cudaSuccess && s->dim == 2 && !knn2_direct(n, step_params(s)))
+      e = cudaMemsetAsync(s->b.ovf_count, 0, 2 * sizeof(int32_t), s->stream);
     if (e == cudaSuccess) {
       ids_h.resize((size_t)n * k);
       e = cudaMemcpyAsync(ids_h.data(), out_d, sizeof(int32_t) * n * k, cudaMemcpyDeviceToHost, s->stream);

@@ -732,6 +732,7 @@ cudaError_t launch_knn2_step(const Geometry& g, const Buffers& b, const StepPara
 // called where the first launch serves every particle
 bool knn2_direct(int64_t n, const StepParams& P);
 cudaError_t launch_knn2_finish(const Geometry& g, const Buffers& b, const StepParams& P, cudaStream_t st);
+// (uses the lists unless knn2_direct(n): the caller has them empty before and clears ovf_count after)
 cudaError_t launch_knn2_export(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out, cudaStream_t st,
                                const StepParams& P);
 // one-time kernel attributes for k neighbors (shared memory of the radius-first search)

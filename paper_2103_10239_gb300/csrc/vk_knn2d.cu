@@ -468,6 +468,12 @@ __device__ __noinline__ float box_radius_estimate(const Rep* __restrict__ rep, G
   const int ux0 = ucell2(p.x - a, nx, R.sh[0], Lx), ux1 = ucell2(p.x + a, nx, R.sh[0], Lx);
   const int uy0 = ucell2(p.y - a, ny, R.sh[1], Ly), uy1 = ucell2(p.y + a, ny, R.sh[1], Ly);
   if (ux1 - ux0 > kMaxCells || uy1 - uy0 > kMaxCells) return r;
+  if (ux0 >= 0 && ux1 < nx && uy1 - uy0 <= 1) {  // (the usual case: whole cells hold no more)
+    const int64_t c0 = R.c0 + (int64_t)(uy0 < 0 ? uy0 + ny : uy0) * nx, c1 = R.c0 + (int64_t)(uy1 >= ny ? uy1 - ny : uy1) * nx;
+    const uint32_t m0 = __ldg(G.off + c0 + ux1 + 1) - __ldg(G.off + c0 + ux0);
+    const uint32_t m1 = __ldg(G.off + c1 + ux1 + 1) - __ldg(G.off + c1 + ux0);
+    if (m0 + m1 <= (uint32_t)kMaxCand) return r;
+  }
   float n = 0.f;
   for (int uy = uy0; uy <= uy1; ++uy)
     for (int ux = ux0; ux <= ux1; ++ux) {
@@ -861,14 +867,13 @@ template <int KC, bool FOV>
 cudaError_t export2(const Geometry& g, const Buffers& b, int rep, int n, int32_t* out_ids, cudaStream_t st,
                     const StepParams& P) {
   if (n == 0) return cudaSuccess;
-  // the lists are empty between steps; the export clears what it used
+  // the lists are empty between steps; the caller clears what the export used
   const RowOut<KC> out{(const float2*)b.S_dir, b.S_id, out_ids, b.U_hint, P};
   if (knn2_direct(n, P)) return group_all<KC, FOV>(g, b, out, n, nullptr, rep, st);
   knn2_box_export_kernel<KC, FOV><<<(n + kBlk - 1) / kBlk, kBlk, sizeof(BoxShared<KC>), st>>>(
       g.reps, rep, (const int2*)b.S_pos, b.S_id, b.S_hint, view_of(b), out, b.ovf_list, b.ovf_count);
   finish_lists<KC, FOV>(g, b, out, n, st);
-  cudaError_t e = cudaMemsetAsync(b.ovf_count, 0, 2 * sizeof(int32_t), st);
-  return e == cudaSuccess ? cudaGetLastError() : e;
+  return cudaGetLastError();
 }
 
 template <int KC>
