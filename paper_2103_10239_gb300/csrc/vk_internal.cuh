@@ -615,13 +615,13 @@ inline void plan_grid2(Rep& R, double side) {
 }
 
 // Metric rule, 2D: may the rectangle of the particles of one coarse cell (at
-// most 2^sh + 2 r0q wide) reach half a period, or meet a coarse cell twice?  (It
-// meets at most one cell more than its width says, and one for the last cell of
-// the axis, which may be narrower.)
+// most 2^sh + 2 r0q wide) reach half a period, or meet a coarse cell twice?  (A last
+// cell much narrower than the others can still make one do so; that is left to
+// the kernel's fallback.)
 inline bool metric_wide(const Rep& R) {
   for (int a = 0; a < 2; ++a) {
     const int64_t w = (1ll << R.sh[a]) + 2 * (int64_t)R.r0q;
-    if (2 * w >= (int64_t)R.L[a] || (w >> R.sh[a]) + 2 >= R.nc[a]) return true;
+    if (2 * w >= (int64_t)R.L[a] || (w >> R.sh[a]) + 1 >= R.nc[a]) return true;
   }
   return false;
 }

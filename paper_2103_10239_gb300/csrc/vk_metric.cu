@@ -108,12 +108,12 @@ struct MetricStage {
 
 constexpr int kMetricBlk = 128;
 
-// WIDE: some rectangle of some replica may reach half a period or meet a coarse
-// cell twice (metric_wide).  The rectangle is then cut per axis, and minimum
-// images are taken one by one (20,000 particles, r0 a fifth and a quarter of the
-// box: 464 and 682 us per step; the whole box for such rectangles 2148 and 3424, one
-// thread per square 1179 and 1459).  The narrow kernel has no code for that: with
-// it, it loses 5 to 10 %.
+// WIDE: rectangles that reach half a period or meet a coarse cell twice are to be
+// expected (metric_wide).  Such a one is then cut per axis, and minimum images are
+// taken one by one (20,000 particles, r0 a fifth and a quarter of the box: 464 and 682
+// us per step; the whole replica for such rectangles 2148 and 3424, one thread per
+// square 1179 and 1459).  The narrow kernel takes the whole replica: with the other
+// code in it, it loses 5 to 10 %.
 template <bool WIDE>
 __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
     const Rep* __restrict__ reps, const BlockTask* __restrict__ tasks, const int2* __restrict__ S_pos,
@@ -151,28 +151,32 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
     const int32_t x0 = __reduce_min_sync(0xffffffffu, on ? p.x : INT_MAX), x1 = __reduce_max_sync(0xffffffffu, on ? p.x : -1);
     const int32_t y0 = __reduce_min_sync(0xffffffffu, on ? p.y : INT_MAX), y1 = __reduce_max_sync(0xffffffffu, on ? p.y : -1);
     // their rectangle.  Offsets within it are exact in one image while it is
-    // narrower than half a period; otherwise minimum images are taken one by
-    // one.  An axis that it covers, or on which it meets a coarse cell twice, is
-    // covered whole.
+    // narrower than half a period and meets no coarse cell twice.  Otherwise
+    // minimum images are taken one by one, of the whole replica, or (WIDE) of
+    // the axes that it covers or meets a cell twice on and its part of the others.
     const int64_t ax = x0 - r, bx = x1 + r, ay = y0 - r, by = y1 + r;
     const long long lim = on ? r2 : -1;  // squared distances are >= 0: the other lanes find nothing
-    bool fullx = WIDE && bx - ax + 1 >= Lx, fully = WIDE && by - ay + 1 >= Ly;
+    bool image = 2 * (bx - ax + 1) >= Lx || 2 * (by - ay + 1) >= Ly;
+    bool fullx = WIDE ? bx - ax + 1 >= Lx : image, fully = WIDE ? by - ay + 1 >= Ly : image;
     int ux0 = 0, ux1 = nx - 1, uy0 = 0, uy1 = ny - 1;
     if (!fullx) {
       ux0 = ucell2(ax, nx, shx, Lx);
       ux1 = ucell2(bx, nx, shx, Lx);
-      fullx = WIDE && ux1 - ux0 >= nx;
-      if (fullx) ux0 = 0, ux1 = nx - 1;
+      fullx = ux1 - ux0 >= nx;
     }
     if (!fully) {
       uy0 = ucell2(ay, ny, shy, Ly);
       uy1 = ucell2(by, ny, shy, Ly);
-      fully = WIDE && uy1 - uy0 >= ny;
+      fully = uy1 - uy0 >= ny;
+    }
+    image = image || fullx || fully;
+    if (WIDE) {
+      if (fullx) ux0 = 0, ux1 = nx - 1;
       if (fully) uy0 = 0, uy1 = ny - 1;
     }
-    const bool image = WIDE && (fullx || fully || 2 * (bx - ax + 1) >= Lx || 2 * (by - ay + 1) >= Ly);
-    // candidates [qb, qe); (ox, oy): the period added to their coordinates (unless `image`)
-    auto scan = [&](int64_t qb, int64_t qe, uint32_t ox, uint32_t oy) {
+    // candidates [qb, qe); (ox, oy): the period added to their coordinates, or
+    // (wrap) minimum images taken one by one
+    auto scan = [&](int64_t qb, int64_t qe, uint32_t ox, uint32_t oy, bool wrap) {
       n_cand += on ? (uint32_t)(qe - qb) : 0u;
       for (int64_t q0 = qb; q0 < qe; q0 += 32) {
         const int n = (int)min(qe - q0, (int64_t)32);
@@ -184,10 +188,13 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
           M.head[lane] = make_longlong2(phi_fixed(d.x), phi_fixed(d.y));
         }
         __syncwarp();
-        auto test = [&](int j, bool wrap) {
+        auto test = [&](int j, bool image_j) {
           const int2 pj = M.pos[j];
           int32_t dx = (int32_t)((uint32_t)pj.x - (uint32_t)p.x), dy = (int32_t)((uint32_t)pj.y - (uint32_t)p.y);
-          if (wrap) {  // a distance of half a period is the same in both images
+          if (image_j && !WIDE) {  // (seldom; short code for it costs the other loop registers)
+            dx = (int32_t)min_image((int64_t)pj.x - p.x, Lx);
+            dy = (int32_t)min_image((int64_t)pj.y - p.y, Ly);
+          } else if (image_j) {  // a distance of half a period is the same in both images
             dx = (uint32_t)abs(dx) > R.L[0] / 2 ? (int32_t)(R.L[0] - (uint32_t)abs(dx)) : dx;
             dy = (uint32_t)abs(dy) > R.L[1] / 2 ? (int32_t)(R.L[1] - (uint32_t)abs(dy)) : dy;
           }
@@ -198,7 +205,9 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
             ++S.m;
           }
         };
-        if (image) {
+        if (wrap && !WIDE) {
+          for (int j = 0; j < n; ++j) test(j, true);
+        } else if (wrap) {
 #pragma unroll 4
           for (int j = 0; j < n; ++j) test(j, true);
         } else {
@@ -207,10 +216,11 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
         }
       }
     };
-    if (fullx && fully) {
-      scan(R.p0, R.p0 + R.n, 0u, 0u);
+    if (WIDE ? fullx && fully : image) {
+      scan(R.p0, R.p0 + R.n, 0u, 0u, true);
       continue;
     }
+    const bool wrap = WIDE && image;
     const uint32_t fx0 = cell_frac((uint32_t)(ax < 0 ? ax + Lx : ax), shx);
     const uint32_t fx1 = cell_frac((uint32_t)(bx >= Lx ? bx - Lx : bx), shx);
     const uint32_t fy0 = cell_frac((uint32_t)(ay < 0 ? ay + Ly : ay), shy);
@@ -219,15 +229,16 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
       for (int ux = ux0; ux <= ux1; ++ux) {
         const int wy = uy < 0 ? uy + ny : (uy >= ny ? uy - ny : uy);
         const int wx = ux < 0 ? ux + nx : (ux >= nx ? ux - nx : ux);
-        const uint32_t ox = image ? 0u : ux < 0 ? 0u - R.L[0] : (ux >= nx ? R.L[0] : 0u);
-        const uint32_t oy = image ? 0u : uy < 0 ? 0u - R.L[1] : (uy >= ny ? R.L[1] : 0u);
+        const uint32_t ox = wrap ? 0u : ux < 0 ? 0u - R.L[0] : (ux >= nx ? R.L[0] : 0u);
+        const uint32_t oy = wrap ? 0u : uy < 0 ? 0u - R.L[1] : (uy >= ny ? R.L[1] : 0u);
         const int64_t gc = R.c0 + (int64_t)wy * nx + wx;
         const uint32_t base = __ldg(G.sub_base + gc);
         const int sd = __ldg(G.sub_s + gc);
-        const int c0 = ux == ux0 && !fullx ? sub_of(fx0, sd) : 0, c1 = ux == ux1 && !fullx ? sub_of(fx1, sd) : sd - 1;
-        const int r0 = uy == uy0 && !fully ? sub_of(fy0, sd) : 0, r1 = uy == uy1 && !fully ? sub_of(fy1, sd) : sd - 1;
+        const bool allx = WIDE && fullx, ally = WIDE && fully;
+        const int c0 = ux == ux0 && !allx ? sub_of(fx0, sd) : 0, c1 = ux == ux1 && !allx ? sub_of(fx1, sd) : sd - 1;
+        const int r0 = uy == uy0 && !ally ? sub_of(fy0, sd) : 0, r1 = uy == uy1 && !ally ? sub_of(fy1, sd) : sd - 1;
         if (c0 == 0 && c1 == sd - 1) {  // whole rows follow one another
-          scan(__ldg(G.sub_off + base + r0 * sd), __ldg(G.sub_off + base + (r1 + 1) * sd), ox, oy);
+          scan(__ldg(G.sub_off + base + r0 * sd), __ldg(G.sub_off + base + (r1 + 1) * sd), ox, oy, wrap);
           continue;
         }
         for (int rr = r0; rr <= r1; rr += 32) {
@@ -241,7 +252,7 @@ __global__ void __launch_bounds__(kMetricBlk) metric2_step_kernel(
           while (rows) {
             const int j = __ffs(rows) - 1;
             rows &= rows - 1u;
-            scan(__shfl_sync(0xffffffffu, qb, j), __shfl_sync(0xffffffffu, qe, j), ox, oy);
+            scan(__shfl_sync(0xffffffffu, qb, j), __shfl_sync(0xffffffffu, qe, j), ox, oy, wrap);
           }
         }
       }
