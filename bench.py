@@ -48,15 +48,14 @@ def parse():
     ap.add_argument("--cpu-seconds", type=float, default=12.0)
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--voronoi3-kernel", type=int, choices=[0, 1], default=None,
-                    help="voronoi3d scenario: 0 one thread per cell, 1 one warp per cell (default: the library's)")
+                    help="voronoi3d scenario: passed to the library, where 0 and 1 are the same kernel")
     ap.add_argument("--scenario-n", type=int, default=0,
                     help="particles of the voronoi3d / knn3d scenario (0: the workload's default)")
-    ap.add_argument("--occupancy", type=float, default=256.0,
-                    help="coarse-grid occupancy (particles per cell) of the headline run; 256 was the "
-                         "fastest of a sweep on the clustered 4M workload (steps 5-25 / 100-130, halo "
-                         "1.15: 128: 3.43/2.52, 256: 3.49/2.51, 512: 3.63/2.55 ms/step)")
+    ap.add_argument("--occupancy", type=float, default=64.0,
+                    help="coarse-grid occupancy (particles per cell) of the headline run; 64 is what the "
+                         "library takes for a flock of this size when it is left to it")
     ap.add_argument("--search", choices=["radius", "walk"], default="radius",
-                    help="2D kNN search: radius-first squares (default) or the per-particle walk only")
+                    help="2D kNN search: radius-first squares (default) or the general search of lane groups only")
     ap.add_argument("--halo", type=float, default=0.0,
                     help="radius-first search square half-width as a multiple of the previous k-th "
                          "distance (0: library default)")

@@ -26,9 +26,9 @@
 //
 // Measured (GB300, us per step, 64-bit list / 32-bit keys and power-of-two
 // cells): 4M clustered, k = 7, ten steps from a set state: first square 2372 /
-// 1175, listed particles 1232 / 594 (thirty steps on, with cells of 64 particles,
-// 905 and 332); 50,021 uniform, k = 16, vectorial noise: 178 / 35, 183 / 36.  2048
-// uniform: 45 + 48 / 26 + 26, and 27 by the groups alone.
+// 1175 (913 in cells of 64 particles, with the guess of first radii out of line), listed
+// particles 1232 / 594; 50,021 uniform, k = 16, vectorial noise: 178 / 34, 183 / 35.  2048
+// uniform: 45 + 48 / 26 + 26, and 25 by the groups alone.
 #include <algorithm>
 #include <climits>
 #include <type_traits>

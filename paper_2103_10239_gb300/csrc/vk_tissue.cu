@@ -23,8 +23,8 @@
 // The FP64 units are few (about 0.6 Tops/s): recomputing circumcenters, edge
 // lengths and quotients at every vertex took 780 FP64 operations per vertex and
 // cell; with the stored edges it is about 110.  Measured (GB300, 1M uniform
-// particles, ms, recomputed by one thread per cell / stored): cells 13.6 / 4.05,
-// forces 11.1 / 2.31, energy 3.1 / 0.03.  Packed rows in place of 32 entries per
+// particles, ms, recomputed by one thread per cell / stored): cells 13.6 / 3.74,
+// forces 11.1 / 2.32, energy 3.1 / 0.03.  Packed rows in place of 32 entries per
 // cell: 273 instead of 1185 bytes a particle, and 6.45 / 6.11 ms for all three.
 #include "vk_voronoi_fast.cuh"
 
