@@ -298,8 +298,9 @@ struct Group : GroupTop<GS, CAP> {
   // sub-cells that meet the square of half-width min(a, sqrt(tau)): a list
   // that has filled up on the way leaves little to scan.  Near cells and rows
   // go first: of a cluster that the square reaches from outside, met from its far
-  // side, every particle would be nearer than the last (65,536 particles around one
-  // point, k = 32: 7890 / 634 us for all lists, with kMaxCand below 1024).  True when the square is the whole box.
+  // side, every particle would be nearer than the last (all lists of 65,536 particles
+  // around one point, k = 32, before first radii looked at their cells: 7890 / 634 us).
+  // True when the square is the whole box.
   __device__ __forceinline__ bool square(const Rep& R, const GridView& G, int64_t a) {
     const int64_t Lx = C.Lx, Ly = C.Ly;
     const int nx = R.nc[0], ny = R.nc[1], shx = R.sh[0], shy = R.sh[1];
